@@ -17,6 +17,7 @@
 #include "simt_gemm.cuh"
 #include "umma_gemm.cuh"
 #include "tc_gemm.cuh"
+#include "quantize_block.cuh"
 
 using namespace gptaq;
 
@@ -103,8 +104,8 @@ struct WsLayout {
     size_t s_off[6];        // split operand matrices (n x n each): S1 hi/lo, S2 hi/lo, S3 hi/lo
     size_t pan_off[2];      // split copy of factor panels, hi/lo: n x 128 float32 (TF32) or n x SUPER_NB fp16
     // [-Err | Wpre]: float32 (m x 2B, or m x 2 * QSUPER * B for the FP16-split update), second part
-    // (TF32 remainder, or the fp16 hi / lo parts of the wide matrix), fp16 hi / lo of one block, row scales
-    size_t ew_off, ew_lo_off, ew16_off, rs_off, total;
+    // (TF32 remainder, or the fp16 hi / lo parts), row scales
+    size_t ew_off, ew_lo_off, rs_off, total;
     bool tensor;
 };
 
@@ -112,8 +113,8 @@ struct WsLayout {
 // the rank-128 update only touches the super-panel's remaining columns, the rest of the matrix receives
 // one rank-SUPER_NB update per super-panel (8x less read-modify-write traffic, longer contractions)
 constexpr int SUPER_NB = 8 * NB;
-// The lazy-batch update of gptaq_quantize likewise: QSUPER blocks form a super-block; a block's errors
-// are applied to the rest of its super-block at once and to everything beyond once per super-block.
+// The lazy-batch update of gptaq_quantize likewise: a launch of quant_block_kernel takes up to QSUPER blocks
+// (at most QB_SUPER columns), everything beyond them receives their errors at once.
 constexpr int QSUPER = 8;
 
 WsLayout ws_layout(int64_t n, int64_t m_max, int blocksize) {
@@ -137,9 +138,8 @@ WsLayout ws_layout(int64_t n, int64_t m_max, int blocksize) {
     const size_t ew = f16 ? QSUPER * ew1 : ew1;
     w.ew_off = off;
     w.ew_lo_off = off + ew;
-    w.ew16_off = off + (w.tensor ? 2 * ew : ew);
-    w.rs_off = w.ew16_off + (f16 ? ew1 : 0);
-    w.total = w.rs_off + (f16 ? round_up(2 * (size_t)m_max * sizeof(float), ALIGN) : 0);
+    w.rs_off = off + (w.tensor ? 2 * ew : ew);
+    w.total = w.rs_off + (f16 ? round_up((size_t)m_max * sizeof(float), ALIGN) : 0);
     return w;
 }
 
@@ -525,15 +525,11 @@ struct QuantizeTarget {
     const float *UT_hi, *UT_lo, *PT_hi, *PT_lo;
     float *EW_lo;
     // the same update with FP16-split operands (takes precedence when set): U^T and P^T as fp16 hi / lo
-    // (lo = hi + n * n), each with the scale of its recorded maximum, [-Err | Wpre] as fp16 hi / lo with
-    // one scale per row
+    // (lo = hi + n * n), each with the scale of its recorded maximum; EW is then m x 2 * SW wide (SW columns per
+    // launch), EW16 holds its fp16 hi / lo parts (lo = hi + m * 2 * SW) with one scale per row
     const __half *UT16 = nullptr, *PT16 = nullptr;
     __half *EW16 = nullptr;
     float *row_inv = nullptr;
-    // ... in super-blocks: EW is then m x 2 * QSUPER * B wide; EWS16 its fp16 hi / lo parts (lo = hi +
-    // m * 2 * QSUPER * B) with the row scales row_inv_s
-    __half *EWS16 = nullptr;
-    float *row_inv_s = nullptr;
     const unsigned *amax_u = nullptr, *amax_p = nullptr;
     int terms = GPTAQ_TERM_ERR | GPTAQ_TERM_ASYM;   // which terms of the weight update are applied
     const int *perm = nullptr;                      // act_order: working column c is the caller's column perm[c]
@@ -541,6 +537,53 @@ struct QuantizeTarget {
     const uint8_t *dead_orig = nullptr;             // static groups: dead-input flags in the caller's column order
     bool static_groups = false;
 };
+
+// One launch of quant_block_kernel: columns [i0, i1) of the loop, SW columns per launch at most.
+cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, int64_t m, int i0, int i1, int blocksize, int SW,
+                               int bits, int group, int sym, uint8_t *codes, float *scales, float *zeros, int G,
+                               bool static_groups, cudaStream_t s) {
+    const bool far_form = t.UT16 != nullptr;
+    const size_t nn = (size_t)t.n * t.n;
+    QuantBlockArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.W = W; a.ldw = ldw; a.m = (int)m; a.n = t.n; a.U = t.U; a.P = t.P; a.dead = t.dead;
+    a.i0 = i0; a.i1 = i1; a.bw = far_form ? QB_W : blocksize;
+    a.bits = bits; a.group = group; a.sym = sym;
+    a.codes = codes; a.scales = scales; a.zeros = zeros; a.G = G;
+    a.ew_ld = 2 * SW; a.ew_pre = SW;
+    if (i1 < t.n) {
+        a.EW = t.EW;
+        if (far_form) { a.EWS_hi = t.EW16; a.EWS_lo = t.EW16 + (size_t)m * 2 * SW; a.row_inv = t.row_inv; }
+        else a.EW_lo = t.EW_lo;
+    }
+    a.amax_u = t.amax_u; a.amax_p = t.amax_p; a.hd = t.hd;
+    a.err_scale = (t.terms & GPTAQ_TERM_ERR) ? 1.f : 0.f; a.asym_scale = (t.terms & GPTAQ_TERM_ASYM) ? 1.f : 0.f;
+    a.perm = t.perm; a.clip_steps = t.clip_steps; a.clip_min = t.clip_min;
+    CUtensorMap uh, ul, ph, pl;
+    std::memset(&uh, 0, sizeof(uh)); ul = ph = pl = uh;
+    if (far_form && (!make_f16_map(&uh, t.UT16, t.n, t.n, t.n, 128) || !make_f16_map(&ul, t.UT16 + nn, t.n, t.n, t.n, 128) ||
+                     !make_f16_map(&ph, t.PT16, t.n, t.n, t.n, 128) || !make_f16_map(&pl, t.PT16 + nn, t.n, t.n, t.n, 128)))
+        return cudaErrorUnknown;
+    const dim3 grid((unsigned)((m + QB_ROWS - 1) / QB_ROWS));
+    const size_t smem = quant_block_smem_bytes(far_form, static_groups);
+    if (far_form && static_groups) quant_block_kernel<true, true><<<grid, QB_THREADS_FAR, smem, s>>>(uh, ul, ph, pl, a);
+    else if (far_form) quant_block_kernel<true, false><<<grid, QB_THREADS_FAR, smem, s>>>(uh, ul, ph, pl, a);
+    else if (static_groups) quant_block_kernel<false, true><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
+    else quant_block_kernel<false, false><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
+    return cudaGetLastError();
+}
+
+// Raises the shared-memory limits of the kernels of the column loop.
+cudaError_t configure_quantize_kernels() {
+    const cudaFuncAttribute attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(column_loop_kernel<4>, attr, 2 * 128 * 128 * (int)sizeof(float));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(column_loop_kernel<2>, attr, 2 * 64 * 64 * (int)sizeof(float));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, true>, attr, (int)quant_block_smem_bytes(true, true));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, false>, attr, (int)quant_block_smem_bytes(true, false));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true>, attr, (int)quant_block_smem_bytes(false, true));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false>, attr, (int)quant_block_smem_bytes(false, false));
+    return e;
+}
 
 gptaq_status_t check_quantize_args(int64_t n, const void *d_W, int w_dtype, int64_t m, int64_t ldw, int bits,
                                    int group, int blocksize, const uint8_t *d_codes, const float *d_scales,
@@ -613,114 +656,73 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
         QLAUNCHED();
     }
 
-    int nw = (int)((m + t.num_sms - 1) / t.num_sms);
-    nw = std::max(1, std::min(32, nw));
-    const unsigned cl_grid = (unsigned)((m + nw - 1) / nw);
-    const int T = blocksize / 32;
-    // rows per CTA of the block kernel: enough CTAs for every SM, at most 128 rows each
-    const int cb_rows = 32 * std::max(1, std::min(4, (int)((m + 32 * (int64_t)t.num_sms - 1) / (32 * (int64_t)t.num_sms))));
-    const unsigned cb_grid = (unsigned)((m + cb_rows - 1) / cb_rows);
-    const size_t cl_smem = 2 * (size_t)blocksize * blocksize * sizeof(float);
-
-    const bool tensor16 = t.EW16 != nullptr;
+    // grids per output channel, per group of whole 32-column steps, or per column (static groups): quant_block_kernel.
+    // Smaller groups take column_loop_kernel (one warp per row, any group).
+    const bool steps = group <= 0 || (group % 32) == 0 || static_groups;
+    const bool tensor16 = t.UT16 != nullptr;
     const bool tensor = tensor16 || t.EW_lo != nullptr;
-    TcMaps maps, maps_super;
-    const int SBW = QSUPER * blocksize;           // super-block width (FP16-split update)
+    // columns per launch: as many blocks as the slab holds where the tensor cores carry the updates between them
+    // (the workspace holds the errors of QSUPER blocks), one block otherwise
+    const int SW = tensor16 && steps ? std::min(QB_SUPER, QSUPER * blocksize) : blocksize;
+    TcMaps maps;
     if (tensor16) {
-        const size_t nn = (size_t)n * n, me = (size_t)m * 2 * blocksize;
-        const SplitOperand A{t.EW16, t.EW16 + me, m, 2 * blocksize, 2 * blocksize, true};
-        const SplitOperand AS{t.EWS16, t.EWS16 + (size_t)m * 2 * SBW, m, 2 * SBW, 2 * SBW, true};
+        const size_t nn = (size_t)n * n, me = (size_t)m * 2 * SW;
+        const SplitOperand A{t.EW16, t.EW16 + me, m, 2 * SW, 2 * SW, true};
         const SplitOperand B{t.UT16, t.UT16 + nn, n, n, n, true}, B2{t.PT16, t.PT16 + nn, n, n, n, true};
-        if (!make_tc_maps(&maps, A, B, &B2) || !make_tc_maps(&maps_super, AS, B, &B2)) {
-            *err = cudaErrorUnknown;
-            return GPTAQ_ERR_CUDA;
-        }
+        if (!make_tc_maps(&maps, A, B, &B2)) { *err = cudaErrorUnknown; return GPTAQ_ERR_CUDA; }
     } else if (tensor) {
         const SplitOperand A{EW, t.EW_lo, m, 2 * blocksize, 2 * blocksize};
         const SplitOperand B{t.UT_hi, t.UT_lo, n, n, n}, B2{t.PT_hi, t.PT_lo, n, n, n};
         if (!make_tc_maps(&maps, A, B, &B2)) { *err = cudaErrorUnknown; return GPTAQ_ERR_CUDA; }
     }
-    for (int i0 = 0; i0 < n; i0 += blocksize) {
-        ColumnLoopArgs a;
-        a.W = Wk; a.ldw = ldk; a.m = (int)m; a.n = n; a.U = t.U; a.P = t.P; a.dead = t.dead;
-        a.i0 = i0; a.bw = std::min(blocksize, n - i0);
-        a.bits = bits; a.group = group; a.sym = sym;
-        a.codes = d_codes; a.scales = d_scales; a.zeros = d_zeros; a.G = G; a.EW = EW; a.EW_lo = tensor16 ? nullptr : t.EW_lo; a.hd = t.hd;
-        a.ew_ld = 2 * blocksize; a.ew_pre = blocksize;
-        a.EW16_hi = tensor16 ? t.EW16 : nullptr; a.EW16_lo = tensor16 ? t.EW16 + (size_t)m * 2 * blocksize : nullptr;
-        a.row_inv = t.row_inv; a.amax_u = t.amax_u; a.amax_p = t.amax_p;
-        a.perm = t.perm; a.clip_steps = t.clip_steps; a.clip_min = t.clip_min; a.err_scale = (t.terms & GPTAQ_TERM_ERR) ? 1.f : 0.f; a.asym_scale = (t.terms & GPTAQ_TERM_ASYM) ? 1.f : 0.f;
-        a.static_groups = static_groups ? 1 : 0;
-        // (every full block of one call takes the same kernel: the conditions do not depend on the block)
-        const bool fast = a.bw == blocksize && (group <= 0 || (group % 32) == 0) && (i0 % 4) == 0 &&
-                          (reinterpret_cast<uintptr_t>(t.dead) & 3) == 0 && !static_groups;
-        const int sb0 = i0 / SBW * SBW, sb_end = std::min(sb0 + SBW, n);
-        if (fast && tensor16) {
-            // this block's columns of the super-block's [-Err | Wpre]
-            a.EW = EW + (i0 - sb0); a.ew_ld = 2 * SBW; a.ew_pre = SBW;
-        }
-        if (fast) {
-            const int lanes = column_block_lanes(cb_rows);
-            if (lanes == 4) column_block_kernel<4><<<cb_grid, CB_THREADS, column_block_smem(cb_rows), s>>>(a, cb_rows, blocksize);
-            else if (lanes == 2) column_block_kernel<2><<<cb_grid, CB_THREADS, column_block_smem(cb_rows), s>>>(a, cb_rows, blocksize);
-            else column_block_kernel<1><<<cb_grid, CB_THREADS, column_block_smem(cb_rows), s>>>(a, cb_rows, blocksize);
-        }
-        else if (T == 4) column_loop_kernel<4><<<cl_grid, nw * 32, cl_smem, s>>>(a);
-        else if (T == 2) column_loop_kernel<2><<<cl_grid, nw * 32, cl_smem, s>>>(a);
-        else column_loop_kernel<1><<<cl_grid, nw * 32, cl_smem, s>>>(a);
-        QLAUNCHED();
-        const int i2 = i0 + blocksize;
-        if (tensor16 && !fast) {
-            // grids per group of fewer than 32 columns: every full block takes column_loop_kernel, which
-            // leaves [-Err | rho Wpre] in float32; scaled row by row and split here, then applied to all
-            // columns to the right (the ragged last block has none)
-            if (i2 < n) {
-                rowscale_split16_kernel<<<(unsigned)((m + 7) / 8), 256, 0, s>>>(EW, 2 * blocksize, (int)m, 2 * blocksize, t.EW16,
-                                                                              t.EW16 + (size_t)m * 2 * blocksize, t.row_inv);
+    for (int i0 = 0; i0 < n; i0 += SW) {
+        const int i1 = std::min(i0 + SW, n);
+        if (steps) {
+            *err = launch_quant_block(t, Wk, ldk, m, i0, i1, blocksize, SW, bits, group, sym, d_codes, d_scales, d_zeros, G,
+                                      static_groups, s);
+            if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
+            ++*launches;
+        } else {
+            ColumnLoopArgs a;
+            a.W = Wk; a.ldw = ldk; a.m = (int)m; a.n = n; a.U = t.U; a.P = t.P; a.dead = t.dead;
+            a.i0 = i0; a.bw = i1 - i0;
+            a.bits = bits; a.group = group; a.sym = sym;
+            a.codes = d_codes; a.scales = d_scales; a.zeros = d_zeros; a.G = G; a.EW = EW; a.EW_lo = tensor16 ? nullptr : t.EW_lo; a.hd = t.hd;
+            a.amax_u = t.amax_u; a.amax_p = t.amax_p;
+            a.perm = t.perm; a.clip_steps = t.clip_steps; a.clip_min = t.clip_min;
+            a.err_scale = (t.terms & GPTAQ_TERM_ERR) ? 1.f : 0.f; a.asym_scale = (t.terms & GPTAQ_TERM_ASYM) ? 1.f : 0.f;
+            const int nw = std::max(1, std::min(32, (int)((m + t.num_sms - 1) / t.num_sms)));
+            const unsigned cl_grid = (unsigned)((m + nw - 1) / nw);
+            const size_t cl_smem = 2 * (size_t)blocksize * blocksize * sizeof(float);
+            const int T = blocksize / 32;
+            if (T == 4) column_loop_kernel<4><<<cl_grid, nw * 32, cl_smem, s>>>(a);
+            else if (T == 2) column_loop_kernel<2><<<cl_grid, nw * 32, cl_smem, s>>>(a);
+            else column_loop_kernel<1><<<cl_grid, nw * 32, cl_smem, s>>>(a);
+            QLAUNCHED();
+            if (tensor16 && i1 < n) {
+                // [-Err | rho Wpre] scaled row by row and split here (quant_block_kernel does so itself)
+                rowscale_split16_kernel<<<(unsigned)((m + 7) / 8), 256, 0, s>>>(EW, 2 * SW, (int)m, 2 * SW, t.EW16,
+                                                                              t.EW16 + (size_t)m * 2 * SW, t.row_inv);
                 QLAUNCHED();
-                TcGemmArgs g = tc_args(Wk + i2, ldk, (int)m, n - i2, 2 * blocksize, 1.f, 1.f, TC_FULL, TC_MASK_NONE, t.hd);
-                g.b_row0 = i2; g.b_k0 = i0; g.k_split = blocksize; g.b2_k0 = i0;
-                g.row_inv = t.row_inv; g.amax_b = t.amax_u;
-                *err = launch_tc_gemm(maps, g, *t.sched, t.num_sms, s, false);
-                if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
-                ++*launches;
             }
-        } else if (tensor16) {
-            if (i2 < sb_end) {
-                // rest of the super-block: W[:, i2:sb_end] += [-Err | Wpre] * [U[blk, i2:sb_end] ; P[blk, i2:sb_end]]
-                TcGemmArgs g = tc_args(Wk + i2, ldk, (int)m, sb_end - i2, 2 * blocksize, 1.f, 1.f, TC_FULL, TC_MASK_NONE, t.hd);
-                g.b_row0 = i2; g.b_k0 = i0; g.k_split = blocksize; g.b2_k0 = i0;
-                g.row_inv = t.row_inv; g.amax_b = t.amax_u;
-                *err = launch_tc_gemm(maps, g, *t.sched, t.num_sms, s, false);
-                if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
-                ++*launches;
-            } else if (i2 == sb_end && sb_end < n) {
-                // super-block done: everything to its right receives all of its errors at once
-                rowscale_split16_kernel<<<(unsigned)((m + 7) / 8), 256, 0, s>>>(EW, 2 * SBW, (int)m, 2 * SBW, t.EWS16,
-                                                                              t.EWS16 + (size_t)m * 2 * SBW, t.row_inv_s);
-                QLAUNCHED();
-                TcGemmArgs g = tc_args(Wk + sb_end, ldk, (int)m, n - sb_end, 2 * SBW, 1.f, 1.f, TC_FULL, TC_MASK_NONE, t.hd);
-                g.b_row0 = sb_end; g.b_k0 = sb0; g.k_split = SBW; g.b2_k0 = sb0;
-                g.row_inv = t.row_inv_s; g.amax_b = t.amax_u;
-                *err = launch_tc_gemm(maps_super, g, *t.sched, t.num_sms, s, false);
-                if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
-                ++*launches;
-            }
-        } else if (i2 < n && tensor) {
-            // W[:, i2:] += [-Err | Wpre] * [U[blk, i2:] ; P[blk, i2:]] on the tensor cores: B operand rows
-            // are rows i2.. of U^T (first B contraction steps) and of P^T (the next B)
-            TcGemmArgs g = tc_args(Wk + i2, ldk, (int)m, n - i2, 2 * blocksize, 1.f, 1.f, TC_FULL, TC_MASK_NONE, t.hd);
-            g.b_row0 = i2; g.b_k0 = i0; g.k_split = blocksize; g.b2_k0 = i0;
+        }
+        if (i1 >= n) break;
+        if (tensor) {
+            // W[:, i1:] += [-Err | Wpre] * [U[blk, i1:] ; P[blk, i1:]] on the tensor cores: B operand rows
+            // are rows i1.. of U^T (first SW contraction steps) and of P^T (the next SW)
+            TcGemmArgs g = tc_args(Wk + i1, ldk, (int)m, n - i1, 2 * SW, 1.f, 1.f, TC_FULL, TC_MASK_NONE, t.hd);
+            g.b_row0 = i1; g.b_k0 = i0; g.k_split = SW; g.b2_k0 = i0;
+            if (tensor16) { g.row_inv = t.row_inv; g.amax_b = t.amax_u; }
             *err = launch_tc_gemm(maps, g, *t.sched, t.num_sms, s, false);
             if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
             ++*launches;
-        } else if (i2 < n) {
-            // W[:, i2:] += [-Err | Wpre] * [U[blk, i2:] ; P[blk, i2:]]   (lazy-batch update)
-            Operand bop = make_operand(t.U + (int64_t)i0 * n + i2, 1, n);
-            bop.p2 = t.P + (int64_t)i0 * n + i2;
+        } else {
+            // W[:, i1:] += [-Err | Wpre] * [U[blk, i1:] ; P[blk, i1:]]   (lazy-batch update)
+            Operand bop = make_operand(t.U + (int64_t)i0 * n + i1, 1, n);
+            bop.p2 = t.P + (int64_t)i0 * n + i1;
             bop.k_split = blocksize;
-            GemmProblem pt = make_problem(make_operand(EW, 2 * blocksize, 1), bop, Wk + i2, ldk,
-                                          (int)m, n - i2, 2 * blocksize, 1.f, 1.f, GEMM_FULL);
+            GemmProblem pt = make_problem(make_operand(EW, 2 * blocksize, 1), bop, Wk + i1, ldk,
+                                          (int)m, n - i1, 2 * blocksize, 1.f, 1.f, GEMM_FULL);
             *err = launch_simt_gemm(pt, false, true, s);
             if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
             ++*launches;
@@ -778,17 +780,7 @@ cudaError_t static_scratch_for_current_device(StaticScratch **out) {
         if (e != cudaSuccess) return e;
         e = cudaDeviceGetAttribute(&sc.num_sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(column_loop_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 2 * 128 * 128 * (int)sizeof(float));
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(column_loop_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 2 * 64 * 64 * (int)sizeof(float));
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(column_block_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)column_block_smem(128));
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(column_block_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)column_block_smem(128));
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(column_block_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)column_block_smem(128));
+        e = configure_quantize_kernels();
         if (e != cudaSuccess) return e;
         sc.base = static_cast<uint8_t *>(ptr);
         sc.ready = true;
@@ -851,9 +843,7 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(factor_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FP_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(column_loop_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 2 * 128 * 128 * (int)sizeof(float));
+    if (e == cudaSuccess) e = configure_quantize_kernels();
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(invert_diag_blocks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ID_SMEM);
     if (e == cudaSuccess)
@@ -870,15 +860,6 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
         e = cudaFuncSetAttribute(convert_transpose_kernel<0>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(convert_transpose_kernel<1>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(column_loop_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 2 * 64 * 64 * (int)sizeof(float));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(column_block_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)column_block_smem(128));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(column_block_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)column_block_smem(128));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(column_block_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)column_block_smem(128));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(unpermute_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ACT_ORDER_MAX_N * 4);
     if (e != cudaSuccess) {
@@ -1324,16 +1305,14 @@ gptaq_status_t gptaq_quantize(gptaq_handle_t h, void *d_W, int w_dtype, int64_t 
     t.clip_steps = h->clip_steps; t.clip_min = h->clip_min;
     t.static_groups = h->static_groups; t.dead_orig = h->dead_raw;
     t.UT_hi = t.UT_lo = t.PT_hi = t.PT_lo = nullptr; t.EW_lo = nullptr;
-    // FP16-split trailing update where a block is a whole number of 64-step K-blocks; TF32-split for
-    // widths that are multiples of 4 only; plain float32 products otherwise (blocks of 32 columns)
-    const bool f16 = h->f16 && (blocksize % 64) == 0;
+    // FP16-split updates; TF32-split for widths that are multiples of 4 only; plain float32 products otherwise.
+    // (Groups of fewer than 32 columns update block by block, and blocks of 32 columns are no whole K-block of 64.)
+    const bool f16 = h->f16 && ((blocksize % 64) == 0 || group <= 0 || (group % 32) == 0 || h->static_groups);
     if (f16) {
         t.UT16 = reinterpret_cast<const __half *>(h->ws + wl.s_off[0]);
         t.PT16 = reinterpret_cast<const __half *>(h->ws + wl.s_off[1]);
-        t.EWS16 = reinterpret_cast<__half *>(h->ws + wl.ew_lo_off);
-        t.EW16 = reinterpret_cast<__half *>(h->ws + wl.ew16_off);
+        t.EW16 = reinterpret_cast<__half *>(h->ws + wl.ew_lo_off);
         t.row_inv = reinterpret_cast<float *>(h->ws + wl.rs_off);
-        t.row_inv_s = t.row_inv + m;
         t.amax_u = h->hd->tc_amax + AMAX_U; t.amax_p = h->hd->tc_amax + AMAX_P;
     } else if (h->tensor && !h->f16) {
         float *S[6];

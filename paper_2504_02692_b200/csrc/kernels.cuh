@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(256) static_group_grid_kernel(const T *W, int6
 
 // ---------------------------------------------------------------------------
 // Column loop over one lazy-batch block [i0, i0 + bw) (Algorithm 1, inner
-// loop).  One warp per weight row; the row's block lives in registers (lane
+// loop), for grids per group of fewer than 32 columns (quant_block_kernel takes all others).  One warp per weight row; the row's block lives in registers (lane
 // owns columns lane, lane + 32, ...), the B x B diagonal tiles of U and P live
 // in shared memory.  Outputs: codes, dequantized columns (in place in W),
 // -Err and the pre-quantization columns (for the trailing update), group grids.
@@ -746,22 +746,14 @@ struct ColumnLoopArgs {
     float *scales, *zeros;     // m x G
     int G;
     float *EW;                 // m x (2 * 32 * T): [-Err | Wpre]
-    int ew_ld, ew_pre;         // column_block_kernel: row pitch of EW / EW_lo and the offset of Wpre in a row (2B and B
-                               //   for the layout above; a block's slice of a wider [-Err | Wpre] otherwise)
     float *EW_lo;              // nullptr, or: EW receives the TF32 value of each entry and EW_lo the remainder
-    // FP16 operand for the tensor-core update (column_block_kernel only; EW_lo is null then), or nullptr:
-    // row i of [-Err | rho * Wpre] times a power of two s_i, as fp16 hi / lo parts, m x (2 * block) each;
-    // row_inv[i] = 1 / s_i.  rho = scale of U^T / scale of P^T (from the two recorded maxima) lets the two
-    // halves of the B operand keep scales of their own.
-    __half *EW16_hi, *EW16_lo;
-    float *row_inv;
+    // fp16-split handles (else nullptr): Wpre is stored times rho = scale of U^T / scale of P^T (from the two recorded
+    // maxima), which lets the two halves of the update's B operand keep scales of their own
     const unsigned *amax_u, *amax_p;
     StateHeader *hd;
     float err_scale, asym_scale;   // 1 or 0: switches of the two terms of the weight update (ablation)
     const int *perm;               // nullptr, or: working column c is original column perm[c] (codes go there)
     int clip_steps; float clip_min; // clipping-range search of the group grids (0: plain min/max)
-    int static_groups;             // column_loop_kernel: scales / zeros hold ready grids per group of ORIGINAL columns
-                                   //   (static_group_grid_kernel); column c uses group (perm ? perm[c] : c) / group
 };
 
 template <int T>
@@ -811,11 +803,7 @@ __global__ void __launch_bounds__(1024) column_loop_kernel(ColumnLoopArgs a) {
         for (int jj = 0; jj < 32; ++jj) {
             const int j = t * 32 + jj;
             if (j >= bw) break;
-            if (a.static_groups) {
-                const int cj = a.perm ? a.perm[i0 + j] : i0 + j;
-                scale = a.scales[(int64_t)row * a.G + cj / a.group];
-                zero = a.zeros[(int64_t)row * a.G + cj / a.group];
-            } else if (a.group > 0 && ((i0 + j) % a.group) == 0) {
+            if (a.group > 0 && ((i0 + j) % a.group) == 0) {
                 // grid of the group that starts here, from the current values
                 const int gend = min(j + a.group, bw);
                 float lo = 0.f, hi = 0.f, am = 0.f;
@@ -872,10 +860,8 @@ __global__ void __launch_bounds__(1024) column_loop_kernel(ColumnLoopArgs a) {
     }
 
     bool bad = false;
-    // fp16-split handles (row_inv set): Wpre is stored times rho = scale of U^T / scale of P^T, like
-    // column_block_kernel does, so that the two halves of the update's B operand keep scales of their own
     float rho = 1.f;
-    if (a.row_inv) {
+    if (a.amax_u) {
         const float ap = __uint_as_float(*a.amax_p);
         rho = ap > 0.f ? split_scale(__uint_as_float(*a.amax_u)) / split_scale(ap) : 0.f;
     }
@@ -901,408 +887,6 @@ __global__ void __launch_bounds__(1024) column_loop_kernel(ColumnLoopArgs a) {
         }
     }
     if (bad) record_status(a.hd, ST_NONFINITE, row);
-}
-
-// ---------------------------------------------------------------------------
-// Column loop over one full lazy-batch block [i0, i0 + B), B in {32, 64, 128}, for grids per
-// output channel or per group of a multiple of 32 columns.  One CTA owns `rows` weight rows
-// (a multiple of 32); their block lives in shared memory.  The block is processed 32 columns
-// at a time:
-//   - LANES threads per row (4 for 32 rows per CTA, 2 for 64, 1 beyond) take the 32 columns into
-//     registers, 32 / LANES consecutive columns each, and run the sequential part (quantize column
-//     k, scaled error, rank-1 update of the later columns of the 32): the lane that holds column k
-//     quantizes it and passes the scaled error and the pre-quantization value to the row's other
-//     lanes by shuffles, every lane updates its own later columns from the rows k of U and P in
-//     shared memory.  The dependent chain of a column is then the quantizer plus one update, not
-//     the up to 31 updates of one thread (154 cycles per column with one thread per row);
-//   - all threads then apply the 32 columns' errors and pre-quantization values to the rest
-//     of the block, a (rows x 64) x (64 x rest) product out of shared memory.
-// Same outputs as column_loop_kernel.
-// ---------------------------------------------------------------------------
-constexpr int CB_THREADS = 256;
-constexpr int CB_LD = 128 + 4;
-
-__host__ __device__ inline size_t column_block_smem(int rows) {
-    // the block, two buffers of 32 rows of U and P, [-Err | Wpre] of 32 columns transposed, two sets of 32
-    // reciprocal pivots, and per row: the chosen clipping candidate and the largest operand magnitude
-    return ((size_t)rows * CB_LD + 2 * 2 * 32 * CB_LD + 64 * (rows + 4) + 2 * 32 + 2 * rows) * sizeof(float);
-}
-__host__ __device__ inline int column_block_lanes(int rows) { return rows <= 32 ? 4 : (rows <= 64 ? 2 : 1); }
-
-// Round to nearest, ties to even, for a value that is clamped to [0, 255] afterwards: adding and
-// subtracting 1.5 * 2^23 rounds exactly like rintf wherever |v| < 2^22 and leaves larger values large
-// (the clamp decides those), in two additions instead of a trip through the conversion unit, which
-// was 30 of the 154 cycles of a column step.
-__device__ __forceinline__ float round_for_clamp(float v) {
-    const float magic = 12582912.f;
-    return __fsub_rn(__fadd_rn(v, magic), magic);
-}
-
-// Step K of the sequential part for one row held by LANES lanes (lane `sub` of the row holds columns
-// sub * CPL .. + CPL - 1 of the 32 in x).  The arithmetic of every column is that of a single thread per
-// row: the results do not depend on LANES.
-template <int LANES, int K>
-struct QuantStep {
-    static constexpr int CPL = 32 / LANES;
-    static __device__ __forceinline__ void run(float (&x)[CPL], float (&nerr)[CPL], float (&pre)[CPL], uint32_t (&code)[CPL / 4],
-                                               int sub, const float *Us, const float *Ps, const float *udinv,
-                                               float scale, float inv_scale, float zero, float maxq, float err_scale,
-                                               float asym_scale) {
-        constexpr int OWNER = K / CPL, KK = K % CPL;
-        // Straight-line code for all lanes (no divergent branches, so that the loads of U and P for the next
-        // steps can move ahead of this step's arithmetic): every lane quantizes its own column KK, the owner's
-        // result is the one that is kept and passed on.
-        const bool own = LANES == 1 || sub == OWNER;
-        const float w0 = x[KK];
-        // w / scale as w * (1 / scale): one rounding more (about 1e-7 of a step, far inside the tie band)
-        // for a much shorter dependent chain
-        const float cq = fminf(fmaxf(round_for_clamp(w0 * inv_scale) + zero, 0.f), maxq);
-        const float q = scale * (cq - zero);
-        float ne = err_scale * ((q - w0) * udinv[K]);           // -(w - q) / U_kk
-        float w = asym_scale * w0;
-        if (own) { x[KK] = q; nerr[KK] = ne; pre[KK] = w; code[KK >> 2] |= (uint32_t)cq << (8 * (KK & 3)); }
-        if (LANES > 1) {
-            ne = __shfl_sync(0xffffffffu, ne, OWNER, LANES);
-            w = __shfl_sync(0xffffffffu, w, OWNER, LANES);
-        }
-        // this lane's columns beyond K
-        const float *ur = Us + K * CB_LD + sub * CPL, *pr = Ps + K * CB_LD + sub * CPL;
-#pragma unroll
-        for (int j4 = 0; j4 < CPL / 4; ++j4) {
-            // (compile-time skip of the quads that no lane needs any more)
-            if ((LANES - 1) * CPL + 4 * j4 + 3 <= K) continue;
-            const float4 u = *reinterpret_cast<const float4 *>(ur + 4 * j4);
-            const float4 p = *reinterpret_cast<const float4 *>(pr + 4 * j4);
-            const int c0 = sub * CPL + 4 * j4;
-            const float y0 = fmaf(w, p.x, fmaf(ne, u.x, x[4 * j4 + 0]));
-            const float y1 = fmaf(w, p.y, fmaf(ne, u.y, x[4 * j4 + 1]));
-            const float y2 = fmaf(w, p.z, fmaf(ne, u.z, x[4 * j4 + 2]));
-            const float y3 = fmaf(w, p.w, fmaf(ne, u.w, x[4 * j4 + 3]));
-            x[4 * j4 + 0] = c0 + 0 > K ? y0 : x[4 * j4 + 0];
-            x[4 * j4 + 1] = c0 + 1 > K ? y1 : x[4 * j4 + 1];
-            x[4 * j4 + 2] = c0 + 2 > K ? y2 : x[4 * j4 + 2];
-            x[4 * j4 + 3] = c0 + 3 > K ? y3 : x[4 * j4 + 3];
-        }
-        QuantStep<LANES, K + 1>::run(x, nerr, pre, code, sub, Us, Ps, udinv, scale, inv_scale, zero, maxq, err_scale, asym_scale);
-    }
-};
-template <int LANES>
-struct QuantStep<LANES, 32> {
-    static constexpr int CPL = 32 / LANES;
-    static __device__ __forceinline__ void run(float (&)[CPL], float (&)[CPL], float (&)[CPL], uint32_t (&)[CPL / 4], int,
-                                               const float *, const float *, const float *, float, float, float, float, float, float) {}
-};
-
-template <int LANES>
-__global__ void __launch_bounds__(CB_THREADS, 1) column_block_kernel(ColumnLoopArgs a, int rows, int B) {
-    extern __shared__ __align__(16) float smem_f[];
-    float (*Wt)[CB_LD] = reinterpret_cast<float (*)[CB_LD]>(smem_f);                       // [rows][B]
-    // rows o..o+31 of U and of P (block columns), two buffers: the next 32 rows are fetched while the
-    // current 32 columns are quantized
-    float (*UP)[CB_LD] = reinterpret_cast<float (*)[CB_LD]>(smem_f + rows * CB_LD);        // [2 buffers][U, P][32]
-    float *St = smem_f + rows * CB_LD + 2 * 2 * 32 * CB_LD;                                // [64][rows + 4]: -Err, then Wpre
-    const int sld = rows + 4;
-    float *udinv2 = St + 64 * sld;                                                         // [2][32]
-    int *bsel = reinterpret_cast<int *>(udinv2 + 2 * 32);                                  // [rows]: chosen clipping candidate
-    float *rmax_s = reinterpret_cast<float *>(bsel + rows);                                // [rows]: largest |operand| of the row
-    const int tid = threadIdx.x;
-    const int n = a.n, i0 = a.i0;
-    const int row0 = blockIdx.x * rows;
-    const int nrows = min(rows, a.m - row0);
-    const int bq = B / 4;
-    // sequential part: thread tid < rows * LANES holds columns sub * CPL .. of row lrow (whole warps take part,
-    // rows beyond the matrix run on zeros and store nothing)
-    constexpr int CPL = 32 / LANES;
-    const int lrow = tid / LANES, sub = tid % LANES;
-    const bool chain = tid < rows * LANES;
-
-    // the block of W (dead inputs read as zero), along rows; four loads in flight per thread
-    for (int base = 0; base < rows * bq; base += 4 * CB_THREADS) {
-        float4 v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int idx = base + u * CB_THREADS + tid;
-            const int r = idx / bq, c4 = idx - r * bq;
-            v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (idx < rows * bq && r < nrows) {
-                const float *src = a.W + (int64_t)(row0 + r) * a.ldw + i0 + 4 * c4;
-                if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) v[u] = *reinterpret_cast<const float4 *>(src);
-                else { v[u].x = src[0]; v[u].y = src[1]; v[u].z = src[2]; v[u].w = src[3]; }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int idx = base + u * CB_THREADS + tid;
-            if (idx >= rows * bq) continue;
-            const int r = idx / bq, c4 = idx - r * bq;
-            const uchar4 dd = *reinterpret_cast<const uchar4 *>(a.dead + i0 + 4 * c4);
-            if (dd.x) v[u].x = 0.f;
-            if (dd.y) v[u].y = 0.f;
-            if (dd.z) v[u].z = 0.f;
-            if (dd.w) v[u].w = 0.f;
-            // a non-finite weight is reported from the value that was read: its code and dequantized value
-            // come out finite (the clamp absorbs NaN and Inf), so the results alone would not show it
-            if (r < nrows && (!isfinite(v[u].x) || !isfinite(v[u].y) || !isfinite(v[u].z) || !isfinite(v[u].w)))
-                record_status(a.hd, ST_NONFINITE, row0 + r);
-            *reinterpret_cast<float4 *>(&Wt[r][4 * c4]) = v[u];
-        }
-    }
-
-    const float maxq = (float)((1 << a.bits) - 1);
-    float scale = 1.f, zero = 0.f;
-    const bool owner = chain && lrow < nrows;
-    const int row = row0 + lrow;
-    if (a.group <= 0 && owner) { scale = a.scales[row]; zero = a.zeros[row]; }
-    const bool f16 = a.EW16_hi != nullptr;
-    float rho = 1.f, rmax = 0.f;
-    if (f16) {
-        const float ap = __uint_as_float(*a.amax_p);
-        rho = ap > 0.f ? split_scale(__uint_as_float(*a.amax_u)) / split_scale(ap) : 0.f;
-    }
-
-    // rows [o, o + 32) of U and P of this block into buffer `buf`, by `nthr` threads starting at `t0`
-    auto fetch_up = [&](int o, int buf, int t0, int nthr) {
-        float (*Ub)[CB_LD] = UP + buf * 64;
-        float (*Pb)[CB_LD] = Ub + 32;
-        const int t = tid - t0;
-        for (int idx = t; idx < 32 * bq; idx += nthr) {
-            const int k = idx / bq, c4 = idx - k * bq;
-            const int64_t off = (int64_t)(i0 + o + k) * n + i0 + 4 * c4;
-            float4 u, p;
-            if ((n & 3) == 0) {
-                u = *reinterpret_cast<const float4 *>(a.U + off);
-                p = *reinterpret_cast<const float4 *>(a.P + off);
-            } else {
-                u = make_float4(a.U[off], a.U[off + 1], a.U[off + 2], a.U[off + 3]);
-                p = make_float4(a.P[off], a.P[off + 1], a.P[off + 2], a.P[off + 3]);
-            }
-            *reinterpret_cast<float4 *>(&Ub[k][4 * c4]) = u;
-            *reinterpret_cast<float4 *>(&Pb[k][4 * c4]) = p;
-        }
-        if (t < 32) udinv2[buf * 32 + t] = 1.f / a.U[(int64_t)(i0 + o + t) * n + i0 + o + t];
-    };
-    fetch_up(0, 0, 0, CB_THREADS);
-
-    for (int o = 0; o < B; o += 32) {
-        const int buf = (o >> 5) & 1;
-        float (*Us)[CB_LD] = UP + buf * 64;
-        float (*Ps)[CB_LD] = Us + 32;
-        const float *udinv = udinv2 + buf * 32;
-        __syncthreads();        // the block is current; this buffer of U / P is loaded; St and the other buffer are free
-        const bool group_start = a.group > 0 && ((i0 + o) % a.group) == 0;
-        int best_k = 0;
-        if (group_start && a.clip_steps > 0) {
-            // clipping-range search, all threads: thread = (row, share of the candidates); the shares'
-            // best (error, candidate) pairs meet in St, which is free until the columns are quantized
-            const int ncg = CB_THREADS / rows;
-            const int r = tid % rows, cgi = tid / rows;
-            float *berr = St;
-            int *bk = reinterpret_cast<int *>(St + CB_THREADS);
-            if (cgi < ncg) {
-                float lo = 0.f, hi = 0.f, am = 0.f;
-                const int gend = min(o + a.group, B);
-                for (int c = o; c < gend; ++c) {
-                    const float v = Wt[r][c];
-                    lo = fminf(lo, v); hi = fmaxf(hi, v); am = fmaxf(am, fabsf(v));
-                }
-                float best = INFINITY;
-                int kb = 0;
-                for (int k = cgi; k < a.clip_steps; k += ncg) {
-                    const float p = clip_ratio(k, a.clip_steps, a.clip_min);
-                    float sk, zk;
-                    make_grid(p * lo, p * hi, p * am, a.bits, a.sym, sk, zk);
-                    float err = 0.f;
-                    for (int c = o; c < gend; ++c) err += rounding_error_sq(Wt[r][c], sk, zk, maxq);
-                    if (err < best) { best = err; kb = k; }
-                }
-                berr[cgi * rows + r] = best;
-                bk[cgi * rows + r] = kb;
-            }
-            __syncthreads();
-            if (tid < rows) {
-                float best = INFINITY;
-                int kbest = 0;
-                for (int c = 0; c < ncg; ++c) {
-                    const float e = berr[c * rows + tid];
-                    const int k = bk[c * rows + tid];
-                    if (e < best || (e == best && k < kbest)) { best = e; kbest = k; }
-                }
-                bsel[tid] = kbest;
-            }
-            __syncthreads();
-            if (chain) best_k = bsel[lrow];
-        }
-        if (tid >= CB_THREADS / 2 && o + 32 < B) fetch_up(o + 32, buf ^ 1, CB_THREADS / 2, CB_THREADS / 2);
-        if (chain) {
-            if (group_start) {
-                // grid of the group that starts here, from the current values (the row's lanes share the scan)
-                float lo = 0.f, hi = 0.f, am = 0.f;
-                const int gend = min(o + a.group, B);
-                for (int c = o + sub; c < gend; c += LANES) {
-                    const float v = Wt[lrow][c];
-                    lo = fminf(lo, v); hi = fmaxf(hi, v); am = fmaxf(am, fabsf(v));
-                }
-#pragma unroll
-                for (int d = 1; d < LANES; d <<= 1) {
-                    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, d));
-                    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, d));
-                    am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, d));
-                }
-                const float p = a.clip_steps > 0 ? clip_ratio(best_k, a.clip_steps, a.clip_min) : 1.f;
-                make_grid(p * lo, p * hi, p * am, a.bits, a.sym, scale, zero);
-                if (owner && sub == 0) {
-                    const int g = (i0 + o) / a.group;
-                    a.scales[(int64_t)row * a.G + g] = scale;
-                    a.zeros[(int64_t)row * a.G + g] = zero;
-                }
-            }
-            float x[CPL], nerr[CPL], pre[CPL];
-            uint32_t code[CPL / 4];
-            const int c_lane = o + sub * CPL;                 // this lane's first column in the block
-#pragma unroll
-            for (int k4 = 0; k4 < CPL / 4; ++k4) {
-                const float4 v = *reinterpret_cast<const float4 *>(&Wt[lrow][c_lane + 4 * k4]);
-                x[4 * k4] = v.x; x[4 * k4 + 1] = v.y; x[4 * k4 + 2] = v.z; x[4 * k4 + 3] = v.w;
-                code[k4] = 0u;
-            }
-            QuantStep<LANES, 0>::run(x, nerr, pre, code, sub, &Us[0][o], &Ps[0][o], udinv, scale, 1.f / scale, zero, maxq,
-                                     a.err_scale, a.asym_scale);
-            if (owner) {
-                uint8_t *crow = a.codes + (int64_t)row * n + i0 + c_lane;
-                if (a.perm) {
-                    uint8_t *cbase = a.codes + (int64_t)row * n;
-                    const int *pp = a.perm + i0 + c_lane;
-#pragma unroll
-                    for (int k = 0; k < CPL; ++k) cbase[pp[k]] = (uint8_t)(code[k >> 2] >> (8 * (k & 3)));
-                } else if ((reinterpret_cast<uintptr_t>(crow) & (CPL >= 16 ? 15 : 7)) == 0) {
-                    if constexpr (CPL == 32) {
-                        *reinterpret_cast<uint4 *>(crow) = make_uint4(code[0], code[1], code[2], code[3]);
-                        *reinterpret_cast<uint4 *>(crow + 16) = make_uint4(code[4], code[5], code[6], code[7]);
-                    } else if constexpr (CPL == 16) {
-                        *reinterpret_cast<uint4 *>(crow) = make_uint4(code[0], code[1], code[2], code[3]);
-                    } else {
-                        *reinterpret_cast<uint2 *>(crow) = make_uint2(code[0], code[1]);
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < CPL; ++k) crow[k] = (uint8_t)(code[k >> 2] >> (8 * (k & 3)));
-                }
-            }
-            float *ew = a.EW + (int64_t)row * a.ew_ld + c_lane;
-            float *ewl = a.EW_lo ? a.EW_lo + (int64_t)row * a.ew_ld + c_lane : nullptr;
-#pragma unroll
-            for (int k4 = 0; k4 < CPL / 4; ++k4) {
-                *reinterpret_cast<float4 *>(&Wt[lrow][c_lane + 4 * k4]) = make_float4(x[4 * k4], x[4 * k4 + 1], x[4 * k4 + 2], x[4 * k4 + 3]);
-                float e4[4] = {nerr[4 * k4], nerr[4 * k4 + 1], nerr[4 * k4 + 2], nerr[4 * k4 + 3]};
-                float p4[4] = {pre[4 * k4], pre[4 * k4 + 1], pre[4 * k4 + 2], pre[4 * k4 + 3]};
-                if (f16) {
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) {
-                        p4[f] *= rho;
-                        rmax = fmaxf(rmax, fmaxf(fabsf(e4[f]), fabsf(p4[f])));
-                    }
-                }
-                if (!owner) continue;
-                if (ewl) {
-                    float el[4], pl[4];
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) {
-                        const float eh = tf32_rn(e4[f]), ph = tf32_rn(p4[f]);
-                        el[f] = tf32_rn(e4[f] - eh); pl[f] = tf32_rn(p4[f] - ph);
-                        e4[f] = eh; p4[f] = ph;
-                    }
-                    *reinterpret_cast<float4 *>(ewl + 4 * k4) = make_float4(el[0], el[1], el[2], el[3]);
-                    *reinterpret_cast<float4 *>(ewl + a.ew_pre + 4 * k4) = make_float4(pl[0], pl[1], pl[2], pl[3]);
-                }
-                *reinterpret_cast<float4 *>(ew + 4 * k4) = make_float4(e4[0], e4[1], e4[2], e4[3]);
-                *reinterpret_cast<float4 *>(ew + a.ew_pre + 4 * k4) = make_float4(p4[0], p4[1], p4[2], p4[3]);
-            }
-#pragma unroll
-            for (int k = 0; k < CPL; ++k) {
-                St[(sub * CPL + k) * sld + lrow] = nerr[k];
-                St[(32 + sub * CPL + k) * sld + lrow] = pre[k];
-            }
-        }
-        __syncthreads();
-        // rest of the block: Wt[:, c] += sum_k (-Err)[:, k] U[o + k][c] + Wpre[:, k] P[o + k][c], c >= o + 32
-        const int c_begin = o + 32;
-        if (c_begin < B) {
-            const int tr = rows / 4, tc = (B - c_begin) / 4;
-            for (int t = tid; t < tr * tc; t += CB_THREADS) {
-                const int tj = t / tr, ti = t - tj * tr;            // consecutive threads: consecutive row tiles
-                const int c0 = c_begin + 4 * tj;
-                float acc[4][4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
-#pragma unroll 4
-                for (int k = 0; k < 64; ++k) {
-                    const float4 av4 = *reinterpret_cast<const float4 *>(St + k * sld + 4 * ti);
-                    const float4 bv4 = *reinterpret_cast<const float4 *>(k < 32 ? &Us[k][c0] : &Ps[k - 32][c0]);
-                    const float av[4] = {av4.x, av4.y, av4.z, av4.w}, bv[4] = {bv4.x, bv4.y, bv4.z, bv4.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-#pragma unroll
-                        for (int f = 0; f < 4; ++f) acc[e][f] = fmaf(av[e], bv[f], acc[e][f]);
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    float4 *cp = reinterpret_cast<float4 *>(&Wt[4 * ti + e][c0]);
-                    float4 v = *cp;
-                    v.x += acc[e][0]; v.y += acc[e][1]; v.z += acc[e][2]; v.w += acc[e][3];
-                    *cp = v;
-                }
-            }
-        }
-    }
-    if (f16 && chain) {
-        // the row's largest operand magnitude, over its lanes
-#pragma unroll
-        for (int d = 1; d < LANES; d <<= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, d));
-        if (sub == 0) rmax_s[lrow] = rmax;
-    }
-    __syncthreads();
-    // dequantized block back to W
-    for (int idx = tid; idx < nrows * bq; idx += CB_THREADS) {
-        const int r = idx / bq, c4 = idx - r * bq;
-        const float4 v = *reinterpret_cast<const float4 *>(&Wt[r][4 * c4]);
-        const bool bad = !isfinite(v.x) || !isfinite(v.y) || !isfinite(v.z) || !isfinite(v.w);
-        float *dst = a.W + (int64_t)(row0 + r) * a.ldw + i0 + 4 * c4;
-        if ((reinterpret_cast<uintptr_t>(dst) & 15) == 0) *reinterpret_cast<float4 *>(dst) = v;
-        else { dst[0] = v.x; dst[1] = v.y; dst[2] = v.z; dst[3] = v.w; }
-        if (bad) record_status(a.hd, ST_NONFINITE, row0 + r);
-    }
-    if (f16) {
-        // this CTA's rows of [-Err | rho * Wpre], scaled row by row into the fp16 range and split
-        float *srow = St;                       // free since the last rank update
-        if (tid < rows) {
-            const bool live = tid < nrows;
-            const float sc = live ? split_scale(rmax_s[tid]) : 1.f;
-            srow[tid] = sc;
-            if (live) a.row_inv[row0 + tid] = 1.f / sc;
-        }
-        __syncthreads();                        // (also: the rows written above are visible to the whole CTA)
-        const int q = 2 * B / 4;
-        for (int idx = tid; idx < nrows * q; idx += CB_THREADS) {
-            const int r = idx / q, c4 = idx - r * q;
-            const int64_t off = (int64_t)(row0 + r) * (2 * B) + 4 * c4;
-            const int cc = 4 * c4;
-            const float4 v = *reinterpret_cast<const float4 *>(a.EW + (int64_t)(row0 + r) * a.ew_ld +
-                                                               (cc < B ? cc : a.ew_pre + cc - B));
-            const float sc = srow[r];
-            const float x[4] = {sc * v.x, sc * v.y, sc * v.z, sc * v.w};
-            __half h[4], l[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { h[e] = __float2half_rn(x[e]); l[e] = __float2half_rn(x[e] - __half2float(h[e])); }
-            const __half2 h01 = __halves2half2(h[0], h[1]), h23 = __halves2half2(h[2], h[3]);
-            const __half2 l01 = __halves2half2(l[0], l[1]), l23 = __halves2half2(l[2], l[3]);
-            *reinterpret_cast<uint2 *>(a.EW16_hi + off) =
-                make_uint2(*reinterpret_cast<const uint32_t *>(&h01), *reinterpret_cast<const uint32_t *>(&h23));
-            *reinterpret_cast<uint2 *>(a.EW16_lo + off) =
-                make_uint2(*reinterpret_cast<const uint32_t *>(&l01), *reinterpret_cast<const uint32_t *>(&l23));
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------

@@ -1,0 +1,723 @@
+// The column loop of Algorithm 1 over several lazy-batch blocks of columns in ONE launch.
+//
+// Rows of W are independent, so a CTA that owns 32 rows can run the sequential part of the loop over many
+// lazy-batch blocks without ever meeting another CTA.  Its slab of W (32 x 512 float32) stays in shared
+// memory; what would be a launch per block and a product per block over the whole matrix is a pipeline of
+// warp roles inside the CTA:
+//
+//   chain   (4 warps)  quantizes 32 columns at a time, four lanes per row with 8 consecutive columns each;
+//   near    (8 warps)  applies a step's errors to the rest of its 128-column block (float32 FMA), 8 columns
+//                      behind the chain, fetches the rows of U and P of the next step, writes results out;
+//   drain   (4 warps)  adds the products of the tensor cores to the later blocks of the slab;
+//   load, mma (1 + 1)  stream U^T and P^T (fp16 hi / lo parts) and issue
+//                      D[128 later columns][32 rows] = [U^T | P^T] [-Err | rho Wpre]^T   (tcgen05, M = 128, N = 32)
+//                      for every 64 quantized columns, as lo*hi + hi*lo + hi*hi.
+//
+// What bounds it: the chain.  A column is 6 dependent float32 operations (24 cycles) as long as the next
+// column belongs to the same lane -- the lane goes on with its own error and pre-quantization value, the
+// shuffled copies that the other lanes need are off the chain -- and a shuffle more at every 8th column.
+#pragma once
+#include "tc_gemm.cuh"
+
+namespace gptaq {
+
+constexpr int QB_ROWS = 32;             // rows of W per CTA
+constexpr int QB_W = 128;               // columns per block (float32 updates inside, tensor cores beyond)
+constexpr int QB_SUPER = 512;           // most columns per launch
+constexpr int QB_CHAIN = 128, QB_NEAR = 256, QB_DRAIN = 128;
+constexpr int QB_THREADS_NEAR = QB_CHAIN + QB_NEAR;                   // one block per launch, no tensor cores
+constexpr int QB_THREADS_FAR = QB_THREADS_NEAR + QB_DRAIN + 64;
+constexpr int QB_ULD0 = QB_W + 4, QB_ULD1 = QB_W - 32 + 4;            // pitch of U / P rows in the even / odd step's buffer
+constexpr int QB_SLD = QB_ROWS + 4;                                   // pitch of the published errors
+// 128 x 64 fp16 tiles of U^T / P^T in flight (one less makes room for the grids per column)
+__host__ __device__ constexpr int qb_aslots(bool percol) { return percol ? 2 : 3; }
+constexpr int QB_A_BYTES = 128 * 64 * 2;
+constexpr int QB_E_BYTES = QB_ROWS * 64 * 2;                          // one K-block (64 columns) of one part of the errors
+constexpr int QB_HALF_BYTES = 4 * QB_E_BYTES;                         // (hi, lo) x (-Err, Wpre) of 64 columns
+constexpr int QB_TMEM_COLS = 256;                                     // 2 halves x 3 blocks x 32 columns, a power of two
+
+struct QuantBlockArgs {
+    float *W; int64_t ldw; int m, n;
+    const float *U, *P;        // n x n, ld n; entries below the diagonals are not used
+    const uint8_t *dead;
+    int i0, i1;                // columns of this launch: [i0, i1); i1 - i0 <= QB_SUPER (tensor-core form) or one block
+    int bw;                    // columns per block: QB_W (tensor-core form); 32, 64 or 128
+    int bits, group, sym;
+    uint8_t *codes;            // m x n
+    float *scales, *zeros;     // m x G
+    int G;
+    float *EW; int ew_ld, ew_pre;   // [-Err | rho * Wpre] of this launch, row pitch, offset of Wpre in a row
+    float *EW_lo;              // nullptr, or: EW receives the TF32 value of each entry and EW_lo the remainder
+    // fp16 parts of [-Err | rho * Wpre] for the update beyond i1, one power-of-two scale per row (row_inv = 1 / scale),
+    // or nullptr (nothing beyond); pitch ew_ld
+    __half *EWS_hi, *EWS_lo;
+    float *row_inv;
+    const unsigned *amax_u, *amax_p;   // fp16-split handles: recorded maxima of U and P (rho = scale of U / scale of P)
+    StateHeader *hd;
+    float err_scale, asym_scale;   // 1 or 0: switches of the two terms of the weight update (ablation)
+    const int *perm;               // nullptr, or: working column c is original column perm[c] (codes go there)
+    int clip_steps; float clip_min;
+};
+
+// Shared memory, in bytes from a 1024-byte boundary.  The tensor-core operands come first (alignment).
+struct QuantBlockSmem {
+    int a, e, w, up, st, grid, udinv, perm, inv, bars, total, wld;
+};
+__host__ __device__ constexpr QuantBlockSmem quant_block_smem(bool far_form, bool percol) {
+    QuantBlockSmem s{};
+    s.wld = (far_form ? QB_SUPER : QB_W) + 4;
+    s.a = 0;
+    s.e = s.a + (far_form ? qb_aslots(percol) * QB_A_BYTES : 0);
+    s.w = s.e + (far_form ? 2 * QB_HALF_BYTES : 0);
+    s.up = s.w + QB_ROWS * s.wld * 4;
+    s.st = s.up + 2 * 32 * (QB_ULD0 + QB_ULD1) * 4;
+    s.grid = s.st + 2 * 64 * QB_SLD * 4;
+    s.udinv = s.grid + (percol ? 2 * 32 * QB_SLD * 4 : 0);
+    s.perm = s.udinv + 2 * 32 * 4;
+    s.inv = s.perm + 2 * 32 * 4;
+    s.bars = s.inv + 2 * QB_ROWS * 4;
+    s.total = s.bars + 256;
+    return s;
+}
+constexpr size_t quant_block_smem_bytes(bool far_form, bool percol) {
+    return (size_t)quant_block_smem(far_form, percol).total + 1024;        // (alignment slack)
+}
+static_assert(quant_block_smem_bytes(true, false) <= 227 * 1024 && quant_block_smem_bytes(true, true) <= 227 * 1024, "shared memory of one SM");
+
+// kind::f16 instruction descriptor: fp16 A and B (K-major), fp32 D, M = 128, N = QB_ROWS.
+constexpr uint32_t QB_IDESC = (1u << 4) | ((QB_ROWS >> 3) << 17) | ((128 >> 4) << 24);
+
+// Named barriers.  Chunk barriers are used once per step each; the step barrier keeps the chain from lapping them.
+enum { QBAR_CHUNK = 1, QBAR_STEP = 5, QBAR_NEAR = 6, QBAR_DRAIN = 7, QBAR_CLIP = 8 };
+__device__ __forceinline__ void named_bar_arrive(int id, int nthreads) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
+// Position of a row in a column of the published errors: the near warps' threads take rows ti, ti + 8, .. as
+// one 16-byte read.
+__device__ __forceinline__ int qb_pos(int row) { return (row & 7) * 4 + (row >> 3); }
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+// Two float32 FMAs in one instruction: the roles share their schedulers' issue slots, which the chain is short of.
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float lo2(unsigned long long v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(unsigned long long v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ float pick2(const unsigned long long (&v)[4], int j) { return (j & 1) ? hi2(v[j >> 1]) : lo2(v[j >> 1]); }
+
+// Range of a row over columns [c0, c1) of the slab, by the row's four lanes.
+__device__ __forceinline__ void row_range(const float *w, int c0, int c1, int sub, float &lo, float &hi, float &am) {
+    lo = 0.f; hi = 0.f;
+    for (int c = c0 + sub; c < c1; c += 4) {
+        const float v = w[c];
+        lo = fminf(lo, v); hi = fmaxf(hi, v);
+    }
+#pragma unroll
+    for (int d = 1; d < 4; d <<= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, d));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, d));
+    }
+    am = fmaxf(-lo, hi);
+}
+
+// FAR: several blocks per launch, updates between them on the tensor cores.  PERCOL: static groups, a grid per column.
+template <bool FAR, bool PERCOL>
+__global__ void __launch_bounds__(FAR ? QB_THREADS_FAR : QB_THREADS_NEAR, 1)
+quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_constant__ CUtensorMap mapUlo,
+                   const __grid_constant__ CUtensorMap mapPhi, const __grid_constant__ CUtensorMap mapPlo, QuantBlockArgs a) {
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    uint8_t *sm = smem_raw + (base - raw);
+    constexpr QuantBlockSmem L = quant_block_smem(FAR, PERCOL);
+    constexpr int ASLOTS = qb_aslots(PERCOL);
+    constexpr int WLD = L.wld;
+    constexpr int NTHREADS = FAR ? QB_THREADS_FAR : QB_THREADS_NEAR;
+    float *Ws = reinterpret_cast<float *>(sm + L.w);               // [32][WLD]: the slab
+    float *UPs = reinterpret_cast<float *>(sm + L.up);             // rows of U and P of the current and the next step
+    float *Sts = reinterpret_cast<float *>(sm + L.st);             // [2 steps][64][QB_SLD]: -Err, then Wpre, of 32 columns
+    float *grid_s = reinterpret_cast<float *>(sm + L.grid);        // PERCOL: scales, then zero points, [32 columns][QB_SLD] each
+    float *udinv2 = reinterpret_cast<float *>(sm + L.udinv);       // [2 steps][32]: err_scale / U_kk
+    int *perm2 = reinterpret_cast<int *>(sm + L.perm);             // [2 steps][32]: where a column's codes go
+    float *inv_s = reinterpret_cast<float *>(sm + L.inv);          // [2 halves][32]: 1 / scale of a row's errors
+    const uint32_t bar0 = base + L.bars;
+    // mbarriers (8 bytes each): afull[3], aempty[3], efull[2], efree[2], tfull[6], tempty[6]; tmem slot, abort flag
+    auto afull = [&](int s) { return bar0 + 8u * s; };
+    auto aempty = [&](int s) { return bar0 + 8u * (3 + s); };
+    auto efull = [&](int s) { return bar0 + 8u * (6 + s); };
+    auto efree = [&](int s) { return bar0 + 8u * (8 + s); };
+    auto tfull = [&](int s) { return bar0 + 8u * (10 + s); };
+    auto tempty = [&](int s) { return bar0 + 8u * (16 + s); };
+    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(sm + L.bars + 8 * 22);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n = a.n, i0 = a.i0, B = a.bw;
+    const int row0 = blockIdx.x * QB_ROWS;
+    const int nrows = min(QB_ROWS, a.m - row0);
+    const int cols = a.i1 - i0;
+    const int nblk = FAR ? (cols + QB_W - 1) / QB_W : 1;
+    auto nsteps = [&](int b) { return min(B / 32, (cols - b * QB_W + 31) / 32); };     // 32-column steps of block b
+    const float maxq = (float)((1 << a.bits) - 1);
+    const bool aligned_up = (n & 3) == 0 && ((reinterpret_cast<uintptr_t>(a.U) | reinterpret_cast<uintptr_t>(a.P)) & 15) == 0;
+
+    // U / P rows of step s of the block that starts at column cb: buffer s & 1, columns cb + 32 s ..
+    auto up_ld = [&](int s) { return (s & 1) ? QB_ULD1 : QB_ULD0; };
+    auto up_buf = [&](int s) { return UPs + (s & 1) * (2 * 32 * QB_ULD0); };
+    auto fetch_up = [&](int cb, int s, int t, int nthr) {
+        const int ld = up_ld(s), q = (B - 32 * s) / 4, r0 = cb + 32 * s;
+        float *ub = up_buf(s), *pb = ub + 32 * ld;
+        for (int idx = t; idx < 32 * q; idx += nthr) {
+            const int k = idx / q, c4 = idx - k * q;
+            const int row = r0 + k, col = r0 + 4 * c4;
+            float *du = ub + k * ld + 4 * c4, *dp = pb + k * ld + 4 * c4;
+            const int64_t off = (int64_t)row * n + col;
+            if (aligned_up && row < n && col + 3 < n) {
+                cp_async16(du, a.U + off);
+                cp_async16(dp, a.P + off);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const bool in = row < n && col + e < n;
+                    du[e] = in ? a.U[off + e] : 0.f;
+                    dp[e] = in ? a.P[off + e] : 0.f;
+                }
+            }
+        }
+    };
+    // per column of a step: err_scale / U_kk (padded columns beyond n have no error: 0) and the column's original index
+    auto load_pivot = [&](int c) { return c < n ? a.err_scale * (1.f / a.U[(int64_t)c * n + c]) : 0.f; };
+    auto load_perm = [&](int c) { return a.perm && c < n ? a.perm[c] : c; };
+    // PERCOL: grids of four columns c .. c + 3 of a row
+    auto load_grid = [&](int r, int c, float (&sc)[4], float (&zp)[4]) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            sc[e] = 1.f; zp[e] = 0.f;
+            if (r < nrows && c + e < n) {
+                const int64_t g = (int64_t)(row0 + r) * a.G + load_perm(c + e) / a.group;
+                sc[e] = a.scales[g]; zp[e] = a.zeros[g];
+            }
+        }
+    };
+    auto store_grid = [&](int r, int c, const float (&sc)[4], const float (&zp)[4]) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            grid_s[(c + e) * QB_SLD + r] = sc[e];
+            grid_s[(32 + c + e) * QB_SLD + r] = zp[e];
+        }
+    };
+
+    // ---------------------------------------------------------------- set-up: barriers, tensor memory, slab, first rows of U / P
+    if (FAR) {
+        if (tid == 0) {
+            for (int s = 0; s < ASLOTS; ++s) { mbar_init(afull(s), 1); mbar_init(aempty(s), 1); }
+            for (int s = 0; s < 2; ++s) { mbar_init(efull(s), QB_CHAIN / 32); mbar_init(efree(s), QB_DRAIN / 32); }
+            for (int s = 0; s < 6; ++s) { mbar_init(tfull(s), 1); mbar_init(tempty(s), QB_DRAIN / 32); }
+            *abort_flag = 0;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        if (warp == NTHREADS / 32 - 1) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                         ::"r"(smem_u32(const_cast<uint32_t *>(tmem_slot))), "r"((uint32_t)QB_TMEM_COLS) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
+    }
+    fetch_up(i0, 0, tid, NTHREADS);
+    if (tid < 32) { udinv2[tid] = load_pivot(i0 + tid); perm2[tid] = load_perm(i0 + tid); }
+    if (PERCOL && tid < QB_NEAR) {
+        float sc[4], zp[4];
+        load_grid(tid >> 3, i0 + 4 * (tid & 7), sc, zp);
+        store_grid(tid >> 3, 4 * (tid & 7), sc, zp);
+    }
+    {
+        const int cq = FAR ? nblk * (QB_W / 4) : B / 4;            // quads per row, padded columns included
+        for (int idx0 = 0; idx0 < QB_ROWS * cq; idx0 += 4 * NTHREADS) {
+            float4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int idx = idx0 + u * NTHREADS + tid;
+                const int r = idx / cq, c = 4 * (idx - r * cq);
+                v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (r < nrows && c < cols) {
+                    const float *src = a.W + (int64_t)(row0 + r) * a.ldw + i0 + c;
+                    if (c + 3 < cols && (reinterpret_cast<uintptr_t>(src) & 15) == 0) v[u] = *reinterpret_cast<const float4 *>(src);
+                    else {
+                        v[u].x = src[0];
+                        if (c + 1 < cols) v[u].y = src[1];
+                        if (c + 2 < cols) v[u].z = src[2];
+                        if (c + 3 < cols) v[u].w = src[3];
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int idx = idx0 + u * NTHREADS + tid;
+                const int r = idx / cq, c = 4 * (idx - r * cq);
+                if (r >= QB_ROWS) continue;
+                float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+                bool bad = false;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (c + e < cols && a.dead[i0 + c + e]) x[e] = 0.f;       // dead inputs read as zero
+                    bad |= !isfinite(x[e]);
+                }
+                // a non-finite weight is reported from the value that was read: its code and dequantized value
+                // come out finite (the clamp absorbs NaN and Inf), so the results alone would not show it
+                if (bad) record_status(a.hd, ST_NONFINITE, row0 + r);
+                *reinterpret_cast<float4 *>(Ws + r * WLD + c) = make_float4(x[0], x[1], x[2], x[3]);
+            }
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (FAR) tc_fence_before();
+    __syncthreads();
+    if (FAR) tc_fence_after();
+
+    float rho = 1.f, su = 1.f;
+    if (a.amax_u) {
+        su = split_scale(__uint_as_float(*a.amax_u));
+        const float ap = __uint_as_float(*a.amax_p);
+        rho = ap > 0.f ? su / split_scale(ap) : 0.f;
+    }
+    const int last_groups = nblk - 1;                               // blocks 0 .. nblk - 2 have later blocks in this launch
+
+    if (tid < QB_CHAIN) {
+        // ================================================================ chain
+        const int lrow = tid >> 2, sub = tid & 3;
+        const int row = row0 + lrow;
+        const bool live = lrow < nrows;
+        float *wrow = Ws + lrow * WLD;
+        const int pos = qb_pos(lrow);
+        float scale = 1.f, zero = 0.f;
+        float row_max = 0.f;                                        // largest magnitude of the row's errors in this launch
+        if (!PERCOL && a.group <= 0 && live) { scale = a.scales[row]; zero = a.zeros[row]; }
+        for (int b = 0; b < nblk; ++b) {
+            const int nst = nsteps(b);
+            for (int s = 0; s < nst; ++s) {
+                const int co = b * QB_W + 32 * s;                   // first column of the step in the slab
+                const int cg = i0 + co;                             // ... in W
+                if (b + s > 0) named_bar_sync(QBAR_STEP, QB_THREADS_NEAR);
+                if (FAR && s == 0 && b > 0) named_bar_sync(QBAR_DRAIN, QB_CHAIN + QB_DRAIN);
+                float *St = Sts + (s & 1) * 64 * QB_SLD;
+                float scv[8], ivv[8], zv[8];
+                if (PERCOL) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        scv[e] = grid_s[(8 * sub + e) * QB_SLD + lrow];
+                        zv[e] = grid_s[(32 + 8 * sub + e) * QB_SLD + lrow];
+                        ivv[e] = 1.f / scv[e];
+                    }
+                } else if (a.group > 0 && (cg % a.group) == 0) {
+                    // grid of the group that starts here, from the current values
+                    float lo, hi, am;
+                    row_range(wrow, co, min(co + a.group, cols), sub, lo, hi, am);
+                    float p = 1.f;
+                    if (a.clip_steps > 0) {
+                        named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);          // the near warps search
+                        named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);
+                        p = clip_ratio(reinterpret_cast<int *>(St)[lrow], a.clip_steps, a.clip_min);
+                    }
+                    make_grid(p * lo, p * hi, p * am, a.bits, a.sym, scale, zero);
+                    if (live && sub == 0) {
+                        const int g = cg / a.group;
+                        a.scales[(int64_t)row * a.G + g] = scale;
+                        a.zeros[(int64_t)row * a.G + g] = zero;
+                    }
+                    if (a.clip_steps > 0) named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);   // the search's scratch is free again
+                }
+                const float inv_scale = 1.f / scale, qlo = -zero, qhi = maxq - zero;
+                const int ld = up_ld(s);
+                const float *Us = up_buf(s) + 8 * sub, *Ps = Us + 32 * ld;
+                const float *ud = udinv2 + (s & 1) * 32;
+                unsigned long long x[4];                            // this lane's 8 columns, in pairs
+                {
+                    const ulonglong2 v0 = *reinterpret_cast<const ulonglong2 *>(wrow + co + 8 * sub);
+                    const ulonglong2 v1 = *reinterpret_cast<const ulonglong2 *>(wrow + co + 8 * sub + 4);
+                    x[0] = v0.x; x[1] = v0.y; x[2] = v1.x; x[3] = v1.y;
+                }
+                // `c` is the chain: the current column's value in the lane that owns it.  Every lane runs the same
+                // instructions on its own column; only the owner's results are used.  Entries of x that belong to
+                // columns already done are garbage (entries of U and P at or below the diagonal are applied to them)
+                // and never read again.
+                float c = lo2(x[0]);
+#pragma unroll
+                for (int ph = 0; ph < 4; ++ph) {
+                    float nerr[8], pre[8], qv[8];
+                    uint32_t code[2] = {0u, 0u};
+                    const float4 ud0 = *reinterpret_cast<const float4 *>(ud + 8 * ph), ud1 = *reinterpret_cast<const float4 *>(ud + 8 * ph + 4);
+                    const float udv[8] = {ud0.x, ud0.y, ud0.z, ud0.w, ud1.x, ud1.y, ud1.z, ud1.w};
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk) {
+                        const int K = 8 * ph + kk;
+                        const ulonglong2 u0 = *reinterpret_cast<const ulonglong2 *>(Us + K * ld), u1 = *reinterpret_cast<const ulonglong2 *>(Us + K * ld + 4);
+                        const ulonglong2 p0 = *reinterpret_cast<const ulonglong2 *>(Ps + K * ld), p1 = *reinterpret_cast<const ulonglong2 *>(Ps + K * ld + 4);
+                        const unsigned long long u[4] = {u0.x, u0.y, u1.x, u1.y}, pp[4] = {p0.x, p0.y, p1.x, p1.y};
+                        const float sc = PERCOL ? scv[kk] : scale;
+                        const float iv = PERCOL ? ivv[kk] : inv_scale;
+                        const float z = PERCOL ? zv[kk] : zero;
+                        const float w0 = c;
+                        // round(w / scale), clamped to the grid, minus the zero point.  Adding 1.5 * 2^23 rounds to nearest even
+                        // wherever |v| < 2^22 and leaves larger values large (the clamp decides those).
+                        const float magic = 12582912.f;
+                        const float r = __fsub_rn(__fadd_rn(__fmul_rn(w0, iv), magic), magic);
+                        const float cz = fminf(fmaxf(r, PERCOL ? -z : qlo), PERCOL ? maxq - z : qhi);
+                        const float d = __fmaf_rn(sc, cz, -w0);                  // -(w - q)
+                        const float ne = d * udv[kk];                            // ... / U_kk
+                        const float wa = a.asym_scale * w0;
+                        qv[kk] = sc * cz; nerr[kk] = ne; pre[kk] = wa;
+                        code[kk >> 2] |= (__float_as_uint(cz + z + magic) & 0xffu) << (8 * (kk & 3));
+                        // the owner's next column, from its own values
+                        if (kk < 7) c = fmaf(d, udv[kk] * pick2(u, kk + 1), fmaf(wa, pick2(pp, kk + 1), pick2(x, kk + 1)));
+                        const float ne_b = __shfl_sync(0xffffffffu, ne, ph, 4);
+                        const float wa_b = __shfl_sync(0xffffffffu, wa, ph, 4);
+                        const unsigned long long ne2 = pack2(ne_b, ne_b), wa2 = pack2(wa_b, wa_b);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            if (ph == 3 && 2 * j + 1 <= kk) continue;            // (no lane needs it any more)
+                            x[j] = fma2(ne2, u[j], fma2(wa2, pp[j], x[j]));
+                        }
+                        if (kk == 7) c = lo2(x[0]);
+                    }
+                    // publish these 8 columns
+                    if (sub == ph) {
+#pragma unroll
+                        for (int kk = 0; kk < 8; ++kk) {
+                            St[(8 * ph + kk) * QB_SLD + pos] = nerr[kk];
+                            St[(32 + 8 * ph + kk) * QB_SLD + pos] = pre[kk];
+                        }
+                        *reinterpret_cast<float4 *>(wrow + co + 8 * sub) = make_float4(qv[0], qv[1], qv[2], qv[3]);
+                        *reinterpret_cast<float4 *>(wrow + co + 8 * sub + 4) = make_float4(qv[4], qv[5], qv[6], qv[7]);
+                        if (live) {
+                            uint8_t *crow = a.codes + (int64_t)row * n;
+                            const int cc = cg + 8 * sub;
+                            if (!a.perm && cc + 7 < n && (reinterpret_cast<uintptr_t>(crow + cc) & 7) == 0) {
+                                *reinterpret_cast<uint2 *>(crow + cc) = make_uint2(code[0], code[1]);
+                            } else {
+#pragma unroll
+                                for (int kk = 0; kk < 8; ++kk)
+                                    if (cc + kk < n) crow[perm2[(s & 1) * 32 + 8 * ph + kk]] = (uint8_t)(code[kk >> 2] >> (8 * (kk & 3)));
+                            }
+                        }
+                    }
+                    named_bar_arrive(QBAR_CHUNK + ph, QB_THREADS_NEAR);
+                }
+                if (FAR && (s & 1)) {
+                    // 64 columns done: their errors as the tensor cores' operand, with one power-of-two scale per row
+                    __syncwarp();
+                    float v[2][2][8];                               // [step of the pair][-Err, Wpre][column]
+                    float mx = 0.f;
+#pragma unroll
+                    for (int d = 0; d < 2; ++d)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const float *S2 = Sts + d * 64 * QB_SLD;
+                            v[d][0][e] = S2[(8 * sub + e) * QB_SLD + pos];
+                            v[d][1][e] = rho * S2[(32 + 8 * sub + e) * QB_SLD + pos];
+                            mx = fmaxf(mx, fmaxf(fabsf(v[d][0][e]), fabsf(v[d][1][e])));
+                        }
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+                    row_max = fmaxf(row_max, mx);
+                    if (b < last_groups) {
+                        const int half = s >> 1;                    // buffer: even and odd halves alternate
+                        // (the drain warps are done with this buffer's row scales, the MMAs with its operands)
+                        if (b > 0) mbar_wait(efree(half), (uint32_t)(b - 1) & 1u, abort_flag);
+                        const float sc = split_scale(mx);
+                        if (sub == 0) inv_s[half * QB_ROWS + lrow] = 1.f / sc / su;
+                        uint8_t *eb = sm + L.e + half * QB_HALF_BYTES + (lrow >> 3) * 1024 + (lrow & 7) * 128;
+#pragma unroll
+                        for (int d = 0; d < 2; ++d)
+#pragma unroll
+                            for (int o = 0; o < 2; ++o) {
+                                const float y0[4] = {sc * v[d][o][0], sc * v[d][o][1], sc * v[d][o][2], sc * v[d][o][3]};
+                                const float y1[4] = {sc * v[d][o][4], sc * v[d][o][5], sc * v[d][o][6], sc * v[d][o][7]};
+                                uint2 h0, l0, h1, l1;
+                                split16_pack(y0, h0, l0);
+                                split16_pack(y1, h1, l1);
+                                const int ch = ((4 * d + sub) ^ (lrow & 7)) << 4;
+                                *reinterpret_cast<uint4 *>(eb + o * QB_E_BYTES + ch) = make_uint4(h0.x, h0.y, h1.x, h1.y);
+                                *reinterpret_cast<uint4 *>(eb + (2 + o) * QB_E_BYTES + ch) = make_uint4(l0.x, l0.y, l1.x, l1.y);
+                            }
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(efull(half));
+                    }
+                }
+            }
+        }
+        if (FAR && a.EWS_hi && sub == 0) {
+            const float sc = live ? split_scale(row_max) : 1.f;
+            udinv2[lrow] = sc;                                      // (free: the last step's pivots are in the other half; read
+                                                                    //  after the barrier below)
+            if (live) a.row_inv[row] = 1.f / sc;
+        }
+    } else if (tid < QB_THREADS_NEAR) {
+        // ================================================================ near
+        const int t = tid - QB_CHAIN;
+        const int ti = t & 7, tj = t >> 3;                          // rows ti, ti + 8, ti + 16, ti + 24; columns 4 tj .. of the rest
+        for (int b = 0; b < nblk; ++b) {
+            const int nst = nsteps(b);
+            for (int s = 0; s < nst; ++s) {
+                const int co = b * QB_W + 32 * s;
+                named_bar_sync(QBAR_NEAR, QB_NEAR);                 // all near warps are done with the other buffer of U / P
+                const bool last = b == nblk - 1 && s == nst - 1;
+                const int nb = s + 1 < nst ? b : b + 1, ns = s + 1 < nst ? s + 1 : 0;       // the next step
+                const int ncol = i0 + nb * QB_W + 32 * ns;
+                float next_ud = 0.f, next_sc[4], next_zp[4];
+                int next_perm = 0;
+                if (!last) {
+                    fetch_up(i0 + nb * QB_W, ns, t, QB_NEAR);
+                    if (t < 32) { next_ud = load_pivot(ncol + t); next_perm = load_perm(ncol + t); }
+                    if (PERCOL) load_grid(t >> 3, ncol + 4 * (t & 7), next_sc, next_zp);
+                }
+                if (!PERCOL && a.group > 0 && a.clip_steps > 0 && ((i0 + co) % a.group) == 0) {
+                    // clipping-range search: thread = (row, one eighth of the candidates)
+                    named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);     // the group's values are current
+                    const int r = t & 31, cgi = t >> 5;
+                    const int gend = min(co + a.group, cols);
+                    const float *w = Ws + r * WLD;
+                    float lo = 0.f, hi = 0.f;
+                    for (int c = co; c < gend; ++c) {
+                        const float v = w[c];
+                        lo = fminf(lo, v); hi = fmaxf(hi, v);
+                    }
+                    const float am = fmaxf(-lo, hi);
+                    float best = INFINITY;
+                    int kb = 0;
+                    for (int k = cgi; k < a.clip_steps; k += QB_NEAR / 32) {
+                        const float p = clip_ratio(k, a.clip_steps, a.clip_min);
+                        float sk, zk;
+                        make_grid(p * lo, p * hi, p * am, a.bits, a.sym, sk, zk);
+                        float err = 0.f;
+                        for (int c = co; c < gend; ++c) err += rounding_error_sq(w[c], sk, zk, maxq);
+                        if (err < best) { best = err; kb = k; }
+                    }
+                    float *scratch = Sts + (s & 1) * 64 * QB_SLD;   // (the chain writes there only after this search)
+                    float *be = scratch + 64;
+                    int *bk = reinterpret_cast<int *>(be + QB_NEAR);
+                    be[t] = best; bk[t] = kb;
+                    named_bar_sync(QBAR_NEAR, QB_NEAR);
+                    if (t < QB_ROWS) {
+                        for (int g = 1; g < QB_NEAR / 32; ++g) {
+                            const float e = be[g * 32 + t];
+                            const int k = bk[g * 32 + t];
+                            if (e < best || (e == best && k < kb)) { best = e; kb = k; }
+                        }
+                        reinterpret_cast<int *>(scratch)[t] = kb;
+                    }
+                    named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);
+                    named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);
+                }
+                const int ld = up_ld(s);
+                const float *Ub = up_buf(s) + 32 + 4 * tj, *Pb = Ub + 32 * ld;      // (columns beyond the step's own 32)
+                const float *St = Sts + (s & 1) * 64 * QB_SLD;
+                const bool active = 32 + 4 * tj < B - 32 * s;
+                unsigned long long acc[4][2];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) { acc[e][0] = 0ull; acc[e][1] = 0ull; }
+                for (int ph = 0; ph < 4; ++ph) {
+                    named_bar_sync(QBAR_CHUNK + ph, QB_THREADS_NEAR);
+                    if (!active) continue;
+#pragma unroll
+                    for (int kk = 0; kk < 16; ++kk) {
+                        const int k = 8 * ph + (kk & 7);
+                        const float4 av = *reinterpret_cast<const float4 *>(St + (k + (kk < 8 ? 0 : 32)) * QB_SLD + 4 * ti);
+                        const ulonglong2 bv = *reinterpret_cast<const ulonglong2 *>((kk < 8 ? Ub : Pb) + k * ld);
+                        const float ae[4] = {av.x, av.y, av.z, av.w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const unsigned long long aa = pack2(ae[e], ae[e]);
+                            acc[e][0] = fma2(aa, bv.x, acc[e][0]);
+                            acc[e][1] = fma2(aa, bv.y, acc[e][1]);
+                        }
+                    }
+                }
+                if (active) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        float4 *cp = reinterpret_cast<float4 *>(Ws + (ti + 8 * e) * WLD + co + 32 + 4 * tj);
+                        float4 v = *cp;
+                        v.x += lo2(acc[e][0]); v.y += hi2(acc[e][0]); v.z += lo2(acc[e][1]); v.w += hi2(acc[e][1]);
+                        *cp = v;
+                    }
+                }
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                if (!last) {
+                    if (t < 32) { udinv2[(ns & 1) * 32 + t] = next_ud; perm2[(ns & 1) * 32 + t] = next_perm; }
+                    if (PERCOL) store_grid(t >> 3, 4 * (t & 7), next_sc, next_zp);      // (the chain has read this step's)
+                    named_bar_arrive(QBAR_STEP, QB_THREADS_NEAR);
+                }
+                // results of the step: dequantized columns, -Err and Wpre (a thread: four columns of a row)
+                {
+                    const int r = t >> 3, c4 = 4 * (t & 7);
+                    const int cw = co + c4;                         // column in the slab
+                    const float4 v = *reinterpret_cast<const float4 *>(Ws + r * WLD + cw);
+                    const int left = cols - cw;                     // columns that exist from here on
+                    if (r < nrows && left > 0) {
+                        float *dst = a.W + (int64_t)(row0 + r) * a.ldw + i0 + cw;
+                        if (left >= 4 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) *reinterpret_cast<float4 *>(dst) = v;
+                        else {
+                            dst[0] = v.x;
+                            if (left > 1) dst[1] = v.y;
+                            if (left > 2) dst[2] = v.z;
+                            if (left > 3) dst[3] = v.w;
+                        }
+                        if (!isfinite(v.x) || !isfinite(v.y) || !isfinite(v.z) || !isfinite(v.w)) record_status(a.hd, ST_NONFINITE, row0 + r);
+                    }
+                    if (a.EW && r < nrows) {
+                        const int pos = qb_pos(r);
+                        float e4[4], p4[4];
+#pragma unroll
+                        for (int f = 0; f < 4; ++f) {
+                            e4[f] = St[(c4 + f) * QB_SLD + pos];
+                            p4[f] = rho * St[(32 + c4 + f) * QB_SLD + pos];
+                        }
+                        float *ew = a.EW + (int64_t)(row0 + r) * a.ew_ld + cw;
+                        if (a.EW_lo) {
+                            float *ewl = a.EW_lo + (int64_t)(row0 + r) * a.ew_ld + cw;
+                            float el[4], pl[4];
+#pragma unroll
+                            for (int f = 0; f < 4; ++f) {
+                                const float eh = tf32_rn(e4[f]), phi = tf32_rn(p4[f]);
+                                el[f] = tf32_rn(e4[f] - eh); pl[f] = tf32_rn(p4[f] - phi);
+                                e4[f] = eh; p4[f] = phi;
+                            }
+                            *reinterpret_cast<float4 *>(ewl) = make_float4(el[0], el[1], el[2], el[3]);
+                            *reinterpret_cast<float4 *>(ewl + a.ew_pre) = make_float4(pl[0], pl[1], pl[2], pl[3]);
+                        }
+                        *reinterpret_cast<float4 *>(ew) = make_float4(e4[0], e4[1], e4[2], e4[3]);
+                        *reinterpret_cast<float4 *>(ew + a.ew_pre) = make_float4(p4[0], p4[1], p4[2], p4[3]);
+                    }
+                }
+            }
+        }
+    } else if (FAR && tid < QB_THREADS_NEAR + QB_DRAIN) {
+        // ================================================================ drain: tensor memory -> later blocks of the slab
+        const int quarter = warp & 3;                               // TMEM lanes 32 * quarter ..: columns of the block
+        const uint32_t tmem_base = *tmem_slot;
+        for (int b = 0; b < last_groups; ++b)
+            for (int half = 0; half < 2; ++half) {
+                mbar_wait(efull(half), (uint32_t)b & 1u, abort_flag);           // the row scales
+                for (int j = b + 1; j < nblk; ++j) {
+                    const int slot = half * 3 + (j - 1);            // (used once per earlier block: b = 0 .. j - 1)
+                    mbar_wait(tfull(slot), (uint32_t)b & 1u, abort_flag);
+                    tc_fence_after();
+                    uint32_t v[32];
+                    tmem_ld32(tmem_base + slot * QB_ROWS + ((uint32_t)(quarter * 32) << 16), v);
+                    tmem_ld_wait();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(tempty(slot));
+                    float *wp = Ws + j * QB_W + quarter * 32 + lane;
+#pragma unroll
+                    for (int r4 = 0; r4 < QB_ROWS / 4; ++r4) {
+                        const float4 iv = *reinterpret_cast<const float4 *>(inv_s + half * QB_ROWS + 4 * r4);
+                        float *w4 = wp + 4 * r4 * WLD;
+                        w4[0] = fmaf(__uint_as_float(v[4 * r4]), iv.x, w4[0]);
+                        w4[WLD] = fmaf(__uint_as_float(v[4 * r4 + 1]), iv.y, w4[WLD]);
+                        w4[2 * WLD] = fmaf(__uint_as_float(v[4 * r4 + 2]), iv.z, w4[2 * WLD]);
+                        w4[3 * WLD] = fmaf(__uint_as_float(v[4 * r4 + 3]), iv.w, w4[3 * WLD]);
+                    }
+                    if (half == 1 && j == b + 1) named_bar_arrive(QBAR_DRAIN, QB_CHAIN + QB_DRAIN);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(efree(half));
+            }
+    } else if (FAR && warp == (QB_THREADS_NEAR + QB_DRAIN) / 32) {
+        // ================================================================ load: tiles of U^T and P^T
+        if (lane == 0) {
+            uint32_t slot = 0, phase = 0;
+            int issued = 0;
+            bool ok = true;
+            for (int b = 0; ok && b < last_groups; ++b)
+                for (int half = 0; ok && half < 2; ++half)
+                    for (int j = b + 1; ok && j < nblk; ++j)
+                        for (int t4 = 0; t4 < 4; ++t4) {            // U lo, U hi, P lo, P hi
+                            if (!mbar_wait(aempty(slot), phase ^ 1u, abort_flag)) { ok = false; break; }
+                            const CUtensorMap *map = t4 == 0 ? &mapUlo : (t4 == 1 ? &mapUhi : (t4 == 2 ? &mapPlo : &mapPhi));
+                            mbar_expect_tx(afull(slot), QB_A_BYTES);
+                            tma_load_2d(base + L.a + slot * QB_A_BYTES, map, i0 + b * QB_W + 64 * half, i0 + j * QB_W, afull(slot));
+                            ++issued;
+                            if (++slot == ASLOTS) { slot = 0; phase ^= 1u; }
+                        }
+            if (!ok) {
+                // give copies that are still in flight time to land before the CTA exits
+                const long long t0 = clock64();
+                while (issued > 0 && clock64() - t0 < 4000000LL) {}
+            }
+        }
+    } else if (FAR) {
+        // ================================================================ mma
+        if (lane == 0) {
+            uint32_t slot = 0, phase = 0;
+            const uint32_t tmem_base = *tmem_slot;
+            bool ok = true;
+            for (int b = 0; ok && b < last_groups; ++b)
+                for (int half = 0; ok && half < 2; ++half) {
+                    if (!mbar_wait(efull(half), (uint32_t)b & 1u, abort_flag)) { ok = false; break; }
+                    const uint32_t eb = base + L.e + half * QB_HALF_BYTES;
+                    for (int j = b + 1; ok && j < nblk; ++j) {
+                        const int acc = half * 3 + (j - 1);
+                        if (b > 0 && !mbar_wait(tempty(acc), (uint32_t)(b - 1) & 1u, abort_flag)) { ok = false; break; }
+                        tc_fence_after();
+                        const uint32_t d = tmem_base + acc * QB_ROWS;
+                        for (int t4 = 0; t4 < 4; ++t4) {
+                            if (!mbar_wait(afull(slot), phase, abort_flag)) { ok = false; break; }
+                            tc_fence_after();
+                            const uint64_t ad = make_kmajor_desc(base + L.a + slot * QB_A_BYTES);
+                            const uint64_t bh = make_kmajor_desc(eb + (t4 >> 1) * QB_E_BYTES);
+                            const uint64_t bl = make_kmajor_desc(eb + (2 + (t4 >> 1)) * QB_E_BYTES);
+                            if (t4 & 1) {
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) umma_f16(d, ad + (uint64_t)(k * 2), bl + (uint64_t)(k * 2), QB_IDESC, 1u);
+                            }
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                umma_f16(d, ad + (uint64_t)(k * 2), bh + (uint64_t)(k * 2), QB_IDESC, (t4 | k) ? 1u : 0u);
+                            umma_commit(aempty(slot));
+                            if (++slot == ASLOTS) { slot = 0; phase ^= 1u; }
+                        }
+                        if (ok) umma_commit(tfull(acc));
+                    }
+                }
+        }
+    }
+
+    if (!FAR) return;
+    tc_fence_before();
+    __syncthreads();
+    if (a.EWS_hi) {
+        // fp16 parts of [-Err | rho Wpre] for everything beyond this launch's columns (the rows were written by this
+        // CTA; one scale per row over the whole launch)
+        const int q = a.ew_ld / 4;
+        for (int idx = tid; idx < nrows * q; idx += NTHREADS) {
+            const int r = idx / q, c = 4 * (idx - r * q);
+            const int64_t off = (int64_t)(row0 + r) * a.ew_ld + c;
+            const float4 v = *reinterpret_cast<const float4 *>(a.EW + off);
+            const float sc = udinv2[r];
+            const float x[4] = {sc * v.x, sc * v.y, sc * v.z, sc * v.w};
+            uint2 h2, l2;
+            split16_pack(x, h2, l2);
+            *reinterpret_cast<uint2 *>(a.EWS_hi + off) = h2;
+            *reinterpret_cast<uint2 *>(a.EWS_lo + off) = l2;
+        }
+    }
+    if (*abort_flag && tid == 0) record_status(a.hd, ST_TIMEOUT, 3000000 + blockIdx.x);
+    if (warp == NTHREADS / 32 - 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"((uint32_t)QB_TMEM_COLS) : "memory");
+    }
+}
+
+}  // namespace gptaq
