@@ -1000,7 +1000,7 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
     } else {
         CU(cudaMemcpyAsync(h->dead, h->dead_raw, (size_t)n, cudaMemcpyDeviceToDevice, s));
     }
-    scale_damp_kernel<<<dim3((n + 63) / 64, (n + 63) / 64), 256, 0, s>>>(H, n, h->hd, h->dead);
+    scale_damp_kernel<<<dim3((n + 63) / 64, (n + 15) / 16), 256, 0, s>>>(H, n, h->hd, h->dead);
     LAUNCHED();
 
     // reverse Cholesky H_d = R R^T, R upper, from the last block column upwards
@@ -1079,7 +1079,10 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
         const int np = (int)((n - sz + 2 * sz - 1) / (2 * sz));
         const int tail = (int)(n - (2 * sz * (np - 1) + sz));
         const int64_t bstride = 2 * sz * ((int64_t)n + 1);
-        if (h->f16 && damp > 0.f && sz >= 2 * NB) {
+        // few tiles: the plain float32 products of 32 x 32 tiles need no operand copies and beat the tensor cores'
+        // two splits and a product per factor
+        const bool few = np * (sz / GBM) * (sz / GBN) <= SIMT_SMALL_TILES;
+        if (h->f16 && damp > 0.f && sz >= 2 * NB && !few) {
             // The two products on the tensor cores with FP16-split operands.  Ranges: B holds entries of R
             // (bounded like the panels), the inverted blocks are bounded by 1 / sqrt(lambda), the
             // intermediate T records its own maximum in the first product's epilogue.
@@ -1114,7 +1117,7 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
             h->launches += 6;
             continue;
         }
-        if (h->tensor && !h->f16 && sz >= 2 * NB) {
+        if (h->tensor && !h->f16 && sz >= 2 * NB && !few) {
             // Same two products on the tensor cores, TF32-split operands (widths that are multiples of 4
             // only).  S1 holds K-major copies of the left operands at
             // their own coordinates (B, then A^-1), S2 the transposed right operands (C^-T, then T^T).
@@ -1144,7 +1147,7 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
             h->launches++;
             continue;
         }
-        // the 128-wide level, and every level of an fp16-split handle without damping (nothing bounds the
+        // the narrow levels, and every level of an fp16-split handle without damping (nothing bounds the
         // inverse in advance then): plain float32 products
         // T = B * C^-1
         GemmProblem p1 = make_problem(make_operand(H + sz, n, 1),

@@ -99,19 +99,35 @@ __global__ void __launch_bounds__(1024) diag_stats_kernel(const float *H, int n,
 
 // Upper triangle: H <- H * inv_tokens (+ lambda on the diagonal, dead -> 1 + lambda);
 // strict lower triangle <- 0.
+// Tiles of 64 columns x 16 rows, four columns of a row per thread: one load in flight per thread everywhere
+// (64 rows in a loop of dependent load-store pairs took 13 us at n = 1024).
 __global__ void __launch_bounds__(256) scale_damp_kernel(float *H, int n, const StateHeader *hd,
                                                          const uint8_t *dead) {
-    int j = blockIdx.x * 64 + (threadIdx.x & 63);
-    int ib = blockIdx.y * 64;
-    if (j >= n) return;
-    float inv = hd->inv_tokens, lam = hd->lambda;
-    for (int r = threadIdx.x >> 6; r < 64; r += 4) {
-        int i = ib + r;
-        if (i >= n) break;
-        float *p = H + (int64_t)i * n + j;
-        if (j < i) *p = 0.f;
-        else if (j == i) *p = (dead[i] ? 1.f : *p * inv) + lam;
-        else *p = *p * inv;
+    const int j = blockIdx.x * 64 + 4 * (threadIdx.x & 15), i = blockIdx.y * 16 + (threadIdx.x >> 4);
+    if (j >= n || i >= n) return;
+    const float inv = hd->inv_tokens, lam = hd->lambda;
+    float *p = H + (int64_t)i * n + j;
+    const bool vec = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(H) & 15) == 0;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (j + 3 >= i) {
+        if (vec) {
+            const float4 q = *reinterpret_cast<const float4 *>(p);
+            v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) if (j + e < n) v[e] = p[e];
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        if (j + e < i) v[e] = 0.f;
+        else if (j + e == i) v[e] = (dead[i] ? 1.f : v[e] * inv) + lam;
+        else v[e] *= inv;
+    }
+    if (vec) *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) if (j + e < n) p[e] = v[e];
     }
 }
 
@@ -522,25 +538,70 @@ __global__ void __launch_bounds__(FP_THREADS, 1) factor_panel_kernel(FactorPanel
 
 // ---------------------------------------------------------------------------
 // Inverts every NB x NB diagonal factor R_pp (one CTA each) and stores the inverse on the
-// diagonal of H (strict lower part of the block zero): the starting point of U = R^-1.
+// diagonal of H (strict lower part of the block zero): the starting point of U = R^-1.  Bound by shared-memory
+// reads: 4 x 4 outputs per thread (one output per thread, and divisions in the substitution, took 36 us; now 11).
 // 32 x 32 diagonal sub-blocks by back substitution (one warp each, lane = column), then
 // X12 = -X11 (R12 X22) for 32 -> 64 -> 128.
 // ---------------------------------------------------------------------------
-constexpr int ID_THREADS = 512;
-constexpr int ID_LD = NB + 1;
-constexpr size_t ID_SMEM = (2 * NB * ID_LD + 2 * 32 * 33) * sizeof(float);
+constexpr int ID_THREADS = 256;
+constexpr int ID_LD = NB + 4;
+constexpr size_t ID_SMEM = (2 * NB * ID_LD + 64 * 68 + NB) * sizeof(float);
+
+// C[i][j] = sign * sum_k A[i][k] B[k][j], S x S outputs, 4 x 4 per thread (rows ti + S / 4 e, four columns), all operands
+// row-major in shared memory; `t` counts the (S / 4)^2 threads of one product.
+template <int S>
+__device__ __forceinline__ void tile_product(float *C, int ldc, const float *A, int lda, const float *B, int ldb, int t, float sign) {
+    const int ti = t / (S / 4), tj = t % (S / 4);
+    float acc[4][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < S; k += 4) {
+        float av[4][4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float4 v = *reinterpret_cast<const float4 *>(A + (ti + S / 4 * e) * lda + k);
+            av[e][0] = v.x; av[e][1] = v.y; av[e][2] = v.z; av[e][3] = v.w;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 b = *reinterpret_cast<const float4 *>(B + (k + q) * ldb + 4 * tj);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                acc[e][0] = fmaf(av[e][q], b.x, acc[e][0]); acc[e][1] = fmaf(av[e][q], b.y, acc[e][1]);
+                acc[e][2] = fmaf(av[e][q], b.z, acc[e][2]); acc[e][3] = fmaf(av[e][q], b.w, acc[e][3]);
+            }
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        *reinterpret_cast<float4 *>(C + (ti + S / 4 * e) * ldc + 4 * tj) =
+            make_float4(sign * acc[e][0], sign * acc[e][1], sign * acc[e][2], sign * acc[e][3]);
+}
 
 __global__ void __launch_bounds__(ID_THREADS, 1) invert_diag_blocks_kernel(float *H, int n, const float *Rdiag) {
     extern __shared__ __align__(16) float smem_f[];
-    float (*S)[ID_LD] = reinterpret_cast<float (*)[ID_LD]>(smem_f);
-    float (*X)[ID_LD] = reinterpret_cast<float (*)[ID_LD]>(smem_f + NB * ID_LD);
-    float (*T32)[32][33] = reinterpret_cast<float (*)[32][33]>(smem_f + 2 * NB * ID_LD);
+    float *S = smem_f, *X = smem_f + NB * ID_LD, *T = X + NB * ID_LD, *dinv = T + 64 * 68;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b0 = blockIdx.x * NB;
     const float *src = Rdiag + (int64_t)blockIdx.x * NB * NB;
-    for (int idx = tid; idx < NB * NB; idx += ID_THREADS) {
-        S[idx >> 7][idx & 127] = src[idx];
-        X[idx >> 7][idx & 127] = 0.f;
+    float4 v[NB * NB / 4 / ID_THREADS];
+#pragma unroll
+    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) v[it] = *reinterpret_cast<const float4 *>(src + 4 * (tid + it * ID_THREADS));
+    if (tid < NB) dinv[tid] = 1.f / src[tid * NB + tid];
+#pragma unroll
+    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) {
+        const int i = (tid + it * ID_THREADS) >> 5, j4 = (tid + it * ID_THREADS) & 31;
+        *reinterpret_cast<float4 *>(S + i * ID_LD + 4 * j4) = v[it];
+        *reinterpret_cast<float4 *>(X + i * ID_LD + 4 * j4) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    // transposes of the 32 x 32 diagonal sub-blocks into their own lower parts, for the substitution
+    for (int idx = tid; idx < 4 * 1024; idx += ID_THREADS) {
+        const int o = 32 * (idx >> 10), i = (idx >> 5) & 31, j = idx & 31;
+        if (j > i) S[(o + j) * ID_LD + o + i] = S[(o + i) * ID_LD + o + j];
     }
     __syncthreads();
     if (warp < NB / 32) {
@@ -548,71 +609,33 @@ __global__ void __launch_bounds__(ID_THREADS, 1) invert_diag_blocks_kernel(float
         float x[32];
 #pragma unroll
         for (int i = 0; i < 32; ++i) x[i] = (i == lane) ? 1.f : 0.f;
+        InvColStep<31>::run(x, S + o * ID_LD + o, dinv + o);
 #pragma unroll
-        for (int i = 31; i >= 0; --i) {
-            x[i] = x[i] / S[o + i][o + i];
+        for (int i = 0; i < 32; ++i) X[(o + i) * ID_LD + o + lane] = x[i];
+    }
+    __syncthreads();
+    // X12 = -X11 (R12 X22), 32 -> 64 for both pairs, then 64 -> 128 (the triangular operands carry explicit zeros)
+    const int pr = tid >> 6, o = 64 * pr;
+    if (tid < 128) tile_product<32>(T + pr * 32 * 36, 36, S + o * ID_LD + o + 32, ID_LD, X + (o + 32) * ID_LD + o + 32, ID_LD, tid & 63, 1.f);
+    __syncthreads();
+    if (tid < 128) tile_product<32>(X + o * ID_LD + o + 32, ID_LD, X + o * ID_LD + o, ID_LD, T + pr * 32 * 36, 36, tid & 63, -1.f);
+    __syncthreads();
+    tile_product<64>(T, 68, S + 64, ID_LD, X + 64 * ID_LD + 64, ID_LD, tid, 1.f);
+    __syncthreads();
+    tile_product<64>(X + 64, ID_LD, X, ID_LD, T, 68, tid, -1.f);
+    __syncthreads();
+    const bool vec = (n & 3) == 0 && b0 + NB <= n;
+    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) {
+        const int i = (tid + it * ID_THREADS) >> 5, j = 4 * ((tid + it * ID_THREADS) & 31);
+        float x[4];
 #pragma unroll
-            for (int i2 = 0; i2 < i; ++i2) x[i2] = fmaf(-S[o + i2][o + i], x[i], x[i2]);
-        }
+        for (int e = 0; e < 4; ++e) x[e] = j + e >= i ? X[i * ID_LD + j + e] : 0.f;
+        float *dst = H + (int64_t)(b0 + i) * n + b0 + j;
+        if (vec) *reinterpret_cast<float4 *>(dst) = make_float4(x[0], x[1], x[2], x[3]);
+        else if (b0 + i < n) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) X[o + i][o + lane] = x[i];
-    }
-    __syncthreads();
-    // (the triangular operands carry explicit zeros, so full-length sums are exact)
-    for (int idx = tid; idx < 2 * 1024; idx += ID_THREADS) {
-        const int pr = idx >> 10, i = (idx >> 5) & 31, j = idx & 31;
-        const int oa = 64 * pr, oc = oa + 32;
-        float s0 = 0.f, s1 = 0.f;
-#pragma unroll 8
-        for (int k = 0; k < 32; k += 2) {
-            s0 = fmaf(S[oa + i][oc + k], X[oc + k][oc + j], s0);
-            s1 = fmaf(S[oa + i][oc + k + 1], X[oc + k + 1][oc + j], s1);
+            for (int e = 0; e < 4; ++e) if (b0 + j + e < n) dst[e] = x[e];
         }
-        T32[pr][i][j] = s0 + s1;
-    }
-    __syncthreads();
-    for (int idx = tid; idx < 2 * 1024; idx += ID_THREADS) {
-        const int pr = idx >> 10, i = (idx >> 5) & 31, j = idx & 31;
-        const int oa = 64 * pr, oc = oa + 32;
-        float s0 = 0.f, s1 = 0.f;
-#pragma unroll 8
-        for (int k = 0; k < 32; k += 2) {
-            s0 = fmaf(X[oa + i][oa + k], T32[pr][k][j], s0);
-            s1 = fmaf(X[oa + i][oa + k + 1], T32[pr][k + 1][j], s1);
-        }
-        X[oa + i][oc + j] = -(s0 + s1);
-    }
-    __syncthreads();
-    // T64 = R[0:64, 64:128] X[64:128, 64:128], parked in the (still unused) lower-left of X
-    for (int idx = tid; idx < 64 * 64; idx += ID_THREADS) {
-        const int i = idx >> 6, j = idx & 63;
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll 4
-        for (int k = 0; k < 64; k += 4) {
-            s0 = fmaf(S[i][64 + k], X[64 + k][64 + j], s0);
-            s1 = fmaf(S[i][64 + k + 1], X[64 + k + 1][64 + j], s1);
-            s2 = fmaf(S[i][64 + k + 2], X[64 + k + 2][64 + j], s2);
-            s3 = fmaf(S[i][64 + k + 3], X[64 + k + 3][64 + j], s3);
-        }
-        X[64 + i][j] = (s0 + s1) + (s2 + s3);
-    }
-    __syncthreads();
-    for (int idx = tid; idx < 64 * 64; idx += ID_THREADS) {
-        const int i = idx >> 6, j = idx & 63;
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll 4
-        for (int k = 0; k < 64; k += 4) {
-            s0 = fmaf(X[i][k], X[64 + k][j], s0);
-            s1 = fmaf(X[i][k + 1], X[64 + k + 1][j], s1);
-            s2 = fmaf(X[i][k + 2], X[64 + k + 2][j], s2);
-            s3 = fmaf(X[i][k + 3], X[64 + k + 3][j], s3);
-        }
-        X[i][64 + j] = -((s0 + s1) + (s2 + s3));
-    }
-    __syncthreads();
-    for (int idx = tid; idx < NB * NB; idx += ID_THREADS) {
-        const int i = idx >> 7, j = idx & 127;
-        if (b0 + i < n && b0 + j < n) H[(int64_t)(b0 + i) * n + (b0 + j)] = (j >= i) ? X[i][j] : 0.f;
     }
 }
 

@@ -7,7 +7,8 @@
 // triangular products with per-tile K ranges, and the stacked [Err | Wpre] *
 // [U ; P] trailing update.  It is the exact-fp32 reference path of the
 // library: the tensor-core kernels replace it where a product is large, and it
-// stays in use for ragged or small shapes.
+// stays in use for ragged or small shapes.  Products of few tiles take
+// simt_small_kernel below.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -244,10 +245,233 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(GemmProblem pr) {
     }
 }
 
-struct LaunchCounter;
+// ---------------------------------------------------------------------------
+// The same products where 128 x 128 tiles are few: 32 x 32 tiles, 64 threads, 4 x 4 outputs per thread, operands
+// through three 32-deep stages of asynchronous copies; the K range of a tile may be shared by a cluster of CTAs,
+// whose partial sums meet in distributed shared memory in a fixed order (deterministic, no scratch).
+// What bounds it: shared-memory reads (two 16-byte reads per 16 FMA: about half the FMA rate of the 128 x 128
+// form), so it pays while those tiles leave the chip idle.  A rank-128 update of 384 columns: 30 us as 128 x 128
+// tiles, 9 here; the statistics of 8192 tokens at n = 200: 2700 us there, 150 here.
+// ---------------------------------------------------------------------------
+constexpr int SGT = 32, SGK = 32, SG_LD = SGK + 4, SG_STAGES = 3, SG_THREADS = 64;
+constexpr int SG_TILE = SGT * SG_LD;                  // floats of one operand tile
+
+__device__ __forceinline__ void sg_copy16(float *dst, const float *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void sg_copy4(float *dst, const float *src, bool valid) {
+    // (a source size of 0 writes a zero and reads nothing)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
+
+// Operand rows row0 .. + 31, contraction steps k0 .. + 31 into a tile.  RC: tile[k][row], else tile[row][k].
+template <bool RC>
+__device__ __forceinline__ void sg_fetch(float *tile, const float *p, const float *p2, int k_split, int64_t rs, int64_t ks,
+                                         int row0, int R, int k0, int ke, int tid) {
+    const bool second = p2 != nullptr && k0 >= k_split;               // (k_split is a multiple of 32)
+    const float *base = second ? p2 : p;
+    const int kk0 = second ? k0 - k_split : k0;
+#pragma unroll
+    for (int it = 0; it < SGT * SGK / 4 / SG_THREADS; ++it) {
+        const int idx = tid + it * SG_THREADS, o = idx >> 3, c4 = (idx & 7) * 4;
+        float *dst = tile + o * SG_LD + c4;
+        const int row = RC ? row0 + c4 : row0 + o, k = RC ? o : c4;   // k: within the tile
+        const float *src = base + (RC ? (int64_t)(kk0 + k) * ks + row : (int64_t)row * rs + kk0 + k);
+        const int left = RC ? (k0 + k < ke ? R - row : 0) : (row < R ? ke - k0 - k : 0);      // valid elements of the four
+        if (left >= 4 && (reinterpret_cast<uintptr_t>(src) & 15) == 0) sg_copy16(dst, src);
+        else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sg_copy4(dst + e, e < left ? src + e : base, e < left);
+        }
+    }
+}
+
+template <bool A_RC, bool B_RC>
+__global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, int ksplit) {
+    extern __shared__ __align__(16) float sg_smem[];
+    const int tid = threadIdx.x;
+    const int z = blockIdx.z / ksplit, part = blockIdx.z - z * ksplit;
+    int M = pr.M, N = pr.N, K = pr.K;
+    if (z == pr.nbatch - 1) {
+        if (pr.batchM_last) M = pr.batchM_last;
+        if (pr.batchN_last) N = pr.batchN_last;
+        if (pr.batchK_last) K = pr.batchK_last;
+    }
+    const int i0 = blockIdx.y * SGT, j0 = blockIdx.x * SGT;
+    if (i0 >= M || j0 >= N) return;                                   // (the same for the CTAs of a cluster)
+    const int mode = pr.mode;
+    bool skip = false;
+    int kb = 0, ke = K;
+    if (mode == GEMM_UPPER_TILES) skip = i0 >= j0 + SGT;
+    else if (mode == GEMM_O) { skip = i0 >= j0 + SGT; kb = j0; }
+    else if (mode == GEMM_P) { skip = i0 >= j0 + SGT; kb = i0; ke = min(K, j0 + SGT); }
+    else if (mode == GEMM_TRI_RIGHT) ke = min(K, j0 + SGT);
+    else if (mode == GEMM_TRI_LEFT) kb = i0;
+    if (skip && mode != GEMM_P) return;
+    if (skip) ke = kb;
+    if (ksplit > 1) {
+        const int steps = max(0, (ke - kb + SGK - 1) / SGK);
+        const int b = kb + steps * part / ksplit * SGK, e = kb + steps * (part + 1) / ksplit * SGK;
+        kb = b; ke = min(ke, e);
+    }
+
+    const float *A = pr.A.p + z * pr.batchA, *B = pr.B.p + z * pr.batchB;
+    const float *A2 = pr.A.p2 ? pr.A.p2 + z * pr.batchA : nullptr, *B2 = pr.B.p2 ? pr.B.p2 + z * pr.batchB : nullptr;
+    const float *Asub = pr.A.sub ? pr.A.sub + z * pr.batchA : nullptr;
+    const int stage_floats = (Asub ? 3 : 2) * SG_TILE;
+    const int nk = max(0, (ke - kb + SGK - 1) / SGK);
+    auto fetch = [&](int t) {
+        if (t < nk) {
+            float *st = sg_smem + (t % SG_STAGES) * stage_floats;
+            const int k0 = kb + t * SGK;
+            sg_fetch<A_RC>(st, A, A2, pr.A.k_split, pr.A.rs, pr.A.ks, i0, M, k0, ke, tid);
+            sg_fetch<B_RC>(st + SG_TILE, B, B2, pr.B.k_split, pr.B.rs, pr.B.ks, j0, N, k0, ke, tid);
+            if (Asub) sg_fetch<A_RC>(st + 2 * SG_TILE, Asub, nullptr, 0, pr.A.rs, pr.A.ks, i0, M, k0, ke, tid);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    const int tj = tid & 7, ti = tid >> 3;
+    float acc[4][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
+    // rows 4 ti + e (tile[k][row]) or ti + 8 e (tile[row][k]), columns likewise
+    auto read4 = [&](const float *tile, bool rc, int t, int k, float (&v)[4][4]) {          // v[k][e]
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 x = *reinterpret_cast<const float4 *>(rc ? tile + (k + q) * SG_LD + 4 * t : tile + (t + 8 * q) * SG_LD + k);
+            const float xx[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { if (rc) v[q][e] = xx[e]; else v[e][q] = xx[e]; }
+        }
+    };
+#pragma unroll
+    for (int t = 0; t < SG_STAGES - 1; ++t) fetch(t);
+    // what C holds arrives under the products (read at the end, each value would wait for its own round trip)
+    float *C = pr.C + z * pr.batchC;
+    const bool masked = mode == GEMM_O || mode == GEMM_P;
+    const bool add_c = pr.beta != 0.f && !masked;
+    float cv[4][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            const int i = i0 + (A_RC ? 4 * ti + e : ti + 8 * e), j = j0 + (B_RC ? 4 * tj + f : tj + 8 * f);
+            cv[e][f] = (add_c && ksplit == 1 && i < M && j < N) ? C[(int64_t)i * pr.ldc + j] : 0.f;
+        }
+    for (int t = 0; t < nk; ++t) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(SG_STAGES - 2) : "memory");
+        __syncthreads();
+        fetch(t + SG_STAGES - 1);                                     // into the stage that was read last step
+        const float *st = sg_smem + (t % SG_STAGES) * stage_floats;
+#pragma unroll 2
+        for (int k = 0; k < SGK; k += 4) {
+            float av[4][4], bv[4][4];
+            read4(st, A_RC, ti, k, av);
+            read4(st + SG_TILE, B_RC, tj, k, bv);
+            if (Asub) {
+                float sv[4][4];
+                read4(st + 2 * SG_TILE, A_RC, ti, k, sv);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) av[q][e] = sv[q][e] - av[q][e];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int f = 0; f < 4; ++f) acc[e][f] = fmaf(av[q][e], bv[q][f], acc[e][f]);
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+
+    auto store = [&](int i, int j, float v, float c) {
+        if (i >= M || j >= N) return;
+        v *= pr.alpha;
+        if (masked && j <= i) v = 0.f;
+        C[(int64_t)i * pr.ldc + j] = add_c ? fmaf(pr.beta, c, v) : v;
+    };
+    if (ksplit == 1) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int f = 0; f < 4; ++f)
+                store(i0 + (A_RC ? 4 * ti + e : ti + 8 * e), j0 + (B_RC ? 4 * tj + f : tj + 8 * f), acc[e][f], cv[e][f]);
+        return;
+    }
+    // partial sums meet: every CTA of the cluster adds up its share of the rows, in the order of the parts
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+            sg_smem[(A_RC ? 4 * ti + e : ti + 8 * e) * SG_LD + (B_RC ? 4 * tj + f : tj + 8 * f)] = acc[e][f];
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const int rows = SGT / ksplit;
+    float own[SGT * SGT / 2 / SG_THREADS];               // (at least two parts)
+#pragma unroll
+    for (int q = 0; q < SGT * SGT / 2 / SG_THREADS; ++q) {
+        const int idx = tid + q * SG_THREADS, i = i0 + part * rows + (idx >> 5), j = j0 + (idx & 31);
+        own[q] = (add_c && idx < rows * SGT && i < M && j < N) ? C[(int64_t)i * pr.ldc + j] : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < SGT * SGT / 2 / SG_THREADS; ++q) {
+        const int idx = tid + q * SG_THREADS;
+        if (idx >= rows * SGT) break;
+        const int i = part * rows + (idx >> 5), j = idx & 31;
+        const uint32_t addr = (uint32_t)__cvta_generic_to_shared(sg_smem + i * SG_LD + j);
+        float v = 0.f;
+        for (int c = 0; c < ksplit; ++c) {
+            uint32_t remote;
+            float x;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(c));
+            asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(remote) : "memory");
+            v += x;
+        }
+        store(i0 + i, j0 + j, v, own[q]);
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// 128 x 128 tiles of a product (all batch entries; the skipped ones of a triangular mode count, a factor of two at most)
+inline int64_t simt_tiles(const GemmProblem &pr) {
+    return (int64_t)pr.nbatch * ((pr.M + GBM - 1) / GBM) * ((pr.N + GBN - 1) / GBN);
+}
+// Up to here the 32 x 32 form is the faster one: T tiles on 148 SMs cost ceil(T / 148) x 128 cycles per contraction
+// step as 128 x 128 tiles and about 16 T / 148 x 20 as 32 x 32 tiles.
+constexpr int64_t SIMT_SMALL_TILES = 60;
+
+template <bool A_RC, bool B_RC>
+inline cudaError_t launch_simt_small(const GemmProblem &pr, cudaStream_t s) {
+    dim3 grid((pr.N + SGT - 1) / SGT, (pr.M + SGT - 1) / SGT, pr.nbatch);
+    // long contractions of few tiles (the statistics of narrow layers) are shared by up to eight CTAs per tile
+    int ksplit = 1;
+    const int64_t tiles = (int64_t)grid.x * grid.y * grid.z;
+    while (ksplit < 8 && tiles * ksplit <= 592 && pr.K / (2 * ksplit) >= 128) ksplit *= 2;      // 592: four CTAs per SM
+    grid.z *= ksplit;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(SG_THREADS); cfg.stream = s;
+    cfg.dynamicSmemBytes = (size_t)SG_STAGES * (pr.A.sub ? 3 : 2) * SG_TILE * sizeof(float);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = (unsigned)ksplit;
+    cfg.attrs = attr; cfg.numAttrs = ksplit > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, simt_small_kernel<A_RC, B_RC>, pr, ksplit);
+}
 
 inline cudaError_t launch_simt_gemm(const GemmProblem &pr, bool a_rc, bool b_rc, cudaStream_t s) {
     if (pr.M <= 0 || pr.N <= 0 || pr.nbatch <= 0) return cudaSuccess;
+    if (simt_tiles(pr) <= SIMT_SMALL_TILES && !pr.B.sub) {
+        if (a_rc && b_rc) return launch_simt_small<true, true>(pr, s);
+        if (a_rc) return launch_simt_small<true, false>(pr, s);
+        if (b_rc) return launch_simt_small<false, true>(pr, s);
+        return launch_simt_small<false, false>(pr, s);
+    }
     dim3 grid((pr.N + GBN - 1) / GBN, (pr.M + GBM - 1) / GBM, pr.nbatch);
     if (a_rc && b_rc) simt_gemm_kernel<true, true><<<grid, 256, 0, s>>>(pr);
     else if (a_rc && !b_rc) simt_gemm_kernel<true, false><<<grid, 256, 0, s>>>(pr);

@@ -621,7 +621,8 @@ stats_umma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
                 } else {
 #pragma unroll
                     for (int q = 0; q < UBN / 2; ++q)
-                        if (col0 + q < a.n) cp[q] = fmaf(acc[q], inv, cp[q]);
+                        if (col0 + q < a.n)
+                            asm volatile("red.global.add.f32 [%0], %1;" ::"l"(cp + q), "f"(acc[q] * inv) : "memory");
                 }
             }
         }

@@ -688,3 +688,22 @@ def test_tensor_core_statistics_rescale_out_of_range_batches(scale, prec):
     assert np.isfinite(H).all() and np.isfinite(D).all()
     assert np.linalg.norm((H - so.H)[iu]) / np.linalg.norm(so.H[iu]) < 2.0 ** -10
     assert hp.rel_fro(np.triu(D, 1), np.triu(so.D, 1)) < 2.0 ** -10
+
+
+@pytest.mark.parametrize("n,m,tokens,group,B", [
+    (31, 5, 40, 0, 32),          # one tile, less than one of its rows and steps
+    (33, 33, 127, 32, 32),       # one row beyond a tile, contraction just below the shortest that is shared
+    (96, 40, 4097, 0, 32),       # contraction shared by eight CTAs, one step beyond whole ones
+    (250, 70, 2050, 32, 64),     # no aligned rows (4-byte copies), ragged in every direction
+    (385, 200, 900, 128, 128),   # more than a panel, one column beyond it
+])
+def test_small_float32_products(n, m, tokens, group, B):
+    """Products of few tiles (32 x 32 tiles, K shared by a cluster) in every step of a narrow float32 layer.  Sums of
+    `tokens` rounded products: each of the at most tokens / 8 additions of a part rounds by 2^-24 of the partial sum,
+    which averages to sqrt(tokens) * 2^-24; twice that is allowed."""
+    cfg = wl.scaled(wl.CONFIGS["cfg1"], name="small", n=n, m=m, batch_tokens=tokens, n_batches=2, group=group, blocksize=B,
+                    outlier_channels=2)
+    out = hp.check_layer(cfg, wl.make_weight(cfg), batches_of(cfg), stats_precision=g.GPTAQ_STATS_FP32)
+    hp.assert_parity(out)
+    bound = 2.0 ** -23 * np.sqrt(2 * tokens)
+    assert out["H_rel"] < bound and out["D_rel"] < 8 * bound, out       # (X~ - X cancels: 20 times smaller terms)
