@@ -116,19 +116,63 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
 }
 __device__ __forceinline__ float pick2(const unsigned long long (&v)[4], int j) { return (j & 1) ? hi2(v[j >> 1]) : lo2(v[j >> 1]); }
 
-// Range of a row over columns [c0, c1) of the slab, by the row's four lanes.
-__device__ __forceinline__ void row_range(const float *w, int c0, int c1, int sub, float &lo, float &hi, float &am) {
+// Range of a row over `len` columns (a multiple of 32) from w, by the row's four lanes.
+__device__ __forceinline__ void row_range(const float *w, int len, int sub, float &lo, float &hi) {
     lo = 0.f; hi = 0.f;
-    for (int c = c0 + sub; c < c1; c += 4) {
-        const float v = w[c];
-        lo = fminf(lo, v); hi = fmaxf(hi, v);
+#pragma unroll 2
+    for (int c = 4 * sub; c < len; c += 16) {
+        const float4 v = *reinterpret_cast<const float4 *>(w + c);
+        lo = fminf(lo, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
+        hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
     }
 #pragma unroll
     for (int d = 1; d < 4; d <<= 1) {
         lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, d));
         hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, d));
     }
-    am = fmaxf(-lo, hi);
+}
+
+// Least squared rounding error of one row's group among candidates k0, k0 + stride, ..: four candidates (two pairs) per
+// pass over the weights (`w`: n weights, n a multiple of 4, 16-byte aligned).
+__device__ __forceinline__ void clip_search(const float *w, int n, float lo, float hi, int bits, int sym, int steps, float clip_min,
+                                            int k0, int stride, float &best, int &kbest) {
+    const float am = fmaxf(-lo, hi), maxq = (float)((1 << bits) - 1), magic = 12582912.f;
+    const unsigned long long mg = pack2(magic, magic), nmg = pack2(-magic, -magic), one = pack2(1.f, 1.f);
+    best = INFINITY; kbest = 0;
+    for (int k = k0; k < steps; k += 4 * stride) {
+        float sc[4], iv[4], ql[4], qh[4];
+        unsigned long long err[2] = {0ull, 0ull};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float p = clip_ratio(min(k + e * stride, steps - 1), steps, clip_min);
+            float z;
+            make_grid(p * lo, p * hi, p * am, bits, sym, sc[e], z);
+            iv[e] = 1.f / sc[e]; ql[e] = -z; qh[e] = maxq - z;
+        }
+        const unsigned long long sc2[2] = {pack2(sc[0], sc[1]), pack2(sc[2], sc[3])}, iv2[2] = {pack2(iv[0], iv[1]), pack2(iv[2], iv[3])};
+        const unsigned long long zero2 = 0ull;
+        for (int c = 0; c < n; c += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(w + c);
+            const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int f = 0; f < 4; ++f) {
+                const unsigned long long x2 = pack2(x[f], x[f]), nx2 = pack2(-x[f], -x[f]);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    // round(w / scale) by adding and subtracting 1.5 * 2^23, products and sums rounded one by one
+                    const unsigned long long q = fma2(x2, iv2[h], zero2);
+                    const unsigned long long r = fma2(fma2(q, one, mg), one, nmg);
+                    const float c0 = fminf(fmaxf(lo2(r), ql[2 * h]), qh[2 * h]), c1 = fminf(fmaxf(hi2(r), ql[2 * h + 1]), qh[2 * h + 1]);
+                    const unsigned long long d = fma2(sc2[h], pack2(c0, c1), nx2);
+                    err[h] = fma2(d, d, err[h]);
+                }
+            }
+        }
+        const float er[4] = {lo2(err[0]), hi2(err[0]), lo2(err[1]), hi2(err[1])};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (k + e * stride < steps && er[e] < best) { best = er[e]; kbest = k + e * stride; }
+    }
 }
 
 // FAR: several blocks per launch, updates between them on the tensor cores.  PERCOL: static groups, a grid per column.
@@ -233,6 +277,20 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
     }
+    // the slab and the first rows of U and P all in flight at once (in batches through registers the prologue took 6 us
+    // of a launch, now 4)
+    const int cq = FAR ? nblk * (QB_W / 4) : B / 4;                // quads per row, padded columns included
+    const bool wvec = (a.ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(a.W) & 15) == 0;       // (i0 is a multiple of 32)
+    for (int idx = tid; idx < QB_ROWS * cq; idx += NTHREADS) {
+        const int r = idx / cq, c = 4 * (idx - r * cq);
+        float *dst = Ws + r * WLD + c;
+        const float *src = a.W + (int64_t)(row0 + r) * a.ldw + i0 + c;
+        if (wvec && r < nrows && c + 3 < cols) cp_async16(dst, src);
+        else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) dst[e] = r < nrows && c + e < cols ? src[e] : 0.f;
+        }
+    }
     fetch_up(i0, 0, tid, NTHREADS);
     if (tid < 32) { udinv2[tid] = load_pivot(i0 + tid); perm2[tid] = load_perm(i0 + tid); }
     if (PERCOL && tid < QB_NEAR) {
@@ -240,46 +298,19 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         load_grid(tid >> 3, i0 + 4 * (tid & 7), sc, zp);
         store_grid(tid >> 3, 4 * (tid & 7), sc, zp);
     }
-    {
-        const int cq = FAR ? nblk * (QB_W / 4) : B / 4;            // quads per row, padded columns included
-        for (int idx0 = 0; idx0 < QB_ROWS * cq; idx0 += 4 * NTHREADS) {
-            float4 v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int idx = idx0 + u * NTHREADS + tid;
-                const int r = idx / cq, c = 4 * (idx - r * cq);
-                v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (r < nrows && c < cols) {
-                    const float *src = a.W + (int64_t)(row0 + r) * a.ldw + i0 + c;
-                    if (c + 3 < cols && (reinterpret_cast<uintptr_t>(src) & 15) == 0) v[u] = *reinterpret_cast<const float4 *>(src);
-                    else {
-                        v[u].x = src[0];
-                        if (c + 1 < cols) v[u].y = src[1];
-                        if (c + 2 < cols) v[u].z = src[2];
-                        if (c + 3 < cols) v[u].w = src[3];
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int idx = idx0 + u * NTHREADS + tid;
-                const int r = idx / cq, c = 4 * (idx - r * cq);
-                if (r >= QB_ROWS) continue;
-                float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-                bool bad = false;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if (c + e < cols && a.dead[i0 + c + e]) x[e] = 0.f;       // dead inputs read as zero
-                    bad |= !isfinite(x[e]);
-                }
-                // a non-finite weight is reported from the value that was read: its code and dequantized value
-                // come out finite (the clamp absorbs NaN and Inf), so the results alone would not show it
-                if (bad) record_status(a.hd, ST_NONFINITE, row0 + r);
-                *reinterpret_cast<float4 *>(Ws + r * WLD + c) = make_float4(x[0], x[1], x[2], x[3]);
-            }
-        }
-    }
     asm volatile("cp.async.wait_all;" ::: "memory");
+    for (int idx = tid; idx < QB_ROWS * cq; idx += NTHREADS) {
+        const int r = idx / cq, c = 4 * (idx - r * cq);            // (the words that this thread has copied)
+        float4 *wp = reinterpret_cast<float4 *>(Ws + r * WLD + c);
+        const float4 v = *wp;
+        // dead inputs read as zero (the flags are 4-byte aligned and padded beyond n)
+        const uchar4 dd = c < cols ? *reinterpret_cast<const uchar4 *>(a.dead + i0 + c) : make_uchar4(0, 0, 0, 0);
+        const float x[4] = {dd.x ? 0.f : v.x, dd.y ? 0.f : v.y, dd.z ? 0.f : v.z, dd.w ? 0.f : v.w};
+        // a non-finite weight is reported from the value that was read: its code and dequantized value
+        // come out finite (the clamp absorbs NaN and Inf), so the results alone would not show it
+        if (!isfinite(x[0]) || !isfinite(x[1]) || !isfinite(x[2]) || !isfinite(x[3])) record_status(a.hd, ST_NONFINITE, row0 + r);
+        if (dd.x | dd.y | dd.z | dd.w) *wp = make_float4(x[0], x[1], x[2], x[3]);
+    }
     if (FAR) tc_fence_before();
     __syncthreads();
     if (FAR) tc_fence_after();
@@ -320,15 +351,16 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     }
                 } else if (a.group > 0 && (cg % a.group) == 0) {
                     // grid of the group that starts here, from the current values
-                    float lo, hi, am;
-                    row_range(wrow, co, min(co + a.group, cols), sub, lo, hi, am);
+                    // (columns of it beyond the layer are zeros)
+                    float lo, hi;
+                    row_range(wrow + co, a.group, sub, lo, hi);
                     float p = 1.f;
                     if (a.clip_steps > 0) {
                         named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);          // the near warps search
                         named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);
                         p = clip_ratio(reinterpret_cast<int *>(St)[lrow], a.clip_steps, a.clip_min);
                     }
-                    make_grid(p * lo, p * hi, p * am, a.bits, a.sym, scale, zero);
+                    make_grid(p * lo, p * hi, p * fmaxf(-lo, hi), a.bits, a.sym, scale, zero);
                     if (live && sub == 0) {
                         const int g = cg / a.group;
                         a.scales[(int64_t)row * a.G + g] = scale;
@@ -485,24 +517,15 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     // clipping-range search: thread = (row, one eighth of the candidates)
                     named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);     // the group's values are current
                     const int r = t & 31, cgi = t >> 5;
-                    const int gend = min(co + a.group, cols);
-                    const float *w = Ws + r * WLD;
-                    float lo = 0.f, hi = 0.f;
-                    for (int c = co; c < gend; ++c) {
-                        const float v = w[c];
-                        lo = fminf(lo, v); hi = fmaxf(hi, v);
+                    const float *w = Ws + r * WLD + co;
+                    float lo = 0.f, hi = 0.f, best;
+                    int kb;
+                    for (int c = 0; c < a.group; c += 4) {          // (columns beyond the layer are zeros)
+                        const float4 v = *reinterpret_cast<const float4 *>(w + c);
+                        lo = fminf(lo, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
+                        hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
                     }
-                    const float am = fmaxf(-lo, hi);
-                    float best = INFINITY;
-                    int kb = 0;
-                    for (int k = cgi; k < a.clip_steps; k += QB_NEAR / 32) {
-                        const float p = clip_ratio(k, a.clip_steps, a.clip_min);
-                        float sk, zk;
-                        make_grid(p * lo, p * hi, p * am, a.bits, a.sym, sk, zk);
-                        float err = 0.f;
-                        for (int c = co; c < gend; ++c) err += rounding_error_sq(w[c], sk, zk, maxq);
-                        if (err < best) { best = err; kb = k; }
-                    }
+                    clip_search(w, a.group, lo, hi, a.bits, a.sym, a.clip_steps, a.clip_min, cgi, QB_NEAR / 32, best, kb);
                     float *scratch = Sts + (s & 1) * 64 * QB_SLD;   // (the chain writes there only after this search)
                     float *be = scratch + 64;
                     int *bk = reinterpret_cast<int *>(be + QB_NEAR);
