@@ -17,6 +17,7 @@
 #include "simt_gemm.cuh"
 #include "umma_gemm.cuh"
 #include "tc_gemm.cuh"
+#include "factor.cuh"
 #include "quantize_block.cuh"
 
 using namespace gptaq;
@@ -101,6 +102,7 @@ inline bool tc_shape_ok(int64_t n) { return n >= TC_MIN_N && (n % 4) == 0; }
 
 struct WsLayout {
     size_t t_off, rinv_off;
+    size_t diag_off;        // inverses of the current diagonal block's sub-blocks, copy of the next diagonal block
     size_t s_off[6];        // split operand matrices (n x n each): S1 hi/lo, S2 hi/lo, S3 hi/lo
     size_t pan_off[2];      // split copy of factor panels, hi/lo: n x 128 float32 (TF32) or n x SUPER_NB fp16
     // [-Err | Wpre]: float32 (m x 2B, or m x 2 * QSUPER * B for the FP16-split update), second part
@@ -124,7 +126,8 @@ WsLayout ws_layout(int64_t n, int64_t m_max, int blocksize) {
     w.tensor = tc_shape_ok(n);
     w.t_off = 0;
     w.rinv_off = w.t_off + mat;
-    size_t off = w.rinv_off + round_up(nb * NB * NB * sizeof(float), ALIGN);
+    w.diag_off = w.rinv_off + round_up(nb * NB * NB * sizeof(float), ALIGN);
+    size_t off = w.diag_off + round_up((4 * 32 * FP_YLD + NB * NB) * sizeof(float), ALIGN);
     const bool f16 = w.tensor && (n % 8) == 0;
     // split operand copies: six float32-sized regions for TF32 parts; fp16 hi / lo parts use three
     // (S0 = U^T, S1 = U then P^T, S4 = dXX^T then O; hi and lo of one matrix fill one region)
@@ -842,7 +845,11 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
     cudaError_t e = cudaGetDevice(&h->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(factor_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FP_SMEM);
+        e = cudaFuncSetAttribute(diag_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DF_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(panel_solve_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(panel_solve_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM);
     if (e == cudaSuccess) e = configure_quantize_kernels();
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(invert_diag_blocks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ID_SMEM);
@@ -1007,32 +1014,17 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
     float *pan_hi = h->tensor ? reinterpret_cast<float *>(h->ws + wl.pan_off[0]) : nullptr;
     float *pan_lo = h->tensor ? reinterpret_cast<float *>(h->ws + wl.pan_off[1]) : nullptr;
     TcMaps pan_maps;
+    std::memset(static_cast<void *>(&pan_maps), 0, sizeof(pan_maps));
     const int pan_ld = h->f16 ? SUPER_NB : NB;
     if (h->tensor) {
         const SplitOperand pan{pan_hi, pan_lo, n, pan_ld, pan_ld, h->f16};
         if (!make_tc_maps(&pan_maps, pan, pan, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
     }
-    for (int p = nb - 1; p >= 0; --p) {
+    float *Y = reinterpret_cast<float *>(h->ws + wl.diag_off), *next_diag = Y + 4 * 32 * FP_YLD;
+    // rank-NB (or super-panel) update of the columns to the left of panel p, on stream `us` with at most `sms` CTAs
+    auto update = [&](int p, cudaStream_t us, int sms) -> gptaq_status_t {
         const int b0 = p * NB;
-        const int s0 = h->f16 ? b0 / SUPER_NB * SUPER_NB : b0;      // first column of this panel's super-panel
-        // diagonal block (factor + inverse) and the panel above it: R[0:b0, blk] = A[0:b0, blk] inv(R_pp)^T
-        FactorPanelArgs fa;
-        fa.H = H; fa.n = n; fa.b0 = b0; fa.Rdiag = Rinv + (size_t)p * NB * NB;
-        fa.pan_hi = pan_hi; fa.pan_lo = pan_lo; fa.pan_f16 = h->f16 ? 1 : 0; fa.hd = h->hd;
-        fa.pan_ld = pan_ld; fa.pan_col0 = b0 - s0;
-        // rows above the block in tiles of 32, 64 or 128 rows: the smallest tile that still gives every
-        // SM at most one tile spreads a short panel over more SMs (the diagonal block is refactored by
-        // every CTA either way)
-        int tr = 32;
-        while (tr < NB && b0 / tr > h->num_sms) tr *= 2;
-        fa.tile_rows = tr;
-        const int fgrid = std::max(1, std::min(b0 / tr, h->num_sms));
-        fa.rows_per_cta = ((b0 + fgrid - 1) / fgrid + tr - 1) / tr * tr;
-        // one more CTA, without a slab, stores the diagonal factor while there is an SM left for it
-        const int fextra = (b0 > 0 && fgrid < h->num_sms) ? 1 : 0;
-        CU(launch_pdl(true, factor_panel_kernel, dim3(fgrid + fextra), dim3(FP_THREADS), FP_SMEM, s, fa));
-        h->launches++;
-        if (p == 0) break;
+        const int s0 = h->f16 ? b0 / SUPER_NB * SUPER_NB : b0;
         if (h->f16 && b0 >= TC_MIN_N) {
             const unsigned *am = h->hd->tc_amax + AMAX_PAN;
             if (b0 > s0) {
@@ -1040,27 +1032,73 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
                 TcGemmArgs g = tc_args(H + s0, n, b0, b0 - s0, NB, -1.f, 1.f, TC_UPPER_TILES, TC_MASK_UPPER_KEEP, h->hd);
                 g.diag_off = s0; g.a_k0 = g.b_k0 = b0 - s0; g.b_row0 = s0;
                 g.amax_a = g.amax_b = am;
-                CU(launch_tc_gemm(pan_maps, g, h->sched, h->num_sms, s));
+                CU(launch_tc_gemm(pan_maps, g, h->sched, sms, us));
             } else {
                 // super-panel [s0, s1) done: A[0:s0, 0:s0] -= R[0:s0, s0:s1] R[0:s0, s0:s1]^T  (upper part)
                 const int s1 = std::min(s0 + SUPER_NB, nb * NB);
                 TcGemmArgs g = tc_args(H, n, s0, s0, s1 - s0, -1.f, 1.f, TC_UPPER_TILES, TC_MASK_UPPER_KEEP, h->hd);
                 g.amax_a = g.amax_b = am;
-                CU(launch_tc_gemm(pan_maps, g, h->sched, h->num_sms, s));
+                CU(launch_tc_gemm(pan_maps, g, h->sched, sms, us));
             }
             h->launches++;
-            continue;
+            return GPTAQ_OK;
         }
         // A[0:b0, 0:b0] -= R[0:b0, blk] R[0:b0, blk]^T  (upper part)
         if (h->tensor && b0 >= TC_MIN_N) {
             TcGemmArgs g = tc_args(H, n, b0, b0, NB, -1.f, 1.f, TC_UPPER_TILES, TC_MASK_UPPER_KEEP, h->hd);
-            CU(launch_tc_gemm(pan_maps, g, h->sched, h->num_sms, s));
+            CU(launch_tc_gemm(pan_maps, g, h->sched, sms, us));
             h->launches++;
-        } else {
-            Operand rp = make_operand(H + b0, n, 1);
-            GemmProblem ps = make_problem(rp, rp, H, n, b0, b0, std::min(NB, n - b0), -1.f, 1.f, GEMM_UPPER_TILES);
-            OK(gemm(h, ps, false, false, s));
+            return GPTAQ_OK;
         }
+        Operand rp = make_operand(H + b0, n, 1);
+        GemmProblem ps = make_problem(rp, rp, H, n, b0, b0, std::min(NB, n - b0), -1.f, 1.f, GEMM_UPPER_TILES);
+        return gemm(h, ps, false, false, us);
+    };
+    auto factor_diag = [&](int p, const float *src, int64_t lds, int syrk, int pan_col0) -> gptaq_status_t {
+        DiagFactorArgs da;
+        da.src = src; da.lds = lds; da.n = n; da.b0 = p * NB; da.Rdiag = Rinv + (size_t)p * NB * NB; da.Y = Y;
+        da.syrk = syrk; da.pan_col0 = pan_col0; da.hd = h->hd;
+        CU(launch_pdl(true, diag_factor_kernel, dim3(1), dim3(DF_THREADS), DF_SMEM, s, pan_maps.a_hi, pan_maps.a_lo, da));
+        h->launches++;
+        return GPTAQ_OK;
+    };
+    bool diag_done = false;                     // the diagonal block of this panel was factored beside the last update
+    for (int p = nb - 1; p >= 0; --p) {
+        const int b0 = p * NB;
+        const int s0 = h->f16 ? b0 / SUPER_NB * SUPER_NB : b0;      // first column of this panel's super-panel
+        if (!diag_done) OK(factor_diag(p, H + (int64_t)b0 * n + b0, n, 0, 0));
+        const bool early = diag_done;           // (then the update of this panel's columns was waited for, not overlapped)
+        diag_done = false;
+        if (p == 0) break;
+        const bool ahead = h->f16 && b0 > s0;   // the next panel is in the same super-panel: its block needs this panel only
+        PanelSolveArgs pa;
+        pa.H = H; pa.n = n; pa.b0 = b0; pa.Rdiag = Rinv + (size_t)p * NB * NB; pa.Y = Y;
+        pa.pan_hi = pan_hi; pa.pan_lo = pan_lo; pa.pan_f16 = h->f16 ? 1 : 0;
+        pa.pan_ld = pan_ld; pa.pan_col0 = b0 - s0; pa.hd = h->hd;
+        pa.next_diag = ahead ? next_diag : nullptr;
+        pa.early = early ? 1 : 0;
+        // a warp per 4 rows while that fills no SM beyond PS_WORKERS warps, per 8 rows beyond; as few warps per CTA as give
+        // every SM at most one CTA
+        const int rpt = b0 / 4 <= PS_WORKERS * h->num_sms ? 1 : 2;
+        const int groups = b0 / (4 * rpt);
+        pa.workers = std::max(1, std::min(PS_WORKERS, (groups + h->num_sms - 1) / h->num_sms));
+        const int slabs = std::min((groups + pa.workers - 1) / pa.workers, h->num_sms);
+        const dim3 pg(slabs + (ahead ? 1 : 0));
+        if (rpt == 1) CU(launch_pdl(true, panel_solve_kernel<1>, pg, dim3(PS_THREADS), PS_SMEM, s, pa));
+        else CU(launch_pdl(true, panel_solve_kernel<2>, pg, dim3(PS_THREADS), PS_SMEM, s, pa));
+        h->launches++;
+        if (!ahead) {
+            OK(update(p, s, h->num_sms));
+            continue;
+        }
+        // the update on the internal stream, the next diagonal block beside it (one SM is left free for it)
+        CU(cudaEventRecord(h->conv_done[0], s));
+        CU(cudaStreamWaitEvent(h->gemm_stream, h->conv_done[0], 0));
+        OK(update(p, h->gemm_stream, h->num_sms - 1));
+        CU(cudaEventRecord(h->gemm_done[0], h->gemm_stream));
+        OK(factor_diag(p - 1, next_diag, NB, 1, b0 - s0));
+        CU(cudaStreamWaitEvent(s, h->gemm_done[0], 0));
+        diag_done = true;
     }
 
     // U = R^-1: inverted diagonal blocks, then off-diagonal blocks by doubling:

@@ -132,514 +132,6 @@ __global__ void __launch_bounds__(256) scale_damp_kernel(float *H, int n, const 
 }
 
 // ---------------------------------------------------------------------------
-// One panel step of the reverse Cholesky  H_d = R R^T  (R upper), block column
-// [b0, b0 + NB):
-//   1. factor the NB x NB diagonal block from its last row/column upwards in shared memory,
-//      32 columns at a time: one warp factors the 32 x 32 diagonal sub-block in registers
-//      (lane = row, shuffles), the rows above it are solved against the sub-block one thread per
-//      row, and the leading part receives the rank-32 update (all threads, the tiles of the upper
-//      triangle numbered densely);
-//   2. rows above the block:  R[0:b0, blk] = A[0:b0, blk] * R_pp^-T, 32 columns at a time: a product
-//      with the inverse of the 32 x 32 diagonal sub-block (the four inverses: one warp each, lane =
-//      column), then a rank-32 update of the columns to the left, all threads on both; written back in place and, if asked for, as split parts for the tensor-core rank update.
-// Every CTA repeats step 1 (it is short and the other SMs would idle) and then takes a
-// slab of rows of step 2, whose first tile is fetched while step 1 runs; the last CTA stores R_pp for
-// invert_diag_blocks_kernel.  Rows/columns beyond n are padded with the identity.
-// ---------------------------------------------------------------------------
-constexpr int NB = 128;
-constexpr int FP_THREADS = 512;
-constexpr int FP_WARPS = FP_THREADS / 32;
-constexpr int FP_LD = NB + 4;
-constexpr int FP_YLD = 36;
-constexpr size_t FP_SMEM = (2 * NB * FP_LD + 32 * FP_LD + 4 * 32 * FP_YLD + NB + 64) * sizeof(float);
-
-struct FactorPanelArgs {
-    float *H; int n; int b0;
-    float *Rdiag;              // NB x NB (ld NB): the diagonal factor R_pp (upper, zeros below)
-    float *pan_hi, *pan_lo;    // nullptr, or [n][NB]: TF32 parts of the panel rows
-    int pan_f16;               // the two arrays hold __half instead: fp16 parts of split_scale(tc_amax[AMAX_PAN]) * row,
-    int pan_ld, pan_col0;      //   row pitch pan_ld, this panel at columns pan_col0 .. + NB (several panels side by side)
-    int rows_per_cta;          // slab of step 2, a multiple of tile_rows
-    int tile_rows;             // rows of the slab processed at a time: 32, 64 or 128
-    StateHeader *hd;
-};
-
-template <int K, int LEN>
-struct SolveRowStep {
-    static __device__ __forceinline__ void run(float (&a)[LEN], const float *Rt, int ld, const float *dinv) {
-        const float x = a[K] * dinv[K];
-        a[K] = x;
-        const float *col = Rt + K * ld;
-#pragma unroll
-        for (int j4 = 0; j4 < (K + 3) / 4; ++j4) {
-            const float4 r = *reinterpret_cast<const float4 *>(col + 4 * j4);
-            if (4 * j4 + 0 < K) a[4 * j4 + 0] = fmaf(-x, r.x, a[4 * j4 + 0]);
-            if (4 * j4 + 1 < K) a[4 * j4 + 1] = fmaf(-x, r.y, a[4 * j4 + 1]);
-            if (4 * j4 + 2 < K) a[4 * j4 + 2] = fmaf(-x, r.z, a[4 * j4 + 2]);
-            if (4 * j4 + 3 < K) a[4 * j4 + 3] = fmaf(-x, r.w, a[4 * j4 + 3]);
-        }
-        SolveRowStep<K - 1, LEN>::run(a, Rt, ld, dinv);
-    }
-};
-template <int LEN>
-struct SolveRowStep<-1, LEN> {
-    static __device__ __forceinline__ void run(float (&)[LEN], const float *, int, const float *) {}
-};
-template <int LEN>
-__device__ __forceinline__ void solve_row(float (&a)[LEN], const float *Rt, int ld, const float *dinv) {
-    SolveRowStep<LEN - 1, LEN>::run(a, Rt, ld, dinv);
-}
-
-// One column step (K, then K - 1, ... 0) of the 32 x 32 reverse Cholesky held one row per lane.
-// `piv` is the pivot of this step, already broadcast: the dependent chain from one pivot to the
-// next runs through lane K - 1 alone (its own c), the other lanes' updates overlap with it.
-// The scaled column c reaches the other lanes through shared memory (cv: two buffers of 32 floats,
-// read back as broadcast float4s): K shuffles per step, one per element, cost three times as much.
-// A pivot that is not a positive normal number is replaced by 1 without a branch, and off the chain
-// (the estimate is taken from the pivot as it comes, the test runs beside it); the first such column
-// is remembered in bad_col (-1: none) and reported after the block.
-template <int K>
-struct Chol32Step {
-    static __device__ __forceinline__ void run(float (&d)[32], float piv, int lane, float *dinv, float *cv, int &bad_col) {
-        // 1/sqrt(piv): hardware estimate plus one Newton step (to about one ulp)
-        float rinv;
-        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rinv) : "f"(piv));
-        rinv = rinv * fmaf(-0.5f * piv, rinv * rinv, 1.5f);
-        const bool bad = !(piv >= 1.17549435e-38f) || !(piv < INFINITY);
-        bad_col = (bad && bad_col < 0) ? K : bad_col;
-        piv = bad ? 1.f : piv;
-        rinv = bad ? 1.f : rinv;
-        const float c = lane < K ? d[K] * rinv : 0.f;
-        d[K] = lane < K ? c : (lane == K ? piv * rinv : 0.f);
-        if (lane == K) dinv[K] = rinv;
-        float next = 0.f;
-        if (K > 0) {
-            next = __shfl_sync(0xffffffffu, fmaf(-c, c, d[K - 1]), K - 1);
-            float *buf = cv + 32 * (K & 1);
-            buf[lane] = c;
-            __syncwarp();
-#pragma unroll
-            for (int j4 = (K - 1) / 4; j4 >= 0; --j4) {
-                const float4 cj = *reinterpret_cast<const float4 *>(buf + 4 * j4);
-                if (4 * j4 + 3 < K) d[4 * j4 + 3] = fmaf(-c, cj.w, d[4 * j4 + 3]);
-                if (4 * j4 + 2 < K) d[4 * j4 + 2] = fmaf(-c, cj.z, d[4 * j4 + 2]);
-                if (4 * j4 + 1 < K) d[4 * j4 + 1] = fmaf(-c, cj.y, d[4 * j4 + 1]);
-                if (4 * j4 + 0 < K) d[4 * j4 + 0] = fmaf(-c, cj.x, d[4 * j4 + 0]);
-            }
-        }
-        Chol32Step<K - 1>::run(d, next, lane, dinv, cv, bad_col);
-    }
-};
-template <>
-struct Chol32Step<-1> {
-    static __device__ __forceinline__ void run(float (&)[32], float, int, float *, float *, int &) {}
-};
-
-// One column step (from 31 down to 0) of the inversion of a 32 x 32 upper triangular block held in
-// shared memory as its transpose (Rt[k][i] = R[i][k], leading dimension FP_LD): lane = column of the
-// inverse, y = that column, dinv = reciprocal diagonal of R.
-template <int K>
-struct InvColStep {
-    static __device__ __forceinline__ void run(float (&y)[32], const float *Rt, const float *dinv) {
-        const float x = y[K] * dinv[K];
-        y[K] = x;
-        const float *col = Rt + K * FP_LD;
-#pragma unroll
-        for (int j4 = 0; j4 < (K + 3) / 4; ++j4) {
-            const float4 r = *reinterpret_cast<const float4 *>(col + 4 * j4);
-            if (4 * j4 + 0 < K) y[4 * j4 + 0] = fmaf(-x, r.x, y[4 * j4 + 0]);
-            if (4 * j4 + 1 < K) y[4 * j4 + 1] = fmaf(-x, r.y, y[4 * j4 + 1]);
-            if (4 * j4 + 2 < K) y[4 * j4 + 2] = fmaf(-x, r.z, y[4 * j4 + 2]);
-            if (4 * j4 + 3 < K) y[4 * j4 + 3] = fmaf(-x, r.w, y[4 * j4 + 3]);
-        }
-        InvColStep<K - 1>::run(y, Rt, dinv);
-    }
-};
-template <>
-struct InvColStep<-1> {
-    static __device__ __forceinline__ void run(float (&)[32], const float *, const float *) {}
-};
-
-// C[0:rows, 0:o] -= X * Rt-columns:  C[r][j] -= sum_l Xt[l][r] * Rt[l][j]  with Xt (32 x rows) and Rt (32 x o)
-// in shared memory, leading dimension FP_LD.  RT rows x 4 columns per thread, all threads of the CTA.
-template <int RT>
-__device__ __forceinline__ void slab_rank32_update(float (*C)[FP_LD], const float (*Xt)[FP_LD], const float (*Rt)[FP_LD],
-                                                   int o, int tid, int rows) {
-    const int tj = o / 4;
-    for (int t = tid; t < (rows / RT) * tj; t += FP_THREADS) {
-        const int ti = t / tj, j0 = 4 * (t - ti * tj);
-        float acc[RT][4];
-#pragma unroll
-        for (int e = 0; e < RT; ++e)
-#pragma unroll
-            for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
-#pragma unroll 8
-        for (int l = 0; l < 32; ++l) {
-            float xv[RT];
-            if (RT == 2) {
-                const float2 x2 = *reinterpret_cast<const float2 *>(&Xt[l][2 * ti]);
-                xv[0] = x2.x; xv[RT - 1] = x2.y;
-            } else {
-                xv[0] = Xt[l][ti];
-            }
-            const float4 rv = *reinterpret_cast<const float4 *>(&Rt[l][j0]);
-#pragma unroll
-            for (int e = 0; e < RT; ++e) {
-                acc[e][0] = fmaf(xv[e], rv.x, acc[e][0]); acc[e][1] = fmaf(xv[e], rv.y, acc[e][1]);
-                acc[e][2] = fmaf(xv[e], rv.z, acc[e][2]); acc[e][3] = fmaf(xv[e], rv.w, acc[e][3]);
-            }
-        }
-#pragma unroll
-        for (int e = 0; e < RT; ++e) {
-            float4 *cp = reinterpret_cast<float4 *>(&C[RT * ti + e][j0]);
-            float4 v = *cp;
-            v.x -= acc[e][0]; v.y -= acc[e][1]; v.z -= acc[e][2]; v.w -= acc[e][3];
-            *cp = v;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(FP_THREADS, 1) factor_panel_kernel(FactorPanelArgs a) {
-    extern __shared__ __align__(16) float smem_f[];
-    // S: the block as it is read, then R in the upper part and R^T in the lower part
-    float (*S)[FP_LD] = reinterpret_cast<float (*)[FP_LD]>(smem_f);
-    float (*At)[FP_LD] = reinterpret_cast<float (*)[FP_LD]>(smem_f + NB * FP_LD);         // step 2: a tile of panel rows
-    float (*Pt)[FP_LD] = reinterpret_cast<float (*)[FP_LD]>(smem_f + 2 * NB * FP_LD);     // Pt[k][i]: 32 solved columns, transposed
-    float *Yt = smem_f + 2 * NB * FP_LD + 32 * FP_LD;       // [4][32][FP_YLD]: Yt[c][l][j] = inv(R_cc)[j][l]
-    float *dinv = Yt + 4 * 32 * FP_YLD;                     // [NB] 1 / R_jj
-    float *cv = dinv + NB;                                  // 2 x 32: the scaled column of the running 32 x 32 step
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n = a.n, b0 = a.b0;
-    const int nv = min(NB, n - b0);
-    const bool vec = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(a.H) & 15) == 0 && nv == NB;
-    const int TR = a.tile_rows;
-    const int r_begin = blockIdx.x * a.rows_per_cta;
-    const int r_end = min(b0, r_begin + a.rows_per_cta);
-    pdl_launch_dependents();
-    pdl_wait();
-
-    // the block, read along rows (all loads in flight before the first store); only j >= i is used
-    if (vec) {
-        float4 v[NB * NB / 4 / FP_THREADS];
-#pragma unroll
-        for (int it = 0; it < NB * NB / 4 / FP_THREADS; ++it) {
-            const int idx = tid + it * FP_THREADS, i = idx >> 5, j4 = idx & 31;
-            v[it] = *reinterpret_cast<const float4 *>(a.H + (int64_t)(b0 + i) * n + b0 + 4 * j4);
-        }
-        // the first tile of this CTA's slab follows asynchronously
-        if (r_begin < r_end) {
-            for (int idx = tid; idx < TR * (NB / 4); idx += FP_THREADS) {
-                const int i = idx >> 5, j4 = idx & 31;
-                const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&At[i][4 * j4]);
-                const float *src = a.H + (int64_t)(r_begin + i) * n + b0 + 4 * j4;
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-            }
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-#pragma unroll
-        for (int it = 0; it < NB * NB / 4 / FP_THREADS; ++it) {
-            const int idx = tid + it * FP_THREADS, i = idx >> 5, j4 = idx & 31;
-            *reinterpret_cast<float4 *>(&S[i][4 * j4]) = v[it];
-        }
-    } else {
-        for (int i = warp; i < NB; i += FP_WARPS) {
-            const float *src = a.H + (int64_t)(b0 + i) * n + b0;
-            for (int j = lane; j < NB; j += 32) {
-                float v = (i == j) ? 1.f : 0.f;
-                if (i < nv && j < nv && j >= i) v = src[j];
-                S[i][j] = v;
-            }
-        }
-    }
-    __syncthreads();
-
-    // ---- step 1
-    for (int sb = NB / 32 - 1; sb >= 0; --sb) {
-        const int o = 32 * sb;
-        if (warp == 0) {
-            // 32 x 32 reverse Cholesky in registers, lane = row
-            float d[32];
-#pragma unroll
-            for (int j = 0; j < 32; ++j) d[j] = (j >= lane) ? S[o + lane][o + j] : S[o + j][o + lane];
-            int bad_col = -1;
-            Chol32Step<31>::run(d, __shfl_sync(0xffffffffu, d[31], 31), lane, dinv + o, cv, bad_col);
-            if (bad_col >= 0 && lane == 0 && blockIdx.x == 0) record_status(a.hd, ST_NOT_SPD, b0 + o + bad_col);
-            // R_ss to the upper part, its transpose to the lower part
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-                if (j >= lane) { S[o + lane][o + j] = d[j]; S[o + j][o + lane] = d[j]; }
-        }
-        if (o == 0) break;
-        __syncthreads();
-        // rows above: x R_ss^T = S[i, sub], one thread per row; results go to the upper part,
-        // to the lower part (transposed) and to Pt for the update
-        if (tid < o) {
-            const int i = tid;
-            float x[32];
-#pragma unroll
-            for (int k = 0; k < 32; ++k) x[k] = S[i][o + k];
-            solve_row<32>(x, &S[o][o], FP_LD, dinv + o);
-#pragma unroll
-            for (int k = 0; k < 32; ++k) { S[i][o + k] = x[k]; S[o + k][i] = x[k]; Pt[k][i] = x[k]; }
-        }
-        __syncthreads();
-        // leading part: S[i][j] -= X[i] . X[j] for i <= j < o, 4 x 4 per thread; the tiles of the upper
-        // triangle are numbered through a (q / 2) x (q + 1) rectangle so that the active threads are dense
-        {
-            const int q = o / 4;
-            for (int t = tid; t < (q / 2) * (q + 1); t += FP_THREADS) {
-                const int r = t / (q + 1), c = t - r * (q + 1);
-                const int ti = c > r ? r : q - 1 - r, tj = c > r ? c - 1 : q - 1 - r + c;
-                float acc[4][4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
-#pragma unroll 8
-                for (int k = 0; k < 32; ++k) {
-                    const float4 ri = *reinterpret_cast<const float4 *>(&Pt[k][4 * ti]);
-                    const float4 rj = *reinterpret_cast<const float4 *>(&Pt[k][4 * tj]);
-                    const float av[4] = {ri.x, ri.y, ri.z, ri.w}, bv[4] = {rj.x, rj.y, rj.z, rj.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-#pragma unroll
-                        for (int f = 0; f < 4; ++f) acc[e][f] = fmaf(av[e], bv[f], acc[e][f]);
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    float4 *cp = reinterpret_cast<float4 *>(&S[4 * ti + e][4 * tj]);
-                    float4 v = *cp;
-                    v.x -= acc[e][0]; v.y -= acc[e][1]; v.z -= acc[e][2]; v.w -= acc[e][3];
-                    *cp = v;
-                }
-            }
-        }
-        __syncthreads();
-    }
-    __syncthreads();
-
-    // (the last CTA: the host adds one without a slab while there are SMs left)
-    if (blockIdx.x == gridDim.x - 1)
-        for (int idx = tid; idx < NB * NB; idx += FP_THREADS) {
-            const int i = idx >> 7, j = idx & 127;
-            a.Rdiag[idx] = j >= i ? S[i][j] : 0.f;
-        }
-    if (b0 == 0 || r_begin >= r_end) return;
-
-    // the inverses of the four 32 x 32 diagonal sub-blocks (one warp each, lane = column)
-    if (warp < NB / 32) {
-        const int o = 32 * warp;
-        float y[32];
-#pragma unroll
-        for (int k = 0; k < 32; ++k) y[k] = (k == lane) ? 1.f : 0.f;
-        InvColStep<31>::run(y, &S[o][o], dinv + o);
-        float *dst = Yt + (warp * 32 + lane) * FP_YLD;
-#pragma unroll
-        for (int k4 = 0; k4 < 8; ++k4)
-            *reinterpret_cast<float4 *>(dst + 4 * k4) = make_float4(y[4 * k4], y[4 * k4 + 1], y[4 * k4 + 2], y[4 * k4 + 3]);
-    }
-
-    // ---- step 2: rows [r_begin, r_end) of the panel in tiles of TR rows
-    for (int r0 = r_begin; r0 < r_end; r0 += TR) {        // b0 and the slabs are multiples of TR
-        if (vec) {
-            if (r0 != r_begin) {
-                for (int idx = tid; idx < TR * (NB / 4); idx += FP_THREADS) {
-                    const int i = idx >> 5, j4 = idx & 31;
-                    *reinterpret_cast<float4 *>(&At[i][4 * j4]) =
-                        *reinterpret_cast<const float4 *>(a.H + (int64_t)(r0 + i) * n + b0 + 4 * j4);
-                }
-            } else {
-                asm volatile("cp.async.wait_all;" ::: "memory");
-            }
-        } else {
-            for (int i = warp; i < TR; i += FP_WARPS) {
-                const float *src = a.H + (int64_t)(r0 + i) * n + b0;
-                for (int k = lane; k < NB; k += 32) At[i][k] = k < nv ? src[k] : 0.f;
-            }
-        }
-        __syncthreads();
-        for (int sb = NB / 32 - 1; sb >= 0; --sb) {
-            const int o = 32 * sb;
-            // X = At[:, o : o + 32] * inv(R_ss)^T, a row and four columns per thread; to Pt (transposed)
-            const float *Ys = Yt + sb * 32 * FP_YLD;
-            for (int t = tid; t < TR * 8; t += FP_THREADS) {
-                const int r = t >> 3, j0 = 4 * (t & 7);
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int l4 = 0; l4 < 8; ++l4) {
-                    const float4 av = *reinterpret_cast<const float4 *>(&At[r][o + 4 * l4]);
-                    const float al[4] = {av.x, av.y, av.z, av.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float4 yv = *reinterpret_cast<const float4 *>(Ys + (4 * l4 + e) * FP_YLD + j0);
-                        acc[0] = fmaf(al[e], yv.x, acc[0]);
-                        acc[1] = fmaf(al[e], yv.y, acc[1]);
-                        acc[2] = fmaf(al[e], yv.z, acc[2]);
-                        acc[3] = fmaf(al[e], yv.w, acc[3]);
-                    }
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) Pt[j0 + e][r] = acc[e];
-            }
-            __syncthreads();
-            // the solved columns back into the tile; columns to the left: At[r][j] -= sum_l X[r][l] R[j][o + l]
-            for (int t = tid; t < TR * 8; t += FP_THREADS) {
-                const int r = t >> 3, j0 = 4 * (t & 7);
-                *reinterpret_cast<float4 *>(&At[r][o + j0]) = make_float4(Pt[j0][r], Pt[j0 + 1][r], Pt[j0 + 2][r], Pt[j0 + 3][r]);
-            }
-            if (o > 0) {
-                const float (*Rt)[FP_LD] = reinterpret_cast<const float (*)[FP_LD]>(&S[o][0]);
-                slab_rank32_update<2>(At, Pt, Rt, o, tid, TR);
-            }
-            __syncthreads();
-        }
-        // store the tile (and its TF32 parts)
-#pragma unroll
-        for (int it = 0; it < NB * NB / 4 / FP_THREADS; ++it) {
-            const int idx = tid + it * FP_THREADS, i = idx >> 5, j4 = idx & 31;
-            if (i >= TR) continue;
-            const float4 v = *reinterpret_cast<const float4 *>(&At[i][4 * j4]);
-            float *dst = a.H + (int64_t)(r0 + i) * n + b0 + 4 * j4;
-            if (vec) {
-                *reinterpret_cast<float4 *>(dst) = v;
-            } else {
-                if (4 * j4 + 0 < nv) dst[0] = v.x;
-                if (4 * j4 + 1 < nv) dst[1] = v.y;
-                if (4 * j4 + 2 < nv) dst[2] = v.z;
-                if (4 * j4 + 3 < nv) dst[3] = v.w;
-            }
-            if (a.pan_hi && a.pan_f16) {
-                const float sc = split_scale(__uint_as_float(a.hd->tc_amax[AMAX_PAN]));
-                const float xs[4] = {sc * v.x, sc * v.y, sc * v.z, sc * v.w};
-                __half2 hv[2], lv[2];
-#pragma unroll
-                for (int f = 0; f < 2; ++f) {
-                    const __half h0 = __float2half_rn(xs[2 * f]), h1 = __float2half_rn(xs[2 * f + 1]);
-                    hv[f] = __halves2half2(h0, h1);
-                    lv[f] = __halves2half2(__float2half_rn(xs[2 * f] - __half2float(h0)),
-                                           __float2half_rn(xs[2 * f + 1] - __half2float(h1)));
-                }
-                __half *ph = reinterpret_cast<__half *>(a.pan_hi) + (int64_t)(r0 + i) * a.pan_ld + a.pan_col0 + 4 * j4;
-                __half *pl = reinterpret_cast<__half *>(a.pan_lo) + (int64_t)(r0 + i) * a.pan_ld + a.pan_col0 + 4 * j4;
-                *reinterpret_cast<uint2 *>(ph) = make_uint2(*reinterpret_cast<uint32_t *>(&hv[0]), *reinterpret_cast<uint32_t *>(&hv[1]));
-                *reinterpret_cast<uint2 *>(pl) = make_uint2(*reinterpret_cast<uint32_t *>(&lv[0]), *reinterpret_cast<uint32_t *>(&lv[1]));
-            } else if (a.pan_hi) {
-                const float xs[4] = {v.x, v.y, v.z, v.w};
-                float hv[4], lv[4];
-#pragma unroll
-                for (int f = 0; f < 4; ++f) { hv[f] = tf32_rn(xs[f]); lv[f] = tf32_rn(xs[f] - hv[f]); }
-                *reinterpret_cast<float4 *>(a.pan_hi + (int64_t)(r0 + i) * NB + 4 * j4) = make_float4(hv[0], hv[1], hv[2], hv[3]);
-                *reinterpret_cast<float4 *>(a.pan_lo + (int64_t)(r0 + i) * NB + 4 * j4) = make_float4(lv[0], lv[1], lv[2], lv[3]);
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Inverts every NB x NB diagonal factor R_pp (one CTA each) and stores the inverse on the
-// diagonal of H (strict lower part of the block zero): the starting point of U = R^-1.  Bound by shared-memory
-// reads: 4 x 4 outputs per thread (one output per thread, and divisions in the substitution, took 36 us; now 11).
-// 32 x 32 diagonal sub-blocks by back substitution (one warp each, lane = column), then
-// X12 = -X11 (R12 X22) for 32 -> 64 -> 128.
-// ---------------------------------------------------------------------------
-constexpr int ID_THREADS = 256;
-constexpr int ID_LD = NB + 4;
-constexpr size_t ID_SMEM = (2 * NB * ID_LD + 64 * 68 + NB) * sizeof(float);
-
-// C[i][j] = sign * sum_k A[i][k] B[k][j], S x S outputs, 4 x 4 per thread (rows ti + S / 4 e, four columns), all operands
-// row-major in shared memory; `t` counts the (S / 4)^2 threads of one product.
-template <int S>
-__device__ __forceinline__ void tile_product(float *C, int ldc, const float *A, int lda, const float *B, int ldb, int t, float sign) {
-    const int ti = t / (S / 4), tj = t % (S / 4);
-    float acc[4][4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-#pragma unroll
-        for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
-#pragma unroll 4
-    for (int k = 0; k < S; k += 4) {
-        float av[4][4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float4 v = *reinterpret_cast<const float4 *>(A + (ti + S / 4 * e) * lda + k);
-            av[e][0] = v.x; av[e][1] = v.y; av[e][2] = v.z; av[e][3] = v.w;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float4 b = *reinterpret_cast<const float4 *>(B + (k + q) * ldb + 4 * tj);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                acc[e][0] = fmaf(av[e][q], b.x, acc[e][0]); acc[e][1] = fmaf(av[e][q], b.y, acc[e][1]);
-                acc[e][2] = fmaf(av[e][q], b.z, acc[e][2]); acc[e][3] = fmaf(av[e][q], b.w, acc[e][3]);
-            }
-        }
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-        *reinterpret_cast<float4 *>(C + (ti + S / 4 * e) * ldc + 4 * tj) =
-            make_float4(sign * acc[e][0], sign * acc[e][1], sign * acc[e][2], sign * acc[e][3]);
-}
-
-__global__ void __launch_bounds__(ID_THREADS, 1) invert_diag_blocks_kernel(float *H, int n, const float *Rdiag) {
-    extern __shared__ __align__(16) float smem_f[];
-    float *S = smem_f, *X = smem_f + NB * ID_LD, *T = X + NB * ID_LD, *dinv = T + 64 * 68;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int b0 = blockIdx.x * NB;
-    const float *src = Rdiag + (int64_t)blockIdx.x * NB * NB;
-    float4 v[NB * NB / 4 / ID_THREADS];
-#pragma unroll
-    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) v[it] = *reinterpret_cast<const float4 *>(src + 4 * (tid + it * ID_THREADS));
-    if (tid < NB) dinv[tid] = 1.f / src[tid * NB + tid];
-#pragma unroll
-    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) {
-        const int i = (tid + it * ID_THREADS) >> 5, j4 = (tid + it * ID_THREADS) & 31;
-        *reinterpret_cast<float4 *>(S + i * ID_LD + 4 * j4) = v[it];
-        *reinterpret_cast<float4 *>(X + i * ID_LD + 4 * j4) = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    __syncthreads();
-    // transposes of the 32 x 32 diagonal sub-blocks into their own lower parts, for the substitution
-    for (int idx = tid; idx < 4 * 1024; idx += ID_THREADS) {
-        const int o = 32 * (idx >> 10), i = (idx >> 5) & 31, j = idx & 31;
-        if (j > i) S[(o + j) * ID_LD + o + i] = S[(o + i) * ID_LD + o + j];
-    }
-    __syncthreads();
-    if (warp < NB / 32) {
-        const int o = 32 * warp;
-        float x[32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) x[i] = (i == lane) ? 1.f : 0.f;
-        InvColStep<31>::run(x, S + o * ID_LD + o, dinv + o);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) X[(o + i) * ID_LD + o + lane] = x[i];
-    }
-    __syncthreads();
-    // X12 = -X11 (R12 X22), 32 -> 64 for both pairs, then 64 -> 128 (the triangular operands carry explicit zeros)
-    const int pr = tid >> 6, o = 64 * pr;
-    if (tid < 128) tile_product<32>(T + pr * 32 * 36, 36, S + o * ID_LD + o + 32, ID_LD, X + (o + 32) * ID_LD + o + 32, ID_LD, tid & 63, 1.f);
-    __syncthreads();
-    if (tid < 128) tile_product<32>(X + o * ID_LD + o + 32, ID_LD, X + o * ID_LD + o, ID_LD, T + pr * 32 * 36, 36, tid & 63, -1.f);
-    __syncthreads();
-    tile_product<64>(T, 68, S + 64, ID_LD, X + 64 * ID_LD + 64, ID_LD, tid, 1.f);
-    __syncthreads();
-    tile_product<64>(X + 64, ID_LD, X, ID_LD, T, 68, tid, -1.f);
-    __syncthreads();
-    const bool vec = (n & 3) == 0 && b0 + NB <= n;
-    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) {
-        const int i = (tid + it * ID_THREADS) >> 5, j = 4 * ((tid + it * ID_THREADS) & 31);
-        float x[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) x[e] = j + e >= i ? X[i * ID_LD + j + e] : 0.f;
-        float *dst = H + (int64_t)(b0 + i) * n + b0 + j;
-        if (vec) *reinterpret_cast<float4 *>(dst) = make_float4(x[0], x[1], x[2], x[3]);
-        else if (b0 + i < n) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) if (b0 + j + e < n) dst[e] = x[e];
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
 // quant(.)  -- min/max grid that contains zero, round half to even.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void make_grid(float lo, float hi, float amax, int bits, int sym,

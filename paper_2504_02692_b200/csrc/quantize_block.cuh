@@ -89,9 +89,6 @@ constexpr uint32_t QB_IDESC = (1u << 4) | ((QB_ROWS >> 3) << 17) | ((128 >> 4) <
 
 // Named barriers.  Chunk barriers are used once per step each; the step barrier keeps the chain from lapping them.
 enum { QBAR_CHUNK = 1, QBAR_STEP = 5, QBAR_NEAR = 6, QBAR_DRAIN = 7, QBAR_CLIP = 8 };
-__device__ __forceinline__ void named_bar_arrive(int id, int nthreads) {
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
 
 // Position of a row in a column of the published errors: the near warps' threads take rows ti, ti + 8, .. as
 // one 16-byte read.
