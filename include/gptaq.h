@@ -91,7 +91,7 @@ size_t gptaq_state_bytes(int64_t n);
  * gptaq_accumulate will be given in one call (larger batches still work: they
  * are processed in chunks that fit).  For n >= 512 the scratch holds split (high part / low part)
  * operand copies of U^T and P^T for the tensor cores: about 4 n^2 floats in all where n is a multiple
- * of 8 (fp16 parts), about 7 n^2 where it is a multiple of 4 only (TF32 parts).  The library reads them
+ * of 4 (fp16 parts).  The library reads them
  * in every gptaq_quantize, so the workspace must be left untouched from gptaq_factor until the last
  * gptaq_quantize on this state. */
 size_t gptaq_workspace_bytes(int64_t n, int64_t m_max, int64_t max_batch_tokens, int blocksize);

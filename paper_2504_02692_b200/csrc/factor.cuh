@@ -424,9 +424,8 @@ constexpr size_t PS_SMEM = (size_t)(NB * FP_LD + 4 * 32 * FP_YLD + PS_WORKERS * 
 struct PanelSolveArgs {
     float *H; int n; int b0;
     const float *Rdiag, *Y;    // as diag_factor_kernel leaves them (R_pp^T in the lower part)
-    float *pan_hi, *pan_lo;    // nullptr, or [n][NB]: TF32 parts of the panel rows
-    int pan_f16;               // the two arrays hold __half instead: fp16 parts of split_scale(tc_amax[AMAX_PAN]) * row,
-    int pan_ld, pan_col0;      //   row pitch pan_ld, this panel at columns pan_col0 .. + NB (several panels side by side)
+    __half *pan_hi, *pan_lo;   // nullptr, or fp16 parts of split_scale(tc_amax[AMAX_PAN]) * row: row pitch pan_ld, this panel
+    int pan_ld, pan_col0;      //   at columns pan_col0 .. + NB (several panels side by side)
     int workers;               // warps of a CTA that take rows
     int early;                 // the panel is up to date before the diagonal block is: rows may be read before pdl_wait()
     float *next_diag;          // nullptr, or [NB][NB]: receives the block at b0 - NB (by the last CTA)
@@ -485,7 +484,7 @@ __global__ void __launch_bounds__(PS_THREADS) panel_solve_kernel(PanelSolveArgs 
     __syncthreads();
     if (warp >= nwarps) return;
     float *buf = Yt + 4 * 32 * FP_YLD + (warp * ROWS + RPT * rp) * FP_YLD;                          // this lane's rows, 32 values each
-    const float sc = a.pan_hi && a.pan_f16 ? split_scale(__uint_as_float(a.hd->tc_amax[AMAX_PAN])) : 1.f;
+    const float sc = a.pan_hi ? split_scale(__uint_as_float(a.hd->tc_amax[AMAX_PAN])) : 1.f;
     bool first = true;
     for (; g < ngroups; g += slabs * nwarps) {
         if (!first) load_rows(g);
@@ -568,18 +567,12 @@ __global__ void __launch_bounds__(PS_THREADS) panel_solve_kernel(PanelSolveArgs 
 #pragma unroll
                     for (int f = 0; f < 4; ++f) if (c + f < nv) dst[f] = v[f];
                 }
-                if (a.pan_hi && a.pan_f16) {
+                if (a.pan_hi) {
                     const float s4[4] = {sc * v[0], sc * v[1], sc * v[2], sc * v[3]};
                     uint2 hi, lo;
                     split16_pack(s4, hi, lo);
-                    *reinterpret_cast<uint2 *>(reinterpret_cast<__half *>(a.pan_hi) + row * a.pan_ld + a.pan_col0 + c) = hi;
-                    *reinterpret_cast<uint2 *>(reinterpret_cast<__half *>(a.pan_lo) + row * a.pan_ld + a.pan_col0 + c) = lo;
-                } else if (a.pan_hi) {
-                    float hv[4], lv[4];
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) { hv[f] = tf32_rn(v[f]); lv[f] = tf32_rn(v[f] - hv[f]); }
-                    *reinterpret_cast<float4 *>(a.pan_hi + row * NB + c) = make_float4(hv[0], hv[1], hv[2], hv[3]);
-                    *reinterpret_cast<float4 *>(a.pan_lo + row * NB + c) = make_float4(lv[0], lv[1], lv[2], lv[3]);
+                    *reinterpret_cast<uint2 *>(a.pan_hi + row * a.pan_ld + a.pan_col0 + c) = hi;
+                    *reinterpret_cast<uint2 *>(a.pan_lo + row * a.pan_ld + a.pan_col0 + c) = lo;
                 }
             }
         }

@@ -51,8 +51,7 @@ struct gptaq_ctx {
     int64_t tokens;
     int64_t launches;
     int stats_precision;   // GPTAQ_STATS_*
-    bool tensor;           // float32-grade tensor-core GEMMs for factor / P / trailing update
-    bool f16;              // ... with FP16-split operands where the producer can record their range (n % 8 == 0)
+    bool tensor;           // float32-grade tensor-core GEMMs (fp16-split operands) for factor / P / trailing update
     TcSched sched;         // tile numbering of the float32-grade GEMM launches (see StateHeader::sched_counter)
     int terms;             // GPTAQ_TERM_* switches of gptaq_quantize
     bool static_groups;    // group grids from the original weights, per group of the caller's columns
@@ -95,18 +94,19 @@ Layout state_layout(int64_t n) {
     return l;
 }
 
-// float32-grade tensor-core path (tc_gemm.cuh): widths whose rows are 16-byte multiples (a TMA
-// stride rule) and that are large enough for 128 x 256 tiles to pay.
+// float32-grade tensor-core path (tc_gemm.cuh): widths whose float32 rows are 16-byte multiples (the epilogue's tensor
+// map) and that are large enough for 128 x 256 tiles to pay.  The fp16 copies of n x n operands have a row pitch of their
+// own, the next multiple of 8 (a TMA stride rule).
 constexpr int64_t TC_MIN_N = 512;
 inline bool tc_shape_ok(int64_t n) { return n >= TC_MIN_N && (n % 4) == 0; }
+inline int64_t split_pitch(int64_t n) { return (n + 7) / 8 * 8; }
 
 struct WsLayout {
     size_t t_off, rinv_off;
     size_t diag_off;        // inverses of the current diagonal block's sub-blocks, copy of the next diagonal block
-    size_t s_off[6];        // split operand matrices (n x n each): S1 hi/lo, S2 hi/lo, S3 hi/lo
-    size_t pan_off[2];      // split copy of factor panels, hi/lo: n x 128 float32 (TF32) or n x SUPER_NB fp16
-    // [-Err | Wpre]: float32 (m x 2B, or m x 2 * QSUPER * B for the FP16-split update), second part
-    // (TF32 remainder, or the fp16 hi / lo parts), row scales
+    size_t s_off[3];        // split operand matrices, fp16 hi then lo (n x split_pitch(n) each)
+    size_t pan_off[2];      // split copy of factor panels, hi / lo: n x SUPER_NB fp16
+    // [-Err | Wpre]: float32 (m x 2B, or m x 2 * QSUPER * B for the tensor-core update), its fp16 hi / lo parts, row scales
     size_t ew_off, ew_lo_off, rs_off, total;
     bool tensor;
 };
@@ -128,21 +128,17 @@ WsLayout ws_layout(int64_t n, int64_t m_max, int blocksize) {
     w.rinv_off = w.t_off + mat;
     w.diag_off = w.rinv_off + round_up(nb * NB * NB * sizeof(float), ALIGN);
     size_t off = w.diag_off + round_up((4 * 32 * FP_YLD + NB * NB) * sizeof(float), ALIGN);
-    const bool f16 = w.tensor && (n % 8) == 0;
-    // split operand copies: six float32-sized regions for TF32 parts; fp16 hi / lo parts use three
-    // (S0 = U^T, S1 = U then P^T, S4 = dXX^T then O; hi and lo of one matrix fill one region)
-    for (int i = 0; i < 6; ++i) {
-        w.s_off[i] = off;
-        if (w.tensor && (!f16 || i == 0 || i == 1 || i == 4)) off += mat;
-    }
-    const size_t pan = std::max((size_t)n * NB * sizeof(float), (size_t)n * SUPER_NB * sizeof(__half));
+    // S0 = U^T, S1 = U then P^T, S2 = dXX^T then O
+    const size_t smat = round_up(2 * (size_t)n * (size_t)split_pitch(n) * sizeof(__half), ALIGN);
+    for (int i = 0; i < 3; ++i) { w.s_off[i] = off; if (w.tensor) off += smat; }
+    const size_t pan = (size_t)n * SUPER_NB * sizeof(__half);
     for (int i = 0; i < 2; ++i) { w.pan_off[i] = off; if (w.tensor) off += round_up(pan, ALIGN); }
     const size_t ew1 = round_up((size_t)m_max * 2 * (size_t)blocksize * sizeof(float), ALIGN);
-    const size_t ew = f16 ? QSUPER * ew1 : ew1;
+    const size_t ew = w.tensor ? QSUPER * ew1 : ew1;
     w.ew_off = off;
     w.ew_lo_off = off + ew;
     w.rs_off = off + (w.tensor ? 2 * ew : ew);
-    w.total = w.rs_off + (f16 ? round_up((size_t)m_max * sizeof(float), ALIGN) : 0);
+    w.total = w.rs_off + (w.tensor ? round_up((size_t)m_max * sizeof(float), ALIGN) : 0);
     return w;
 }
 
@@ -209,25 +205,10 @@ bool make_kmajor_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t kp
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// float32 matrix [rows][ld] with `cols` valid K-contiguous elements per row; box = 32 x box_rows,
-// 128-byte swizzle, out-of-range elements read as zero.
-bool make_f32_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
-    EncodeTiledFn fn = encode_tiled_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
-    cuuint32_t box[2] = {(cuuint32_t)TBK, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void *>(ptr), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // A split operand (hi / lo arrays of the same shape) as seen by the tensor-core GEMM.
 struct SplitOperand {
-    const void *hi, *lo;       // float32 arrays holding TF32 values, or __half arrays (f16)
+    const __half *hi, *lo;
     int64_t rows, cols, ld;
-    bool f16 = false;
 };
 
 // __half matrix [rows][ld] with `cols` valid K-contiguous elements per row; box = 64 x box_rows.
@@ -236,26 +217,23 @@ bool make_f16_map(CUtensorMap *map, const void *ptr, int64_t rows, int64_t cols,
     if (!fn) return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {(cuuint32_t)(2 * TBK), (cuuint32_t)box_rows};
+    cuuint32_t box[2] = {(cuuint32_t)TBK, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool make_operand_map(CUtensorMap *map, const void *ptr, const SplitOperand &o, int box_rows) {
-    return o.f16 ? make_f16_map(map, ptr, o.rows, o.cols, o.ld, box_rows)
-                 : make_f32_map(map, ptr, o.rows, o.cols, o.ld, box_rows);
+bool make_operand_map(CUtensorMap *map, const __half *ptr, const SplitOperand &o, int box_rows) {
+    return make_f16_map(map, ptr, o.rows, o.cols, o.ld, box_rows);
 }
 
 struct TcMaps {
     CUtensorMap a_hi, a_lo, b_hi, b_lo, b2_hi, b2_lo;
-    bool f16 = false;
 };
 
 bool make_tc_maps(TcMaps *m, const SplitOperand &A, const SplitOperand &B, const SplitOperand *B2) {
     const SplitOperand &b2 = B2 ? *B2 : B;
-    m->f16 = A.f16;
     return make_operand_map(&m->a_hi, A.hi, A, TBM) && make_operand_map(&m->a_lo, A.lo, A, TBM) &&
            make_operand_map(&m->b_hi, B.hi, B, TBN) && make_operand_map(&m->b_lo, B.lo, B, TBN) &&
            make_operand_map(&m->b2_hi, b2.hi, b2, TBN) && make_operand_map(&m->b2_lo, b2.lo, b2, TBN);
@@ -314,8 +292,7 @@ cudaError_t launch_tc_gemm(const TcMaps &m, const TcGemmArgs &a_in, TcSched &sch
     if (a.beta == 1.f && a.nbatch == 1 && !a.amax_out && (a.mask == TC_MASK_NONE || a.mask == TC_MASK_UPPER_KEEP) &&
         (reinterpret_cast<uintptr_t>(a.C) & 15) == 0 && (a.ldc & 3) == 0 && make_c_map(&mapC, a.C, a.M, a.N, a.ldc))
         a.c_tma = 1;
-    if (m.f16) return launch_pdl(pdl, tc_gemm_kernel<true>, dim3(grid), dim3(TC_THREADS), TC_SMEM, s, m.a_hi, m.a_lo, m.b_hi, m.b_lo, m.b2_hi, m.b2_lo, mapC, a);
-    return launch_pdl(pdl, tc_gemm_kernel<false>, dim3(grid), dim3(TC_THREADS), TC_SMEM, s, m.a_hi, m.a_lo, m.b_hi, m.b_lo, m.b2_hi, m.b2_lo, mapC, a);
+    return launch_pdl(pdl, tc_gemm_kernel, dim3(grid), dim3(TC_THREADS), TC_SMEM, s, m.a_hi, m.a_lo, m.b_hi, m.b_lo, m.b2_hi, m.b2_lo, mapC, a);
 }
 
 // Slots of StateHeader::tc_amax (largest magnitudes of FP16-split operands).
@@ -346,19 +323,6 @@ cudaError_t launch_split16(const float *src, int64_t lds, __half *hi, __half *lo
     a.hi_t = hi_t; a.lo_t = lo_t;
     dim3 grid((cols + 63) / 64, (rows + 63) / 64, b.nbatch);
     split16_kernel<<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_split(const float *src, int64_t lds, float *hi, float *lo, int64_t ldd, int rows, int cols,
-                         bool transpose, int mask, float scale, cudaStream_t s, const SplitBatch &b = SplitBatch()) {
-    if (rows <= 0 || cols <= 0 || b.nbatch <= 0) return cudaSuccess;
-    SplitArgs a;
-    a.src = src; a.lds = lds; a.src_bstride = b.src_bstride; a.hi = hi; a.lo = lo; a.ldd = ldd;
-    a.dst_bstride = b.dst_bstride;
-    a.rows = rows; a.cols = cols; a.rows_last = b.rows_last; a.cols_last = b.cols_last; a.nbatch = b.nbatch;
-    a.transpose = transpose ? 1 : 0; a.mask = mask; a.scale = scale;
-    dim3 grid((cols + 63) / 64, (rows + 63) / 64, b.nbatch);
-    split_kernel<<<grid, 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -523,14 +487,11 @@ struct QuantizeTarget {
     TcSched *sched;            // host-side count of the tile numbers drawn from hd->sched_counter
     float *EW;
     int num_sms;
-    // float32-grade tensor-core trailing update: split copies of U^T and P^T (n x n, ld n) and
-    // the low part of [-Err | Wpre]; all null on the plain-FMA path
-    const float *UT_hi, *UT_lo, *PT_hi, *PT_lo;
-    float *EW_lo;
-    // the same update with FP16-split operands (takes precedence when set): U^T and P^T as fp16 hi / lo
-    // (lo = hi + n * n), each with the scale of its recorded maximum; EW is then m x 2 * SW wide (SW columns per
+    // tensor-core trailing update (null: plain float32 products): U^T and P^T as fp16 hi / lo (row pitch ldt,
+    // lo = hi + n * ldt), each with the scale of its recorded maximum; EW is then m x 2 * SW wide (SW columns per
     // launch), EW16 holds its fp16 hi / lo parts (lo = hi + m * 2 * SW) with one scale per row
     const __half *UT16 = nullptr, *PT16 = nullptr;
+    int64_t ldt = 0;
     __half *EW16 = nullptr;
     float *row_inv = nullptr;
     const unsigned *amax_u = nullptr, *amax_p = nullptr;
@@ -546,7 +507,7 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
                                int bits, int group, int sym, uint8_t *codes, float *scales, float *zeros, int G,
                                bool static_groups, cudaStream_t s) {
     const bool far_form = t.UT16 != nullptr;
-    const size_t nn = (size_t)t.n * t.n;
+    const size_t nn = (size_t)t.n * t.ldt;
     QuantBlockArgs a;
     std::memset(&a, 0, sizeof(a));
     a.W = W; a.ldw = ldw; a.m = (int)m; a.n = t.n; a.U = t.U; a.P = t.P; a.dead = t.dead;
@@ -557,15 +518,14 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
     if (i1 < t.n) {
         a.EW = t.EW;
         if (far_form) { a.EWS_hi = t.EW16; a.EWS_lo = t.EW16 + (size_t)m * 2 * SW; a.row_inv = t.row_inv; }
-        else a.EW_lo = t.EW_lo;
     }
     a.amax_u = t.amax_u; a.amax_p = t.amax_p; a.hd = t.hd;
     a.err_scale = (t.terms & GPTAQ_TERM_ERR) ? 1.f : 0.f; a.asym_scale = (t.terms & GPTAQ_TERM_ASYM) ? 1.f : 0.f;
     a.perm = t.perm; a.clip_steps = t.clip_steps; a.clip_min = t.clip_min;
     CUtensorMap uh, ul, ph, pl;
     std::memset(&uh, 0, sizeof(uh)); ul = ph = pl = uh;
-    if (far_form && (!make_f16_map(&uh, t.UT16, t.n, t.n, t.n, 128) || !make_f16_map(&ul, t.UT16 + nn, t.n, t.n, t.n, 128) ||
-                     !make_f16_map(&ph, t.PT16, t.n, t.n, t.n, 128) || !make_f16_map(&pl, t.PT16 + nn, t.n, t.n, t.n, 128)))
+    if (far_form && (!make_f16_map(&uh, t.UT16, t.n, t.n, t.ldt, 128) || !make_f16_map(&ul, t.UT16 + nn, t.n, t.n, t.ldt, 128) ||
+                     !make_f16_map(&ph, t.PT16, t.n, t.n, t.ldt, 128) || !make_f16_map(&pl, t.PT16 + nn, t.n, t.n, t.ldt, 128)))
         return cudaErrorUnknown;
     const dim3 grid((unsigned)((m + QB_ROWS - 1) / QB_ROWS));
     const size_t smem = quant_block_smem_bytes(far_form, static_groups);
@@ -662,20 +622,15 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
     // grids per output channel, per group of whole 32-column steps, or per column (static groups): quant_block_kernel.
     // Smaller groups take column_loop_kernel (one warp per row, any group).
     const bool steps = group <= 0 || (group % 32) == 0 || static_groups;
-    const bool tensor16 = t.UT16 != nullptr;
-    const bool tensor = tensor16 || t.EW_lo != nullptr;
+    const bool tensor = t.UT16 != nullptr;
     // columns per launch: as many blocks as the slab holds where the tensor cores carry the updates between them
     // (the workspace holds the errors of QSUPER blocks), one block otherwise
-    const int SW = tensor16 && steps ? std::min(QB_SUPER, QSUPER * blocksize) : blocksize;
+    const int SW = tensor && steps ? std::min(QB_SUPER, QSUPER * blocksize) : blocksize;
     TcMaps maps;
-    if (tensor16) {
-        const size_t nn = (size_t)n * n, me = (size_t)m * 2 * SW;
-        const SplitOperand A{t.EW16, t.EW16 + me, m, 2 * SW, 2 * SW, true};
-        const SplitOperand B{t.UT16, t.UT16 + nn, n, n, n, true}, B2{t.PT16, t.PT16 + nn, n, n, n, true};
-        if (!make_tc_maps(&maps, A, B, &B2)) { *err = cudaErrorUnknown; return GPTAQ_ERR_CUDA; }
-    } else if (tensor) {
-        const SplitOperand A{EW, t.EW_lo, m, 2 * blocksize, 2 * blocksize};
-        const SplitOperand B{t.UT_hi, t.UT_lo, n, n, n}, B2{t.PT_hi, t.PT_lo, n, n, n};
+    if (tensor) {
+        const size_t nn = (size_t)n * t.ldt, me = (size_t)m * 2 * SW;
+        const SplitOperand A{t.EW16, t.EW16 + me, m, 2 * SW, 2 * SW};
+        const SplitOperand B{t.UT16, t.UT16 + nn, n, n, t.ldt}, B2{t.PT16, t.PT16 + nn, n, n, t.ldt};
         if (!make_tc_maps(&maps, A, B, &B2)) { *err = cudaErrorUnknown; return GPTAQ_ERR_CUDA; }
     }
     for (int i0 = 0; i0 < n; i0 += SW) {
@@ -690,7 +645,7 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
             a.W = Wk; a.ldw = ldk; a.m = (int)m; a.n = n; a.U = t.U; a.P = t.P; a.dead = t.dead;
             a.i0 = i0; a.bw = i1 - i0;
             a.bits = bits; a.group = group; a.sym = sym;
-            a.codes = d_codes; a.scales = d_scales; a.zeros = d_zeros; a.G = G; a.EW = EW; a.EW_lo = tensor16 ? nullptr : t.EW_lo; a.hd = t.hd;
+            a.codes = d_codes; a.scales = d_scales; a.zeros = d_zeros; a.G = G; a.EW = EW; a.hd = t.hd;
             a.amax_u = t.amax_u; a.amax_p = t.amax_p;
             a.perm = t.perm; a.clip_steps = t.clip_steps; a.clip_min = t.clip_min;
             a.err_scale = (t.terms & GPTAQ_TERM_ERR) ? 1.f : 0.f; a.asym_scale = (t.terms & GPTAQ_TERM_ASYM) ? 1.f : 0.f;
@@ -702,7 +657,7 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
             else if (T == 2) column_loop_kernel<2><<<cl_grid, nw * 32, cl_smem, s>>>(a);
             else column_loop_kernel<1><<<cl_grid, nw * 32, cl_smem, s>>>(a);
             QLAUNCHED();
-            if (tensor16 && i1 < n) {
+            if (tensor && i1 < n) {
                 // [-Err | rho Wpre] scaled row by row and split here (quant_block_kernel does so itself)
                 rowscale_split16_kernel<<<(unsigned)((m + 7) / 8), 256, 0, s>>>(EW, 2 * SW, (int)m, 2 * SW, t.EW16,
                                                                               t.EW16 + (size_t)m * 2 * SW, t.row_inv);
@@ -715,7 +670,7 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
             // are rows i1.. of U^T (first SW contraction steps) and of P^T (the next SW)
             TcGemmArgs g = tc_args(Wk + i1, ldk, (int)m, n - i1, 2 * SW, 1.f, 1.f, TC_FULL, TC_MASK_NONE, t.hd);
             g.b_row0 = i1; g.b_k0 = i0; g.k_split = SW; g.b2_k0 = i0;
-            if (tensor16) { g.row_inv = t.row_inv; g.amax_b = t.amax_u; }
+            g.row_inv = t.row_inv; g.amax_b = t.amax_u;
             *err = launch_tc_gemm(maps, g, *t.sched, t.num_sms, s, false);
             if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
             ++*launches;
@@ -836,7 +791,6 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
     h->launches = 0;
     h->stats_precision = GPTAQ_STATS_FP16_SPLIT_TENSOR;
     h->tensor = tc_shape_ok(n) && encode_tiled_fn() != nullptr;
-    h->f16 = h->tensor && (n % 8) == 0;
     h->terms = GPTAQ_TERM_ERR | GPTAQ_TERM_ASYM;
     h->clip_steps = 0; h->clip_min = 1.f;
     h->static_groups = false;
@@ -856,9 +810,7 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(stats_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UMMA_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
+        e = cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
     // the conversion of the next batch shares the SMs with the running product: both kernels ask for
     // the largest shared-memory carve-out, so that a conversion CTA fits beside a product CTA
     if (e == cudaSuccess)
@@ -1011,21 +963,20 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
     LAUNCHED();
 
     // reverse Cholesky H_d = R R^T, R upper, from the last block column upwards
-    float *pan_hi = h->tensor ? reinterpret_cast<float *>(h->ws + wl.pan_off[0]) : nullptr;
-    float *pan_lo = h->tensor ? reinterpret_cast<float *>(h->ws + wl.pan_off[1]) : nullptr;
+    __half *pan_hi = h->tensor ? reinterpret_cast<__half *>(h->ws + wl.pan_off[0]) : nullptr;
+    __half *pan_lo = h->tensor ? reinterpret_cast<__half *>(h->ws + wl.pan_off[1]) : nullptr;
     TcMaps pan_maps;
     std::memset(static_cast<void *>(&pan_maps), 0, sizeof(pan_maps));
-    const int pan_ld = h->f16 ? SUPER_NB : NB;
     if (h->tensor) {
-        const SplitOperand pan{pan_hi, pan_lo, n, pan_ld, pan_ld, h->f16};
+        const SplitOperand pan{pan_hi, pan_lo, n, SUPER_NB, SUPER_NB};
         if (!make_tc_maps(&pan_maps, pan, pan, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
     }
     float *Y = reinterpret_cast<float *>(h->ws + wl.diag_off), *next_diag = Y + 4 * 32 * FP_YLD;
     // rank-NB (or super-panel) update of the columns to the left of panel p, on stream `us` with at most `sms` CTAs
     auto update = [&](int p, cudaStream_t us, int sms) -> gptaq_status_t {
         const int b0 = p * NB;
-        const int s0 = h->f16 ? b0 / SUPER_NB * SUPER_NB : b0;
-        if (h->f16 && b0 >= TC_MIN_N) {
+        const int s0 = b0 / SUPER_NB * SUPER_NB;
+        if (h->tensor && b0 >= TC_MIN_N) {
             const unsigned *am = h->hd->tc_amax + AMAX_PAN;
             if (b0 > s0) {
                 // inside the super-panel: A[0:b0, s0:b0] -= R[0:b0, blk] R[s0:b0, blk]^T  (upper part)
@@ -1044,12 +995,6 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
             return GPTAQ_OK;
         }
         // A[0:b0, 0:b0] -= R[0:b0, blk] R[0:b0, blk]^T  (upper part)
-        if (h->tensor && b0 >= TC_MIN_N) {
-            TcGemmArgs g = tc_args(H, n, b0, b0, NB, -1.f, 1.f, TC_UPPER_TILES, TC_MASK_UPPER_KEEP, h->hd);
-            CU(launch_tc_gemm(pan_maps, g, h->sched, sms, us));
-            h->launches++;
-            return GPTAQ_OK;
-        }
         Operand rp = make_operand(H + b0, n, 1);
         GemmProblem ps = make_problem(rp, rp, H, n, b0, b0, std::min(NB, n - b0), -1.f, 1.f, GEMM_UPPER_TILES);
         return gemm(h, ps, false, false, us);
@@ -1065,16 +1010,16 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
     bool diag_done = false;                     // the diagonal block of this panel was factored beside the last update
     for (int p = nb - 1; p >= 0; --p) {
         const int b0 = p * NB;
-        const int s0 = h->f16 ? b0 / SUPER_NB * SUPER_NB : b0;      // first column of this panel's super-panel
+        const int s0 = h->tensor ? b0 / SUPER_NB * SUPER_NB : b0;      // first column of this panel's super-panel
         if (!diag_done) OK(factor_diag(p, H + (int64_t)b0 * n + b0, n, 0, 0));
         const bool early = diag_done;           // (then the update of this panel's columns was waited for, not overlapped)
         diag_done = false;
         if (p == 0) break;
-        const bool ahead = h->f16 && b0 > s0;   // the next panel is in the same super-panel: its block needs this panel only
+        const bool ahead = h->tensor && b0 > s0;   // the next panel is in the same super-panel: its block needs this panel only
         PanelSolveArgs pa;
         pa.H = H; pa.n = n; pa.b0 = b0; pa.Rdiag = Rinv + (size_t)p * NB * NB; pa.Y = Y;
-        pa.pan_hi = pan_hi; pa.pan_lo = pan_lo; pa.pan_f16 = h->f16 ? 1 : 0;
-        pa.pan_ld = pan_ld; pa.pan_col0 = b0 - s0; pa.hd = h->hd;
+        pa.pan_hi = pan_hi; pa.pan_lo = pan_lo;
+        pa.pan_ld = SUPER_NB; pa.pan_col0 = b0 - s0; pa.hd = h->hd;
         pa.next_diag = ahead ? next_diag : nullptr;
         pa.early = early ? 1 : 0;
         // a warp per 4 rows while that fills no SM beyond PS_WORKERS warps, per 8 rows beyond; as few warps per CTA as give
@@ -1105,14 +1050,6 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
     // inv([[A, B], [0, C]]) = [[A^-1, -A^-1 B C^-1], [0, C^-1]]
     invert_diag_blocks_kernel<<<nb, ID_THREADS, ID_SMEM, s>>>(H, n, Rinv);
     LAUNCHED();
-    float *S1h = nullptr, *S1l = nullptr, *S2h = nullptr, *S2l = nullptr;
-    TcMaps inv_maps;
-    if (h->tensor && !h->f16) {
-        S1h = reinterpret_cast<float *>(h->ws + wl.s_off[0]); S1l = reinterpret_cast<float *>(h->ws + wl.s_off[1]);
-        S2h = reinterpret_cast<float *>(h->ws + wl.s_off[2]); S2l = reinterpret_cast<float *>(h->ws + wl.s_off[3]);
-        const SplitOperand A{S1h, S1l, n, n, n}, B{S2h, S2l, n, n, n};
-        if (!make_tc_maps(&inv_maps, A, B, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
-    }
     for (int64_t sz = NB; sz < n; sz *= 2) {
         const int np = (int)((n - sz + 2 * sz - 1) / (2 * sz));
         const int tail = (int)(n - (2 * sz * (np - 1) + sz));
@@ -1120,23 +1057,24 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
         // few tiles: the plain float32 products of 32 x 32 tiles need no operand copies and beat the tensor cores'
         // two splits and a product per factor
         const bool few = np * (sz / GBM) * (sz / GBN) <= SIMT_SMALL_TILES;
-        if (h->f16 && damp > 0.f && sz >= 2 * NB && !few) {
+        if (h->tensor && damp > 0.f && sz >= 2 * NB && !few) {
             // The two products on the tensor cores with FP16-split operands.  Ranges: B holds entries of R
             // (bounded like the panels), the inverted blocks are bounded by 1 / sqrt(lambda), the
             // intermediate T records its own maximum in the first product's epilogue.
-            const size_t nn = (size_t)n * n;
+            const int64_t ldt = split_pitch(n);
+            const size_t nn = (size_t)n * ldt;
             __half *A1 = reinterpret_cast<__half *>(h->ws + wl.s_off[0]);     // left operands, K-major at their own coordinates
             __half *B2 = reinterpret_cast<__half *>(h->ws + wl.s_off[1]);     // transposed right operands
             unsigned *am = h->hd->tc_amax;
-            const SplitOperand Aop{A1, A1 + nn, n, n, n, true}, Bop{B2, B2 + nn, n, n, n, true};
+            const SplitOperand Aop{A1, A1 + nn, n, n, ldt}, Bop{B2, B2 + nn, n, n, ldt};
             TcMaps m16;
             if (!make_tc_maps(&m16, Aop, Bop, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
-            SplitBatch sb; sb.nbatch = np; sb.src_bstride = sb.dst_bstride = bstride;
+            SplitBatch sb; sb.nbatch = np; sb.src_bstride = bstride; sb.dst_bstride = 2 * sz * (ldt + 1);
             SplitBatch sbt = sb; sbt.cols_last = tail;
             SplitBatch sbc = sb; sbc.rows_last = tail; sbc.cols_last = tail;
             CU(cudaMemsetAsync(am + AMAX_T, 0, sizeof(unsigned), s));
-            CU(launch_split16(H + sz, n, A1 + sz, A1 + nn + sz, n, (int)sz, (int)sz, false, SPLIT_ALL, 1.f, am + AMAX_PAN, s, sbt));
-            CU(launch_split16(H + sz * n + sz, n, B2 + sz * n + sz, B2 + nn + sz * n + sz, n, (int)sz, (int)sz, true,
+            CU(launch_split16(H + sz, n, A1 + sz, A1 + nn + sz, ldt, (int)sz, (int)sz, false, SPLIT_ALL, 1.f, am + AMAX_PAN, s, sbt));
+            CU(launch_split16(H + sz * n + sz, n, B2 + sz * ldt + sz, B2 + nn + sz * ldt + sz, ldt, (int)sz, (int)sz, true,
                               SPLIT_UPPER, 1.f, am + AMAX_INV, s, sbc));
             TcGemmArgs g1 = tc_args(T + sz, n, (int)sz, (int)sz, (int)sz, 1.f, 0.f, TC_TRI_RIGHT, TC_MASK_NONE, h->hd);
             g1.nbatch = np; g1.c_bstride = bstride; g1.N_last = tail; g1.K_last = tail;
@@ -1144,8 +1082,8 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
             g1.b_row0 = (int)sz; g1.b_row_bs = (int)(2 * sz); g1.b_k0 = (int)sz; g1.b_k_bs = (int)(2 * sz);
             g1.amax_a = am + AMAX_PAN; g1.amax_b = am + AMAX_INV; g1.amax_out = am + AMAX_T;
             CU(launch_tc_gemm(m16, g1, h->sched, h->num_sms, s));
-            CU(launch_split16(H, n, A1, A1 + nn, n, (int)sz, (int)sz, false, SPLIT_UPPER, 1.f, am + AMAX_INV, s, sb));
-            CU(launch_split16(T + sz, n, B2 + sz * n, B2 + nn + sz * n, n, (int)sz, (int)sz, true, SPLIT_ALL, 1.f, am + AMAX_T, s, sbt));
+            CU(launch_split16(H, n, A1, A1 + nn, ldt, (int)sz, (int)sz, false, SPLIT_UPPER, 1.f, am + AMAX_INV, s, sb));
+            CU(launch_split16(T + sz, n, B2 + sz * ldt, B2 + nn + sz * ldt, ldt, (int)sz, (int)sz, true, SPLIT_ALL, 1.f, am + AMAX_T, s, sbt));
             TcGemmArgs g2 = tc_args(H + sz, n, (int)sz, (int)sz, (int)sz, -1.f, 0.f, TC_TRI_LEFT, TC_MASK_NONE, h->hd);
             g2.nbatch = np; g2.c_bstride = bstride; g2.N_last = tail;
             g2.a_row0 = 0; g2.a_row_bs = (int)(2 * sz); g2.a_k0 = 0; g2.a_k_bs = (int)(2 * sz);
@@ -1155,37 +1093,7 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
             h->launches += 6;
             continue;
         }
-        if (h->tensor && !h->f16 && sz >= 2 * NB && !few) {
-            // Same two products on the tensor cores, TF32-split operands (widths that are multiples of 4
-            // only).  S1 holds K-major copies of the left operands at
-            // their own coordinates (B, then A^-1), S2 the transposed right operands (C^-T, then T^T).
-            SplitBatch sb; sb.nbatch = np; sb.src_bstride = sb.dst_bstride = bstride;
-            SplitBatch sbt = sb; sbt.cols_last = tail;                 // blocks with `tail` columns
-            SplitBatch sbc = sb; sbc.rows_last = tail; sbc.cols_last = tail;
-            CU(launch_split(H + sz, n, S1h + sz, S1l + sz, n, (int)sz, (int)sz, false, SPLIT_ALL, 1.f, s, sbt));
-            h->launches++;
-            CU(launch_split(H + sz * n + sz, n, S2h + sz * n + sz, S2l + sz * n + sz, n, (int)sz, (int)sz, true,
-                            SPLIT_UPPER, 1.f, s, sbc));
-            h->launches++;
-            TcGemmArgs g1 = tc_args(T + sz, n, (int)sz, (int)sz, (int)sz, 1.f, 0.f, TC_TRI_RIGHT, TC_MASK_NONE, h->hd);
-            g1.nbatch = np; g1.c_bstride = bstride; g1.N_last = tail; g1.K_last = tail;
-            g1.a_row0 = 0; g1.a_row_bs = (int)(2 * sz); g1.a_k0 = (int)sz; g1.a_k_bs = (int)(2 * sz);
-            g1.b_row0 = (int)sz; g1.b_row_bs = (int)(2 * sz); g1.b_k0 = (int)sz; g1.b_k_bs = (int)(2 * sz);
-            CU(launch_tc_gemm(inv_maps, g1, h->sched, h->num_sms, s));
-            h->launches++;
-            CU(launch_split(H, n, S1h, S1l, n, (int)sz, (int)sz, false, SPLIT_UPPER, 1.f, s, sb));
-            h->launches++;
-            CU(launch_split(T + sz, n, S2h + sz * n, S2l + sz * n, n, (int)sz, (int)sz, true, SPLIT_ALL, 1.f, s, sbt));
-            h->launches++;
-            TcGemmArgs g2 = tc_args(H + sz, n, (int)sz, (int)sz, (int)sz, -1.f, 0.f, TC_TRI_LEFT, TC_MASK_NONE, h->hd);
-            g2.nbatch = np; g2.c_bstride = bstride; g2.N_last = tail;
-            g2.a_row0 = 0; g2.a_row_bs = (int)(2 * sz); g2.a_k0 = 0; g2.a_k_bs = (int)(2 * sz);
-            g2.b_row0 = (int)sz; g2.b_row_bs = (int)(2 * sz); g2.b_k0 = 0; g2.b_k_bs = (int)(2 * sz);
-            CU(launch_tc_gemm(inv_maps, g2, h->sched, h->num_sms, s));
-            h->launches++;
-            continue;
-        }
-        // the narrow levels, and every level of an fp16-split handle without damping (nothing bounds the
+        // the narrow levels, and every level without damping (nothing bounds the
         // inverse in advance then): plain float32 products
         // T = B * C^-1
         GemmProblem p1 = make_problem(make_operand(H + sz, n, 1),
@@ -1201,14 +1109,6 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
         p2.batchN_last = tail;
         OK(gemm(h, p2, false, true, s));
     }
-    if (h->tensor && !h->f16) {
-        // operand copies of U for the products that follow: S1 = split(U), S2 = split(U^T)
-        // (FP16-split handles make theirs in gptaq_build_P, once the range of U is known)
-        CU(launch_split(H, n, S1h, S1l, n, n, n, false, SPLIT_UPPER, 1.f, s));
-        h->launches++;
-        CU(launch_split(H, n, S2h, S2l, n, n, n, true, SPLIT_UPPER, 1.f, s));
-        h->launches++;
-    }
     h->stage = STAGE_FACTORED;
     return GPTAQ_OK;
 }
@@ -1220,65 +1120,43 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
     const int n = (int)h->n;
     WsLayout wl = ws_layout(h->n, 0, 32);
     float *O = reinterpret_cast<float *>(h->ws + wl.t_off);
-    if (h->tensor && h->f16) {
-        // FP16-split operands (half the bytes and twice the MMA rate of the TF32 form): every operand is
+    if (h->tensor) {
+        // every operand is
         // scaled by a power of two into the fp16 range, so its largest magnitude is recorded first (by a
         // reduction kernel for U and dXX^T, by the producing GEMM's epilogue for O and P).
-        // Workspace: S[0] = U^T (kept for gptaq_quantize), S[1] = U, then P^T (kept), S[4] = dXX^T, then O.
-        const size_t nn = (size_t)n * n;
+        // Workspace: S[0] = U^T (kept for gptaq_quantize), S[1] = U, then P^T (kept), S[2] = dXX^T, then O.
+        const int64_t ldt = split_pitch(n);
+        const size_t nn = (size_t)n * ldt;
         __half *UT16 = reinterpret_cast<__half *>(h->ws + wl.s_off[0]);
         __half *U16 = reinterpret_cast<__half *>(h->ws + wl.s_off[1]);
-        __half *A16 = reinterpret_cast<__half *>(h->ws + wl.s_off[4]);
+        __half *A16 = reinterpret_cast<__half *>(h->ws + wl.s_off[2]);
         unsigned *am = h->hd->tc_amax;
         const float inv_tokens = (float)(1.0 / (double)h->tokens);
         CU(cudaMemsetAsync(am + AMAX_U, 0, 4 * sizeof(unsigned), s));      // slots U, D, O, P
         CU(launch_absmax(h->H, n, n, n, SPLIT_UPPER, 1.f, am + AMAX_U, h->num_sms, s));
         // (of dXX^T only the entries above the diagonal reach O: row j of U starts at column j and M_U keeps j > i)
         CU(launch_absmax(h->D, n, n, n, SPLIT_STRICT_UPPER, inv_tokens, am + AMAX_D, h->num_sms, s));
-        CU(launch_split16(h->H, n, U16, U16 + nn, n, n, n, false, SPLIT_UPPER, 1.f, am + AMAX_U, s, SplitBatch(),
+        CU(launch_split16(h->H, n, U16, U16 + nn, ldt, n, n, false, SPLIT_UPPER, 1.f, am + AMAX_U, s, SplitBatch(),
                           UT16, UT16 + nn));        // U and U^T in one pass
-        CU(launch_split16(h->D, n, A16, A16 + nn, n, n, n, false, SPLIT_STRICT_UPPER, inv_tokens, am + AMAX_D, s));
+        CU(launch_split16(h->D, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, inv_tokens, am + AMAX_D, s));
         h->launches += 4;
-        const SplitOperand Uop{U16, U16 + nn, n, n, n, true}, UTop{UT16, UT16 + nn, n, n, n, true};
-        const SplitOperand Aop{A16, A16 + nn, n, n, n, true};
+        const SplitOperand Uop{U16, U16 + nn, n, n, ldt}, UTop{UT16, UT16 + nn, n, n, ldt};
+        const SplitOperand Aop{A16, A16 + nn, n, n, ldt};
         TcMaps maps;
         // O = ((dXX^T / tokens) U^T) .* M_U  (contraction over k >= column, U[a][k] = 0 below)
         if (!make_tc_maps(&maps, Aop, Uop, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
         TcGemmArgs go = tc_args(O, n, n, n, n, 1.f, 0.f, TC_O, TC_MASK_STRICT_ZERO, h->hd);
         go.amax_a = am + AMAX_D; go.amax_b = am + AMAX_U; go.amax_out = am + AMAX_O;
         CU(launch_tc_gemm(maps, go, h->sched, h->num_sms, s));
-        CU(launch_split16(O, n, A16, A16 + nn, n, n, n, false, SPLIT_STRICT_UPPER, 1.f, am + AMAX_O, s));
+        CU(launch_split16(O, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, 1.f, am + AMAX_O, s));
         // P = alpha * O U  (B operand rows are rows of U^T)
         if (!make_tc_maps(&maps, Aop, UTop, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
         TcGemmArgs gp = tc_args(h->D, n, n, n, n, alpha, 0.f, TC_P, TC_MASK_STRICT_ZERO, h->hd);
         gp.amax_a = am + AMAX_O; gp.amax_b = am + AMAX_U; gp.amax_out = am + AMAX_P;
         CU(launch_tc_gemm(maps, gp, h->sched, h->num_sms, s));
         // P^T for the lazy-batch updates of gptaq_quantize, over the copy of U that is no longer needed
-        CU(launch_split16(h->D, n, U16, U16 + nn, n, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P, s));
+        CU(launch_split16(h->D, n, U16, U16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P, s));
         h->launches += 4;
-        h->stage = STAGE_P;
-        return GPTAQ_OK;
-    }
-    if (h->tensor) {
-        float *S[6];
-        for (int i = 0; i < 6; ++i) S[i] = reinterpret_cast<float *>(h->ws + wl.s_off[i]);
-        const SplitOperand Us{S[0], S[1], n, n, n}, UTs{S[2], S[3], n, n, n}, S3{S[4], S[5], n, n, n};
-        TcMaps maps;
-        // S3 = split(dXX^T / tokens);  O = (S3 U^T) .* M_U  (contraction over k >= column, U[a][k] = 0 below)
-        CU(launch_split(h->D, n, S[4], S[5], n, n, n, false, SPLIT_ALL, (float)(1.0 / (double)h->tokens), s));
-        h->launches++;
-        if (!make_tc_maps(&maps, S3, Us, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
-        CU(launch_tc_gemm(maps, tc_args(O, n, n, n, n, 1.f, 0.f, TC_O, TC_MASK_STRICT_ZERO, h->hd), h->sched, h->num_sms, s));
-        h->launches++;
-        // S3 = split(O);  P = alpha * O U  (B operand rows are rows of U^T)
-        CU(launch_split(O, n, S[4], S[5], n, n, n, false, SPLIT_STRICT_UPPER, 1.f, s));
-        h->launches++;
-        if (!make_tc_maps(&maps, S3, UTs, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
-        CU(launch_tc_gemm(maps, tc_args(h->D, n, n, n, n, alpha, 0.f, TC_P, TC_MASK_STRICT_ZERO, h->hd), h->sched, h->num_sms, s));
-        h->launches++;
-        // S3 = split(P^T) for the lazy-batch updates of gptaq_quantize
-        CU(launch_split(h->D, n, S[4], S[5], n, n, n, true, SPLIT_STRICT_UPPER, 1.f, s));
-        h->launches++;
         h->stage = STAGE_P;
         return GPTAQ_OK;
     }
@@ -1305,21 +1183,18 @@ gptaq_status_t gptaq_build_P_rowwise(gptaq_handle_t h, float alpha, gptaq_stream
     LAUNCHED();
     // the operand copies that gptaq_quantize reads, as gptaq_build_P leaves them
     WsLayout wl = ws_layout(h->n, 0, 32);
-    if (h->tensor && h->f16) {
-        const size_t nn = (size_t)n * n;
+    if (h->tensor) {
+        const int64_t ldt = split_pitch(n);
+        const size_t nn = (size_t)n * ldt;
         __half *UT16 = reinterpret_cast<__half *>(h->ws + wl.s_off[0]);
         __half *PT16 = reinterpret_cast<__half *>(h->ws + wl.s_off[1]);
         unsigned *am = h->hd->tc_amax;
         CU(cudaMemsetAsync(am + AMAX_U, 0, 4 * sizeof(unsigned), s));
         CU(launch_absmax(h->H, n, n, n, SPLIT_UPPER, 1.f, am + AMAX_U, h->num_sms, s));
         CU(launch_absmax(h->D, n, n, n, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P, h->num_sms, s));
-        CU(launch_split16(h->H, n, UT16, UT16 + nn, n, n, n, true, SPLIT_UPPER, 1.f, am + AMAX_U, s));
-        CU(launch_split16(h->D, n, PT16, PT16 + nn, n, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P, s));
+        CU(launch_split16(h->H, n, UT16, UT16 + nn, ldt, n, n, true, SPLIT_UPPER, 1.f, am + AMAX_U, s));
+        CU(launch_split16(h->D, n, PT16, PT16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P, s));
         h->launches += 4;
-    } else if (h->tensor) {
-        float *S4 = reinterpret_cast<float *>(h->ws + wl.s_off[4]), *S5 = reinterpret_cast<float *>(h->ws + wl.s_off[5]);
-        CU(launch_split(h->D, n, S4, S5, n, n, n, true, SPLIT_STRICT_UPPER, 1.f, s));
-        h->launches++;
     }
     h->stage = STAGE_P;
     return GPTAQ_OK;
@@ -1345,21 +1220,16 @@ gptaq_status_t gptaq_quantize(gptaq_handle_t h, void *d_W, int w_dtype, int64_t 
     t.perm = h->act_order ? h->perm : nullptr;
     t.clip_steps = h->clip_steps; t.clip_min = h->clip_min;
     t.static_groups = h->static_groups; t.dead_orig = h->dead_raw;
-    t.UT_hi = t.UT_lo = t.PT_hi = t.PT_lo = nullptr; t.EW_lo = nullptr;
-    // FP16-split updates; TF32-split for widths that are multiples of 4 only; plain float32 products otherwise.
-    // (Groups of fewer than 32 columns update block by block, and blocks of 32 columns are no whole K-block of 64.)
-    const bool f16 = h->f16 && ((blocksize % 64) == 0 || group <= 0 || (group % 32) == 0 || h->static_groups);
+    // fp16-split updates, plain float32 products otherwise
+    // (groups of fewer than 32 columns update block by block, and blocks of 32 columns are no whole K-block of 64)
+    const bool f16 = h->tensor && ((blocksize % 64) == 0 || group <= 0 || (group % 32) == 0 || h->static_groups);
     if (f16) {
+        t.ldt = split_pitch(h->n);
         t.UT16 = reinterpret_cast<const __half *>(h->ws + wl.s_off[0]);
         t.PT16 = reinterpret_cast<const __half *>(h->ws + wl.s_off[1]);
         t.EW16 = reinterpret_cast<__half *>(h->ws + wl.ew_lo_off);
         t.row_inv = reinterpret_cast<float *>(h->ws + wl.rs_off);
         t.amax_u = h->hd->tc_amax + AMAX_U; t.amax_p = h->hd->tc_amax + AMAX_P;
-    } else if (h->tensor && !h->f16) {
-        float *S[6];
-        for (int i = 0; i < 6; ++i) S[i] = reinterpret_cast<float *>(h->ws + wl.s_off[i]);
-        t.UT_hi = S[2]; t.UT_lo = S[3]; t.PT_hi = S[4]; t.PT_lo = S[5];
-        t.EW_lo = reinterpret_cast<float *>(h->ws + wl.ew_lo_off);
     }
     cudaError_t e = cudaSuccess;
     st = quantize_core(t, d_W, w_dtype, m, ldw, bits, group, sym, blocksize, d_codes, d_scales, d_zeros, d_Wq,
@@ -1431,7 +1301,6 @@ gptaq_status_t gptaq_quantize_static(const float *d_U, const float *d_P, int64_t
     t.dead = sc->base + STATIC_FLAGS_OFFSET;
     t.EW = reinterpret_cast<float *>(sc->base + STATIC_EW_OFFSET);
     t.num_sms = sc->num_sms;
-    t.UT_hi = t.UT_lo = t.PT_hi = t.PT_lo = nullptr; t.EW_lo = nullptr;
     int64_t launches = 0;
     st = quantize_core(t, d_W, w_dtype, m, ldw, bits, group, sym, blocksize, d_codes, d_scales, d_zeros, d_Wq, s,
                        &launches, &e);

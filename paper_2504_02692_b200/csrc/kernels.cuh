@@ -36,13 +36,6 @@ __host__ __device__ __forceinline__ float split_scale(float amax) {
     return ldexpf(1.f, 14 - e);
 }
 
-// Round to the nearest TF32 value (10 explicit mantissa bits), kept in a float.
-__device__ __forceinline__ float tf32_rn(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
-}
-
 // Programmatic dependent launch: a kernel launched with the stream-serialization attribute may be
 // scheduled while its predecessor in the stream drains; pdl_wait() returns once the predecessor has
 // completed and its writes are visible (a no-op for a plain launch), pdl_launch_dependents() lets the
@@ -261,7 +254,6 @@ struct ColumnLoopArgs {
     float *scales, *zeros;     // m x G
     int G;
     float *EW;                 // m x (2 * 32 * T): [-Err | Wpre]
-    float *EW_lo;              // nullptr, or: EW receives the TF32 value of each entry and EW_lo the remainder
     // fp16-split handles (else nullptr): Wpre is stored times rho = scale of U^T / scale of P^T (from the two recorded
     // maxima), which lets the two halves of the update's B operand keep scales of their own
     const unsigned *amax_u, *amax_p;
@@ -381,19 +373,12 @@ __global__ void __launch_bounds__(1024) column_loop_kernel(ColumnLoopArgs a) {
         rho = ap > 0.f ? split_scale(__uint_as_float(*a.amax_u)) / split_scale(ap) : 0.f;
     }
     float *ew = a.EW + (int64_t)row * (2 * BW);
-    float *ewl = a.EW_lo ? a.EW_lo + (int64_t)row * (2 * BW) : nullptr;
     uint8_t *crow = a.codes + (int64_t)row * n + i0;
 #pragma unroll
     for (int t = 0; t < T; ++t) {
         int c = lane + 32 * t;
-        if (ewl) {
-            const float eh = tf32_rn(nerr[t]), ph = tf32_rn(pre[t]);
-            ew[c] = eh; ewl[c] = tf32_rn(nerr[t] - eh);
-            ew[BW + c] = ph; ewl[BW + c] = tf32_rn(pre[t] - ph);
-        } else {
-            ew[c] = nerr[t];
-            ew[BW + c] = rho * pre[t];
-        }
+        ew[c] = nerr[t];
+        ew[BW + c] = rho * pre[t];
         if (c < bw) {
             wrow[c] = w[t];
             if (a.perm) a.codes[(int64_t)row * n + a.perm[i0 + c]] = (uint8_t)code[t];

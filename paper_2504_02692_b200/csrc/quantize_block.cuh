@@ -47,7 +47,6 @@ struct QuantBlockArgs {
     float *scales, *zeros;     // m x G
     int G;
     float *EW; int ew_ld, ew_pre;   // [-Err | rho * Wpre] of this launch, row pitch, offset of Wpre in a row
-    float *EW_lo;              // nullptr, or: EW receives the TF32 value of each entry and EW_lo the remainder
     // fp16 parts of [-Err | rho * Wpre] for the update beyond i1, one power-of-two scale per row (row_inv = 1 / scale),
     // or nullptr (nothing beyond); pitch ew_ld
     __half *EWS_hi, *EWS_lo;
@@ -604,18 +603,6 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                             p4[f] = rho * St[(32 + c4 + f) * QB_SLD + pos];
                         }
                         float *ew = a.EW + (int64_t)(row0 + r) * a.ew_ld + cw;
-                        if (a.EW_lo) {
-                            float *ewl = a.EW_lo + (int64_t)(row0 + r) * a.ew_ld + cw;
-                            float el[4], pl[4];
-#pragma unroll
-                            for (int f = 0; f < 4; ++f) {
-                                const float eh = tf32_rn(e4[f]), phi = tf32_rn(p4[f]);
-                                el[f] = tf32_rn(e4[f] - eh); pl[f] = tf32_rn(p4[f] - phi);
-                                e4[f] = eh; p4[f] = phi;
-                            }
-                            *reinterpret_cast<float4 *>(ewl) = make_float4(el[0], el[1], el[2], el[3]);
-                            *reinterpret_cast<float4 *>(ewl + a.ew_pre) = make_float4(pl[0], pl[1], pl[2], pl[3]);
-                        }
                         *reinterpret_cast<float4 *>(ew) = make_float4(e4[0], e4[1], e4[2], e4[3]);
                         *reinterpret_cast<float4 *>(ew + a.ew_pre) = make_float4(p4[0], p4[1], p4[2], p4[3]);
                     }

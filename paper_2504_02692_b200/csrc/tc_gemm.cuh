@@ -18,11 +18,11 @@
 // the non-zero part of triangular operands, a B operand that switches to a second matrix
 // after k_split ([U ; P] of the lazy-batch update), and masked stores.
 //
-// The kernel exists for two operand kinds.  TF32: hi / lo are float32 arrays holding TF32 values, no
-// range limits, 32 contraction steps per 128-byte row.  FP16: hi = fp16(s x), lo = fp16(s x - hi) with a
-// power-of-two scale s per operand that puts the largest magnitude at 2^14 (split16_kernel; the scale
-// is recomputed from the recorded maximum wherever it is needed), 64 contraction steps per row and
-// tcgen05.mma.kind::f16: half the operand bytes and twice the MMA rate for the same 22 bits.
+// The operands are hi = fp16(s x), lo = fp16(s x - hi) with a power-of-two scale s per operand that puts the largest
+// magnitude at 2^14 (split16_kernel; the scale is recomputed from the recorded maximum wherever it is needed), 64
+// contraction steps per 128-byte row and tcgen05.mma.kind::f16: half the operand bytes and twice the MMA rate of TF32
+// parts for the same 22 bits.  (Widths that are multiples of 4 only used to take TF32 parts, because a TMA row pitch has to
+// be a multiple of 16 bytes; the fp16 copies have a padded pitch instead.  777 x 2052: 2142 -> 1673 us.)
 //
 // Every wait on an mbarrier is bounded; see umma_gemm.cuh.
 #pragma once
@@ -30,11 +30,11 @@
 
 namespace gptaq {
 
-constexpr int TBM = 128, TBN = 256, TBK = 32, TSTAGES = 2;
-constexpr int TA_BYTES = TBM * TBK * 4;
-constexpr int TB_BYTES = TBN * TBK * 4;
+constexpr int TBM = 128, TBN = 256, TBK = 64, TSTAGES = 2;
+constexpr int TA_BYTES = TBM * TBK * 2;
+constexpr int TB_BYTES = TBN * TBK * 2;
 constexpr int TSTAGE_BYTES = 2 * TA_BYTES + 2 * TB_BYTES;
-constexpr int TCHUNK = 4;            // K-blocks (of 32) per accumulation chain in tensor memory
+constexpr int TCHUNK = 4;            // K-blocks per accumulation chain in tensor memory
 constexpr int TC_THREADS = 64 + 32 * UEPI_WARPS;
 // staging of the "C += ..." epilogue: per column half one 128 x 32 float32 box (128-byte rows, swizzled),
 // handed to the TMA unit as a bulk reduction
@@ -70,10 +70,10 @@ struct TcGemmArgs {
     float alpha, beta;
     int mode, mask;
     StateHeader *hd;
-    // FP16 operands: bit patterns of the operands' largest magnitudes (the B matrices share one scale);
-    // the result is divided by the two scales.  nullptr for TF32 operands.
+    // bit patterns of the operands' largest magnitudes (the B matrices share one scale); the result is divided by the two
+    // scales
     const unsigned *amax_a, *amax_b;
-    const float *row_inv;            // FP16 operands with one scale per row of A: 1 / scale of row i (amax_a null)
+    const float *row_inv;            // operands with one scale per row of A: 1 / scale of row i (amax_a null)
     unsigned *amax_out;              // if set: receives (atomicMax) the bit pattern of max |C| over what is stored
     int c_tma;                       // beta == 1, one batch entry: C += through bulk tensor reductions (mapC)
     int diag_off;                    // C is a block of columns of a square matrix: its column j is column j + diag_off there
@@ -126,17 +126,6 @@ __device__ __forceinline__ void tc_decode(const TcGemmArgs &a, int t, TcTile &ti
     ti.work = !ti.skip && ti.kb0 < ti.kb1;
 }
 
-__device__ __forceinline__ void umma_tf32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
-}
-
-// kind::tf32 instruction descriptor: TF32 A and B (both K-major), fp32 D, M = 128, N = 256.
-constexpr uint32_t UMMA_IDESC_TF32 = (1u << 4) | (2u << 7) | (2u << 10) | ((TBN >> 3) << 17) | ((TBM >> 4) << 24);
-
 // C[c1 .. , c0 ..] += box in shared memory (float32 add at the memory side, one request per box)
 __device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap *map, uint32_t src, int c0, int c1) {
     asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3}], [%1];"
@@ -164,14 +153,13 @@ __device__ __forceinline__ bool named_bar_any(int id, int nthreads, bool flag) {
     return r != 0;
 }
 
-template <bool F16>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant__ CUtensorMap mapAlo,
                const __grid_constant__ CUtensorMap mapBhi, const __grid_constant__ CUtensorMap mapBlo,
                const __grid_constant__ CUtensorMap mapB2hi, const __grid_constant__ CUtensorMap mapB2lo,
                const __grid_constant__ CUtensorMap mapC, TcGemmArgs a) {
-    constexpr int BK = F16 ? 2 * TBK : TBK;        // contraction steps per K-block (one 128-byte row)
-    constexpr int KSTEP = F16 ? 16 : 8;            // contraction steps per MMA (32 bytes)
+    constexpr int BK = TBK;                        // contraction steps per K-block (one 128-byte row)
+    constexpr int KSTEP = 16;                      // contraction steps per MMA (32 bytes)
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -297,8 +285,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                         const uint64_t blo = make_kmajor_desc(s0 + 2 * TA_BYTES + TB_BYTES);
                         // small terms first, the hi * hi term last
                         auto mma = [&](uint64_t ad, uint64_t bd, uint32_t accumulate) {
-                            if (F16) umma_f16(d_tmem, ad, bd, UMMA_IDESC_F16, accumulate);
-                            else umma_tf32(d_tmem, ad, bd, UMMA_IDESC_TF32, accumulate);
+                            umma_f16(d_tmem, ad, bd, UMMA_IDESC_F16, accumulate);
                         };
 #pragma unroll
                         for (int k = 0; k < BK / KSTEP; ++k)
@@ -325,10 +312,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
         float acc[TBN / 2];
         float out_max = 0.f;
         float op_scale = 1.f;            // 1 / (scale of A * scale of B), without the per-row part
-        if (F16) {
-            if (a.amax_a) op_scale /= split_scale(__uint_as_float(*a.amax_a));
-            if (a.amax_b) op_scale /= split_scale(__uint_as_float(*a.amax_b));
-        }
+        if (a.amax_a) op_scale /= split_scale(__uint_as_float(*a.amax_a));
+        if (a.amax_b) op_scale /= split_scale(__uint_as_float(*a.amax_b));
         TcTile ti;
         for (uint32_t taken = 0; ok; ++taken) {
             const uint32_t slot = taken % NR, sph = (taken / NR) & 1u;
@@ -370,7 +355,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                 // columns beyond the matrix are clipped by the tensor map.
                 if (named_bar_any(1 + half, 128, !ok)) { ok = false; break; }       // a wait gave up: all leave together
                 float alpha = a.alpha;
-                if (F16) alpha *= (a.row_inv && row < ti.Mz) ? op_scale * a.row_inv[row] : op_scale;
+                alpha *= (a.row_inv && row < ti.Mz) ? op_scale * a.row_inv[row] : op_scale;
                 const bool issuer = quarter == 2 && lane == 0;                       // first warp of the half
                 const int r_in = quarter * 32 + lane;
                 const uint32_t box = stg0 + half * TC_STG_BOX_BYTES;
@@ -403,7 +388,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
             float *cp = a.C + (long long)ti.z * a.c_bstride + (long long)row * a.ldc + col0;
             const float beta = a.beta;
             float alpha = a.alpha;
-            if (F16) alpha *= a.row_inv ? op_scale * a.row_inv[(long long)ti.z * a.M + row] : op_scale;
+            alpha *= a.row_inv ? op_scale * a.row_inv[(long long)ti.z * a.M + row] : op_scale;
             const bool vec_ok = (reinterpret_cast<uintptr_t>(cp) & 15) == 0;
 #pragma unroll
             for (int q = 0; q < TBN / 2 / 4; ++q) {
@@ -463,71 +448,18 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
 }
 
 // ---------------------------------------------------------------------------
-// Operand preparation: dst_hi / dst_lo <- split(scale * src), optionally transposed and
-// masked to the (strictly) upper triangle of the source, tile by tile through shared memory.
-//   src element (r, c), r < rows, c < cols, at src[r * lds + c];
-//   plain:      dst[r * ldd + c];   transposed: dst[c * ldd + r].
-// Elements outside the mask are written as zero.  blockIdx.z walks batch entries.
-// ---------------------------------------------------------------------------
-enum SplitMask { SPLIT_ALL = 0, SPLIT_UPPER = 1, SPLIT_STRICT_UPPER = 2 };
-
-struct SplitArgs {
-    const float *src; long long lds, src_bstride;
-    float *hi, *lo; long long ldd, dst_bstride;
-    int rows, cols, rows_last, cols_last, nbatch;
-    int transpose, mask;
-    float scale;
-};
-
-__global__ void __launch_bounds__(256) split_kernel(SplitArgs a) {
-    __shared__ float th[64][65], tl[64][65];
-    const int z = blockIdx.z;
-    const bool last = z == a.nbatch - 1;
-    const int rows = (last && a.rows_last) ? a.rows_last : a.rows;
-    const int cols = (last && a.cols_last) ? a.cols_last : a.cols;
-    const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
-    if (r0 >= rows || c0 >= cols) return;
-    const float *src = a.src + (long long)z * a.src_bstride;
-    float *hi = a.hi + (long long)z * a.dst_bstride, *lo = a.lo + (long long)z * a.dst_bstride;
-    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
-    for (int rr = ty; rr < 64; rr += 4) {
-        const int r = r0 + rr, c = c0 + tx;
-        float x = 0.f;
-        if (r < rows && c < cols) {
-            const bool keep = a.mask == SPLIT_ALL || (a.mask == SPLIT_UPPER ? c >= r : c > r);
-            if (keep) x = a.scale * src[(long long)r * a.lds + c];
-        }
-        const float h = tf32_rn(x);
-        const float l = tf32_rn(x - h);
-        if (!a.transpose) {
-            if (r < rows && c < cols) {
-                hi[(long long)r * a.ldd + c] = h;
-                lo[(long long)r * a.ldd + c] = l;
-            }
-        } else {
-            th[rr][tx] = h; tl[rr][tx] = l;
-        }
-    }
-    if (a.transpose) {
-        __syncthreads();
-        for (int cc = ty; cc < 64; cc += 4) {
-            const int c = c0 + cc, r = r0 + tx;
-            if (r < rows && c < cols) {
-                hi[(long long)c * a.ldd + r] = th[tx][cc];
-                lo[(long long)c * a.ldd + r] = tl[tx][cc];
-            }
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
 // FP16 operand preparation.  absmax_kernel (a CTA per row, strided) records max |scale * src| over the
 // (masked) region as a float bit pattern (atomicMax on the bits orders non-negative floats);
 // split16_kernel then writes
-// hi = fp16(s x), lo = fp16(s x - hi), x = scale * src, s = split_scale(recorded maximum), with the
-// same options as split_kernel.  The slot has to be zeroed before the first absmax_kernel into it;
-// several matrices that share a scale are reduced into the same slot.
+// hi = fp16(s x), lo = fp16(s x - hi), x = scale * src, s = split_scale(recorded maximum), optionally transposed and
+// masked to the (strictly) upper triangle of the source (elements outside are written as zero), tile by tile through
+// shared memory.  The slot has to be zeroed before the first absmax_kernel into it; several matrices that share a scale
+// are reduced into the same slot.
+//   src element (r, c), r < rows, c < cols, at src[r * lds + c];
+//   plain:      dst[r * ldd + c];   transposed: dst[c * ldd + r].
 // ---------------------------------------------------------------------------
+enum SplitMask { SPLIT_ALL = 0, SPLIT_UPPER = 1, SPLIT_STRICT_UPPER = 2 };
+
 __global__ void __launch_bounds__(256) absmax_kernel(const float *src, long long lds, int rows, int cols, int mask,
                                                      float scale, unsigned *slot) {
     __shared__ float red[8];
@@ -567,7 +499,7 @@ __global__ void __launch_bounds__(256) absmax_kernel(const float *src, long long
 struct Split16Args {
     const float *src; long long lds, src_bstride;
     __half *hi, *lo; long long ldd, dst_bstride;
-    int rows, cols, rows_last, cols_last, nbatch;      // blockIdx.z walks batch entries, as in split_kernel
+    int rows, cols, rows_last, cols_last, nbatch;      // blockIdx.z walks batch entries
     int transpose, mask;       // transpose 2: both forms, the plain one to (hi, lo), the transposed one to (hi_t, lo_t)
     float scale;
     const unsigned *amax;

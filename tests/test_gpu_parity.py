@@ -739,3 +739,28 @@ def test_factor_panels(n):
     sv = np.linalg.svd(ref, compute_uv=False)
     bound = (sv[0] / sv[-1]) ** 2 * np.sqrt(n) * 2.0 ** -22
     assert np.linalg.norm(U - ref) <= bound * np.linalg.norm(ref), (hp.rel_fro(U, ref), bound)
+
+
+@pytest.mark.parametrize("n", [512, 516, 1036, 1284])
+def test_split_operand_row_pitch(n):
+    """Tensor-core products whose fp16 operand copies have rows of 8 k and of 8 k + 4 columns (row pitch padded to a multiple
+    of 8): P from the device's own U and dXX^T.  Two products after one another, each an n-term sum whose factors and
+    roundings are good to 2^-22 of the products of the magnitudes."""
+    torch.manual_seed(n)
+    tokens, alpha = 2 * n, 0.5
+    X = torch.randn(tokens, n, device="cuda")
+    Xfp = X + 0.05 * torch.randn(tokens, n, device="cuda")
+    st = g.LayerState(n, 1, tokens, 32, "cuda")
+    try:
+        g.gptaq_accumulate(st.handle, X, Xfp)
+        D = np.triu(st.D().cpu().numpy().astype(np.float64), 1) / tokens
+        g.gptaq_factor(st.handle, 0.05)
+        g.gptaq_build_P(st.handle, alpha)
+        U = np.triu(st.H().cpu().numpy().astype(np.float64))
+        P = np.triu(st.D().cpu().numpy().astype(np.float64), 1)
+        assert g.gptaq_sync_status(st.handle)[0] == g.GPTAQ_OK
+    finally:
+        st.close()
+    ref = alpha * np.triu(np.triu(D @ U.T, 1) @ U, 1)
+    size = alpha * np.triu(np.triu(abs(D) @ abs(U).T, 1) @ abs(U), 1)
+    assert np.linalg.norm(P - ref) <= 2.0 ** -21 * np.linalg.norm(size), np.linalg.norm(P - ref) / np.linalg.norm(size)
