@@ -568,6 +568,9 @@ gptaq_status_t check_quantize_args(int64_t n, const void *d_W, int w_dtype, int6
         ++*launches;                                         \
     } while (0)
 
+// Rows per CTA of the column permutations: PERM_ROWS while two CTAs fit an SM, then fewer.
+int perm_rows(int n, size_t element) { return std::max(1, std::min(PERM_ROWS, (int)(100 * 1024 / (n * element)))); }
+
 // Algorithm 1, the blocked loop: launch sequence shared by the entry points that quantize.
 gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, int64_t m, int64_t ldw,
                              int bits, int group, int sym, int blocksize, uint8_t *d_codes, float *d_scales,
@@ -578,22 +581,22 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
     int64_t ldk = ldw;
     if (t.perm) {
         // working copy in sorted column order (the caller's d_Wq; checked to be a second buffer)
+        const size_t esz = w_dtype == GPTAQ_W_BF16 ? sizeof(__nv_bfloat16) : sizeof(float);
+        const int rows = perm_rows(n, esz);
+        const unsigned grid = (unsigned)std::min<int64_t>((m + rows - 1) / rows, t.num_sms * 8);
         if (w_dtype == GPTAQ_W_BF16)
-            gather_cols_kernel<__nv_bfloat16><<<t.num_sms * 8, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(d_W), ldw,
-                                                                           d_Wq, n, (int)m, n, t.perm);
+            gather_cols_kernel<__nv_bfloat16><<<grid, 256, rows * n * esz, s>>>(static_cast<const __nv_bfloat16 *>(d_W), ldw, d_Wq, n,
+                                                                              (int)m, n, t.perm, nullptr, rows);
         else
-            gather_cols_kernel<float><<<t.num_sms * 8, 256, 0, s>>>(static_cast<const float *>(d_W), ldw, d_Wq, n,
-                                                                   (int)m, n, t.perm);
+            gather_cols_kernel<float><<<grid, 256, rows * n * esz, s>>>(static_cast<const float *>(d_W), ldw, d_Wq, n, (int)m, n,
+                                                                      t.perm, nullptr, rows);
         QLAUNCHED();
         Wk = d_Wq; ldk = n;
-    } else if (w_dtype == GPTAQ_W_BF16) {
-        bf16_to_f32_kernel<<<t.num_sms * 8, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(d_W), ldw,
-                                                        d_Wq, n, (int)m, n);
-        QLAUNCHED();
-        Wk = d_Wq; ldk = n;
-    } else if (d_Wq && d_Wq != d_W) {
-        copy2d_kernel<<<t.num_sms * 8, 256, 0, s>>>(static_cast<const float *>(d_W), ldw, d_Wq, n,
-                                                   (int)m, n);
+    } else if (w_dtype == GPTAQ_W_BF16 || (d_Wq && d_Wq != d_W)) {
+        const dim3 grid((unsigned)((n + 1023) / 1024), (unsigned)std::min<int64_t>((m + WIDEN_ROWS - 1) / WIDEN_ROWS, 65535));
+        if (w_dtype == GPTAQ_W_BF16)
+            widen_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(d_W), ldw, d_Wq, n, (int)m, n);
+        else widen_kernel<float><<<grid, 256, 0, s>>>(static_cast<const float *>(d_W), ldw, d_Wq, n, (int)m, n);
         QLAUNCHED();
         Wk = d_Wq; ldk = n;
     }
@@ -688,7 +691,9 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
     }
     if (t.perm) {
         // dequantized weights back to the caller's column order
-        unpermute_rows_kernel<<<(unsigned)m, 256, (size_t)n * sizeof(float), s>>>(Wk, ldk, n, t.perm);
+        const int rows = perm_rows(n, sizeof(float));
+        const unsigned grid = (unsigned)std::min<int64_t>((m + rows - 1) / rows, t.num_sms * 8);
+        unpermute_rows_kernel<<<grid, 256, rows * n * sizeof(float), s>>>(Wk, ldk, (int)m, n, t.perm, rows);
         QLAUNCHED();
     }
     return GPTAQ_OK;
@@ -821,6 +826,10 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
         e = cudaFuncSetAttribute(convert_transpose_kernel<1>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(unpermute_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ACT_ORDER_MAX_N * 4);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(gather_cols_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ACT_ORDER_MAX_N * 4);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(gather_cols_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ACT_ORDER_MAX_N * 4);
     if (e != cudaSuccess) {
         delete h;
         return GPTAQ_ERR_CUDA;
@@ -946,20 +955,20 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
     diag_stats_kernel<<<1, 1024, 0, s>>>(H, n, (float)(1.0 / (double)h->tokens), damp, h->hd, h->dead_raw);
     LAUNCHED();
     if (h->act_order) {
-        // columns in order of decreasing diag(H): H and dXX^T are permuted on both sides, through T
-        rank_desc_kernel<<<(n + 255) / 256, 256, 0, s>>>(H, n, (float)(1.0 / (double)h->tokens), h->dead_raw, h->perm, h->dead);
+        // columns in order of decreasing diag(H): dXX^T and H are permuted on both sides, through T (H stays there until it
+        // is scaled)
+        rank_desc_kernel<<<(n + RANK_COLS - 1) / RANK_COLS, 256, 0, s>>>(H, n, (float)(1.0 / (double)h->tokens), h->dead_raw, h->perm, h->dead);
         LAUNCHED();
-        const dim3 pg((n + 255) / 256, n);
-        permute_matrix_kernel<<<pg, 256, 0, s>>>(H, T, n, h->perm, 1);
-        LAUNCHED();
-        CU(cudaMemcpyAsync(H, T, (size_t)n * n * sizeof(float), cudaMemcpyDeviceToDevice, s));
-        permute_matrix_kernel<<<pg, 256, 0, s>>>(h->D, T, n, h->perm, 0);
+        const int rows = perm_rows(n, sizeof(float));
+        gather_cols_kernel<float><<<std::min((n + rows - 1) / rows, h->num_sms * 8), 256, rows * n * sizeof(float), s>>>(h->D, n, T, n, n, n, h->perm, h->perm, rows);
         LAUNCHED();
         CU(cudaMemcpyAsync(h->D, T, (size_t)n * n * sizeof(float), cudaMemcpyDeviceToDevice, s));
+        permute_symmetric_kernel<<<dim3((n + 255) / 256, n), 256, 0, s>>>(H, T, n, h->perm);
+        LAUNCHED();
     } else {
         CU(cudaMemcpyAsync(h->dead, h->dead_raw, (size_t)n, cudaMemcpyDeviceToDevice, s));
     }
-    scale_damp_kernel<<<dim3((n + 63) / 64, (n + 15) / 16), 256, 0, s>>>(H, n, h->hd, h->dead);
+    scale_damp_kernel<<<dim3((n + 63) / 64, (n + 15) / 16), 256, 0, s>>>(h->act_order ? T : H, H, n, h->hd, h->dead);
     LAUNCHED();
 
     // reverse Cholesky H_d = R R^T, R upper, from the last block column upwards

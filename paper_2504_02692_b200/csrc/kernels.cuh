@@ -94,21 +94,23 @@ __global__ void __launch_bounds__(1024) diag_stats_kernel(const float *H, int n,
 // strict lower triangle <- 0.
 // Tiles of 64 columns x 16 rows, four columns of a row per thread: one load in flight per thread everywhere
 // (64 rows in a loop of dependent load-store pairs took 13 us at n = 1024).
-__global__ void __launch_bounds__(256) scale_damp_kernel(float *H, int n, const StateHeader *hd,
+// (src: H itself, or the matrix in sorted order.)
+__global__ void __launch_bounds__(256) scale_damp_kernel(const float *src, float *H, int n, const StateHeader *hd,
                                                          const uint8_t *dead) {
     const int j = blockIdx.x * 64 + 4 * (threadIdx.x & 15), i = blockIdx.y * 16 + (threadIdx.x >> 4);
     if (j >= n || i >= n) return;
     const float inv = hd->inv_tokens, lam = hd->lambda;
     float *p = H + (int64_t)i * n + j;
-    const bool vec = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(H) & 15) == 0;
+    const float *sp = src + (int64_t)i * n + j;
+    const bool vec = (n & 3) == 0 && ((reinterpret_cast<uintptr_t>(H) | reinterpret_cast<uintptr_t>(src)) & 15) == 0;
     float v[4] = {0.f, 0.f, 0.f, 0.f};
     if (j + 3 >= i) {
         if (vec) {
-            const float4 q = *reinterpret_cast<const float4 *>(p);
+            const float4 q = *reinterpret_cast<const float4 *>(sp);
             v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
         } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) if (j + e < n) v[e] = p[e];
+            for (int e = 0; e < 4; ++e) if (j + e < n) v[e] = sp[e];
         }
     }
 #pragma unroll
@@ -431,79 +433,126 @@ __global__ void __launch_bounds__(PR_THREADS) p_rowwise_kernel(float *D, const f
 // act_order: columns sorted by decreasing diag(H).
 // ---------------------------------------------------------------------------
 // perm[rank] = q, rank = number of inputs that sort before q: larger value v (v = 1 for dead
-// inputs, else H_qq / tokens), ties by smaller index (a stable descending sort).  O(n^2) compares.
+// inputs, else H_qq / tokens), ties by smaller index (a stable descending sort).  O(n^2) compares, RANK_COLS inputs
+// per CTA against all of them, in shared memory in chunks (a thread per input kept n / 256 CTAs busy: 63 us at n = 4096,
+// now 15).
+constexpr int RANK_COLS = 32, RANK_CHUNK = 4096;
 __global__ void __launch_bounds__(256) rank_desc_kernel(const float *H, int n, float inv_tokens, const uint8_t *dead,
                                                         int *perm, uint8_t *dead_perm) {
-    __shared__ float tile[256];
-    const int q = blockIdx.x * 256 + threadIdx.x;
-    const float vq = q < n ? (dead[q] ? 1.f : H[(int64_t)q * n + q] * inv_tokens) : 0.f;
-    int rank = 0;
-    for (int j0 = 0; j0 < n; j0 += 256) {
-        const int j = j0 + threadIdx.x;
-        tile[threadIdx.x] = j < n ? (dead[j] ? 1.f : H[(int64_t)j * n + j] * inv_tokens) : -1.f;
+    __shared__ float v[RANK_CHUNK];
+    const int lane = threadIdx.x & 31, q0 = blockIdx.x * RANK_COLS + (threadIdx.x >> 5) * (RANK_COLS / 8);
+    auto value = [&](int j) { return dead[j] ? 1.f : H[(int64_t)j * n + j] * inv_tokens; };
+    float vq[RANK_COLS / 8];
+    int rank[RANK_COLS / 8];
+#pragma unroll
+    for (int e = 0; e < RANK_COLS / 8; ++e) { vq[e] = q0 + e < n ? value(q0 + e) : 0.f; rank[e] = 0; }
+    for (int j0 = 0; j0 < n; j0 += RANK_CHUNK) {
+        const int lim = min(RANK_CHUNK, n - j0);
+        for (int t = threadIdx.x; t < lim; t += 256) v[t] = value(j0 + t);
         __syncthreads();
-        const int lim = min(256, n - j0);
-        for (int t = 0; t < lim; ++t) {
-            const float v = tile[t];
-            rank += (v > vq) || (v == vq && j0 + t < q);
+        for (int t = lane; t < lim; t += 32) {
+            const float x = v[t];
+#pragma unroll
+            for (int e = 0; e < RANK_COLS / 8; ++e) rank[e] += (x > vq[e]) || (x == vq[e] && j0 + t < q0 + e);
         }
         __syncthreads();
     }
-    if (q < n) { perm[rank] = q; dead_perm[rank] = dead[q]; }
+#pragma unroll
+    for (int e = 0; e < RANK_COLS / 8; ++e) {
+        const int r = __reduce_add_sync(0xffffffffu, rank[e]);
+        if (lane == 0 && q0 + e < n) { perm[r] = q0 + e; dead_perm[r] = dead[q0 + e]; }
+    }
 }
 
-// dst[i][j] = src[perm[i]][perm[j]]; `symmetric_upper`: src holds a symmetric matrix in its upper
-// triangle (element (a, b) is read at (min, max)) and only j >= i is written.
-__global__ void __launch_bounds__(256) permute_matrix_kernel(const float *src, float *dst, int n, const int *perm,
-                                                             int symmetric_upper) {
+// dst[i][j] = src[perm[i]][perm[j]], j >= i only, of a symmetric matrix given by its upper triangle (element (a, b) is read
+// at (min, max)).
+__global__ void __launch_bounds__(256) permute_symmetric_kernel(const float *src, float *dst, int n, const int *perm) {
     const int j = blockIdx.x * 256 + threadIdx.x;
     const int i = blockIdx.y;
-    if (j >= n) return;
-    if (symmetric_upper && j < i) return;
-    int a = perm[i], b = perm[j];
-    if (symmetric_upper && a > b) { const int t = a; a = b; b = t; }
-    dst[(int64_t)i * n + j] = src[(int64_t)a * n + b];
+    if (j >= n || j < i) return;
+    const int a = perm[i], b = perm[j];
+    dst[(int64_t)i * n + j] = src[(int64_t)min(a, b) * n + max(a, b)];
 }
 
-// dst[r][c] = src[r][perm[c]] as float32 (src float32 or bf16): the working copy of W in sorted order.
+// Rows in the two kernels below: as many as PERM_ROWS per CTA at a time, so that the order is read once for all of them;
+// staged in shared memory, so that device memory sees whole rows only.
+constexpr int PERM_ROWS = 4;
+
+// dst[r][c] = src[r][perm[c]] as float32 (src float32 or bf16), or src[row_perm[r]][perm[c]]: the working copy of W, and
+// dXX^T, in sorted order.  Bound by device
+// memory (4096 x 4096 bf16: 30 us; gathered from device memory element by element 51).
 template <typename T>
 __global__ void __launch_bounds__(256) gather_cols_kernel(const T *src, int64_t lds, float *dst, int64_t ldd, int m, int n,
-                                                          const int *perm) {
-    int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    const int64_t total = (int64_t)m * n;
-    for (; idx < total; idx += (int64_t)gridDim.x * 256) {
-        const int64_t r = idx / n, c = idx % n;
-        dst[r * ldd + c] = (float)src[r * lds + perm[c]];
+                                                          const int *perm, const int *row_perm, int rows) {
+    extern __shared__ __align__(16) float row_s[];
+    T *rs = reinterpret_cast<T *>(row_s);
+    for (int r0 = blockIdx.x * rows; r0 < m; r0 += gridDim.x * rows) {
+        const int nr = min(rows, m - r0);
+        for (int r = 0; r < nr; ++r) {
+            const T *sp = src + (int64_t)(row_perm ? row_perm[r0 + r] : r0 + r) * lds;
+#pragma unroll 8
+            for (int c = threadIdx.x; c < n; c += 256) rs[(size_t)r * n + c] = sp[c];
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int c = threadIdx.x; c < n; c += 256) {
+            const int p = perm[c];
+#pragma unroll
+            for (int r = 0; r < PERM_ROWS; ++r)
+                if (r < nr) dst[(int64_t)(r0 + r) * ldd + c] = (float)rs[(size_t)r * n + p];
+        }
+        __syncthreads();
     }
 }
 
-// In place, one CTA per row: W[r][perm[c]] <- W[r][c] (back to the original column order); the
-// row is staged in shared memory (n floats).
-__global__ void __launch_bounds__(256) unpermute_rows_kernel(float *W, int64_t ldw, int n, const int *perm) {
-    extern __shared__ float row_s[];
-    float *w = W + (int64_t)blockIdx.x * ldw;
-    for (int c = threadIdx.x; c < n; c += 256) row_s[c] = w[c];
-    __syncthreads();
-    for (int c = threadIdx.x; c < n; c += 256) w[perm[c]] = row_s[c];
-}
-
-__global__ void __launch_bounds__(256) bf16_to_f32_kernel(const __nv_bfloat16 *src, int64_t lds,
-                                                          float *dst, int64_t ldd, int m, int n) {
-    int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    int64_t total = (int64_t)m * n;
-    for (; idx < total; idx += (int64_t)gridDim.x * 256) {
-        int64_t r = idx / n, c = idx % n;
-        dst[r * ldd + c] = __bfloat162float(src[r * lds + c]);
+// In place: W[r][perm[c]] <- W[r][c] (back to the original column order).  Bound by device memory (4096 x 4096: 43 us;
+// scattered to device memory 81).
+__global__ void __launch_bounds__(256) unpermute_rows_kernel(float *W, int64_t ldw, int m, int n, const int *perm, int rows) {
+    extern __shared__ __align__(16) float row_s[];
+    for (int r0 = blockIdx.x * rows; r0 < m; r0 += gridDim.x * rows) {
+        const int nr = min(rows, m - r0);
+#pragma unroll 4
+        for (int c = threadIdx.x; c < n; c += 256) {
+            const int p = perm[c];
+            float v[PERM_ROWS];
+#pragma unroll
+            for (int r = 0; r < PERM_ROWS; ++r) if (r < nr) v[r] = W[(int64_t)(r0 + r) * ldw + c];
+#pragma unroll
+            for (int r = 0; r < PERM_ROWS; ++r) if (r < nr) row_s[(size_t)r * n + p] = v[r];
+        }
+        __syncthreads();
+        for (int r = 0; r < nr; ++r)
+#pragma unroll 8
+            for (int c = threadIdx.x; c < n; c += 256) W[(int64_t)(r0 + r) * ldw + c] = row_s[(size_t)r * n + c];
+        __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(256) copy2d_kernel(const float *src, int64_t lds, float *dst,
-                                                     int64_t ldd, int m, int n) {
-    int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    int64_t total = (int64_t)m * n;
-    for (; idx < total; idx += (int64_t)gridDim.x * 256) {
-        int64_t r = idx / n, c = idx % n;
-        dst[r * ldd + c] = src[r * lds + c];
+// dst[r][c] = src[r][c] as float32: the working copy of W.  A thread takes 4 columns of WIDEN_ROWS rows, all loads before the
+// first store.  Bound by device memory (16384 x 4096 bf16 58 us, one element at a time 160; 4096 x 4096 float32 18, 43).
+constexpr int WIDEN_ROWS = 8;
+template <typename T> struct alignas(4 * sizeof(T)) Quad { T v[4]; };
+template <typename T>
+__global__ void __launch_bounds__(256) widen_kernel(const T *src, int64_t lds, float *dst, int64_t ldd, int m, int n) {
+    const int c = (blockIdx.x * 256 + threadIdx.x) * 4;
+    if (c >= n) return;
+    const bool vec = c + 3 < n && (lds & 3) == 0 && (ldd & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & (4 * sizeof(T) - 1)) == 0 &&
+                     (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
+    for (int r0 = blockIdx.y * WIDEN_ROWS; r0 < m; r0 += gridDim.y * WIDEN_ROWS) {
+        if (vec) {
+            Quad<T> q[WIDEN_ROWS];
+#pragma unroll
+            for (int i = 0; i < WIDEN_ROWS; ++i)
+                if (r0 + i < m) q[i] = *reinterpret_cast<const Quad<T> *>(src + (int64_t)(r0 + i) * lds + c);
+#pragma unroll
+            for (int i = 0; i < WIDEN_ROWS; ++i)
+                if (r0 + i < m)
+                    *reinterpret_cast<float4 *>(dst + (int64_t)(r0 + i) * ldd + c) =
+                        make_float4((float)q[i].v[0], (float)q[i].v[1], (float)q[i].v[2], (float)q[i].v[3]);
+        } else {
+            for (int i = 0; i < WIDEN_ROWS && r0 + i < m; ++i)
+                for (int e = 0; e < 4 && c + e < n; ++e) dst[(int64_t)(r0 + i) * ldd + c + e] = (float)src[(int64_t)(r0 + i) * lds + c + e];
+        }
     }
 }
 
