@@ -529,10 +529,15 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
         return cudaErrorUnknown;
     const dim3 grid((unsigned)((m + QB_ROWS - 1) / QB_ROWS));
     const size_t smem = quant_block_smem_bytes(far_form, static_groups);
-    if (far_form && static_groups) quant_block_kernel<true, true><<<grid, QB_THREADS_FAR, smem, s>>>(uh, ul, ph, pl, a);
-    else if (far_form) quant_block_kernel<true, false><<<grid, QB_THREADS_FAR, smem, s>>>(uh, ul, ph, pl, a);
-    else if (static_groups) quant_block_kernel<false, true><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
-    else quant_block_kernel<false, false><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
+    // Near form, more CTAs than SMs: two to an SM, one works while the other waits for its own chain (16384 rows of 400
+    // columns 455 us, with one 498); below that one, which has the registers of both (1024 rows of 1024 columns 288 us, 301).
+    const bool two = grid.x > (unsigned)t.num_sms;
+    if (far_form && static_groups) quant_block_kernel<true, true, 1><<<grid, QB_THREADS_FAR, smem, s>>>(uh, ul, ph, pl, a);
+    else if (far_form) quant_block_kernel<true, false, 1><<<grid, QB_THREADS_FAR, smem, s>>>(uh, ul, ph, pl, a);
+    else if (static_groups && two) quant_block_kernel<false, true, 2><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
+    else if (static_groups) quant_block_kernel<false, true, 1><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
+    else if (two) quant_block_kernel<false, false, 2><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
+    else quant_block_kernel<false, false, 1><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
     return cudaGetLastError();
 }
 
@@ -541,10 +546,12 @@ cudaError_t configure_quantize_kernels() {
     const cudaFuncAttribute attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(column_loop_kernel<4>, attr, 2 * 128 * 128 * (int)sizeof(float));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(column_loop_kernel<2>, attr, 2 * 64 * 64 * (int)sizeof(float));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, true>, attr, (int)quant_block_smem_bytes(true, true));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, false>, attr, (int)quant_block_smem_bytes(true, false));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true>, attr, (int)quant_block_smem_bytes(false, true));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false>, attr, (int)quant_block_smem_bytes(false, false));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, true, 1>, attr, (int)quant_block_smem_bytes(true, true));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, false, 1>, attr, (int)quant_block_smem_bytes(true, false));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true, 1>, attr, (int)quant_block_smem_bytes(false, true));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true, 2>, attr, (int)quant_block_smem_bytes(false, true));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false, 1>, attr, (int)quant_block_smem_bytes(false, false));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false, 2>, attr, (int)quant_block_smem_bytes(false, false));
     return e;
 }
 

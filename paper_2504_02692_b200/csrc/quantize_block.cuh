@@ -5,7 +5,9 @@
 // memory; what would be a launch per block and a product per block over the whole matrix is a pipeline of
 // warp roles inside the CTA:
 //
-//   chain   (4 warps)  quantizes 32 columns at a time, four lanes per row with 8 consecutive columns each;
+//   chain   (4 warps)  quantizes 32 columns at a time, four lanes per row with 8 consecutive columns each (lanes 8 s .. 8 s + 7
+//                      hold columns 8 s .. of eight rows: a 16-byte read of U or P by 8 lanes is one word broadcast; with
+//                      the four lanes of a row side by side a launch took 4 % longer);
 //   near    (8 warps)  applies a step's errors to the rest of its 128-column block (float32 FMA), 8 columns
 //                      behind the chain, fetches the rows of U and P of the next step, writes results out;
 //   drain   (4 warps)  adds the products of the tensor cores to the later blocks of the slab;
@@ -13,9 +15,12 @@
 //                      D[128 later columns][32 rows] = [U^T | P^T] [-Err | rho Wpre]^T   (tcgen05, M = 128, N = 32)
 //                      for every 64 quantized columns, as lo*hi + hi*lo + hi*hi.
 //
-// What bounds it: the chain.  A column is 6 dependent float32 operations (24 cycles) as long as the next
+// What bounds it: the chain.  A column is 7 dependent float32 operations (28 cycles) as long as the next
 // column belongs to the same lane -- the lane goes on with its own error and pre-quantization value, the
-// shuffled copies that the other lanes need are off the chain -- and a shuffle more at every 8th column.
+// shuffled copies that the other lanes need are off the chain -- and a shuffle more at every 8th column.  It takes 110
+// (alone) to 200 cycles (beside the near warps of a block's first step), though: shared memory returns 128 bytes a cycle,
+// and a column's rows of U and P are 64 such words for the chain's four warps and up to 96 for the near warps.
+// A launch of 512 columns takes 80 us: 13 % of it the copies and products between blocks, 8 % filling the slab.
 #pragma once
 #include "tc_gemm.cuh"
 
@@ -71,7 +76,7 @@ __host__ __device__ constexpr QuantBlockSmem quant_block_smem(bool far_form, boo
     s.up = s.w + QB_ROWS * s.wld * 4;
     s.st = s.up + 2 * 32 * (QB_ULD0 + QB_ULD1) * 4;
     s.grid = s.st + 2 * 64 * QB_SLD * 4;
-    s.udinv = s.grid + (percol ? 2 * 32 * QB_SLD * 4 : 0);
+    s.udinv = s.grid + (percol ? 3 * 32 * QB_SLD * 4 : 0);
     s.perm = s.udinv + 2 * 32 * 4;
     s.inv = s.perm + 2 * 32 * 4;
     s.bars = s.inv + 2 * QB_ROWS * 4;
@@ -112,6 +117,12 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
 }
 __device__ __forceinline__ float pick2(const unsigned long long (&v)[4], int j) { return (j & 1) ? hi2(v[j >> 1]) : lo2(v[j >> 1]); }
 
+// 16 bytes of shared memory into (x, y) where `on`.
+__device__ __forceinline__ void lds128_if(bool on, const float *p, unsigned long long &x, unsigned long long &y) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q ld.shared.v2.u64 {%0, %1}, [%2];\n\t}"
+                 : "+l"(x), "+l"(y) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"((uint32_t)on));
+}
+
 // Range of a row over `len` columns (a multiple of 32) from w, by the row's four lanes.
 __device__ __forceinline__ void row_range(const float *w, int len, int sub, float &lo, float &hi) {
     lo = 0.f; hi = 0.f;
@@ -122,7 +133,7 @@ __device__ __forceinline__ void row_range(const float *w, int len, int sub, floa
         hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
     }
 #pragma unroll
-    for (int d = 1; d < 4; d <<= 1) {
+    for (int d = 8; d < 32; d <<= 1) {
         lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, d));
         hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, d));
     }
@@ -172,8 +183,9 @@ __device__ __forceinline__ void clip_search(const float *w, int n, float lo, flo
 }
 
 // FAR: several blocks per launch, updates between them on the tensor cores.  PERCOL: static groups, a grid per column.
-template <bool FAR, bool PERCOL>
-__global__ void __launch_bounds__(FAR ? QB_THREADS_FAR : QB_THREADS_NEAR, 1)
+// CTAS: CTAs that share an SM (shared memory allows one of the tensor-core form).
+template <bool FAR, bool PERCOL, int CTAS>
+__global__ void __launch_bounds__(FAR ? QB_THREADS_FAR : QB_THREADS_NEAR, CTAS)
 quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_constant__ CUtensorMap mapUlo,
                    const __grid_constant__ CUtensorMap mapPhi, const __grid_constant__ CUtensorMap mapPlo, QuantBlockArgs a) {
     extern __shared__ uint8_t smem_raw[];
@@ -187,7 +199,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     float *Ws = reinterpret_cast<float *>(sm + L.w);               // [32][WLD]: the slab
     float *UPs = reinterpret_cast<float *>(sm + L.up);             // rows of U and P of the current and the next step
     float *Sts = reinterpret_cast<float *>(sm + L.st);             // [2 steps][64][QB_SLD]: -Err, then Wpre, of 32 columns
-    float *grid_s = reinterpret_cast<float *>(sm + L.grid);        // PERCOL: scales, then zero points, [32 columns][QB_SLD] each
+    float *grid_s = reinterpret_cast<float *>(sm + L.grid);        // PERCOL: scales, zero points, 1 / scales, [32 columns][QB_SLD] each
     float *udinv2 = reinterpret_cast<float *>(sm + L.udinv);       // [2 steps][32]: err_scale / U_kk
     int *perm2 = reinterpret_cast<int *>(sm + L.perm);             // [2 steps][32]: where a column's codes go
     float *inv_s = reinterpret_cast<float *>(sm + L.inv);          // [2 halves][32]: 1 / scale of a row's errors
@@ -255,6 +267,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         for (int e = 0; e < 4; ++e) {
             grid_s[(c + e) * QB_SLD + r] = sc[e];
             grid_s[(32 + c + e) * QB_SLD + r] = zp[e];
+            grid_s[(64 + c + e) * QB_SLD + r] = 1.f / sc[e];
         }
     };
 
@@ -318,10 +331,12 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         rho = ap > 0.f ? su / split_scale(ap) : 0.f;
     }
     const int last_groups = nblk - 1;                               // blocks 0 .. nblk - 2 have later blocks in this launch
+    // a grid is made at column c (groups have 32, 64 or 128 columns)
+    auto grid_starts = [&](int c) { return !PERCOL && a.group > 0 && (c & (a.group - 1)) == 0; };
 
     if (tid < QB_CHAIN) {
         // ================================================================ chain
-        const int lrow = tid >> 2, sub = tid & 3;
+        const int lrow = 8 * warp + (lane & 7), sub = lane >> 3;
         const int row = row0 + lrow;
         const bool live = lrow < nrows;
         float *wrow = Ws + lrow * WLD;
@@ -329,6 +344,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         float scale = 1.f, zero = 0.f;
         float row_max = 0.f;                                        // largest magnitude of the row's errors in this launch
         if (!PERCOL && a.group <= 0 && live) { scale = a.scales[row]; zero = a.zeros[row]; }
+        float inv_scale = 1.f / scale, qlo = -zero, qhi = maxq - zero;
         for (int b = 0; b < nblk; ++b) {
             const int nst = nsteps(b);
             for (int s = 0; s < nst; ++s) {
@@ -343,9 +359,9 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     for (int e = 0; e < 8; ++e) {
                         scv[e] = grid_s[(8 * sub + e) * QB_SLD + lrow];
                         zv[e] = grid_s[(32 + 8 * sub + e) * QB_SLD + lrow];
-                        ivv[e] = 1.f / scv[e];
+                        ivv[e] = grid_s[(64 + 8 * sub + e) * QB_SLD + lrow];
                     }
-                } else if (a.group > 0 && (cg % a.group) == 0) {
+                } else if (grid_starts(cg)) {
                     // grid of the group that starts here, from the current values
                     // (columns of it beyond the layer are zeros)
                     float lo, hi;
@@ -363,8 +379,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         a.zeros[(int64_t)row * a.G + g] = zero;
                     }
                     if (a.clip_steps > 0) named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);   // the search's scratch is free again
+                    inv_scale = 1.f / scale; qlo = -zero; qhi = maxq - zero;
                 }
-                const float inv_scale = 1.f / scale, qlo = -zero, qhi = maxq - zero;
                 const int ld = up_ld(s);
                 const float *Us = up_buf(s) + 8 * sub, *Ps = Us + 32 * ld;
                 const float *ud = udinv2 + (s & 1) * 32;
@@ -407,8 +423,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         code[kk >> 2] |= (__float_as_uint(cz + z + magic) & 0xffu) << (8 * (kk & 3));
                         // the owner's next column, from its own values
                         if (kk < 7) c = fmaf(d, udv[kk] * pick2(u, kk + 1), fmaf(wa, pick2(pp, kk + 1), pick2(x, kk + 1)));
-                        const float ne_b = __shfl_sync(0xffffffffu, ne, ph, 4);
-                        const float wa_b = __shfl_sync(0xffffffffu, wa, ph, 4);
+                        const float ne_b = __shfl_sync(0xffffffffu, ne, 8 * ph + (lane & 7));
+                        const float wa_b = __shfl_sync(0xffffffffu, wa, 8 * ph + (lane & 7));
                         const unsigned long long ne2 = pack2(ne_b, ne_b), wa2 = pack2(wa_b, wa_b);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
@@ -454,8 +470,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                             v[d][1][e] = rho * S2[(32 + 8 * sub + e) * QB_SLD + pos];
                             mx = fmaxf(mx, fmaxf(fabsf(v[d][0][e]), fabsf(v[d][1][e])));
                         }
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
                     row_max = fmaxf(row_max, mx);
                     if (b < last_groups) {
                         const int half = s >> 1;                    // buffer: even and odd halves alternate
@@ -509,7 +525,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     if (t < 32) { next_ud = load_pivot(ncol + t); next_perm = load_perm(ncol + t); }
                     if (PERCOL) load_grid(t >> 3, ncol + 4 * (t & 7), next_sc, next_zp);
                 }
-                if (!PERCOL && a.group > 0 && a.clip_steps > 0 && ((i0 + co) % a.group) == 0) {
+                if (a.clip_steps > 0 && grid_starts(i0 + co)) {
                     // clipping-range search: thread = (row, one eighth of the candidates)
                     named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);     // the group's values are current
                     const int r = t & 31, cgi = t >> 5;

@@ -764,3 +764,18 @@ def test_split_operand_row_pitch(n):
     ref = alpha * np.triu(np.triu(D @ U.T, 1) @ U, 1)
     size = alpha * np.triu(np.triu(abs(D) @ abs(U).T, 1) @ abs(U), 1)
     assert np.linalg.norm(P - ref) <= 2.0 ** -21 * np.linalg.norm(size), np.linalg.norm(P - ref) / np.linalg.norm(size)
+
+
+@pytest.mark.parametrize("n,m,group,B", [
+    (96, 4737, 32, 32),         # block by block, one row more than a CTA of 32 on each of 148 SMs: two to an SM
+    (321, 31, 0, 128),          # odd width, a row short of a CTA
+    (512, 33, 64, 64),          # the narrowest tensor-core form, exactly one launch; a row more than a CTA
+    (516, 32, 128, 128),        # a launch of 512 columns and one of 4
+    (1060, 40, 32, 64),         # a grid at every step; the last block has two steps, the last of them 4 columns
+])
+def test_quantize_launch_edges(n, m, group, B):
+    """Forms of the column loop at the edges of their rows, blocks and launches (bounds as in the other parity tests)."""
+    cfg = wl.scaled(wl.CONFIGS["cfg2"], name="edges", n=n, m=m, batch_tokens=3 * n, n_batches=1, group=group, blocksize=B,
+                    outlier_channels=4)
+    out = hp.check_layer(cfg, wl.make_weight(cfg), batches_of(cfg), rows=np.unique(np.r_[0:m:max(1, m // 16), m - 1]))
+    hp.assert_parity(out)
