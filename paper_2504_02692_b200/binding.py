@@ -111,7 +111,8 @@ def _ptr(t) -> int | None:
 
 def _stream(stream) -> int | None:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream or None
+        # the current stream's handle without building a Stream object (3 us, as much as a launch)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream or None
     return int(stream) or None
@@ -126,11 +127,15 @@ def _check(status: int, what: str, handle=None):
 
 
 def _need_cuda(*tensors):
-    if not torch.cuda.is_available():
-        raise RuntimeError("the GPTAQ kernels need a CUDA device (no CPU fallback)")
+    on_device = False
     for t in tensors:
-        if t is not None and isinstance(t, torch.Tensor) and not t.is_cuda:
-            raise ValueError("expected a CUDA tensor")
+        if isinstance(t, torch.Tensor):
+            if not t.is_cuda:
+                _need_cuda()
+                raise ValueError("expected a CUDA tensor")
+            on_device = True
+    if not on_device and not torch.cuda.is_available():
+        raise RuntimeError("the GPTAQ kernels need a CUDA device (no CPU fallback)")
 
 
 # ---------------------------------------------------------------- size queries
@@ -368,15 +373,15 @@ class LayerState:
         if sb == 0 or wb == 0:
             raise ValueError("bad sizes")
         self.state = torch.empty(sb, dtype=torch.uint8, device=self.device)
+        self._state_f32 = self.state.view(torch.float32)
         self.workspace = torch.empty(wb, dtype=torch.uint8, device=self.device)
         self.handle = gptaq_create(n, self.state, self.workspace, stream)
         if total_tokens is not None:
             gptaq_set_stats_precision(self.handle, gptaq_recommended_stats_precision(n, total_tokens))
 
     def _view(self, ptr: int) -> torch.Tensor:
-        off = ptr - self.state.data_ptr()
-        nbytes = self.n * self.n * 4
-        return self.state[off:off + nbytes].view(torch.float32).view(self.n, self.n)
+        # float32 [n, n] at ptr in the state (one operation on a float32 view of the whole of it)
+        return self._state_f32.as_strided((self.n, self.n), (self.n, 1), (ptr - self.state.data_ptr()) // 4)
 
     def H(self) -> torch.Tensor:
         """View of H (before factor) / U (after), ``[n, n]`` float32, current on torch's stream."""

@@ -64,6 +64,8 @@ struct gptaq_ctx {
     bool gemm_pending[2];
     bool relayout;         // the operand buffers change size: wait for the products in flight first
     int next_buf;
+    // tensor maps of a buffer's operands (they lie in the workspace: only the padded token count and the layout matter)
+    struct StatsMaps { CUtensorMap x, d, xlo, dlo; int64_t kp, chunk; int narr; } stats_maps[2];
     // partial sums of the cut tiles of the statistics products wait in the workspace (fix_args.scratch) until
     // the sums are needed or the cut changes; fix_pending: they have not been added to H / dXX^T yet
     bool fix_pending;
@@ -106,7 +108,7 @@ struct WsLayout {
     size_t diag_off;        // inverses of the current diagonal block's sub-blocks, copy of the next diagonal block
     size_t s_off[3];        // split operand matrices, fp16 hi then lo (n x split_pitch(n) each)
     size_t pan_off[2];      // split copy of factor panels, hi / lo: n x SUPER_NB fp16
-    // [-Err | Wpre]: float32 (m x 2B, or m x 2 * QSUPER * B for the tensor-core update), its fp16 hi / lo parts, row scales
+    // [-Err | Wpre] of a launch: float32, its fp16 hi / lo parts (tensor cores), row scales
     size_t ew_off, ew_lo_off, rs_off, total;
     bool tensor;
 };
@@ -115,11 +117,11 @@ struct WsLayout {
 // the rank-128 update only touches the super-panel's remaining columns, the rest of the matrix receives
 // one rank-SUPER_NB update per super-panel (8x less read-modify-write traffic, longer contractions)
 constexpr int SUPER_NB = 8 * NB;
-// The lazy-batch update of gptaq_quantize likewise: a launch of quant_block_kernel takes up to QSUPER blocks
-// (at most QB_SUPER columns), everything beyond them receives their errors at once.
-constexpr int QSUPER = 8;
+// The lazy-batch update of gptaq_quantize likewise: a launch of quant_block_kernel takes QB_SUPER columns (QB_W without the
+// tensor cores), everything beyond them receives their errors at once.  The result does not depend on where the launches
+// end, so the caller's block size does not set their width (128 x 128 with blocks of 32: 3 launches for 9, 67 -> 28 us).
 
-WsLayout ws_layout(int64_t n, int64_t m_max, int blocksize) {
+WsLayout ws_layout(int64_t n, int64_t m_max) {
     WsLayout w;
     size_t nb = (size_t)((n + NB - 1) / NB);
     const size_t mat = round_up((size_t)n * (size_t)n * sizeof(float), ALIGN);
@@ -133,8 +135,7 @@ WsLayout ws_layout(int64_t n, int64_t m_max, int blocksize) {
     for (int i = 0; i < 3; ++i) { w.s_off[i] = off; if (w.tensor) off += smat; }
     const size_t pan = (size_t)n * SUPER_NB * sizeof(__half);
     for (int i = 0; i < 2; ++i) { w.pan_off[i] = off; if (w.tensor) off += round_up(pan, ALIGN); }
-    const size_t ew1 = round_up((size_t)m_max * 2 * (size_t)blocksize * sizeof(float), ALIGN);
-    const size_t ew = w.tensor ? QSUPER * ew1 : ew1;
+    const size_t ew = round_up((size_t)m_max * 2 * (w.tensor ? QB_SUPER : QB_W) * sizeof(float), ALIGN);
     w.ew_off = off;
     w.ew_lo_off = off + ew;
     w.rs_off = off + (w.tensor ? 2 * ew : ew);
@@ -408,7 +409,6 @@ gptaq_status_t accumulate_tc(gptaq_ctx *h, const float *X, const float *Xfp, int
             CU(cudaStreamWaitEvent(s, h->gemm_done[buf], 0));
             h->gemm_pending[buf] = false;
         }
-        CU(cudaMemsetAsync(amax, 0, 2 * sizeof(unsigned), s));
         ConvertArgs ca;
         ca.X = X + t0 * ld; ca.Xfp = Xfp + t0 * ld; ca.ld = ld; ca.tokens = tk; ca.n = n; ca.kp = kp;
         ca.Xt = Xt; ca.dXt = dXt; ca.Xlo = Xlo; ca.dXlo = dXlo; ca.amax = amax;
@@ -419,13 +419,17 @@ gptaq_status_t accumulate_tc(gptaq_ctx *h, const float *X, const float *Xfp, int
         LAUNCHED();
         CU(cudaEventRecord(h->conv_done[buf], s));
         CU(cudaStreamWaitEvent(gs, h->conv_done[buf], 0));
-        CUtensorMap mX, mD, mL, mDL;
-        const __half *lo = split ? Xlo : Xt;    // unused maps still have to be valid
-        const __half *dlo = splitd ? dXlo : dXt;
-        if (!make_kmajor_map(&mX, Xt, n, kp, UBM) || !make_kmajor_map(&mD, dXt, n, kp, UBM) ||
-            !make_kmajor_map(&mL, lo, n, kp, UBM) || !make_kmajor_map(&mDL, dlo, n, kp, UBM)) {
-            h->cuda_error = "cuTensorMapEncodeTiled failed";
-            return GPTAQ_ERR_CUDA;
+        gptaq_ctx::StatsMaps &mp = h->stats_maps[buf];
+        if (mp.kp != kp || mp.chunk != chunk || mp.narr != narr) {
+            const __half *lo = split ? Xlo : Xt;    // unused maps still have to be valid
+            const __half *dlo = splitd ? dXlo : dXt;
+            mp.kp = 0;
+            if (!make_kmajor_map(&mp.x, Xt, n, kp, UBM) || !make_kmajor_map(&mp.d, dXt, n, kp, UBM) ||
+                !make_kmajor_map(&mp.xlo, lo, n, kp, UBM) || !make_kmajor_map(&mp.dlo, dlo, n, kp, UBM)) {
+                h->cuda_error = "cuTensorMapEncodeTiled failed";
+                return GPTAQ_ERR_CUDA;
+            }
+            mp.kp = kp; mp.chunk = chunk; mp.narr = narr;
         }
         StatsGemmArgs ga;
         ga.H = h->H; ga.D = h->D; ga.n = n; ga.kblocks = kp / UBK; ga.nseg_h = split ? 3 : 1; ga.nseg_d = splitd ? 3 : 1; ga.amax = amax; ga.hd = h->hd;
@@ -465,7 +469,7 @@ gptaq_status_t accumulate_tc(gptaq_ctx *h, const float *X, const float *Xfp, int
             h->fix_args = ga;
             h->fix_pending = true;
         }
-        stats_umma_kernel<<<sgrid, UMMA_THREADS, UMMA_SMEM, gs>>>(mX, mD, mL, mDL, ga);
+        stats_umma_kernel<<<sgrid, UMMA_THREADS, UMMA_SMEM, gs>>>(mp.x, mp.d, mp.xlo, mp.dlo, ga);
         LAUNCHED();
         if (tev) CU(cudaEventRecord(tev->second, gs));
         CU(cudaEventRecord(h->gemm_done[buf], gs));
@@ -486,6 +490,7 @@ struct QuantizeTarget {
     StateHeader *hd;
     TcSched *sched;            // host-side count of the tile numbers drawn from hd->sched_counter
     float *EW;
+    int64_t ew_floats;         // its size
     int num_sms;
     // tensor-core trailing update (null: plain float32 products): U^T and P^T as fp16 hi / lo (row pitch ldt,
     // lo = hi + n * ldt), each with the scale of its recorded maximum; EW is then m x 2 * SW wide (SW columns per
@@ -503,7 +508,7 @@ struct QuantizeTarget {
 };
 
 // One launch of quant_block_kernel: columns [i0, i1) of the loop, SW columns per launch at most.
-cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, int64_t m, int i0, int i1, int blocksize, int SW,
+cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, int64_t m, int i0, int i1, int SW,
                                int bits, int group, int sym, uint8_t *codes, float *scales, float *zeros, int G,
                                bool static_groups, cudaStream_t s) {
     const bool far_form = t.UT16 != nullptr;
@@ -511,7 +516,7 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
     QuantBlockArgs a;
     std::memset(&a, 0, sizeof(a));
     a.W = W; a.ldw = ldw; a.m = (int)m; a.n = t.n; a.U = t.U; a.P = t.P; a.dead = t.dead;
-    a.i0 = i0; a.i1 = i1; a.bw = far_form ? QB_W : blocksize;
+    a.i0 = i0; a.i1 = i1; a.bw = far_form ? QB_W : SW;
     a.bits = bits; a.group = group; a.sym = sym;
     a.codes = codes; a.scales = scales; a.zeros = zeros; a.G = G;
     a.ew_ld = 2 * SW; a.ew_pre = SW;
@@ -633,9 +638,8 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
     // Smaller groups take column_loop_kernel (one warp per row, any group).
     const bool steps = group <= 0 || (group % 32) == 0 || static_groups;
     const bool tensor = t.UT16 != nullptr;
-    // columns per launch: as many blocks as the slab holds where the tensor cores carry the updates between them
-    // (the workspace holds the errors of QSUPER blocks), one block otherwise
-    const int SW = tensor && steps ? std::min(QB_SUPER, QSUPER * blocksize) : blocksize;
+    // columns per launch: as many as the slab holds (and the scratch has room for the errors of), else the caller's block
+    const int SW = !steps ? blocksize : tensor ? QB_SUPER : (n <= QB_W || t.ew_floats >= m * 2 * QB_W) ? QB_W : blocksize;
     TcMaps maps;
     if (tensor) {
         const size_t nn = (size_t)n * t.ldt, me = (size_t)m * 2 * SW;
@@ -646,7 +650,7 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
     for (int i0 = 0; i0 < n; i0 += SW) {
         const int i1 = std::min(i0 + SW, n);
         if (steps) {
-            *err = launch_quant_block(t, Wk, ldk, m, i0, i1, blocksize, SW, bits, group, sym, d_codes, d_scales, d_zeros, G,
+            *err = launch_quant_block(t, Wk, ldk, m, i0, i1, SW, bits, group, sym, d_codes, d_scales, d_zeros, G,
                                       static_groups, s);
             if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
             ++*launches;
@@ -688,9 +692,8 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
             // W[:, i1:] += [-Err | Wpre] * [U[blk, i1:] ; P[blk, i1:]]   (lazy-batch update)
             Operand bop = make_operand(t.U + (int64_t)i0 * n + i1, 1, n);
             bop.p2 = t.P + (int64_t)i0 * n + i1;
-            bop.k_split = blocksize;
-            GemmProblem pt = make_problem(make_operand(EW, 2 * blocksize, 1), bop, Wk + i1, ldk,
-                                          (int)m, n - i1, 2 * blocksize, 1.f, 1.f, GEMM_FULL);
+            bop.k_split = SW;
+            GemmProblem pt = make_problem(make_operand(EW, 2 * SW, 1), bop, Wk + i1, ldk, (int)m, n - i1, 2 * SW, 1.f, 1.f, GEMM_FULL);
             *err = launch_simt_gemm(pt, false, true, s);
             if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
             ++*launches;
@@ -773,7 +776,7 @@ size_t gptaq_workspace_bytes(int64_t n, int64_t m_max, int64_t max_batch_tokens,
     // the fp16 operand copies of one token batch share the space of the later steps' scratch
     size_t kp = round_up((size_t)max_batch_tokens, (size_t)UBK);
     size_t xt = 2 * round_up(3 * (size_t)n * kp * 2, ALIGN) + stats_scratch_bytes(MAX_SMS_FOR_SIZING);
-    return std::max(ws_layout(n, m_max, blocksize).total, xt);
+    return std::max(ws_layout(n, m_max).total, xt);
 }
 
 gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_t state_bytes,
@@ -785,7 +788,7 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
         return GPTAQ_ERR_INVALID_ARG;
     Layout l = state_layout(n);
     if (state_bytes < l.total) return GPTAQ_ERR_WORKSPACE;
-    if (workspace_bytes < ws_layout(n, 0, 32).total) return GPTAQ_ERR_WORKSPACE;
+    if (workspace_bytes < ws_layout(n, 0).total) return GPTAQ_ERR_WORKSPACE;
     gptaq_ctx *h = new (std::nothrow) gptaq_ctx();
     if (!h) return GPTAQ_ERR_INVALID_ARG;
     h->n = n;
@@ -844,6 +847,7 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
     h->gemm_stream = nullptr;
     h->relayout = false;
     h->next_buf = 0;
+    h->stats_maps[0].kp = h->stats_maps[1].kp = 0;
     h->fix_pending = false;
     h->d_upper_only = false;
     for (int i = 0; i < 2; ++i) { h->conv_done[i] = h->gemm_done[i] = nullptr; h->gemm_pending[i] = false; }
@@ -912,6 +916,14 @@ gptaq_status_t gptaq_accumulate(gptaq_handle_t h, const float *d_X, const float 
     // H (upper tiles) += X X^T
     Operand xa = make_operand(d_X, 1, ld);
     GemmProblem ph = make_problem(xa, xa, h->H, n, n, n, (int)tokens, 1.f, 1.f, GEMM_UPPER_TILES);
+    // (narrow layers: with the second sum in one launch)
+    GemmProblem both = ph;
+    both.nbatch = 2; both.paired = 1; both.pair_mode = GEMM_FULL; both.pair_sub = d_Xfp; both.pair_C = h->D;
+    if (simt_tiles(both) <= SIMT_SMALL_TILES) {
+        OK(gemm(h, both, true, true, s));
+        h->tokens += tokens;
+        return GPTAQ_OK;
+    }
     OK(gemm(h, ph, true, true, s));
     // dXX^T += (X~ - X) X^T, the difference taken in float32 at load time
     Operand da = xa;
@@ -954,7 +966,7 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
     OK(join_statistics(h, s));
     const int n = (int)h->n;
     const int nb = (n + NB - 1) / NB;
-    WsLayout wl = ws_layout(h->n, 0, 32);
+    WsLayout wl = ws_layout(h->n, 0);
     float *T = reinterpret_cast<float *>(h->ws + wl.t_off);
     float *Rinv = reinterpret_cast<float *>(h->ws + wl.rinv_off);
     float *H = h->H;
@@ -1134,7 +1146,7 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
     if (h->stage != STAGE_FACTORED) return GPTAQ_ERR_BAD_STATE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int n = (int)h->n;
-    WsLayout wl = ws_layout(h->n, 0, 32);
+    WsLayout wl = ws_layout(h->n, 0);
     float *O = reinterpret_cast<float *>(h->ws + wl.t_off);
     if (h->tensor) {
         // every operand is
@@ -1198,7 +1210,7 @@ gptaq_status_t gptaq_build_P_rowwise(gptaq_handle_t h, float alpha, gptaq_stream
     p_rowwise_kernel<<<n, PR_THREADS, 2 * (size_t)n * sizeof(float), s>>>(h->D, h->H, n, (float)((double)alpha / (double)h->tokens));
     LAUNCHED();
     // the operand copies that gptaq_quantize reads, as gptaq_build_P leaves them
-    WsLayout wl = ws_layout(h->n, 0, 32);
+    WsLayout wl = ws_layout(h->n, 0);
     if (h->tensor) {
         const int64_t ldt = split_pitch(n);
         const size_t nn = (size_t)n * ldt;
@@ -1226,11 +1238,12 @@ gptaq_status_t gptaq_quantize(gptaq_handle_t h, void *d_W, int w_dtype, int64_t 
                                             d_scales, d_zeros, d_Wq);
     if (st != GPTAQ_OK || m == 0) return st;
     if (h->act_order && (!d_Wq || d_Wq == d_W)) return GPTAQ_ERR_INVALID_ARG;
-    WsLayout wl = ws_layout(h->n, m, blocksize);
+    WsLayout wl = ws_layout(h->n, m);
     if (h->ws_bytes < wl.total) return GPTAQ_ERR_WORKSPACE;
     QuantizeTarget t;
     t.n = (int)h->n; t.U = h->H; t.P = h->D; t.dead = h->dead; t.hd = h->hd; t.sched = &h->sched;
     t.EW = reinterpret_cast<float *>(h->ws + wl.ew_off);
+    t.ew_floats = (int64_t)((wl.ew_lo_off - wl.ew_off) / sizeof(float));
     t.num_sms = h->num_sms;
     t.terms = h->terms;
     t.perm = h->act_order ? h->perm : nullptr;
@@ -1316,6 +1329,7 @@ gptaq_status_t gptaq_quantize_static(const float *d_U, const float *d_P, int64_t
     t.hd = reinterpret_cast<StateHeader *>(sc->base);
     t.dead = sc->base + STATIC_FLAGS_OFFSET;
     t.EW = reinterpret_cast<float *>(sc->base + STATIC_EW_OFFSET);
+    t.ew_floats = GPTAQ_STATIC_SCRATCH_FLOATS;
     t.num_sms = sc->num_sms;
     int64_t launches = 0;
     st = quantize_core(t, d_W, w_dtype, m, ldw, bits, group, sym, blocksize, d_codes, d_scales, d_zeros, d_Wq, s,

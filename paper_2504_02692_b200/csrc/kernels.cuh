@@ -18,7 +18,8 @@ struct StateHeader {
     unsigned amax[2][2]; // per operand buffer: bit patterns of max|X| and max|X~ - X| of the batch converted into it
     unsigned tc_amax[8]; // largest magnitudes of FP16-split operands of the float32-grade GEMMs (see tc_gemm.cuh)
     unsigned sched_counter; // tile numbers drawn by the float32-grade GEMM launches so far (never reset between launches)
-    int pad1[13];
+    unsigned stats_done;    // CTAs of the running statistics product that have finished
+    int pad1[12];
 };
 static_assert(sizeof(StateHeader) == 128, "header size");
 

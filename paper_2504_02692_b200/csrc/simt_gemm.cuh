@@ -46,6 +46,10 @@ struct GemmProblem {
     int64_t batchA, batchB, batchC;
     int batchM_last, batchN_last, batchK_last;  // dims of the last batch entry (ragged tail), 0 = same
     int nbatch;
+    // `paired` (32 x 32 tiles only, nbatch 2): entry 1 is the product (pair_sub - A) B into pair_C with its own mode
+    int paired, pair_mode;
+    const float *pair_sub;
+    float *pair_C;
 };
 
 constexpr int GBM = 128, GBN = 128, GBK = 16, GPAD = 4;
@@ -299,7 +303,8 @@ __global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, 
     }
     const int i0 = blockIdx.y * SGT, j0 = blockIdx.x * SGT;
     if (i0 >= M || j0 >= N) return;                                   // (the same for the CTAs of a cluster)
-    const int mode = pr.mode;
+    const bool pair1 = pr.paired && z == 1;
+    const int mode = pair1 ? pr.pair_mode : pr.mode;
     bool skip = false;
     int kb = 0, ke = K;
     if (mode == GEMM_UPPER_TILES) skip = i0 >= j0 + SGT;
@@ -317,7 +322,7 @@ __global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, 
 
     const float *A = pr.A.p + z * pr.batchA, *B = pr.B.p + z * pr.batchB;
     const float *A2 = pr.A.p2 ? pr.A.p2 + z * pr.batchA : nullptr, *B2 = pr.B.p2 ? pr.B.p2 + z * pr.batchB : nullptr;
-    const float *Asub = pr.A.sub ? pr.A.sub + z * pr.batchA : nullptr;
+    const float *Asub = pair1 ? pr.pair_sub : (pr.A.sub ? pr.A.sub + z * pr.batchA : nullptr);
     const int stage_floats = (Asub ? 3 : 2) * SG_TILE;
     const int nk = max(0, (ke - kb + SGK - 1) / SGK);
     auto fetch = [&](int t) {
@@ -349,7 +354,7 @@ __global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, 
 #pragma unroll
     for (int t = 0; t < SG_STAGES - 1; ++t) fetch(t);
     // what C holds arrives under the products (read at the end, each value would wait for its own round trip)
-    float *C = pr.C + z * pr.batchC;
+    float *C = pair1 ? pr.pair_C : pr.C + z * pr.batchC;
     const bool masked = mode == GEMM_O || mode == GEMM_P;
     const bool add_c = pr.beta != 0.f && !masked;
     float cv[4][4];
@@ -456,7 +461,7 @@ inline cudaError_t launch_simt_small(const GemmProblem &pr, cudaStream_t s) {
     grid.z *= ksplit;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(SG_THREADS); cfg.stream = s;
-    cfg.dynamicSmemBytes = (size_t)SG_STAGES * (pr.A.sub ? 3 : 2) * SG_TILE * sizeof(float);
+    cfg.dynamicSmemBytes = (size_t)SG_STAGES * (pr.A.sub || pr.paired ? 3 : 2) * SG_TILE * sizeof(float);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = (unsigned)ksplit;
@@ -488,7 +493,8 @@ inline GemmProblem make_problem(Operand A, Operand B, float *C, int64_t ldc, int
                                 float alpha, float beta, int mode) {
     GemmProblem p; p.A = A; p.B = B; p.C = C; p.ldc = ldc; p.M = M; p.N = N; p.K = K;
     p.alpha = alpha; p.beta = beta; p.mode = mode; p.batchA = p.batchB = p.batchC = 0;
-    p.batchM_last = p.batchN_last = p.batchK_last = 0; p.nbatch = 1; return p;
+    p.batchM_last = p.batchN_last = p.batchK_last = 0; p.nbatch = 1;
+    p.paired = p.pair_mode = 0; p.pair_sub = nullptr; p.pair_C = nullptr; return p;
 }
 
 }  // namespace gptaq

@@ -353,7 +353,7 @@ struct StatsGemmArgs {
     int kblocks;             // kp / 64
     int nseg_h;              // 1: H = hi hi^T;  3: H = hi hi^T + hi lo^T + lo hi^T (split operands)
     int nseg_d;              // 1: dXX^T = dh xh^T;  3: dh xh^T + dh xl^T + dl xh^T
-    const unsigned *amax;    // scales are recomputed from the recorded maxima
+    unsigned *amax;          // scales are recomputed from the recorded maxima; zero again when the launch is done
     StateHeader *hd;
     // Work items of a CTA pair: tiles [0, full_tiles) are whole 256 x 256 tiles; each of the remaining
     // `ntiles - full_tiles` tiles (the last, partial wave) is cut along K into `ksplit` items so that every
@@ -634,6 +634,12 @@ stats_umma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     __syncthreads();
     cluster_sync_all();
     if (*abort_flag && threadIdx.x == 0) record_status(a.hd, ST_TIMEOUT, blockIdx.x);
+    // the last CTA clears the maxima for the next batch that is converted into this buffer (which waits for this launch;
+    // launches of one handle run one after the other)
+    if (threadIdx.x == 0 && atomicAdd(&a.hd->stats_done, 1u) == gridDim.x - 1) {
+        a.amax[0] = 0u; a.amax[1] = 0u;
+        a.hd->stats_done = 0u;
+    }
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
