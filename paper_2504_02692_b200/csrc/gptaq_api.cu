@@ -236,8 +236,8 @@ struct TcMaps {
 bool make_tc_maps(TcMaps *m, const SplitOperand &A, const SplitOperand &B, const SplitOperand *B2) {
     const SplitOperand &b2 = B2 ? *B2 : B;
     return make_operand_map(&m->a_hi, A.hi, A, TBM) && make_operand_map(&m->a_lo, A.lo, A, TBM) &&
-           make_operand_map(&m->b_hi, B.hi, B, TBN) && make_operand_map(&m->b_lo, B.lo, B, TBN) &&
-           make_operand_map(&m->b2_hi, b2.hi, b2, TBN) && make_operand_map(&m->b2_lo, b2.lo, b2, TBN);
+           make_operand_map(&m->b_hi, B.hi, B, TBOX) && make_operand_map(&m->b_lo, B.lo, B, TBOX) &&
+           make_operand_map(&m->b2_hi, b2.hi, b2, TBOX) && make_operand_map(&m->b2_lo, b2.lo, b2, TBOX);
 }
 
 // Launch with programmatic stream serialization: the kernel may be scheduled while its predecessor
@@ -281,7 +281,8 @@ bool make_c_map(CUtensorMap *map, float *C, int64_t M, int64_t N, int64_t ldc) {
 cudaError_t launch_tc_gemm(const TcMaps &m, const TcGemmArgs &a_in, TcSched &sched, int num_sms, cudaStream_t s, bool pdl = true) {
     if (a_in.M <= 0 || a_in.N <= 0 || a_in.nbatch <= 0) return cudaSuccess;
     TcGemmArgs a = a_in;
-    const int64_t tiles = (int64_t)a.nbatch * ((a.M + TBM - 1) / TBM) * ((a.N + TBN - 1) / TBN);
+    const int bn = tc_tile_width(a, num_sms);
+    const int64_t tiles = (int64_t)a.nbatch * ((a.M + TBM - 1) / TBM) * ((a.N + bn - 1) / bn);
     const int grid = (int)std::min<int64_t>(tiles, num_sms);
     // "C += ...": bulk tensor reductions where the target qualifies for a tensor map (16-byte aligned base
     // and row pitch); scattered per-thread reductions otherwise
@@ -293,7 +294,8 @@ cudaError_t launch_tc_gemm(const TcMaps &m, const TcGemmArgs &a_in, TcSched &sch
     if (a.beta == 1.f && a.nbatch == 1 && !a.amax_out && (a.mask == TC_MASK_NONE || a.mask == TC_MASK_UPPER_KEEP) &&
         (reinterpret_cast<uintptr_t>(a.C) & 15) == 0 && (a.ldc & 3) == 0 && make_c_map(&mapC, a.C, a.M, a.N, a.ldc))
         a.c_tma = 1;
-    return launch_pdl(pdl, tc_gemm_kernel, dim3(grid), dim3(TC_THREADS), TC_SMEM, s, m.a_hi, m.a_lo, m.b_hi, m.b_lo, m.b2_hi, m.b2_lo, mapC, a);
+    return launch_pdl(pdl, bn == 256 ? tc_gemm_kernel<256> : bn == 128 ? tc_gemm_kernel<128> : tc_gemm_kernel<64>, dim3(grid),
+                      dim3(TC_THREADS), tc_smem(bn), s, m.a_hi, m.a_lo, m.b_hi, m.b_lo, m.b2_hi, m.b2_lo, mapC, a);
 }
 
 // Slots of StateHeader::tc_amax (largest magnitudes of FP16-split operands).
@@ -825,7 +827,11 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(stats_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UMMA_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
+        e = cudaFuncSetAttribute(tc_gemm_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem(256));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(tc_gemm_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem(128));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(tc_gemm_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_smem(64));
     // the conversion of the next batch shares the SMs with the running product: both kernels ask for
     // the largest shared-memory carve-out, so that a conversion CTA fits beside a product CTA
     if (e == cudaSuccess)

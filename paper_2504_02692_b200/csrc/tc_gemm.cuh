@@ -5,7 +5,7 @@
 // on the tensor cores with float32 accumulation in tensor memory: about 22 significant bits
 // per factor, which is what the factorisation, the correction matrix and the propagation of
 // quantization errors need (single TF32/fp16 products flip integer codes).  TMA loads the
-// 128-row (A) and 256-row (B) tiles of both parts, one 128-byte row piece per K-block, into
+// 128-row (A) and up to 256-row (B) tiles of both parts, one 128-byte row piece per K-block, into
 // 128-byte-swizzled shared memory; one thread issues the MMAs into one of two 128 x 256
 // accumulators; eight epilogue warps drain them.  Accumulation chains in tensor memory are
 // cut every TCHUNK K-blocks and added into float32 registers with round-to-nearest (the
@@ -27,20 +27,27 @@
 // Every wait on an mbarrier is bounded; see umma_gemm.cuh.
 #pragma once
 #include "umma_gemm.cuh"
+#include <algorithm>
 
 namespace gptaq {
 
-constexpr int TBM = 128, TBN = 256, TBK = 64, TSTAGES = 2;
+// Tiles of 128 rows x BN columns, BN = 256, 128 or 64 (tc_tile_width chooses): 2, 3 or 4 stages fill the shared memory.
+// Wide tiles read A less often; narrow ones fill the chip where wide ones are few, and shorten the last round.  us, BN =
+// 256 / 128 / 64: P of a 1024-wide layer (32 to 112 tiles) 27 / 16 / 13.7 a product; 4096 x 512 x 1024 26.7 / 16.7 / 22.1;
+// a rank-128 update 10.3 / 6.9 / 5.9; 4096 x 3584 x 1024 91 / 83 / 122.
+constexpr int TBM = 128, TBK = 64;
+constexpr int TBOX = 64;             // rows of B per TMA box
 constexpr int TA_BYTES = TBM * TBK * 2;
-constexpr int TB_BYTES = TBN * TBK * 2;
-constexpr int TSTAGE_BYTES = 2 * TA_BYTES + 2 * TB_BYTES;
+__host__ __device__ constexpr int tc_b_bytes(int bn) { return bn * TBK * 2; }
+__host__ __device__ constexpr int tc_stages(int bn) { return bn == 256 ? 2 : bn == 128 ? 3 : 4; }
+__host__ __device__ constexpr int tc_stage_bytes(int bn) { return 2 * TA_BYTES + 2 * tc_b_bytes(bn); }
 constexpr int TCHUNK = 4;            // K-blocks per accumulation chain in tensor memory
 constexpr int TC_THREADS = 64 + 32 * UEPI_WARPS;
 // staging of the "C += ..." epilogue: per column half one 128 x 32 float32 box (128-byte rows, swizzled),
 // handed to the TMA unit as a bulk reduction
 constexpr int TC_STG_BOX_BYTES = TBM * 32 * 4;
 constexpr int TC_STG_BYTES = 2 * TC_STG_BOX_BYTES;
-constexpr size_t TC_SMEM = (size_t)TSTAGES * TSTAGE_BYTES + TC_STG_BYTES + 1024 + 256;
+constexpr size_t tc_smem(int bn) { return (size_t)tc_stages(bn) * tc_stage_bytes(bn) + TC_STG_BYTES + 1024 + 256; }
 
 enum TcMode {
     TC_FULL = 0,
@@ -85,6 +92,49 @@ struct TcGemmArgs {
     unsigned sched_base;
 };
 
+// Measured cycles: a K-block where every CTA has one tile at most, where the chip is full, and the rest of a tile (epilogue;
+// with several tiles per CTA it runs under the next tile's K-blocks).
+struct TcCost { int bn, block_one, block_full, rest; };
+constexpr TcCost TC_COST[3] = {{256, 2250, 2700, 9000}, {128, 1243, 1400, 4500}, {64, 1040, 1400, 2900}};
+
+// Estimated time of a product with tiles of bn columns on `sms` CTAs: whole rounds of equal tiles, or, where the K range
+// varies, the larger of an equal share of all K-blocks and the longest tile.
+inline int64_t tc_estimate(const TcGemmArgs &a, const TcCost &c, int sms) {
+    const int bn = c.bn;
+    const int TM = (a.M + TBM - 1) / TBM, TN = (a.N + bn - 1) / bn;
+    int64_t tiles = 0, blocks = 0, longest = 0;
+    for (int tn = 0; tn < TN; ++tn) {
+        const int64_t j0 = (int64_t)tn * bn, j1 = std::min<int64_t>(j0 + bn, a.K);
+        // row tiles of this column that are not skipped
+        int64_t rows = TM;
+        if (a.mode == TC_UPPER_TILES) rows = std::min<int64_t>(TM, (j0 + a.diag_off + bn + TBM - 1) / TBM);
+        else if (a.mode == TC_O || a.mode == TC_P) rows = std::min<int64_t>(TM, (j0 + bn + TBM - 1) / TBM);
+        int64_t first = 0, last = a.K;                     // K range of row tile 0
+        if (a.mode == TC_O) first = j0;
+        if (a.mode == TC_P || a.mode == TC_TRI_RIGHT) last = j1;
+        int64_t k = rows * (last - first);
+        if (a.mode == TC_P || a.mode == TC_TRI_LEFT) k -= (int64_t)TBM * rows * (rows - 1) / 2;      // (starts at the row)
+        tiles += rows; blocks += std::max<int64_t>(0, k) / TBK;
+        longest = std::max(longest, (last - first + TBK - 1) / TBK);
+    }
+    tiles *= a.nbatch; blocks *= a.nbatch;
+    const int64_t waves = (tiles + sms - 1) / sms;
+    if (a.mode == TC_FULL || a.mode == TC_UPPER_TILES) {
+        const int64_t k = longest * (waves > 1 ? c.block_full : c.block_one);
+        return waves * std::max<int64_t>(k, c.rest) + std::min<int64_t>(k, c.rest);
+    }
+    return std::max(blocks * c.block_full / sms, longest * c.block_one) + c.rest;
+}
+inline int tc_tile_width(const TcGemmArgs &a, int sms) {
+    int best = 0;
+    int64_t t = 0;
+    for (const TcCost &c : TC_COST) {
+        const int64_t u = tc_estimate(a, c, sms);
+        if (best == 0 || u < t) { t = u; best = c.bn; }
+    }
+    return best;
+}
+
 // Host-side twin of StateHeader::sched_counter: the first tile number of the next launch.
 struct TcSched { unsigned base = 0; };
 
@@ -93,6 +143,7 @@ struct TcTile {
     int z, i0, j0, Mz, Nz, kb0, kb1;   // K-block range [kb0, kb1)
 };
 
+template <int TBN>
 __device__ __forceinline__ void tc_decode(const TcGemmArgs &a, int t, TcTile &ti, int bk) {
     const int TM = (a.M + TBM - 1) / TBM, TN = (a.N + TBN - 1) / TBN;
     const int per = TM * TN;
@@ -153,6 +204,7 @@ __device__ __forceinline__ bool named_bar_any(int id, int nthreads, bool flag) {
     return r != 0;
 }
 
+template <int TBN>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant__ CUtensorMap mapAlo,
                const __grid_constant__ CUtensorMap mapBhi, const __grid_constant__ CUtensorMap mapBlo,
@@ -160,6 +212,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                const __grid_constant__ CUtensorMap mapC, TcGemmArgs a) {
     constexpr int BK = TBK;                        // contraction steps per K-block (one 128-byte row)
     constexpr int KSTEP = 16;                      // contraction steps per MMA (32 bytes)
+    constexpr int TSTAGES = tc_stages(TBN), TB_BYTES = tc_b_bytes(TBN), TSTAGE_BYTES = tc_stage_bytes(TBN);
+    // kind::f16, fp16 A and B (K-major), fp32 D, M = 128, N = TBN
+    constexpr uint32_t IDESC = (1u << 4) | ((TBN >> 3) << 17) | ((TBM >> 4) << 24);
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -215,7 +270,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                 first = false;
                 const int t = ticket < (unsigned)ntiles ? (int)ticket : -1;
                 if (t >= 0) {
-                    tc_decode(a, t, ti, BK);
+                    tc_decode<TBN>(a, t, ti, BK);
                     if (ti.skip && !ti.zero_fill) continue;          // nothing to do for any role
                 }
                 {   // hand the number to the MMA issuer and the epilogue warps
@@ -238,13 +293,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                     mbar_expect_tx(full_bar(stage), TSTAGE_BYTES);
                     tma_load_2d(s0, &mapAhi, ak0 + k, arow, full_bar(stage));
                     tma_load_2d(s0 + TA_BYTES, &mapAlo, ak0 + k, arow, full_bar(stage));
-                    if (!second) {
-                        tma_load_2d(s0 + 2 * TA_BYTES, &mapBhi, bk0 + k, brow, full_bar(stage));
-                        tma_load_2d(s0 + 2 * TA_BYTES + TB_BYTES, &mapBlo, bk0 + k, brow, full_bar(stage));
-                    } else {
-                        const int k2 = a.b2_k0 + (k - a.k_split);
-                        tma_load_2d(s0 + 2 * TA_BYTES, &mapB2hi, k2, brow, full_bar(stage));
-                        tma_load_2d(s0 + 2 * TA_BYTES + TB_BYTES, &mapB2lo, k2, brow, full_bar(stage));
+                    const CUtensorMap *bhi = second ? &mapB2hi : &mapBhi, *blo = second ? &mapB2lo : &mapBlo;
+                    const int kB = second ? a.b2_k0 + (k - a.k_split) : bk0 + k;
+#pragma unroll
+                    for (int q = 0; q < TBN / TBOX; ++q) {
+                        tma_load_2d(s0 + 2 * TA_BYTES + q * TBOX * 128, bhi, kB, brow + q * TBOX, full_bar(stage));
+                        tma_load_2d(s0 + 2 * TA_BYTES + TB_BYTES + q * TBOX * 128, blo, kB, brow + q * TBOX, full_bar(stage));
                     }
                     ++issued;
                     if (++stage == TSTAGES) { stage = 0; phase ^= 1u; }
@@ -268,7 +322,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                 const int t = ring[slot];
                 mbar_arrive(sempty_bar(slot));
                 if (t < 0) break;
-                tc_decode(a, t, ti, BK);
+                tc_decode<TBN>(a, t, ti, BK);
                 if (!ti.work) continue;
                 for (int kc = ti.kb0; kc < ti.kb1 && ok; kc += TCHUNK) {
                     const uint32_t buf = ccount & 1u, cphase = (ccount >> 1) & 1u;
@@ -285,7 +339,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                         const uint64_t blo = make_kmajor_desc(s0 + 2 * TA_BYTES + TB_BYTES);
                         // small terms first, the hi * hi term last
                         auto mma = [&](uint64_t ad, uint64_t bd, uint32_t accumulate) {
-                            umma_f16(d_tmem, ad, bd, UMMA_IDESC_F16, accumulate);
+                            umma_f16(d_tmem, ad, bd, IDESC, accumulate);
                         };
 #pragma unroll
                         for (int k = 0; k < BK / KSTEP; ++k)
@@ -322,7 +376,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
             __syncwarp();
             if (lane == 0) mbar_arrive(sempty_bar(slot));
             if (t < 0) break;
-            tc_decode(a, t, ti, BK);
+            tc_decode<TBN>(a, t, ti, BK);
 #pragma unroll
             for (int i = 0; i < TBN / 2; ++i) acc[i] = 0.f;
             if (ti.work) {
