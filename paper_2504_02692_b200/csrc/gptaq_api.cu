@@ -356,6 +356,12 @@ bool tc_eligible(const gptaq_ctx *h) {
            encode_tiled_fn() != nullptr;
 }
 
+// A small batch of a narrow layer takes the float32 products whatever the precision asked for: no conversions, one launch
+// instead of three.  us a batch, float32 / tensor cores: n = 128 512 tokens 16 / 35, 2048 23 / 37, 4096 37 / 37; n = 256 512
+// tokens 19 / 36, 1024 29 / 37, 2048 43 / 39; n = 384 512 tokens 31 / 35.  Batches after one another overlap on the tensor
+// path (20 to 25 us each), so the line lies at half of where a single one would draw it.
+constexpr int64_t STATS_FP32_WORK = (int64_t)1 << 25;          // tokens n^2
+
 // Adds the waiting partial sums of the cut tiles to H / dXX^T, on the internal stream behind the products.
 gptaq_status_t flush_partials(gptaq_ctx *h) {
     if (!h->fix_pending) return GPTAQ_OK;
@@ -445,11 +451,30 @@ gptaq_status_t accumulate_tc(gptaq_ctx *h, const float *X, const float *Xfp, int
             const int by_pairs = npairs / cut, by_k = ga.kblocks / (2 * UCHUNK);
             ga.ksplit = std::max(1, std::min(std::min(by_pairs, by_k), 8));
         }
-        if (ga.ksplit == 1) ga.full_tiles = (int)ntiles;
+        ga.ksplit_d = 0;
+        int cut_items = cut * ga.ksplit, cut_slots = cut * (ga.ksplit - 1);
+        if (ga.full_tiles == 0 && ga.nseg_h != ga.nseg_d) {
+            // fewer tiles than pairs, those of H several times as long as those of dXX^T (low parts of X): cut so that the
+            // longest item is as short as it gets.  3001 tokens at n = 1416, 21 tiles of 141 and 21 of 47 K-blocks: a batch
+            // 87 us as they are (none could be cut in the same number of items), 67 with two items and one.
+            const int T = (n + UPM - 1) / UPM, nh = T * (T + 1) / 2, nd = (int)ntiles - nh;
+            const int lh = ga.kblocks * ga.nseg_h, ld = ga.kblocks * ga.nseg_d;
+            int best = INT32_MAX;
+            for (int kd = 1; kd <= 8 && nh + nd * kd <= npairs; ++kd) {
+                const int kh = std::min(8, (npairs - nd * kd) / nh);
+                // (pieces of one accumulation chain at least)
+                const int ph = std::max(1, std::min(kh, lh / UCHUNK)), pd = std::max(1, std::min(kd, ld / UCHUNK));
+                const int longest = std::max((lh + ph - 1) / ph, (ld + pd - 1) / pd);
+                if (longest < best) { best = longest; ga.ksplit = ph; ga.ksplit_d = pd; }
+            }
+            cut_items = nh * ga.ksplit + nd * ga.ksplit_d;
+            cut_slots = cut_items - cut;
+        }
+        if (cut_slots == 0) { ga.full_tiles = (int)ntiles; ga.ksplit = 1; ga.ksplit_d = 0; cut_items = 0; }
         // scratch behind the two operand buffers (one partial 128 x 256 tile per CTA at most; the products
         // run one after the other on the internal stream, so one scratch serves both buffers)
         ga.scratch = reinterpret_cast<float *>(h->ws + 2 * buf_bytes);
-        const int nitems = ga.full_tiles + ((int)ntiles - ga.full_tiles) * ga.ksplit;
+        const int nitems = ga.full_tiles + cut_items;
         const int sgrid = 2 * std::min(nitems, npairs);
         std::pair<cudaEvent_t, cudaEvent_t> *tev = nullptr;
         if (h->kernel_timing) {
@@ -462,12 +487,12 @@ gptaq_status_t accumulate_tc(gptaq_ctx *h, const float *X, const float *Xfp, int
             tev = &h->timing_events[h->timing_used++];
             CU(cudaEventRecord(tev->first, gs));
         }
-        if (h->fix_pending && (h->fix_args.ksplit != ga.ksplit || h->fix_args.full_tiles != ga.full_tiles ||
+        if (h->fix_pending && (h->fix_args.ksplit != ga.ksplit || h->fix_args.ksplit_d != ga.ksplit_d || h->fix_args.full_tiles != ga.full_tiles ||
                                h->fix_args.ntiles != ga.ntiles || h->fix_args.d_full != ga.d_full ||
                                h->fix_args.scratch != ga.scratch))
             OK(flush_partials(h));              // another cut: the slots change meaning
-        if (ga.ksplit > 1 && !h->fix_pending) {
-            CU(cudaMemsetAsync(ga.scratch, 0, (size_t)((int)ntiles - ga.full_tiles) * (ga.ksplit - 1) * 2 * UBM * UBN * sizeof(float), gs));
+        if (cut_slots > 0 && !h->fix_pending) {
+            CU(cudaMemsetAsync(ga.scratch, 0, (size_t)cut_slots * 2 * UBM * UBN * sizeof(float), gs));
             h->fix_args = ga;
             h->fix_pending = true;
         }
@@ -917,7 +942,7 @@ gptaq_status_t gptaq_accumulate(gptaq_handle_t h, const float *d_X, const float 
     if (!d_X || !d_Xfp || ld < h->n) return GPTAQ_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int n = (int)h->n;
-    if (tc_eligible(h)) return accumulate_tc(h, d_X, d_Xfp, tokens, ld, s);
+    if (tc_eligible(h) && tokens > STATS_FP32_WORK / (h->n * h->n)) return accumulate_tc(h, d_X, d_Xfp, tokens, ld, s);
     OK(join_statistics(h, s));
     // H (upper tiles) += X X^T
     Operand xa = make_operand(d_X, 1, ld);

@@ -364,6 +364,9 @@ struct StatsGemmArgs {
     // stats_fixup_kernel adds them to the sums in a fixed order once, before the sums are read: the result
     // does not depend on timing.
     int ntiles, full_tiles, ksplit;
+    // ksplit_d > 0 (full_tiles 0): the tiles of H come first, cut in `ksplit` items each, then those of
+    // dXX^T, cut in `ksplit_d`; slots in the same order
+    int ksplit_d;
     float *scratch;
     int d_full;              // 0: only the tiles of dXX^T that reach the diagonal or lie above it (see TileIter)
 };
@@ -418,10 +421,36 @@ static_assert(UBN == UPM, "the diagonal test of TileIter assumes square pair til
 struct StatsItem {
     int g0, g1;          // K-block range
     int part;            // 0: adds into H / dXX^T;  c > 0: partial result number c of a cut tile
-    int cut_index;       // index of the cut tile among the cut tiles
+    int slot;            // where a partial result goes
 };
 
+// ksplit_d > 0: the i-th tile of H (column by column) or of dXX^T
+__device__ __forceinline__ void stats_tile_of(const StatsGemmArgs &a, bool isD, int i, TileIter &it) {
+    if (isD && a.d_full) {
+        it.tn = i / it.T;
+        it.r = it.T + i - it.tn * it.T;
+    } else {
+        int tn = 0;
+        while (i > tn) { i -= tn + 1; ++tn; }
+        it.tn = tn;
+        it.r = (isD ? it.T : 0) + i;
+    }
+}
+
 __device__ __forceinline__ bool stats_item(const StatsGemmArgs &a, int w, TileIter &it, StatsItem &item) {
+    if (a.ksplit_d > 0) {
+        const int nh = it.T * (it.T + 1) / 2, nd = a.ntiles - nh;
+        const bool isD = w >= nh * a.ksplit;
+        const int e = isD ? w - nh * a.ksplit : w, parts = isD ? a.ksplit_d : a.ksplit, i = e / parts;
+        if (isD && i >= nd) return false;
+        stats_tile_of(a, isD, i, it);
+        const int kb = a.kblocks * (isD ? a.nseg_d : a.nseg_h);
+        item.part = e - i * parts;
+        item.g0 = kb * item.part / parts;
+        item.g1 = kb * (item.part + 1) / parts;
+        item.slot = (isD ? nh * (a.ksplit - 1) : 0) + i * (parts - 1) + item.part - 1;
+        return true;
+    }
     const int nitems = a.full_tiles + (a.ntiles - a.full_tiles) * a.ksplit;
     if (w >= nitems) return false;
     int tile = w, part = 0, parts = 1;
@@ -436,7 +465,7 @@ __device__ __forceinline__ bool stats_item(const StatsGemmArgs &a, int w, TileIt
     item.g0 = (int)((long long)kb_total * part / parts);
     item.g1 = (int)((long long)kb_total * (part + 1) / parts);
     item.part = part;
-    item.cut_index = tile - a.full_tiles;
+    item.slot = (tile - a.full_tiles) * (a.ksplit - 1) + part - 1;
     return true;
 }
 
@@ -596,7 +625,7 @@ stats_umma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
             const float inv = 1.f / (sx * (isD ? sd : sx));
             if (item.part > 0) {
                 // partial result of a cut tile: added into its slot, all 128 x 256 entries
-                float *sp = a.scratch + (((int64_t)item.cut_index * (a.ksplit - 1) + item.part - 1) * 2 + (int)rank) * (UBM * UBN) +
+                float *sp = a.scratch + ((int64_t)item.slot * 2 + (int)rank) * (UBM * UBN) +
                             (quarter * 32 + lane) * UBN + half * (UBN / 2);
 #pragma unroll
                 for (int q = 0; q < UBN / 2 / 4; ++q)
@@ -667,12 +696,18 @@ __global__ void bounded_wait_selftest_kernel(StateHeader *hd, long long limit_cy
 constexpr int FIXUP_SLABS = 32;     // CTAs per cut tile, UPM / FIXUP_SLABS rows each
 __global__ void __launch_bounds__(256) stats_fixup_kernel(StatsGemmArgs a) {
     TileIter it(a.n, a.d_full);
-    if (!it.seek_to(a.full_tiles + blockIdx.x)) return;
+    int slot0 = blockIdx.x * (a.ksplit - 1), parts = a.ksplit;
+    if (a.ksplit_d > 0) {
+        const int nh = it.T * (it.T + 1) / 2, i = (int)blockIdx.x;
+        stats_tile_of(a, i >= nh, i >= nh ? i - nh : i, it);
+        if (i >= nh) { slot0 = nh * (a.ksplit - 1) + (i - nh) * (a.ksplit_d - 1); parts = a.ksplit_d; }
+        if (parts == 1) return;
+    } else if (!it.seek_to(a.full_tiles + blockIdx.x)) return;
     const bool isD = it.r >= it.T;
     const int row0 = (isD ? it.r - it.T : it.r) * UPM, col0 = it.tn * UBN;
     float *C = isD ? a.D : a.H;
-    // slot of partial c, CTA rank r: ((blockIdx.x * (ksplit - 1) + c) * 2 + r) * UBM * UBN
-    const float *sp = a.scratch + (int64_t)blockIdx.x * (a.ksplit - 1) * 2 * (UBM * UBN);
+    // slot of partial c, CTA rank r: ((slot0 + c) * 2 + r) * UBM * UBN
+    const float *sp = a.scratch + (int64_t)slot0 * 2 * (UBM * UBN);
     constexpr int ROWS = UPM / FIXUP_SLABS;
     const bool vec = (a.n & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
 #pragma unroll
@@ -685,7 +720,7 @@ __global__ void __launch_bounds__(256) stats_fixup_kernel(StatsGemmArgs a) {
         const int64_t pstride = 2 * (int64_t)(UBM * UBN);
         if (vec && col0 + j + 3 < a.n) {
             float4 v = *reinterpret_cast<const float4 *>(cp);
-            for (int c = 0; c < a.ksplit - 1; ++c) {
+            for (int c = 0; c < parts - 1; ++c) {
                 const float4 p = *reinterpret_cast<const float4 *>(pp + c * pstride);
                 v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
             }
@@ -693,7 +728,7 @@ __global__ void __launch_bounds__(256) stats_fixup_kernel(StatsGemmArgs a) {
         } else {
             for (int f = 0; f < 4 && col0 + j + f < a.n; ++f) {
                 float v = cp[f];
-                for (int c = 0; c < a.ksplit - 1; ++c) v += pp[c * pstride + f];
+                for (int c = 0; c < parts - 1; ++c) v += pp[c * pstride + f];
                 cp[f] = v;
             }
         }

@@ -779,3 +779,35 @@ def test_quantize_launch_edges(n, m, group, B):
                     outlier_channels=4)
     out = hp.check_layer(cfg, wl.make_weight(cfg), batches_of(cfg), rows=np.unique(np.r_[0:m:max(1, m // 16), m - 1]))
     hp.assert_parity(out)
+
+
+@pytest.mark.parametrize("n,tokens,act_order", [
+    (128, 2048, False), (128, 2049, False),     # float32 products up to here / one tile of either sum, cut
+    (640, 520, False), (640, 520, True),        # a few tiles, of dXX^T the upper ones or all
+    (2048, 520, False),                         # as many tiles as pairs allow without a cut
+])
+def test_statistics_cut_by_length(n, tokens, act_order):
+    """Tiles of H three times as long as those of dXX^T, cut into different numbers of items (two batches, so that the
+    partial sums are added to).  Bounds as in test_tensor_core_statistics_against_oracle: operands of 22 bits for H, 11 for
+    dXX^T, relative to sqrt(H_ii H_jj)."""
+    torch.manual_seed(n + tokens)
+    st = g.LayerState(n, 8, tokens, 128)
+    try:
+        g.gptaq_set_stats_precision(st.handle, g.GPTAQ_STATS_FP16_SPLIT_TENSOR)
+        g.gptaq_set_act_order(st.handle, act_order)
+        H, D = np.zeros((n, n)), np.zeros((n, n))
+        d = np.zeros(n)
+        for _ in range(2):
+            X = torch.randn(tokens, n, device="cuda")
+            F = X + 0.05 * torch.randn(tokens, n, device="cuda")
+            g.gptaq_accumulate(st.handle, X, F)
+            x, dx = X.double().cpu().numpy(), (F - X).double().cpu().numpy()
+            H += x.T @ x; D += dx.T @ x; d += (dx ** 2).sum(0)
+        assert g.gptaq_sync_status(st.handle)[0] == g.GPTAQ_OK
+        Hg, Dg = st.H().cpu().numpy().astype(np.float64), st.D().cpu().numpy().astype(np.float64)
+    finally:
+        st.close()
+    h = np.sqrt(np.diag(H))
+    assert (np.abs(np.triu(Hg - H)) / np.outer(h, h)).max() < 1e-5
+    err = Dg - D if act_order else np.triu(Dg - D, 1)
+    assert (np.abs(err) / np.outer(np.sqrt(d), h)).max() < 2.0 ** -10
