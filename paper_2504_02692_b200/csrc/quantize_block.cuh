@@ -228,24 +228,26 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     auto up_ld = [&](int s) { return (s & 1) ? QB_ULD1 : QB_ULD0; };
     auto up_buf = [&](int s) { return UPs + (s & 1) * (2 * 32 * QB_ULD0); };
     auto fetch_up = [&](int cb, int s, int t, int nthr) {
-        const int ld = up_ld(s), q = (B - 32 * s) / 4, r0 = cb + 32 * s;
-        float *ub = up_buf(s), *pb = ub + 32 * ld;
-        for (int idx = t; idx < 32 * q; idx += nthr) {
-            const int k = idx / q, c4 = idx - k * q;
-            const int row = r0 + k, col = r0 + 4 * c4;
-            float *du = ub + k * ld + 4 * c4, *dp = pb + k * ld + 4 * c4;
-            const int64_t off = (int64_t)row * n + col;
-            if (aligned_up && row < n && col + 3 < n) {
+        // a warp per row, a lane per four columns (no divisions: with 32 q quads numbered through, they made up most of it)
+        const int ld = up_ld(s), q = (B - 32 * s) / 4, r0 = cb + 32 * s, c4 = t & 31;
+        if (c4 >= q) return;
+        const int col = r0 + 4 * c4;
+        float *du = up_buf(s) + (t >> 5) * ld + 4 * c4, *dp = du + 32 * ld;
+        int64_t off = (int64_t)(r0 + (t >> 5)) * n + col;
+        const bool whole = aligned_up && col + 3 < n;
+        for (int k = t >> 5; k < 32; k += nthr / 32) {
+            if (whole && r0 + k < n) {
                 cp_async16(du, a.U + off);
                 cp_async16(dp, a.P + off);
             } else {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const bool in = row < n && col + e < n;
+                    const bool in = r0 + k < n && col + e < n;
                     du[e] = in ? a.U[off + e] : 0.f;
                     dp[e] = in ? a.P[off + e] : 0.f;
                 }
             }
+            du += nthr / 32 * ld; dp += nthr / 32 * ld; off += (int64_t)(nthr / 32) * n;
         }
     };
     // per column of a step: err_scale / U_kk (padded columns beyond n have no error: 0) and the column's original index
@@ -287,19 +289,28 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         }
     }
     // the slab and the first rows of U and P all in flight at once (in batches through registers the prologue took 6 us
-    // of a launch, now 4)
+    // of a launch, now 3)
     const int cq = FAR ? nblk * (QB_W / 4) : B / 4;                // quads per row, padded columns included
     const bool wvec = (a.ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(a.W) & 15) == 0;       // (i0 is a multiple of 32)
-    for (int idx = tid; idx < QB_ROWS * cq; idx += NTHREADS) {
-        const int r = idx / cq, c = 4 * (idx - r * cq);
-        float *dst = Ws + r * WLD + c;
-        const float *src = a.W + (int64_t)(row0 + r) * a.ldw + i0 + c;
-        if (wvec && r < nrows && c + 3 < cols) cp_async16(dst, src);
-        else {
+    // a thread: four columns of every RSTEP-th row
+    constexpr int WQ = FAR ? QB_SUPER / 4 : QB_W / 4, RSTEP = NTHREADS / WQ;
+    const int wq = tid % WQ, wr0 = tid / WQ, wc = 4 * wq;
+    const bool fills = wr0 < RSTEP && wq < cq;
+    if (fills) {
+        const bool whole = wvec && wc + 3 < cols;
+        const float *src = a.W + (int64_t)(row0 + wr0) * a.ldw + i0 + wc;
+        float *dst = Ws + wr0 * WLD + wc;
+        for (int r = wr0; r < QB_ROWS; r += RSTEP) {
+            if (whole && r < nrows) cp_async16(dst, src);
+            else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) dst[e] = r < nrows && c + e < cols ? src[e] : 0.f;
+                for (int e = 0; e < 4; ++e) dst[e] = r < nrows && wc + e < cols ? src[e] : 0.f;
+            }
+            src += (int64_t)RSTEP * a.ldw; dst += RSTEP * WLD;
         }
     }
+    // (dead inputs read as zero; the flags are 4-byte aligned and padded beyond n)
+    const uint32_t dead4 = fills && wc < cols ? *reinterpret_cast<const uint32_t *>(a.dead + i0 + wc) : 0u;
     fetch_up(i0, 0, tid, NTHREADS);
     if (tid < 32) { udinv2[tid] = load_pivot(i0 + tid); perm2[tid] = load_perm(i0 + tid); }
     if (PERCOL && tid < QB_NEAR) {
@@ -308,17 +319,21 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         store_grid(tid >> 3, 4 * (tid & 7), sc, zp);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    for (int idx = tid; idx < QB_ROWS * cq; idx += NTHREADS) {
-        const int r = idx / cq, c = 4 * (idx - r * cq);            // (the words that this thread has copied)
-        float4 *wp = reinterpret_cast<float4 *>(Ws + r * WLD + c);
-        const float4 v = *wp;
-        // dead inputs read as zero (the flags are 4-byte aligned and padded beyond n)
-        const uchar4 dd = c < cols ? *reinterpret_cast<const uchar4 *>(a.dead + i0 + c) : make_uchar4(0, 0, 0, 0);
-        const float x[4] = {dd.x ? 0.f : v.x, dd.y ? 0.f : v.y, dd.z ? 0.f : v.z, dd.w ? 0.f : v.w};
-        // a non-finite weight is reported from the value that was read: its code and dequantized value
-        // come out finite (the clamp absorbs NaN and Inf), so the results alone would not show it
-        if (!isfinite(x[0]) || !isfinite(x[1]) || !isfinite(x[2]) || !isfinite(x[3])) record_status(a.hd, ST_NONFINITE, row0 + r);
-        if (dd.x | dd.y | dd.z | dd.w) *wp = make_float4(x[0], x[1], x[2], x[3]);
+    if (fills) {
+        float4 *wp = reinterpret_cast<float4 *>(Ws + wr0 * WLD + wc);                  // (the words that this thread has copied)
+        for (int r = wr0; r < QB_ROWS; r += RSTEP, wp += RSTEP * WLD / 4) {
+            float4 v = *wp;
+            if (dead4) {
+                if (dead4 & 0xffu) v.x = 0.f;
+                if (dead4 & 0xff00u) v.y = 0.f;
+                if (dead4 & 0xff0000u) v.z = 0.f;
+                if (dead4 & 0xff000000u) v.w = 0.f;
+                *wp = v;
+            }
+            // a non-finite weight is reported from the value that was read: its code and dequantized value
+            // come out finite (the clamp absorbs NaN and Inf), so the results alone would not show it
+            if (!isfinite(v.x) || !isfinite(v.y) || !isfinite(v.z) || !isfinite(v.w)) record_status(a.hd, ST_NONFINITE, row0 + r);
+        }
     }
     if (FAR) tc_fence_before();
     __syncthreads();
