@@ -52,7 +52,7 @@ struct gptaq_ctx {
     int64_t launches;
     int stats_precision;   // GPTAQ_STATS_*
     bool tensor;           // float32-grade tensor-core GEMMs (fp16-split operands) for factor / P / trailing update
-    TcSched sched;         // tile numbering of the float32-grade GEMM launches (see StateHeader::sched_counter)
+    TcSched sched, sched2; // tile numbering of the float32-grade GEMM launches (see StateHeader::sched_counter)
     int terms;             // GPTAQ_TERM_* switches of gptaq_quantize
     bool static_groups;    // group grids from the original weights, per group of the caller's columns
     int clip_steps; float clip_min;   // clipping-range search of the grids
@@ -286,7 +286,7 @@ cudaError_t launch_tc_gemm(const TcMaps &m, const TcGemmArgs &a_in, TcSched &sch
     const int grid = (int)std::min<int64_t>(tiles, num_sms);
     // "C += ...": bulk tensor reductions where the target qualifies for a tensor map (16-byte aligned base
     // and row pitch); scattered per-thread reductions otherwise
-    a.sched = &a.hd->sched_counter;
+    a.sched = sched.second ? &a.hd->sched_counter2 : &a.hd->sched_counter;
     a.sched_base = sched.base;
     sched.base += (unsigned)tiles;           // (grid <= tiles)
     CUtensorMap mapC = m.a_hi;       // placeholder, not dereferenced unless c_tma is set
@@ -527,6 +527,10 @@ struct QuantizeTarget {
     __half *EW16 = nullptr;
     float *row_inv = nullptr;
     const unsigned *amax_u = nullptr, *amax_p = nullptr;
+    // a second stream for one half of many rows (null: none), with its own count of tile numbers, and two events
+    cudaStream_t side = nullptr;
+    TcSched *side_sched = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
     int terms = GPTAQ_TERM_ERR | GPTAQ_TERM_ASYM;   // which terms of the weight update are applied
     const int *perm = nullptr;                      // act_order: working column c is the caller's column perm[c]
     int clip_steps = 0; float clip_min = 1.f;       // clipping-range search of the grids (0 steps: min/max)
@@ -534,15 +538,15 @@ struct QuantizeTarget {
     bool static_groups = false;
 };
 
-// One launch of quant_block_kernel: columns [i0, i1) of the loop, SW columns per launch at most.
-cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, int64_t m, int i0, int i1, int SW,
+// One launch of quant_block_kernel: columns [i0, i1) of the loop for rows [r0, r1) of m, SW columns per launch at most.
+cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, int64_t r0, int64_t r1, int64_t m, int i0, int i1, int SW,
                                int bits, int group, int sym, uint8_t *codes, float *scales, float *zeros, int G,
                                bool static_groups, cudaStream_t s) {
     const bool far_form = t.UT16 != nullptr;
     const size_t nn = (size_t)t.n * t.ldt;
     QuantBlockArgs a;
     std::memset(&a, 0, sizeof(a));
-    a.W = W; a.ldw = ldw; a.m = (int)m; a.n = t.n; a.U = t.U; a.P = t.P; a.dead = t.dead;
+    a.W = W; a.ldw = ldw; a.row_first = (int)r0; a.m = (int)r1; a.n = t.n; a.U = t.U; a.P = t.P; a.dead = t.dead;
     a.i0 = i0; a.i1 = i1; a.bw = far_form ? QB_W : SW;
     a.bits = bits; a.group = group; a.sym = sym;
     a.codes = codes; a.scales = scales; a.zeros = zeros; a.G = G;
@@ -559,7 +563,7 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
     if (far_form && (!make_f16_map(&uh, t.UT16, t.n, t.n, t.ldt, 128) || !make_f16_map(&ul, t.UT16 + nn, t.n, t.n, t.ldt, 128) ||
                      !make_f16_map(&ph, t.PT16, t.n, t.n, t.ldt, 128) || !make_f16_map(&pl, t.PT16 + nn, t.n, t.n, t.ldt, 128)))
         return cudaErrorUnknown;
-    const dim3 grid((unsigned)((m + QB_ROWS - 1) / QB_ROWS));
+    const dim3 grid((unsigned)((r1 - r0 + QB_ROWS - 1) / QB_ROWS));
     const size_t smem = quant_block_smem_bytes(far_form, static_groups);
     // Near form, more CTAs than SMs: two to an SM, one works while the other waits for its own chain (16384 rows of 400
     // columns 455 us, with one 498); below that one, which has the registers of both (1024 rows of 1024 columns 288 us, 301).
@@ -674,10 +678,46 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
         const SplitOperand B{t.UT16, t.UT16 + nn, n, n, t.ldt}, B2{t.PT16, t.PT16 + nn, n, n, t.ldt};
         if (!make_tc_maps(&maps, A, B, &B2)) { *err = cudaErrorUnknown; return GPTAQ_ERR_CUDA; }
     }
-    for (int i0 = 0; i0 < n; i0 += SW) {
+    if (steps && tensor) {
+        // More rows than one round of CTAs: two halves of the rows on two streams, so that one half's launches fill the SMs
+        // that the last round of the other's leaves idle (16384 x 4096, four rounds for 3.5: 3455 us, in one piece
+        // 3696; 5000 x 4096, two for 1.06: 1256, 1713).  Rows that one round takes gain nothing (4096 x 4096 1045, 1030).
+        struct Part { int64_t r0, r1; cudaStream_t s; TcSched *sched; } parts[2] = {{0, m, s, t.sched}, {m, m, t.side, t.side_sched}};
+        if (t.side && m > (int64_t)QB_ROWS * t.num_sms) {
+            parts[0].r1 = parts[1].r0 = (m / 2 + TBM - 1) / TBM * TBM;
+            *err = cudaEventRecord(t.fork, s);
+            if (*err == cudaSuccess) *err = cudaStreamWaitEvent(t.side, t.fork, 0);
+            if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
+        }
+        for (int i0 = 0; i0 < n; i0 += SW) {
+            const int i1 = std::min(i0 + SW, n);
+            for (const Part &p : parts) {
+                if (p.r0 == p.r1) continue;
+                *err = launch_quant_block(t, Wk, ldk, p.r0, p.r1, m, i0, i1, SW, bits, group, sym, d_codes, d_scales, d_zeros, G,
+                                          static_groups, p.s);
+                if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
+                ++*launches;
+                if (i1 >= n) continue;
+                // W[:, i1:] += [-Err | Wpre] * [U[blk, i1:] ; P[blk, i1:]] on the tensor cores: B operand rows
+                // are rows i1.. of U^T (first SW contraction steps) and of P^T (the next SW)
+                TcGemmArgs g = tc_args(Wk + p.r0 * ldk + i1, ldk, (int)(p.r1 - p.r0), n - i1, 2 * SW, 1.f, 1.f, TC_FULL, TC_MASK_NONE, t.hd);
+                g.a_row0 = (int)p.r0;
+                g.b_row0 = i1; g.b_k0 = i0; g.k_split = SW; g.b2_k0 = i0;
+                g.row_inv = t.row_inv + p.r0; g.amax_b = t.amax_u;
+                *err = launch_tc_gemm(maps, g, *p.sched, t.num_sms, p.s, false);
+                if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
+                ++*launches;
+            }
+        }
+        if (parts[1].r0 < parts[1].r1) {
+            *err = cudaEventRecord(t.join, t.side);
+            if (*err == cudaSuccess) *err = cudaStreamWaitEvent(s, t.join, 0);
+            if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
+        }
+    } else for (int i0 = 0; i0 < n; i0 += SW) {
         const int i1 = std::min(i0 + SW, n);
         if (steps) {
-            *err = launch_quant_block(t, Wk, ldk, m, i0, i1, SW, bits, group, sym, d_codes, d_scales, d_zeros, G,
+            *err = launch_quant_block(t, Wk, ldk, 0, m, m, i0, i1, SW, bits, group, sym, d_codes, d_scales, d_zeros, G,
                                       static_groups, s);
             if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
             ++*launches;
@@ -707,8 +747,7 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
         }
         if (i1 >= n) break;
         if (tensor) {
-            // W[:, i1:] += [-Err | Wpre] * [U[blk, i1:] ; P[blk, i1:]] on the tensor cores: B operand rows
-            // are rows i1.. of U^T (first SW contraction steps) and of P^T (the next SW)
+            // the same update behind column_loop_kernel
             TcGemmArgs g = tc_args(Wk + i1, ldk, (int)m, n - i1, 2 * SW, 1.f, 1.f, TC_FULL, TC_MASK_NONE, t.hd);
             g.b_row0 = i1; g.b_k0 = i0; g.k_split = SW; g.b2_k0 = i0;
             g.row_inv = t.row_inv; g.amax_b = t.amax_u;
@@ -915,7 +954,8 @@ gptaq_status_t gptaq_reset(gptaq_handle_t h, gptaq_stream_t stream) {
     h->stage = STAGE_ACCUM;
     h->tokens = 0;
     h->d_upper_only = false;
-    h->sched.base = 0;           // the counter in the header was zeroed with the rest of the state
+    h->sched.base = h->sched2.base = 0;           // the counters in the header were zeroed with the rest of the state
+    h->sched2.second = true;
     return GPTAQ_OK;
 }
 
@@ -1280,6 +1320,7 @@ gptaq_status_t gptaq_quantize(gptaq_handle_t h, void *d_W, int w_dtype, int64_t 
     t.perm = h->act_order ? h->perm : nullptr;
     t.clip_steps = h->clip_steps; t.clip_min = h->clip_min;
     t.static_groups = h->static_groups; t.dead_orig = h->dead_raw;
+    t.side = h->gemm_stream; t.side_sched = &h->sched2; t.fork = h->conv_done[0]; t.join = h->gemm_done[0];
     // fp16-split updates, plain float32 products otherwise
     // (groups of fewer than 32 columns update block by block, and blocks of 32 columns are no whole K-block of 64)
     const bool f16 = h->tensor && ((blocksize % 64) == 0 || group <= 0 || (group % 32) == 0 || h->static_groups);

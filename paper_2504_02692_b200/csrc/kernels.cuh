@@ -19,7 +19,8 @@ struct StateHeader {
     unsigned tc_amax[8]; // largest magnitudes of FP16-split operands of the float32-grade GEMMs (see tc_gemm.cuh)
     unsigned sched_counter; // tile numbers drawn by the float32-grade GEMM launches so far (never reset between launches)
     unsigned stats_done;    // CTAs of the running statistics product that have finished
-    int pad1[12];
+    unsigned sched_counter2; // as sched_counter, for launches on the internal stream that run beside those
+    int pad1[11];
 };
 static_assert(sizeof(StateHeader) == 128, "header size");
 

@@ -42,7 +42,7 @@ constexpr int QB_HALF_BYTES = 4 * QB_E_BYTES;                         // (hi, lo
 constexpr int QB_TMEM_COLS = 256;                                     // 2 halves x 3 blocks x 32 columns, a power of two
 
 struct QuantBlockArgs {
-    float *W; int64_t ldw; int m, n;
+    float *W; int64_t ldw; int row_first, m, n;     // rows [row_first, m)
     const float *U, *P;        // n x n, ld n; entries below the diagonals are not used
     const uint8_t *dead;
     int i0, i1;                // columns of this launch: [i0, i1); i1 - i0 <= QB_SUPER (tensor-core form) or one block
@@ -216,7 +216,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = a.n, i0 = a.i0, B = a.bw;
-    const int row0 = blockIdx.x * QB_ROWS;
+    const int row0 = a.row_first + blockIdx.x * QB_ROWS;
     const int nrows = min(QB_ROWS, a.m - row0);
     const int cols = a.i1 - i0;
     const int nblk = FAR ? (cols + QB_W - 1) / QB_W : 1;

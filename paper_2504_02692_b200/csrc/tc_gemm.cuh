@@ -136,7 +136,7 @@ inline int tc_tile_width(const TcGemmArgs &a, int sms) {
 }
 
 // Host-side twin of StateHeader::sched_counter: the first tile number of the next launch.
-struct TcSched { unsigned base = 0; };
+struct TcSched { unsigned base = 0; bool second = false; };    // second: of sched_counter2
 
 struct TcTile {
     bool skip, zero_fill, work;

@@ -772,6 +772,7 @@ def test_split_operand_row_pitch(n):
     (512, 33, 64, 64),          # the narrowest tensor-core form, exactly one launch; a row more than a CTA
     (516, 32, 128, 128),        # a launch of 512 columns and one of 4
     (1060, 40, 32, 64),         # a grid at every step; the last block has two steps, the last of them 4 columns
+    (644, 4737, 64, 64),        # more rows than a round of CTAs: two parts of 2432 and 2305 rows on two streams
 ])
 def test_quantize_launch_edges(n, m, group, B):
     """Forms of the column loop at the edges of their rows, blocks and launches (bounds as in the other parity tests)."""
