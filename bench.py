@@ -363,11 +363,10 @@ def run_ours(args, cfg):
         cpu = {"value": v, "unit": "ms", "cores": threads, "kind": "oracle", "sample": desc}
     # Per-stage rooflines (algorithmic work / stage time against the bound that applies): the products of
     # factor, P and the lazy-batch update run as three tensor-core products on split operands: fp16 hi / lo
-    # parts where the width is a multiple of 8 (at most bf16 peak / 3 of useful flops), TF32 parts otherwise
-    # (bf16 peak / 2 / 3); the column loop is bound by HBM on paper.
-    fp16_split = cfg.n >= 512 and cfg.n % 8 == 0
-    split_peak = peak / 3.0 if fp16_split else peak / 2.0 / 3.0
-    split_name = "tensor (3xFP16 split)" if fp16_split else "tensor (3xTF32)"
+    # parts (at most bf16 peak / 3 of useful flops; narrow and odd widths take float32 products and are held to the
+    # same figure); the column loop is bound by HBM on paper.
+    split_peak = peak / 3.0
+    split_name = "tensor (3xFP16 split)"
     n_, m_, B_ = float(cfg.n), float(cfg.m), float(cfg.blocksize)
     fl_factor, fl_P = 2.0 * n_ ** 3 / 3.0, 2.0 * n_ ** 3 / 3.0
     fl_trail = 2.0 * m_ * n_ * n_ * max(0.0, 1.0 - B_ / n_)

@@ -269,8 +269,7 @@ const int32_t *gptaq_perm(gptaq_handle_t h);
  * `group` consecutive columns of the CALLER's column order; a column keeps the grid of its own group wherever
  * act_order moves it in the processing order.  d_scales / d_zeros [m x G] then index caller column c by
  * c / group, with or without act_order -- no index table is needed to dequantize.  Without act_order the
- * only difference from the default is that grids come from the original instead of the updated weights.
- * Such calls take the general column kernel (one warp per row), not the 32-columns-per-thread one. */
+ * only difference from the default is that grids come from the original instead of the updated weights. */
 gptaq_status_t gptaq_set_static_groups(gptaq_handle_t h, int enable);
 
 /* Clipping-range search of the quantization grids by least squared rounding error (experimental

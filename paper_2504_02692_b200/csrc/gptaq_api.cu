@@ -300,10 +300,8 @@ cudaError_t launch_tc_gemm(const TcMaps &m, const TcGemmArgs &a_in, TcSched &sch
 
 // Slots of StateHeader::tc_amax (largest magnitudes of FP16-split operands).
 
-cudaError_t launch_absmax(const float *src, int64_t lds, int rows, int cols, int mask, float scale, unsigned *slot,
-                          int num_sms, cudaStream_t s) {
-    const int grid = std::max(1, std::min(rows, 8 * num_sms));
-    absmax_kernel<<<grid, 256, 0, s>>>(src, lds, rows, cols, mask, scale, slot);
+cudaError_t launch_absmax(const AbsmaxArgs &a, const AbsmaxArgs &b, int num_sms, cudaStream_t s) {
+    absmax_kernel<<<dim3(std::max(1, std::min(a.rows, 4 * num_sms)), 2), 256, 0, s>>>(a, b);
     return cudaGetLastError();
 }
 
@@ -314,18 +312,21 @@ struct SplitBatch {
 };
 
 // hi_t / lo_t non-null: the transposed form goes there in the same pass (transpose is then ignored)
-cudaError_t launch_split16(const float *src, int64_t lds, __half *hi, __half *lo, int64_t ldd, int rows, int cols,
-                           bool transpose, int mask, float scale, const unsigned *amax, cudaStream_t s,
-                           const SplitBatch &b = SplitBatch(), __half *hi_t = nullptr, __half *lo_t = nullptr) {
-    if (rows <= 0 || cols <= 0 || b.nbatch <= 0) return cudaSuccess;
+Split16Args split16_args(const float *src, int64_t lds, __half *hi, __half *lo, int64_t ldd, int rows, int cols,
+                         bool transpose, int mask, float scale, const unsigned *amax, const SplitBatch &b = SplitBatch(),
+                         __half *hi_t = nullptr, __half *lo_t = nullptr) {
     Split16Args a;
     a.src = src; a.lds = lds; a.src_bstride = b.src_bstride; a.hi = hi; a.lo = lo; a.ldd = ldd;
     a.dst_bstride = b.dst_bstride;
     a.rows = rows; a.cols = cols; a.rows_last = b.rows_last; a.cols_last = b.cols_last; a.nbatch = b.nbatch;
     a.transpose = hi_t ? 2 : (transpose ? 1 : 0); a.mask = mask; a.scale = scale; a.amax = amax;
     a.hi_t = hi_t; a.lo_t = lo_t;
-    dim3 grid((cols + 63) / 64, (rows + 63) / 64, b.nbatch);
-    split16_kernel<<<grid, 256, 0, s>>>(a);
+    return a;
+}
+cudaError_t launch_split16(const Split16Args &a, cudaStream_t s, const Split16Args *second = nullptr) {
+    if (a.rows <= 0 || a.cols <= 0 || a.nbatch <= 0) return cudaSuccess;
+    dim3 grid((a.cols + 63) / 64, (a.rows + 63) / 64, a.nbatch + (second ? 1 : 0));
+    split16_kernel<<<grid, 256, 0, s>>>(a, second ? *second : a);
     return cudaGetLastError();
 }
 
@@ -636,12 +637,14 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
         QLAUNCHED();
         Wk = d_Wq; ldk = n;
     } else if (w_dtype == GPTAQ_W_BF16 || (d_Wq && d_Wq != d_W)) {
-        const dim3 grid((unsigned)((n + 1023) / 1024), (unsigned)std::min<int64_t>((m + WIDEN_ROWS - 1) / WIDEN_ROWS, 65535));
-        if (w_dtype == GPTAQ_W_BF16)
-            widen_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(d_W), ldw, d_Wq, n, (int)m, n);
-        else widen_kernel<float><<<grid, 256, 0, s>>>(static_cast<const float *>(d_W), ldw, d_Wq, n, (int)m, n);
-        QLAUNCHED();
         Wk = d_Wq; ldk = n;
+        if (group > 0) {
+            const dim3 grid((unsigned)((n + 1023) / 1024), (unsigned)std::min<int64_t>((m + WIDEN_ROWS - 1) / WIDEN_ROWS, 65535));
+            if (w_dtype == GPTAQ_W_BF16)
+                widen_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(d_W), ldw, d_Wq, n, (int)m, n);
+            else widen_kernel<float><<<grid, 256, 0, s>>>(static_cast<const float *>(d_W), ldw, d_Wq, n, (int)m, n);
+            QLAUNCHED();
+        }
     }
 
     const int G = group > 0 ? (n + group - 1) / group : 1;
@@ -660,8 +663,15 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
         QLAUNCHED();
     }
     if (group <= 0) {
-        row_grid_kernel<<<(unsigned)((m + 7) / 8), 256, 0, s>>>(Wk, ldk, (int)m, n, t.dead, bits, sym,
-                                                               d_scales, d_zeros, t.clip_steps, t.clip_min);
+        // (from the caller's rows, with the working copy made on the way; in sorted order that exists already)
+        const unsigned rg = (unsigned)((m + 7) / 8);
+        float *copy = t.perm || Wk == d_W ? nullptr : Wk;
+        if (w_dtype == GPTAQ_W_BF16 && copy)
+            row_grid_kernel<__nv_bfloat16><<<rg, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(d_W), ldw, copy, ldk, (int)m, n, t.dead, bits,
+                                                              sym, d_scales, d_zeros, t.clip_steps, t.clip_min);
+        else
+            row_grid_kernel<float><<<rg, 256, 0, s>>>(copy ? static_cast<const float *>(d_W) : Wk, copy ? ldw : ldk, copy, ldk, (int)m, n, t.dead,
+                                                      bits, sym, d_scales, d_zeros, t.clip_steps, t.clip_min);
         QLAUNCHED();
     }
 
@@ -1042,7 +1052,7 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
     float *Rinv = reinterpret_cast<float *>(h->ws + wl.rinv_off);
     float *H = h->H;
 
-    diag_stats_kernel<<<1, 1024, 0, s>>>(H, n, (float)(1.0 / (double)h->tokens), damp, h->hd, h->dead_raw);
+    diag_stats_kernel<<<1, 1024, 0, s>>>(H, n, (float)(1.0 / (double)h->tokens), damp, h->hd, h->dead_raw, h->act_order ? nullptr : h->dead);
     LAUNCHED();
     if (h->act_order) {
         // columns in order of decreasing diag(H): dXX^T and H are permuted on both sides, through T (H stays there until it
@@ -1055,8 +1065,6 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
         CU(cudaMemcpyAsync(h->D, T, (size_t)n * n * sizeof(float), cudaMemcpyDeviceToDevice, s));
         permute_symmetric_kernel<<<dim3((n + 255) / 256, n), 256, 0, s>>>(H, T, n, h->perm);
         LAUNCHED();
-    } else {
-        CU(cudaMemcpyAsync(h->dead, h->dead_raw, (size_t)n, cudaMemcpyDeviceToDevice, s));
     }
     scale_damp_kernel<<<dim3((n + 63) / 64, (n + 15) / 16), 256, 0, s>>>(h->act_order ? T : H, H, n, h->hd, h->dead);
     LAUNCHED();
@@ -1172,17 +1180,17 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
             SplitBatch sbt = sb; sbt.cols_last = tail;
             SplitBatch sbc = sb; sbc.rows_last = tail; sbc.cols_last = tail;
             CU(cudaMemsetAsync(am + AMAX_T, 0, sizeof(unsigned), s));
-            CU(launch_split16(H + sz, n, A1 + sz, A1 + nn + sz, ldt, (int)sz, (int)sz, false, SPLIT_ALL, 1.f, am + AMAX_PAN, s, sbt));
-            CU(launch_split16(H + sz * n + sz, n, B2 + sz * ldt + sz, B2 + nn + sz * ldt + sz, ldt, (int)sz, (int)sz, true,
-                              SPLIT_UPPER, 1.f, am + AMAX_INV, s, sbc));
+            CU(launch_split16(split16_args(H + sz, n, A1 + sz, A1 + nn + sz, ldt, (int)sz, (int)sz, false, SPLIT_ALL, 1.f, am + AMAX_PAN, sbt), s));
+            CU(launch_split16(split16_args(H + sz * n + sz, n, B2 + sz * ldt + sz, B2 + nn + sz * ldt + sz, ldt, (int)sz, (int)sz, true,
+                                           SPLIT_UPPER, 1.f, am + AMAX_INV, sbc), s));
             TcGemmArgs g1 = tc_args(T + sz, n, (int)sz, (int)sz, (int)sz, 1.f, 0.f, TC_TRI_RIGHT, TC_MASK_NONE, h->hd);
             g1.nbatch = np; g1.c_bstride = bstride; g1.N_last = tail; g1.K_last = tail;
             g1.a_row0 = 0; g1.a_row_bs = (int)(2 * sz); g1.a_k0 = (int)sz; g1.a_k_bs = (int)(2 * sz);
             g1.b_row0 = (int)sz; g1.b_row_bs = (int)(2 * sz); g1.b_k0 = (int)sz; g1.b_k_bs = (int)(2 * sz);
             g1.amax_a = am + AMAX_PAN; g1.amax_b = am + AMAX_INV; g1.amax_out = am + AMAX_T;
             CU(launch_tc_gemm(m16, g1, h->sched, h->num_sms, s));
-            CU(launch_split16(H, n, A1, A1 + nn, ldt, (int)sz, (int)sz, false, SPLIT_UPPER, 1.f, am + AMAX_INV, s, sb));
-            CU(launch_split16(T + sz, n, B2 + sz * ldt, B2 + nn + sz * ldt, ldt, (int)sz, (int)sz, true, SPLIT_ALL, 1.f, am + AMAX_T, s, sbt));
+            CU(launch_split16(split16_args(H, n, A1, A1 + nn, ldt, (int)sz, (int)sz, false, SPLIT_UPPER, 1.f, am + AMAX_INV, sb), s));
+            CU(launch_split16(split16_args(T + sz, n, B2 + sz * ldt, B2 + nn + sz * ldt, ldt, (int)sz, (int)sz, true, SPLIT_ALL, 1.f, am + AMAX_T, sbt), s));
             TcGemmArgs g2 = tc_args(H + sz, n, (int)sz, (int)sz, (int)sz, -1.f, 0.f, TC_TRI_LEFT, TC_MASK_NONE, h->hd);
             g2.nbatch = np; g2.c_bstride = bstride; g2.N_last = tail;
             g2.a_row0 = 0; g2.a_row_bs = (int)(2 * sz); g2.a_k0 = 0; g2.a_k_bs = (int)(2 * sz);
@@ -1232,13 +1240,12 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
         unsigned *am = h->hd->tc_amax;
         const float inv_tokens = (float)(1.0 / (double)h->tokens);
         CU(cudaMemsetAsync(am + AMAX_U, 0, 4 * sizeof(unsigned), s));      // slots U, D, O, P
-        CU(launch_absmax(h->H, n, n, n, SPLIT_UPPER, 1.f, am + AMAX_U, h->num_sms, s));
         // (of dXX^T only the entries above the diagonal reach O: row j of U starts at column j and M_U keeps j > i)
-        CU(launch_absmax(h->D, n, n, n, SPLIT_STRICT_UPPER, inv_tokens, am + AMAX_D, h->num_sms, s));
-        CU(launch_split16(h->H, n, U16, U16 + nn, ldt, n, n, false, SPLIT_UPPER, 1.f, am + AMAX_U, s, SplitBatch(),
-                          UT16, UT16 + nn));        // U and U^T in one pass
-        CU(launch_split16(h->D, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, inv_tokens, am + AMAX_D, s));
-        h->launches += 4;
+        CU(launch_absmax({h->H, n, n, n, SPLIT_UPPER, 1.f, am + AMAX_U}, {h->D, n, n, n, SPLIT_STRICT_UPPER, inv_tokens, am + AMAX_D}, h->num_sms, s));
+        // U and U^T in one pass, dXX^T in the same launch
+        const Split16Args split_d = split16_args(h->D, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, inv_tokens, am + AMAX_D);
+        CU(launch_split16(split16_args(h->H, n, U16, U16 + nn, ldt, n, n, false, SPLIT_UPPER, 1.f, am + AMAX_U, SplitBatch(), UT16, UT16 + nn), s, &split_d));
+        h->launches += 2;
         const SplitOperand Uop{U16, U16 + nn, n, n, ldt}, UTop{UT16, UT16 + nn, n, n, ldt};
         const SplitOperand Aop{A16, A16 + nn, n, n, ldt};
         TcMaps maps;
@@ -1247,14 +1254,14 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
         TcGemmArgs go = tc_args(O, n, n, n, n, 1.f, 0.f, TC_O, TC_MASK_STRICT_ZERO, h->hd);
         go.amax_a = am + AMAX_D; go.amax_b = am + AMAX_U; go.amax_out = am + AMAX_O;
         CU(launch_tc_gemm(maps, go, h->sched, h->num_sms, s));
-        CU(launch_split16(O, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, 1.f, am + AMAX_O, s));
+        CU(launch_split16(split16_args(O, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, 1.f, am + AMAX_O), s));
         // P = alpha * O U  (B operand rows are rows of U^T)
         if (!make_tc_maps(&maps, Aop, UTop, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
         TcGemmArgs gp = tc_args(h->D, n, n, n, n, alpha, 0.f, TC_P, TC_MASK_STRICT_ZERO, h->hd);
         gp.amax_a = am + AMAX_O; gp.amax_b = am + AMAX_U; gp.amax_out = am + AMAX_P;
         CU(launch_tc_gemm(maps, gp, h->sched, h->num_sms, s));
         // P^T for the lazy-batch updates of gptaq_quantize, over the copy of U that is no longer needed
-        CU(launch_split16(h->D, n, U16, U16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P, s));
+        CU(launch_split16(split16_args(h->D, n, U16, U16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P), s));
         h->launches += 4;
         h->stage = STAGE_P;
         return GPTAQ_OK;
@@ -1289,11 +1296,10 @@ gptaq_status_t gptaq_build_P_rowwise(gptaq_handle_t h, float alpha, gptaq_stream
         __half *PT16 = reinterpret_cast<__half *>(h->ws + wl.s_off[1]);
         unsigned *am = h->hd->tc_amax;
         CU(cudaMemsetAsync(am + AMAX_U, 0, 4 * sizeof(unsigned), s));
-        CU(launch_absmax(h->H, n, n, n, SPLIT_UPPER, 1.f, am + AMAX_U, h->num_sms, s));
-        CU(launch_absmax(h->D, n, n, n, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P, h->num_sms, s));
-        CU(launch_split16(h->H, n, UT16, UT16 + nn, ldt, n, n, true, SPLIT_UPPER, 1.f, am + AMAX_U, s));
-        CU(launch_split16(h->D, n, PT16, PT16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P, s));
-        h->launches += 4;
+        CU(launch_absmax({h->H, n, n, n, SPLIT_UPPER, 1.f, am + AMAX_U}, {h->D, n, n, n, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P}, h->num_sms, s));
+        const Split16Args split_p = split16_args(h->D, n, PT16, PT16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P);
+        CU(launch_split16(split16_args(h->H, n, UT16, UT16 + nn, ldt, n, n, true, SPLIT_UPPER, 1.f, am + AMAX_U), s, &split_p));
+        h->launches += 2;
     }
     h->stage = STAGE_P;
     return GPTAQ_OK;

@@ -55,7 +55,7 @@ __device__ __forceinline__ void record_status(StateHeader *hd, int code, long lo
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) diag_stats_kernel(const float *H, int n, float inv_tokens,
                                                           float damp, StateHeader *hd,
-                                                          uint8_t *dead) {
+                                                          uint8_t *dead, uint8_t *dead_working) {
     __shared__ double red[1024];
     __shared__ float redmax[1024];
     double s = 0.0;
@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(1024) diag_stats_kernel(const float *H, int n,
         if (!isfinite(d)) record_status(hd, ST_NONFINITE, q);
         bool dd = (d == 0.f);
         dead[q] = dd ? 1 : 0;
+        if (dead_working) dead_working[q] = dd ? 1 : 0;
         const float v = dd ? 1.f : d * inv_tokens;
         s += dd ? 1.0 : (double)d * (double)inv_tokens;
         mx = fmaxf(mx, v);
@@ -160,18 +161,50 @@ __device__ __forceinline__ float rounding_error_sq(float w, float scale, float z
     return d * d;
 }
 
-// Per-channel grids from the original rows (dead inputs count as zero weights).
-__global__ void __launch_bounds__(256) row_grid_kernel(const float *W, int64_t ldw, int m, int n,
+template <typename T> struct alignas(4 * sizeof(T)) Quad { T v[4]; };
+
+// Per-channel grids from the original rows (dead inputs count as zero weights), one warp per row; `copy`: also the rows
+// themselves as float32 (the working copy of W, one pass and one launch less).  The clipping search takes four candidates
+// per pass over the row.
+template <typename T>
+__global__ void __launch_bounds__(256) row_grid_kernel(const T *W, int64_t ldw, float *copy, int64_t ldc, int m, int n,
                                                        const uint8_t *dead, int bits, int sym,
                                                        float *scales, float *zeros, int clip_steps, float clip_min) {
-    int row = blockIdx.x * 8 + (threadIdx.x >> 5);
-    int lane = threadIdx.x & 31;
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
     if (row >= m) return;
-    const float *w = W + (int64_t)row * ldw;
+    const T *w = W + (int64_t)row * ldw;
+    float *cw = copy ? copy + (int64_t)row * ldc : nullptr;
+    const bool vec = (n & 3) == 0 && (ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(W) & (4 * sizeof(T) - 1)) == 0 &&
+                     (!copy || ((ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(copy) & 15) == 0));
+    // four columns from c, dead ones as zero
+    auto load4 = [&](int c, float (&v)[4], bool keep) {
+        if (vec) {
+            const Quad<T> q = *reinterpret_cast<const Quad<T> *>(w + c);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] = (float)q.v[e];
+            if (keep) *reinterpret_cast<float4 *>(cw + c) = make_float4(v[0], v[1], v[2], v[3]);
+            const uint32_t dd = *reinterpret_cast<const uint32_t *>(dead + c);
+            if (dd) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) if (dd >> (8 * e) & 0xffu) v[e] = 0.f;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                v[e] = c + e < n ? (float)w[c + e] : 0.f;
+                if (keep && c + e < n) cw[c + e] = v[e];
+                if (c + e < n && dead[c + e]) v[e] = 0.f;
+            }
+        }
+    };
     float lo = 0.f, hi = 0.f, am = 0.f;
-    for (int c = lane; c < n; c += 32) {
-        float v = dead[c] ? 0.f : w[c];
-        lo = fminf(lo, v); hi = fmaxf(hi, v); am = fmaxf(am, fabsf(v));
+#pragma unroll 4
+    for (int c = 4 * lane; c < n; c += 128) {
+        float v[4];
+        load4(c, v, copy != nullptr);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { lo = fminf(lo, v[e]); hi = fmaxf(hi, v[e]); am = fmaxf(am, fabsf(v[e])); }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -184,15 +217,27 @@ __global__ void __launch_bounds__(256) row_grid_kernel(const float *W, int64_t l
     if (clip_steps > 0) {
         const float maxq = (float)((1 << bits) - 1);
         float best = INFINITY;
-        for (int k = 0; k < clip_steps; ++k) {
-            const float p = clip_ratio(k, clip_steps, clip_min);
-            float sk, zk;
-            make_grid(p * lo, p * hi, p * am, bits, sym, sk, zk);
-            float err = 0.f;
-            for (int c = lane; c < n; c += 32) err += rounding_error_sq(dead[c] ? 0.f : w[c], sk, zk, maxq);
+        for (int k = 0; k < clip_steps; k += 4) {
+            float sk[4], zk[4], err[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) err += __shfl_xor_sync(0xffffffffu, err, o);
-            if (err < best) { best = err; s = sk; z = zk; }
+            for (int t = 0; t < 4; ++t) {
+                const float p = clip_ratio(min(k + t, clip_steps - 1), clip_steps, clip_min);
+                make_grid(p * lo, p * hi, p * am, bits, sym, sk[t], zk[t]);
+            }
+            for (int c = 4 * lane; c < n; c += 128) {
+                float v[4];
+                load4(c, v, false);
+#pragma unroll
+                for (int e = 0; e < 4; ++e)          // (columns beyond n are zeros: on every grid, no error)
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) err[t] += rounding_error_sq(v[e], sk[t], zk[t], maxq);
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) err[t] += __shfl_xor_sync(0xffffffffu, err[t], o);
+                if (k + t < clip_steps && err[t] < best) { best = err[t]; s = sk[t]; z = zk[t]; }
+            }
         }
     }
     if (lane == 0) { scales[row] = s; zeros[row] = z; }
@@ -533,7 +578,6 @@ __global__ void __launch_bounds__(256) unpermute_rows_kernel(float *W, int64_t l
 // dst[r][c] = src[r][c] as float32: the working copy of W.  A thread takes 4 columns of WIDEN_ROWS rows, all loads before the
 // first store.  Bound by device memory (16384 x 4096 bf16 58 us, one element at a time 160; 4096 x 4096 float32 18, 43).
 constexpr int WIDEN_ROWS = 8;
-template <typename T> struct alignas(4 * sizeof(T)) Quad { T v[4]; };
 template <typename T>
 __global__ void __launch_bounds__(256) widen_kernel(const T *src, int64_t lds, float *dst, int64_t ldd, int m, int n) {
     const int c = (blockIdx.x * 256 + threadIdx.x) * 4;

@@ -514,8 +514,15 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
 // ---------------------------------------------------------------------------
 enum SplitMask { SPLIT_ALL = 0, SPLIT_UPPER = 1, SPLIT_STRICT_UPPER = 2 };
 
-__global__ void __launch_bounds__(256) absmax_kernel(const float *src, long long lds, int rows, int cols, int mask,
-                                                     float scale, unsigned *slot) {
+struct AbsmaxArgs { const float *src; long long lds; int rows, cols, mask; float scale; unsigned *slot; };
+// (two matrices per launch, blockIdx.y)
+__global__ void __launch_bounds__(256) absmax_kernel(AbsmaxArgs a0, AbsmaxArgs a1) {
+    const AbsmaxArgs &a = blockIdx.y ? a1 : a0;
+    const float *src = a.src;
+    const long long lds = a.lds;
+    const int rows = a.rows, cols = a.cols, mask = a.mask;
+    const float scale = a.scale;
+    unsigned *slot = a.slot;
     __shared__ float red[8];
     float m = 0.f;
     const bool vec = (lds & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
@@ -573,11 +580,13 @@ __device__ __forceinline__ void split16_pack(const float (&x)[4], uint2 &hi, uin
 // 64 x 64 tiles; a thread handles four consecutive source columns (plain) or four consecutive source
 // rows of one column (transposed), so that every store is 8 bytes.  Needs lds, ldd multiples of 4 and
 // 16- / 8-byte aligned bases (the host checks); rows and cols are arbitrary.
-__global__ void __launch_bounds__(256) split16_kernel(Split16Args a) {
+// With `second` the launch has another matrix's tiles behind its own batch entries (blockIdx.z = a.nbatch: one entry).
+__global__ void __launch_bounds__(256) split16_kernel(Split16Args a, Split16Args second) {
     __shared__ float tile[64][65];
     const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
     {
-        const int z = blockIdx.z;
+        int z = blockIdx.z;
+        if (z == a.nbatch) { a = second; z = 0; }
         const bool last = z == a.nbatch - 1;
         if (last && a.rows_last) a.rows = a.rows_last;
         if (last && a.cols_last) a.cols = a.cols_last;
