@@ -132,8 +132,10 @@ __device__ __forceinline__ int chol32(float (&d)[32], int lane, float *Sd, float
 // being factored).  Warp 16 runs the tensor-core product.
 // What bounds it: the pivot chain (about 150 cycles a column, 5k per sub-block) and the words that shared memory returns
 // (solving the rows 2.2k, the next sub-block 3.5k cycles): solving by substitution, a row per lane, reads R once per row and
-// took as long as the factorisation itself.  The helpers run beside the chain's solve and product on purpose: kept back until
-// the chain factors again, their reads slowed the pivots more (45k against 38k cycles in all).
+// took as long as the factorisation itself.  The helpers start when the chain's rows are solved: beside that solve their
+// reads delay it (n = 2052 761 -> 755 us in all), kept back until the chain factors again they slow the pivots more (45k
+// against 38k cycles).  Two columns per pivot step (two roots and one round of shuffles for both) took longer, 321 -> 328
+// us at n = 1024: the chain is short of issue slots and shared memory by then, not of latency.
 // ---------------------------------------------------------------------------
 constexpr int DF_MAIN = 512, DF_THREADS = DF_MAIN + 32;
 constexpr int DF_CHAIN = 128, DF_HELP = 8 * 32;
@@ -303,7 +305,7 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
     };
     // Named barriers: 1 -- a sub-block is factored and inverted and the helpers' last update is done (warps 0 - 15); 2 -- the
     // rows right above are solved (chain warps arrive, helpers wait); 3 -- the same, among the chain warps; 4 .. 11 -- four
-    // columns of the sub-block are ready for its inverter.
+    // columns of the sub-block are ready for its inverter; 12 -- the rows further up are solved, among the helpers.
     if (tid < DF_CHAIN) {
         float d[32];
         if (warp == 0) {
@@ -322,28 +324,30 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
             if (tid < 64) solve_rows(o, o1, tid);
             named_bar_arrive(2, DF_CHAIN + DF_HELP);
             named_bar_sync(3, DF_CHAIN);
-            // the next sub-block, less their contribution: 4 x 4 outputs of the upper triangle per thread, mirrored
-            if (tid < 36) {
-                int ti = 0, left = tid;
-                while (left >= 8 - ti) { left -= 8 - ti; ++ti; }
-                const int i = o1 + 4 * ti, j = o1 + 4 * (ti + left);
-                float acc[4][4];
-                rows_dot(o, i, j, acc);
+            // the next sub-block, less their contribution: 2 x 4 outputs of the upper triangle per thread, mirrored (n = 2052:
+            // 770 us in all with 4 x 4 outputs in 36 threads, 760)
+            {
+                const int i = o1 + 2 * (tid >> 3), j = o1 + 4 * (tid & 7);
+                if (j + 3 >= i) {
+                    float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll 8
+                    for (int k = 0; k < 32; ++k) {
+                        const float2 ri = *reinterpret_cast<const float2 *>(&S[o + k][i]);
+                        const float4 rj = *reinterpret_cast<const float4 *>(&S[o + k][j]);
+                        acc[0][0] = fmaf(ri.x, rj.x, acc[0][0]); acc[0][1] = fmaf(ri.x, rj.y, acc[0][1]);
+                        acc[0][2] = fmaf(ri.x, rj.z, acc[0][2]); acc[0][3] = fmaf(ri.x, rj.w, acc[0][3]);
+                        acc[1][0] = fmaf(ri.y, rj.x, acc[1][0]); acc[1][1] = fmaf(ri.y, rj.y, acc[1][1]);
+                        acc[1][2] = fmaf(ri.y, rj.z, acc[1][2]); acc[1][3] = fmaf(ri.y, rj.w, acc[1][3]);
+                    }
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float4 q = *reinterpret_cast<const float4 *>(&S[i + e][j]);
-                    acc[e][0] = q.x - acc[e][0]; acc[e][1] = q.y - acc[e][1]; acc[e][2] = q.z - acc[e][2]; acc[e][3] = q.w - acc[e][3];
-                }
-                if (left == 0) {
+                    for (int e = 0; e < 2; ++e)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e)
-#pragma unroll
-                        for (int f = 0; f < e; ++f) acc[e][f] = acc[f][e];
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    *reinterpret_cast<float4 *>(&S[i + e][j]) = make_float4(acc[e][0], acc[e][1], acc[e][2], acc[e][3]);
-                    if (left) *reinterpret_cast<float4 *>(&S[j + e][i]) = make_float4(acc[0][e], acc[1][e], acc[2][e], acc[3][e]);
+                        for (int f = 0; f < 4; ++f)
+                            if (j + f >= i + e) {
+                                const float v = S[i + e][j + f] - acc[e][f];
+                                S[i + e][j + f] = v;
+                                if (j + f > i + e) S[j + f][i + e] = v;
+                            }
                 }
             }
             named_bar_sync(3, DF_CHAIN);
@@ -361,8 +365,9 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
         for (int sb = 3; sb >= 1; --sb) {
             const int o = 32 * sb;
             named_bar_sync(1, DF_MAIN);
-            if (t < 2 * (o - 32)) solve_rows(o, 0, t);
             named_bar_sync(2, DF_CHAIN + DF_HELP);
+            if (t < 2 * (o - 32)) solve_rows(o, 0, t);
+            named_bar_sync(12, DF_HELP);
             // leading part: S[i][j] -= X[i] . X[j] for i <= j < o, the tiles of the upper triangle numbered row by row; the
             // last 32 x 32 sub-block is the chain's own
             const int q = o / 4, ntile = q * (q + 1) / 2 - 36;
