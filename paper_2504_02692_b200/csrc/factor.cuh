@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(PS_THREADS) panel_solve_kernel(PanelSolveArgs 
 }
 
 // ---------------------------------------------------------------------------
-// Inverts every NB x NB diagonal factor R_pp (one CTA each) and stores the inverse on the
+// Inverts NB x NB diagonal factors R_pp from block `first` on (one CTA each) and stores the inverse on the
 // diagonal of H (strict lower part of the block zero): the starting point of U = R^-1.  Bound by shared-memory
 // reads: 4 x 4 outputs per thread (one output per thread, and divisions in the substitution, took 36 us; now 11).
 // 32 x 32 diagonal sub-blocks by back substitution (one warp each, lane = column), then
@@ -629,13 +629,13 @@ __device__ __forceinline__ void tile_product(float *C, int ldc, const float *A, 
             make_float4(sign * acc[e][0], sign * acc[e][1], sign * acc[e][2], sign * acc[e][3]);
 }
 
-__global__ void __launch_bounds__(ID_THREADS, 1) invert_diag_blocks_kernel(float *H, int n, const float *Rdiag) {
+__global__ void __launch_bounds__(ID_THREADS, 1) invert_diag_blocks_kernel(float *H, int n, const float *Rdiag, int first) {
     extern __shared__ __align__(16) float smem_f[];
     float *S = smem_f + 32, *X = S + NB * ID_LD,      // (padding: solve32 reads ahead of its block)
           *T = X + NB * ID_LD, *dinv = T + 64 * 68;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int b0 = blockIdx.x * NB;
-    const float *src = Rdiag + (int64_t)blockIdx.x * NB * NB;
+    const int b0 = (first + blockIdx.x) * NB;
+    const float *src = Rdiag + (int64_t)(first + blockIdx.x) * NB * NB;
     float4 v[NB * NB / 4 / ID_THREADS];
 #pragma unroll
     for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) v[it] = *reinterpret_cast<const float4 *>(src + 4 * (tid + it * ID_THREADS));

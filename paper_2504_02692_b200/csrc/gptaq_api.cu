@@ -60,6 +60,8 @@ struct gptaq_ctx {
     // tensor-core product on `gemm_stream`, so that the (memory-bound) conversion of the next
     // batch overlaps the (tensor-bound) product of this one.  Two operand buffers alternate.
     cudaStream_t gemm_stream;
+    cudaStream_t inv_stream;      // gptaq_factor: the rows of the inverse, beside the factorisation
+    cudaEvent_t inv_ready, inv_done;
     cudaEvent_t conv_done[2], gemm_done[2];
     bool gemm_pending[2];
     bool relayout;         // the operand buffers change size: wait for the products in flight first
@@ -924,7 +926,8 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
         delete h;
         return GPTAQ_ERR_CUDA;
     }
-    h->gemm_stream = nullptr;
+    h->gemm_stream = h->inv_stream = nullptr;
+    h->inv_ready = h->inv_done = nullptr;
     h->relayout = false;
     h->next_buf = 0;
     h->stats_maps[0].kp = h->stats_maps[1].kp = 0;
@@ -939,6 +942,9 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
         e = cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
         if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->gemm_stream, cudaStreamNonBlocking, prio_hi);
     }
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->inv_stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->inv_ready, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->inv_done, cudaEventDisableTiming);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
         e = cudaEventCreateWithFlags(&h->conv_done[i], cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->gemm_done[i], cudaEventDisableTiming);
@@ -975,6 +981,12 @@ gptaq_status_t gptaq_destroy(gptaq_handle_t h) {
         cudaStreamSynchronize(h->gemm_stream);
         cudaStreamDestroy(h->gemm_stream);
     }
+    if (h->inv_stream) {
+        cudaStreamSynchronize(h->inv_stream);
+        cudaStreamDestroy(h->inv_stream);
+    }
+    if (h->inv_ready) cudaEventDestroy(h->inv_ready);
+    if (h->inv_done) cudaEventDestroy(h->inv_done);
     for (int i = 0; i < 2; ++i) {
         if (h->conv_done[i]) cudaEventDestroy(h->conv_done[i]);
         if (h->gemm_done[i]) cudaEventDestroy(h->gemm_done[i]);
@@ -1114,6 +1126,33 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
         h->launches++;
         return GPTAQ_OK;
     };
+    // U = R^-1 of each diagonal block of SUPER_NB columns, a row of NB x NB blocks at a time and beside the factorisation:
+    //   U[p, p] = R_pp^-1,   U[p, > p] = -R_pp^-1 (R[p, > p] U[> p, > p])   (columns > p of the super-panel)
+    // The product in brackets needs the panels to the right only and runs while block p is being factored; when the last
+    // block is, little is left (by doubling 128 -> 1024 afterwards, every level waiting for the one before, 74 us at n = 1024
+    // and 175 at 4096).  Plain float32 products.  R is overwritten: row p comes after panel p is solved, hence after the
+    // update that reads it.  Nothing of this is put on the chain's own stream, where every event costs 4 us.
+    cudaStream_t is = nb > 1 ? h->inv_stream : s;
+    auto invert_diag = [&](int p, cudaStream_t st) -> gptaq_status_t {
+        invert_diag_blocks_kernel<<<1, ID_THREADS, ID_SMEM, st>>>(H, n, Rinv, p);
+        LAUNCHED();
+        return GPTAQ_OK;
+    };
+    auto inverse_row = [&](int p) -> gptaq_status_t {
+        const int b0 = p * NB, b1 = b0 + NB, e1 = std::min(b0 / SUPER_NB * SUPER_NB + SUPER_NB, n);
+        if (b1 >= e1) return GPTAQ_OK;
+        GemmProblem pu = make_problem(make_operand(H + (int64_t)b0 * n + b0, n, 1), make_operand(T + (int64_t)b0 * n + b1, 1, n),
+                                      H + (int64_t)b0 * n + b1, n, NB, e1 - b1, NB, -1.f, 0.f, GEMM_TRI_LEFT);
+        return gemm(h, pu, false, true, is);
+    };
+    // R[p, > p] U[> p, > p], once panel p + 1 is solved
+    auto inverse_product = [&](int p) -> gptaq_status_t {
+        const int b0 = p * NB, b1 = b0 + NB, e1 = std::min(b0 / SUPER_NB * SUPER_NB + SUPER_NB, n);
+        if (b1 >= e1) return GPTAQ_OK;
+        GemmProblem pt = make_problem(make_operand(H + (int64_t)b0 * n + b1, n, 1), make_operand(H + (int64_t)b1 * n + b1, 1, n),
+                                      T + (int64_t)b0 * n + b1, n, NB, e1 - b1, e1 - b1, 1.f, 0.f, GEMM_TRI_RIGHT);
+        return gemm(h, pt, false, true, is);
+    };
     bool diag_done = false;                     // the diagonal block of this panel was factored beside the last update
     for (int p = nb - 1; p >= 0; --p) {
         const int b0 = p * NB;
@@ -1140,6 +1179,11 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
         else CU(launch_pdl(true, panel_solve_kernel<2>, pg, dim3(PS_THREADS), PS_SMEM, s, pa));
         h->launches++;
         if (!ahead) {
+            CU(cudaEventRecord(h->inv_ready, s));
+            CU(cudaStreamWaitEvent(is, h->inv_ready, 0));
+            OK(invert_diag(p, is));
+            OK(inverse_row(p));
+            OK(inverse_product(p - 1));
             OK(update(p, s, h->num_sms));
             continue;
         }
@@ -1151,20 +1195,28 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
         OK(factor_diag(p - 1, next_diag, NB, 1, b0 - s0));
         CU(cudaStreamWaitEvent(s, h->gemm_done[0], 0));
         diag_done = true;
+        OK(invert_diag(p, h->gemm_stream));
+        CU(cudaEventRecord(h->inv_ready, h->gemm_stream));
+        CU(cudaStreamWaitEvent(is, h->inv_ready, 0));
+        OK(inverse_row(p));
+        OK(inverse_product(p - 1));
     }
+    // (block 0 is inverted on the chain's stream while the inverse's own stream ends with the product of row 0)
+    OK(invert_diag(0, s));
+    if (nb > 1) {
+        CU(cudaEventRecord(h->inv_done, is));
+        CU(cudaStreamWaitEvent(s, h->inv_done, 0));
+    }
+    is = s;
+    OK(inverse_row(0));
 
-    // U = R^-1: inverted diagonal blocks, then off-diagonal blocks by doubling:
+    // U beyond the diagonal blocks of SUPER_NB columns, by doubling:
     // inv([[A, B], [0, C]]) = [[A^-1, -A^-1 B C^-1], [0, C^-1]]
-    invert_diag_blocks_kernel<<<nb, ID_THREADS, ID_SMEM, s>>>(H, n, Rinv);
-    LAUNCHED();
-    for (int64_t sz = NB; sz < n; sz *= 2) {
+    for (int64_t sz = SUPER_NB; sz < n; sz *= 2) {
         const int np = (int)((n - sz + 2 * sz - 1) / (2 * sz));
         const int tail = (int)(n - (2 * sz * (np - 1) + sz));
         const int64_t bstride = 2 * sz * ((int64_t)n + 1);
-        // few tiles: the plain float32 products of 32 x 32 tiles need no operand copies and beat the tensor cores'
-        // two splits and a product per factor
-        const bool few = np * (sz / GBM) * (sz / GBN) <= SIMT_SMALL_TILES;
-        if (h->tensor && damp > 0.f && sz >= 2 * NB && !few) {
+        if (h->tensor && damp > 0.f) {
             // The two products on the tensor cores with FP16-split operands.  Ranges: B holds entries of R
             // (bounded like the panels), the inverted blocks are bounded by 1 / sqrt(lambda), the
             // intermediate T records its own maximum in the first product's epilogue.
@@ -1200,7 +1252,7 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
             h->launches += 6;
             continue;
         }
-        // the narrow levels, and every level without damping (nothing bounds the
+        // odd widths, and every level without damping (nothing bounds the
         // inverse in advance then): plain float32 products
         // T = B * C^-1
         GemmProblem p1 = make_problem(make_operand(H + sz, n, 1),
