@@ -9,8 +9,9 @@
 // update: it takes a copy of the block from before the update and subtracts this panel's contribution itself (one
 // 128 x 128 x 128 product on the tensor cores), so that the update runs beside it on another stream.  A panel of a
 // 1024-wide layer took 33 us (every CTA of one kernel factored the diagonal block first) + 12 us for the update, now
-// about 20 us (diagonal) + 7 us (rows above).  Factorisation with the inversion that follows, before and after:
-// n = 1024 404 -> 337 us, n = 4096 2036 -> 1790 us, n = 14336 19.8 -> 15.9 ms.
+// about 20 us (diagonal) + 7 us (rows above).  Factorisation with the inversion that follows it, before and after (the
+// inversion beside the panels included): n = 1024 404 -> 287 us, n = 2052 1118 -> 726 us, n = 4096 2036 -> 1500 to 1700 us,
+// n = 14336 19.8 -> 16.6 ms.
 #pragma once
 #include "tc_gemm.cuh"
 
