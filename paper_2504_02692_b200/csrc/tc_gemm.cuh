@@ -141,6 +141,7 @@ struct TcSched { unsigned base = 0; bool second = false; };    // second: of sch
 struct TcTile {
     bool skip, zero_fill, work;
     int z, i0, j0, Mz, Nz, kb0, kb1;   // K-block range [kb0, kb1)
+    int kc0;                           // accumulation chains are cut every TCHUNK K-blocks from here on (kc0 <= kb0)
 };
 
 template <int TBN>
@@ -174,6 +175,11 @@ __device__ __forceinline__ void tc_decode(const TcGemmArgs &a, int t, TcTile &ti
     }
     ti.kb0 = kb / bk;
     ti.kb1 = (ke + bk - 1) / bk;
+    // Row a of U begins with its diagonal entry, by far the largest term of the sum, and what is added behind it in the same
+    // chain is truncated at that term's last place.  The cuts of TC_O are therefore those of a 256-wide tile for every tile
+    // width: chains that began at a narrow tile's own first column had the term at their beginning (P from the device's own
+    // U and dXX^T, relative error at n = 1024: 1.22e-6 with 64-wide tiles and 1.08e-6 with 128-wide ones, now 9.0e-7).
+    ti.kc0 = a.mode == TC_O ? ti.j0 / (TCHUNK * TBK) * TCHUNK : ti.kb0;
     ti.work = !ti.skip && ti.kb0 < ti.kb1;
 }
 
@@ -324,13 +330,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                 if (t < 0) break;
                 tc_decode<TBN>(a, t, ti, BK);
                 if (!ti.work) continue;
-                for (int kc = ti.kb0; kc < ti.kb1 && ok; kc += TCHUNK) {
+                for (int kc = ti.kc0; kc < ti.kb1 && ok; kc += TCHUNK) {
                     const uint32_t buf = ccount & 1u, cphase = (ccount >> 1) & 1u;
                     if (!mbar_wait(tempty_bar(buf), cphase ^ 1u, abort_flag)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t d_tmem = tmem_base + buf * TBN;
-                    const int kc1 = min(kc + TCHUNK, ti.kb1);
-                    for (int kb = kc; kb < kc1; ++kb) {
+                    const int kfirst = max(kc, ti.kb0), kc1 = min(kc + TCHUNK, ti.kb1);
+                    for (int kb = kfirst; kb < kc1; ++kb) {
                         if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
                         tc_fence_after();
                         const uint32_t s0 = base + stage * TSTAGE_BYTES;
@@ -343,7 +349,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                         };
 #pragma unroll
                         for (int k = 0; k < BK / KSTEP; ++k)
-                            mma(alo + (uint64_t)(k * 2), bhi + (uint64_t)(k * 2), (kb != kc || k != 0) ? 1u : 0u);
+                            mma(alo + (uint64_t)(k * 2), bhi + (uint64_t)(k * 2), (kb != kfirst || k != 0) ? 1u : 0u);
 #pragma unroll
                         for (int k = 0; k < BK / KSTEP; ++k) mma(ahi + (uint64_t)(k * 2), blo + (uint64_t)(k * 2), 1u);
 #pragma unroll
@@ -380,7 +386,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
 #pragma unroll
             for (int i = 0; i < TBN / 2; ++i) acc[i] = 0.f;
             if (ti.work) {
-                for (int kc = ti.kb0; kc < ti.kb1; kc += TCHUNK) {
+                for (int kc = ti.kc0; kc < ti.kb1; kc += TCHUNK) {
                     const uint32_t buf = ccount & 1u, cphase = (ccount >> 1) & 1u;
                     if (!mbar_wait(tfull_bar(buf), cphase, abort_flag)) { ok = false; break; }
                     tc_fence_after();

@@ -812,3 +812,29 @@ def test_statistics_cut_by_length(n, tokens, act_order):
     assert (np.abs(np.triu(Hg - H)) / np.outer(h, h)).max() < 1e-5
     err = Dg - D if act_order else np.triu(Dg - D, 1)
     assert (np.abs(err) / np.outer(np.sqrt(d), h)).max() < 2.0 ** -10
+
+
+@pytest.mark.parametrize("n", [512, 1024, 1416])
+def test_correction_matrix_sums_keep_their_precision_in_narrow_tiles(n):
+    """P from the device's own U and dXX^T where the products take 64-wide tiles.  A chain of 256 contraction steps is 48
+    MMAs, and each of them truncates the running sum.  The largest term of an entry of O is that of the diagonal entry of U;
+    what counts are the MMAs behind it in its chain, 24 on average when chains are cut at multiples of 256.  Half a unit in
+    the last place each, 2^-24 times the mean of one over a mantissa, 1 / (2 ln 2): 24 * 0.72 * 2^-24.  (Chains that begin
+    at a tile's own first column have 42 of them.)"""
+    torch.manual_seed(n)
+    tokens, alpha = 4 * n, 0.25
+    X = torch.randn(tokens, n, device="cuda")
+    Xfp = X + 0.05 * torch.randn(tokens, n, device="cuda")
+    st = g.LayerState(n, 1, tokens, 32, "cuda")
+    try:
+        g.gptaq_accumulate(st.handle, X, Xfp)
+        D = np.triu(st.D().cpu().numpy().astype(np.float64), 1) / tokens
+        g.gptaq_factor(st.handle, 0.01)
+        g.gptaq_build_P(st.handle, alpha)
+        U = np.triu(st.H().cpu().numpy().astype(np.float64))
+        P = np.triu(st.D().cpu().numpy().astype(np.float64), 1)
+        assert g.gptaq_sync_status(st.handle)[0] == g.GPTAQ_OK
+    finally:
+        st.close()
+    err = hp.rel_fro(P, alpha * np.triu(np.triu(D @ U.T, 1) @ U, 1))
+    assert err <= 24 * 0.72 * 2.0 ** -24, err
