@@ -432,7 +432,8 @@ __global__ void __launch_bounds__(1024) column_loop_kernel(ColumnLoopArgs a) {
             wrow[c] = w[t];
             if (a.perm) a.codes[(int64_t)row * n + a.perm[i0 + c]] = (uint8_t)code[t];
             else crow[c] = (uint8_t)code[t];
-            bad |= !isfinite(w[t]);
+            // (of the value before the rounding and of the error: the rounded weight is finite whatever came in)
+            bad |= !isfinite(w[t]) || !isfinite(nerr[t]) || !isfinite(pre[t]);
         }
     }
     if (bad) record_status(a.hd, ST_NONFINITE, row);

@@ -338,20 +338,15 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         store_grid(tid >> 3, 4 * (tid & 7), sc, zp);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    if (fills) {
+    if (fills && dead4) {
         float4 *wp = reinterpret_cast<float4 *>(Ws + wr0 * WLD + wc);                  // (the words that this thread has copied)
         for (int r = wr0; r < QB_ROWS; r += RSTEP, wp += RSTEP * WLD / 4) {
             float4 v = *wp;
-            if (dead4) {
-                if (dead4 & 0xffu) v.x = 0.f;
-                if (dead4 & 0xff00u) v.y = 0.f;
-                if (dead4 & 0xff0000u) v.z = 0.f;
-                if (dead4 & 0xff000000u) v.w = 0.f;
-                *wp = v;
-            }
-            // a non-finite weight is reported from the value that was read: its code and dequantized value
-            // come out finite (the clamp absorbs NaN and Inf), so the results alone would not show it
-            if (!isfinite(v.x) || !isfinite(v.y) || !isfinite(v.z) || !isfinite(v.w)) record_status(a.hd, ST_NONFINITE, row0 + r);
+            if (dead4 & 0xffu) v.x = 0.f;
+            if (dead4 & 0xff00u) v.y = 0.f;
+            if (dead4 & 0xff0000u) v.z = 0.f;
+            if (dead4 & 0xff000000u) v.w = 0.f;
+            *wp = v;
         }
     }
     if (FAR) tc_fence_before();
@@ -642,16 +637,33 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                             if (left > 2) dst[2] = v.z;
                             if (left > 3) dst[3] = v.w;
                         }
-                        if (!isfinite(v.x) || !isfinite(v.y) || !isfinite(v.z) || !isfinite(v.w)) record_status(a.hd, ST_NONFINITE, row0 + r);
                     }
-                    if (a.EW && r < nrows) {
+                    // Non-finite values are reported from every column's value before its rounding (and its error: a range that
+                    // overflows, a pivot of zero).  Codes and dequantized weights come out finite (the clamp absorbs NaN and
+                    // Inf), so the results do not show them, and values checked when the slab is filled miss what a later
+                    // column receives through U and P inside the launch.
+                    auto magnitude = [](float v) { return __float_as_uint(v) & 0x7fffffffu; };
+                    if (!a.EW) {
+                        const int k = t >> 3;                       // column k, rows ti, ti + 8, ..
+                        const float4 e = *reinterpret_cast<const float4 *>(St + k * QB_SLD + 4 * ti);
+                        const float4 p = *reinterpret_cast<const float4 *>(St + (32 + k) * QB_SLD + 4 * ti);
+                        const uint32_t big[4] = {max(magnitude(e.x), magnitude(p.x)), max(magnitude(e.y), magnitude(p.y)),
+                                                 max(magnitude(e.z), magnitude(p.z)), max(magnitude(e.w), magnitude(p.w))};
+#pragma unroll
+                        for (int f = 0; f < 4; ++f)
+                            if (big[f] >= 0x7f800000u && ti + 8 * f < nrows) record_status(a.hd, ST_NONFINITE, row0 + ti + 8 * f);
+                    } else if (r < nrows) {
                         const int pos = qb_pos(r);
                         float e4[4], p4[4];
+                        uint32_t big = 0u;
 #pragma unroll
                         for (int f = 0; f < 4; ++f) {
                             e4[f] = St[(c4 + f) * QB_SLD + pos];
-                            p4[f] = rho * St[(32 + c4 + f) * QB_SLD + pos];
+                            const float p = St[(32 + c4 + f) * QB_SLD + pos];
+                            big = max(big, max(magnitude(e4[f]), magnitude(p)));
+                            p4[f] = rho * p;
                         }
+                        if (big >= 0x7f800000u) record_status(a.hd, ST_NONFINITE, row0 + r);
                         float *ew = a.EW + (int64_t)(row0 + r) * a.ew_ld + cw;
                         *reinterpret_cast<float4 *>(ew) = make_float4(e4[0], e4[1], e4[2], e4[3]);
                         *reinterpret_cast<float4 *>(ew + a.ew_pre) = make_float4(p4[0], p4[1], p4[2], p4[3]);

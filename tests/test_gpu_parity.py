@@ -838,3 +838,59 @@ def test_correction_matrix_sums_keep_their_precision_in_narrow_tiles(n):
         st.close()
     err = hp.rel_fro(P, alpha * np.triu(np.triu(D @ U.T, 1) @ U, 1))
     assert err <= 24 * 0.72 * 2.0 ** -24, err
+
+
+@pytest.mark.parametrize("n,c,group,tokens", [
+    (96, 40, 32, 200),       # one block, inside it
+    (96, 93, 0, 200),        # the last step of a block
+    (512, 100, 128, 700),    # one launch: to later blocks through the tensor cores
+    (1032, 1010, 0, 1100),   # the last block of a launch
+    (1032, 1026, 0, 1100),   # the last launch
+    (64, 40, 8, 200),        # groups of fewer than 32 columns
+])
+def test_a_non_finite_correction_is_reported(n, c, group, tokens):
+    """A NaN in one channel of X~ alone: H and U are finite, row c of P is not, and every column behind c is lost in every
+    row, while all codes and dequantized weights come out finite."""
+    torch.manual_seed(n + c)
+    m = 5
+    X = torch.randn(tokens, n, device="cuda")
+    F = X + 0.05 * torch.randn_like(X)
+    st = g.LayerState(n, m, tokens, 64)
+    try:
+        for poison in (False, True):
+            g.gptaq_reset(st.handle)
+            if poison:
+                F[3, c] = float("nan")
+            g.gptaq_accumulate(st.handle, X, F)
+            g.gptaq_factor(st.handle, 0.01)
+            g.gptaq_build_P(st.handle, 0.25)
+            G = hp.n_groups(n, group)
+            codes = torch.empty((m, n), dtype=torch.uint8, device="cuda")
+            sc, zp = torch.empty((m, G), device="cuda"), torch.empty((m, G), device="cuda")
+            g.gptaq_quantize(st.handle, 0.02 * torch.randn(m, n, device="cuda"), 4, group, False, 128, codes, sc, zp)
+            status, info = g.gptaq_sync_status(st.handle)
+            assert status == (g.GPTAQ_ERR_NONFINITE if poison else g.GPTAQ_OK) and 0 <= info < m, (poison, status, info)
+    finally:
+        st.close()
+
+
+@pytest.mark.parametrize("bad", ["U", "P", "pivot"])
+@pytest.mark.parametrize("n,group,B", [(96, 32, 32), (200, 0, 128), (64, 16, 64)])
+def test_a_non_finite_factor_of_the_static_entry_point_is_reported(n, group, B, bad):
+    torch.manual_seed(n)
+    m, row = 37, n - 12
+    U = torch.eye(n, device="cuda") + torch.triu(0.1 * torch.randn(n, n, device="cuda"), 1)
+    P = torch.triu(0.1 * torch.randn(n, n, device="cuda"), 1)
+    G = hp.n_groups(n, group)
+    codes = torch.empty((m, n), dtype=torch.uint8, device="cuda")
+    sc, zp = torch.empty((m, G), device="cuda"), torch.empty((m, G), device="cuda")
+    W = 0.02 * torch.randn(m, n, device="cuda")
+    status = torch.zeros(2, dtype=torch.int64, device="cuda")
+    g.gptaq_quantize_static(U, P, W.clone(), 4, group, False, B, codes, sc, zp, None, status)
+    assert status.tolist()[0] == g.GPTAQ_OK
+    if bad == "pivot":
+        U[row, row] = 0.0                       # 1 / U_kk
+    else:
+        (U if bad == "U" else P)[row, row + 3] = float("inf")
+    g.gptaq_quantize_static(U, P, W.clone(), 4, group, False, B, codes, sc, zp, None, status)
+    assert status.tolist()[0] == g.GPTAQ_ERR_NONFINITE
