@@ -52,7 +52,6 @@ struct gptaq_ctx {
     int64_t launches;
     int stats_precision;   // GPTAQ_STATS_*
     bool tensor;           // float32-grade tensor-core GEMMs (fp16-split operands) for factor / P / trailing update
-    TcSched sched, sched2; // tile numbering of the float32-grade GEMM launches (see StateHeader::sched_counter)
     int terms;             // GPTAQ_TERM_* switches of gptaq_quantize
     bool static_groups;    // group grids from the original weights, per group of the caller's columns
     int clip_steps; float clip_min;   // clipping-range search of the grids
@@ -280,17 +279,15 @@ bool make_c_map(CUtensorMap *map, float *C, int64_t M, int64_t N, int64_t ldc) {
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-cudaError_t launch_tc_gemm(const TcMaps &m, const TcGemmArgs &a_in, TcSched &sched, int num_sms, cudaStream_t s, bool pdl = true) {
+cudaError_t launch_tc_gemm(const TcMaps &m, const TcGemmArgs &a_in, int num_sms, cudaStream_t s, bool pdl = true, bool beside = false) {
     if (a_in.M <= 0 || a_in.N <= 0 || a_in.nbatch <= 0) return cudaSuccess;
     TcGemmArgs a = a_in;
     const int bn = tc_tile_width(a, num_sms);
     const int64_t tiles = (int64_t)a.nbatch * ((a.M + TBM - 1) / TBM) * ((a.N + bn - 1) / bn);
     const int grid = (int)std::min<int64_t>(tiles, num_sms);
+    a.sched = beside ? &a.hd->sched_counter2 : &a.hd->sched_counter;     // (two launches at the same time: one counter each)
     // "C += ...": bulk tensor reductions where the target qualifies for a tensor map (16-byte aligned base
     // and row pitch); scattered per-thread reductions otherwise
-    a.sched = sched.second ? &a.hd->sched_counter2 : &a.hd->sched_counter;
-    a.sched_base = sched.base;
-    sched.base += (unsigned)tiles;           // (grid <= tiles)
     CUtensorMap mapC = m.a_hi;       // placeholder, not dereferenced unless c_tma is set
     a.c_tma = 0;
     if (a.beta == 1.f && a.nbatch == 1 && !a.amax_out && (a.mask == TC_MASK_NONE || a.mask == TC_MASK_UPPER_KEEP) &&
@@ -518,7 +515,6 @@ struct QuantizeTarget {
     const float *U, *P;
     const uint8_t *dead;
     StateHeader *hd;
-    TcSched *sched;            // host-side count of the tile numbers drawn from hd->sched_counter
     float *EW;
     int64_t ew_floats;         // its size
     int num_sms;
@@ -530,9 +526,8 @@ struct QuantizeTarget {
     __half *EW16 = nullptr;
     float *row_inv = nullptr;
     const unsigned *amax_u = nullptr, *amax_p = nullptr;
-    // a second stream for one half of many rows (null: none), with its own count of tile numbers, and two events
+    // a second stream for one half of many rows (null: none), and two events
     cudaStream_t side = nullptr;
-    TcSched *side_sched = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
     int terms = GPTAQ_TERM_ERR | GPTAQ_TERM_ASYM;   // which terms of the weight update are applied
     const int *perm = nullptr;                      // act_order: working column c is the caller's column perm[c]
@@ -694,7 +689,7 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
         // More rows than one round of CTAs: two halves of the rows on two streams, so that one half's launches fill the SMs
         // that the last round of the other's leaves idle (16384 x 4096, four rounds for 3.5: 3455 us, in one piece
         // 3696; 5000 x 4096, two for 1.06: 1256, 1713).  Rows that one round takes gain nothing (4096 x 4096 1045, 1030).
-        struct Part { int64_t r0, r1; cudaStream_t s; TcSched *sched; } parts[2] = {{0, m, s, t.sched}, {m, m, t.side, t.side_sched}};
+        struct Part { int64_t r0, r1; cudaStream_t s; } parts[2] = {{0, m, s}, {m, m, t.side}};
         if (t.side && m > (int64_t)QB_ROWS * t.num_sms) {
             parts[0].r1 = parts[1].r0 = (m / 2 + TBM - 1) / TBM * TBM;
             *err = cudaEventRecord(t.fork, s);
@@ -716,7 +711,7 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
                 g.a_row0 = (int)p.r0;
                 g.b_row0 = i1; g.b_k0 = i0; g.k_split = SW; g.b2_k0 = i0;
                 g.row_inv = t.row_inv + p.r0; g.amax_b = t.amax_u;
-                *err = launch_tc_gemm(maps, g, *p.sched, t.num_sms, p.s, false);
+                *err = launch_tc_gemm(maps, g, t.num_sms, p.s, false, p.s == t.side);
                 if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
                 ++*launches;
             }
@@ -763,7 +758,7 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
             TcGemmArgs g = tc_args(Wk + i1, ldk, (int)m, n - i1, 2 * SW, 1.f, 1.f, TC_FULL, TC_MASK_NONE, t.hd);
             g.b_row0 = i1; g.b_k0 = i0; g.k_split = SW; g.b2_k0 = i0;
             g.row_inv = t.row_inv; g.amax_b = t.amax_u;
-            *err = launch_tc_gemm(maps, g, *t.sched, t.num_sms, s, false);
+            *err = launch_tc_gemm(maps, g, t.num_sms, s, false);
             if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
             ++*launches;
         } else {
@@ -970,8 +965,6 @@ gptaq_status_t gptaq_reset(gptaq_handle_t h, gptaq_stream_t stream) {
     h->stage = STAGE_ACCUM;
     h->tokens = 0;
     h->d_upper_only = false;
-    h->sched.base = h->sched2.base = 0;           // the counters in the header were zeroed with the rest of the state
-    h->sched2.second = true;
     return GPTAQ_OK;
 }
 
@@ -1102,13 +1095,13 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
                 TcGemmArgs g = tc_args(H + s0, n, b0, b0 - s0, NB, -1.f, 1.f, TC_UPPER_TILES, TC_MASK_UPPER_KEEP, h->hd);
                 g.diag_off = s0; g.a_k0 = g.b_k0 = b0 - s0; g.b_row0 = s0;
                 g.amax_a = g.amax_b = am;
-                CU(launch_tc_gemm(pan_maps, g, h->sched, sms, us));
+                CU(launch_tc_gemm(pan_maps, g, sms, us));
             } else {
                 // super-panel [s0, s1) done: A[0:s0, 0:s0] -= R[0:s0, s0:s1] R[0:s0, s0:s1]^T  (upper part)
                 const int s1 = std::min(s0 + SUPER_NB, nb * NB);
                 TcGemmArgs g = tc_args(H, n, s0, s0, s1 - s0, -1.f, 1.f, TC_UPPER_TILES, TC_MASK_UPPER_KEEP, h->hd);
                 g.amax_a = g.amax_b = am;
-                CU(launch_tc_gemm(pan_maps, g, h->sched, sms, us));
+                CU(launch_tc_gemm(pan_maps, g, sms, us));
             }
             h->launches++;
             return GPTAQ_OK;
@@ -1240,7 +1233,7 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
             g1.a_row0 = 0; g1.a_row_bs = (int)(2 * sz); g1.a_k0 = (int)sz; g1.a_k_bs = (int)(2 * sz);
             g1.b_row0 = (int)sz; g1.b_row_bs = (int)(2 * sz); g1.b_k0 = (int)sz; g1.b_k_bs = (int)(2 * sz);
             g1.amax_a = am + AMAX_PAN; g1.amax_b = am + AMAX_INV; g1.amax_out = am + AMAX_T;
-            CU(launch_tc_gemm(m16, g1, h->sched, h->num_sms, s));
+            CU(launch_tc_gemm(m16, g1, h->num_sms, s));
             CU(launch_split16(split16_args(H, n, A1, A1 + nn, ldt, (int)sz, (int)sz, false, SPLIT_UPPER, 1.f, am + AMAX_INV, sb), s));
             CU(launch_split16(split16_args(T + sz, n, B2 + sz * ldt, B2 + nn + sz * ldt, ldt, (int)sz, (int)sz, true, SPLIT_ALL, 1.f, am + AMAX_T, sbt), s));
             TcGemmArgs g2 = tc_args(H + sz, n, (int)sz, (int)sz, (int)sz, -1.f, 0.f, TC_TRI_LEFT, TC_MASK_NONE, h->hd);
@@ -1248,7 +1241,7 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
             g2.a_row0 = 0; g2.a_row_bs = (int)(2 * sz); g2.a_k0 = 0; g2.a_k_bs = (int)(2 * sz);
             g2.b_row0 = (int)sz; g2.b_row_bs = (int)(2 * sz); g2.b_k0 = 0; g2.b_k_bs = (int)(2 * sz);
             g2.amax_a = am + AMAX_INV; g2.amax_b = am + AMAX_T;
-            CU(launch_tc_gemm(m16, g2, h->sched, h->num_sms, s));
+            CU(launch_tc_gemm(m16, g2, h->num_sms, s));
             h->launches += 6;
             continue;
         }
@@ -1305,13 +1298,13 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
         if (!make_tc_maps(&maps, Aop, Uop, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
         TcGemmArgs go = tc_args(O, n, n, n, n, 1.f, 0.f, TC_O, TC_MASK_STRICT_ZERO, h->hd);
         go.amax_a = am + AMAX_D; go.amax_b = am + AMAX_U; go.amax_out = am + AMAX_O;
-        CU(launch_tc_gemm(maps, go, h->sched, h->num_sms, s));
+        CU(launch_tc_gemm(maps, go, h->num_sms, s));
         CU(launch_split16(split16_args(O, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, 1.f, am + AMAX_O), s));
         // P = alpha * O U  (B operand rows are rows of U^T)
         if (!make_tc_maps(&maps, Aop, UTop, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
         TcGemmArgs gp = tc_args(h->D, n, n, n, n, alpha, 0.f, TC_P, TC_MASK_STRICT_ZERO, h->hd);
         gp.amax_a = am + AMAX_O; gp.amax_b = am + AMAX_U; gp.amax_out = am + AMAX_P;
-        CU(launch_tc_gemm(maps, gp, h->sched, h->num_sms, s));
+        CU(launch_tc_gemm(maps, gp, h->num_sms, s));
         // P^T for the lazy-batch updates of gptaq_quantize, over the copy of U that is no longer needed
         CU(launch_split16(split16_args(h->D, n, U16, U16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P), s));
         h->launches += 4;
@@ -1370,7 +1363,7 @@ gptaq_status_t gptaq_quantize(gptaq_handle_t h, void *d_W, int w_dtype, int64_t 
     WsLayout wl = ws_layout(h->n, m);
     if (h->ws_bytes < wl.total) return GPTAQ_ERR_WORKSPACE;
     QuantizeTarget t;
-    t.n = (int)h->n; t.U = h->H; t.P = h->D; t.dead = h->dead; t.hd = h->hd; t.sched = &h->sched;
+    t.n = (int)h->n; t.U = h->H; t.P = h->D; t.dead = h->dead; t.hd = h->hd;
     t.EW = reinterpret_cast<float *>(h->ws + wl.ew_off);
     t.ew_floats = (int64_t)((wl.ew_lo_off - wl.ew_off) / sizeof(float));
     t.num_sms = h->num_sms;
@@ -1378,7 +1371,7 @@ gptaq_status_t gptaq_quantize(gptaq_handle_t h, void *d_W, int w_dtype, int64_t 
     t.perm = h->act_order ? h->perm : nullptr;
     t.clip_steps = h->clip_steps; t.clip_min = h->clip_min;
     t.static_groups = h->static_groups; t.dead_orig = h->dead_raw;
-    t.side = h->gemm_stream; t.side_sched = &h->sched2; t.fork = h->conv_done[0]; t.join = h->gemm_done[0];
+    t.side = h->gemm_stream; t.fork = h->conv_done[0]; t.join = h->gemm_done[0];
     // fp16-split updates, plain float32 products otherwise
     // (groups of fewer than 32 columns update block by block, and blocks of 32 columns are no whole K-block of 64)
     const bool f16 = h->tensor && ((blocksize % 64) == 0 || group <= 0 || (group % 32) == 0 || h->static_groups);
@@ -1454,8 +1447,7 @@ gptaq_status_t gptaq_quantize_static(const float *d_U, const float *d_P, int64_t
     e = cudaMemsetAsync(sc->base, 0, STATIC_EW_OFFSET, s);
     if (e != cudaSuccess) return GPTAQ_ERR_CUDA;
     QuantizeTarget t;
-    TcSched static_sched;        // (the header is zeroed at every call; this path launches no tensor-core GEMM)
-    t.n = (int)n; t.U = d_U; t.P = d_P; t.sched = &static_sched;
+    t.n = (int)n; t.U = d_U; t.P = d_P;
     t.hd = reinterpret_cast<StateHeader *>(sc->base);
     t.dead = sc->base + STATIC_FLAGS_OFFSET;
     t.EW = reinterpret_cast<float *>(sc->base + STATIC_EW_OFFSET);

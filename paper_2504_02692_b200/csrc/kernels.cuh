@@ -17,9 +17,9 @@ struct StateHeader {
     float inv_tokens;
     unsigned amax[2][2]; // per operand buffer: bit patterns of max|X| and max|X~ - X| of the batch converted into it
     unsigned tc_amax[8]; // largest magnitudes of FP16-split operands of the float32-grade GEMMs (see tc_gemm.cuh)
-    unsigned sched_counter; // tile numbers drawn by the float32-grade GEMM launches so far (never reset between launches)
+    unsigned sched_counter; // tile numbers drawn by the float32-grade GEMM launch that is running (0 between launches)
     unsigned stats_done;    // CTAs of the running statistics product that have finished
-    unsigned sched_counter2; // as sched_counter, for launches on the internal stream that run beside those
+    unsigned sched_counter2; // as sched_counter, for launches that run beside those on the internal stream
     int pad1[11];
 };
 static_assert(sizeof(StateHeader) == 128, "header size");

@@ -84,12 +84,11 @@ struct TcGemmArgs {
     unsigned *amax_out;              // if set: receives (atomicMax) the bit pattern of max |C| over what is stored
     int c_tma;                       // beta == 1, one batch entry: C += through bulk tensor reductions (mapC)
     int diag_off;                    // C is a block of columns of a square matrix: its column j is column j + diag_off there
-    // Tile scheduler: CTA b starts with tile b; further tile numbers come from a counter in global
-    // memory that is never reset: this launch owns its values sched_base .. sched_base + tiles - 1
-    // (tiles - grid numbers of tiles, and every CTA draws exactly one number beyond the last tile before
-    // it stops), the host advances the base by `tiles` per launch.
+    // Tile scheduler: CTA b starts with tile b; further tile numbers come from a counter in global memory.  A launch draws
+    // `tiles` numbers (tiles - grid of tiles, and every CTA exactly one beyond the last tile before it stops); whoever draws
+    // the last of them sets the counter back to 0.  So a launch needs nothing of those before it, and one that was captured
+    // can be replayed.
     unsigned *sched;
-    unsigned sched_base;
 };
 
 // Measured cycles: a K-block where every CTA has one tile at most, where the chip is full, and the rest of a tile (epilogue;
@@ -134,9 +133,6 @@ inline int tc_tile_width(const TcGemmArgs &a, int sms) {
     }
     return best;
 }
-
-// Host-side twin of StateHeader::sched_counter: the first tile number of the next launch.
-struct TcSched { unsigned base = 0; bool second = false; };    // second: of sched_counter2
 
 struct TcTile {
     bool skip, zero_fill, work;
@@ -272,7 +268,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
             while (ok) {
                 // next tile for this CTA; -1 once the list is exhausted.  The first one needs no round trip
                 // to the counter: tile number = CTA number; the counter hands out the numbers from gridDim.x on.
-                const unsigned ticket = first ? blockIdx.x : gridDim.x + (atomicAdd(a.sched, 1u) - a.sched_base);
+                unsigned ticket = blockIdx.x;
+                if (!first) {
+                    const unsigned drawn = atomicAdd(a.sched, 1u);
+                    if (drawn == (unsigned)ntiles - 1u) *a.sched = 0u;
+                    ticket = gridDim.x + drawn;
+                }
                 first = false;
                 const int t = ticket < (unsigned)ntiles ? (int)ticket : -1;
                 if (t >= 0) {

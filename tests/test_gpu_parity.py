@@ -894,3 +894,52 @@ def test_a_non_finite_factor_of_the_static_entry_point_is_reported(n, group, B, 
         (U if bad == "U" else P)[row, row + 3] = float("inf")
     g.gptaq_quantize_static(U, P, W.clone(), 4, group, False, B, codes, sc, zp, None, status)
     assert status.tolist()[0] == g.GPTAQ_ERR_NONFINITE
+
+
+def _replays_match(n, m, B, group, solve_too):
+    """gptaq_quantize, or the whole solve, in a CUDA graph that is replayed twice: the direct calls' results bit for bit."""
+    torch.manual_seed(n)
+    X = torch.randn(2 * n, n, device="cuda")
+    F = X + 0.05 * torch.randn_like(X)
+    W = 0.02 * torch.randn(m, n, device="cuda")
+    G = hp.n_groups(n, group)
+    codes = torch.empty((m, n), dtype=torch.uint8, device="cuda")
+    sc, zp, Wq = torch.empty((m, G), device="cuda"), torch.empty((m, G), device="cuda"), torch.empty((m, n), device="cuda")
+    out = (codes, sc, zp, Wq)
+    st = g.LayerState(n, m, 2 * n, B)
+    h = st.handle
+
+    def solve():
+        g.gptaq_reset(h)
+        g.gptaq_accumulate(h, X, F)
+        g.gptaq_factor(h, 0.01)
+        g.gptaq_build_P(h, 0.25)
+
+    def quantize():
+        g.gptaq_quantize(h, W, 4, group, False, B, *out)
+
+    try:
+        solve()
+        quantize()
+        torch.cuda.synchronize()
+        want = [t.clone() for t in out]
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            if solve_too:
+                solve()
+            quantize()
+        for call in (graph.replay, graph.replay, quantize):           # a direct call last
+            for t in out:
+                t.zero_()
+            call()
+            assert g.gptaq_sync_status(h)[0] == g.GPTAQ_OK
+            assert [int((x != y).sum()) for x, y in zip(out, want)] == [0, 0, 0, 0]
+        del graph
+    finally:
+        st.close()
+
+
+@pytest.mark.parametrize("n,m,B,group", [(2048, 4096, 32, 32), (1024, 9000, 128, 128)])
+def test_captured_quantize_can_be_replayed(n, m, B, group):
+    """Products of more tiles than SMs draw their tile numbers from a counter on the device."""
+    _replays_match(n, m, B, group, False)
