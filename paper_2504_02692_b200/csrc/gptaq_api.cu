@@ -1146,12 +1146,17 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
                                       T + (int64_t)b0 * n + b1, n, NB, e1 - b1, e1 - b1, 1.f, 0.f, GEMM_TRI_RIGHT);
         return gemm(h, pt, false, true, is);
     };
+    // Rows of a panel may be read before the diagonal kernel in front of it has finished, because the update that made them is
+    // waited for by an event.  In a captured graph that event becomes an edge of the same programmatic kind as the one from
+    // the diagonal kernel, and the rows would be read before the update has written them.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const bool plain_stream = cudaStreamIsCapturing(s, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
     bool diag_done = false;                     // the diagonal block of this panel was factored beside the last update
     for (int p = nb - 1; p >= 0; --p) {
         const int b0 = p * NB;
         const int s0 = h->tensor ? b0 / SUPER_NB * SUPER_NB : b0;      // first column of this panel's super-panel
         if (!diag_done) OK(factor_diag(p, H + (int64_t)b0 * n + b0, n, 0, 0));
-        const bool early = diag_done;           // (then the update of this panel's columns was waited for, not overlapped)
+        const bool early = diag_done && plain_stream;        // (diag_done: the update of this panel's columns was waited for)
         diag_done = false;
         if (p == 0) break;
         const bool ahead = h->tensor && b0 > s0;   // the next panel is in the same super-panel: its block needs this panel only

@@ -943,3 +943,9 @@ def _replays_match(n, m, B, group, solve_too):
 def test_captured_quantize_can_be_replayed(n, m, B, group):
     """Products of more tiles than SMs draw their tile numbers from a counter on the device."""
     _replays_match(n, m, B, group, False)
+
+
+@pytest.mark.parametrize("n,m,B,group", [(2048, 300, 128, 128), (520, 9000, 64, 64)])
+def test_captured_solve_can_be_replayed(n, m, B, group):
+    """Launches that overlap their predecessors, and three streams, in one graph."""
+    _replays_match(n, m, B, group, True)
