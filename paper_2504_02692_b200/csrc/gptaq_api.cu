@@ -385,6 +385,16 @@ gptaq_status_t join_statistics(gptaq_ctx *h, cudaStream_t s) {
     return GPTAQ_OK;
 }
 
+// For a step that ends early because a CUDA call failed: `s` is ordered after all that the internal streams were given so
+// far, so that whatever the caller does next (gptaq_reset, other use of its buffers) does not meet it.
+gptaq_status_t join_after_error(gptaq_ctx *h, cudaStream_t s, gptaq_status_t st) {
+    if (st != GPTAQ_OK) {
+        if (cudaEventRecord(h->gemm_done[0], h->gemm_stream) == cudaSuccess) cudaStreamWaitEvent(s, h->gemm_done[0], 0);
+        if (cudaEventRecord(h->inv_done, h->inv_stream) == cudaSuccess) cudaStreamWaitEvent(s, h->inv_done, 0);
+    }
+    return st;
+}
+
 gptaq_status_t accumulate_tc(gptaq_ctx *h, const float *X, const float *Xfp, int64_t tokens, int64_t ld,
                              cudaStream_t s) {
     const int n = (int)h->n;
@@ -997,7 +1007,8 @@ gptaq_status_t gptaq_accumulate(gptaq_handle_t h, const float *d_X, const float 
     if (!d_X || !d_Xfp || ld < h->n) return GPTAQ_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int n = (int)h->n;
-    if (tc_eligible(h) && tokens > STATS_FP32_WORK / (h->n * h->n)) return accumulate_tc(h, d_X, d_Xfp, tokens, ld, s);
+    if (tc_eligible(h) && tokens > STATS_FP32_WORK / (h->n * h->n))
+        return join_after_error(h, s, accumulate_tc(h, d_X, d_Xfp, tokens, ld, s));
     OK(join_statistics(h, s));
     // H (upper tiles) += X X^T
     Operand xa = make_operand(d_X, 1, ld);
@@ -1045,10 +1056,8 @@ gptaq_status_t gptaq_accumulate_host(gptaq_handle_t h, const float *h_X, const f
     return gptaq_accumulate(h, dx, dxfp, tokens, h->n, stream);
 }
 
-gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream) {
-    if (!h || !(damp >= 0.f) || !std::isfinite(damp)) return GPTAQ_ERR_INVALID_ARG;
-    if (h->stage != STAGE_ACCUM || h->tokens <= 0) return GPTAQ_ERR_BAD_STATE;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
+// gptaq_factor behind its argument checks.
+static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
     OK(join_statistics(h, s));
     const int n = (int)h->n;
     const int nb = (n + NB - 1) / NB;
@@ -1270,6 +1279,13 @@ gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream)
     return GPTAQ_OK;
 }
 
+gptaq_status_t gptaq_factor(gptaq_handle_t h, float damp, gptaq_stream_t stream) {
+    if (!h || !(damp >= 0.f) || !std::isfinite(damp)) return GPTAQ_ERR_INVALID_ARG;
+    if (h->stage != STAGE_ACCUM || h->tokens <= 0) return GPTAQ_ERR_BAD_STATE;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    return join_after_error(h, s, factor_core(h, damp, s));
+}
+
 gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t stream) {
     if (!h || !std::isfinite(alpha)) return GPTAQ_ERR_INVALID_ARG;
     if (h->stage != STAGE_FACTORED) return GPTAQ_ERR_BAD_STATE;
@@ -1392,7 +1408,7 @@ gptaq_status_t gptaq_quantize(gptaq_handle_t h, void *d_W, int w_dtype, int64_t 
     st = quantize_core(t, d_W, w_dtype, m, ldw, bits, group, sym, blocksize, d_codes, d_scales, d_zeros, d_Wq,
                        static_cast<cudaStream_t>(stream), &h->launches, &e);
     if (st == GPTAQ_ERR_CUDA) h->cuda_error = cudaGetErrorString(e);
-    return st;
+    return join_after_error(h, static_cast<cudaStream_t>(stream), st);
 }
 
 size_t gptaq_quantize_stage_bytes(int64_t m, int64_t n, int group) {
