@@ -575,10 +575,11 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
     const size_t smem = quant_block_smem_bytes(far_form, static_groups);
     // Near form, more CTAs than SMs: two to an SM, one works while the other waits for its own chain (16384 rows of 400
     // columns 455 us, with one 498); below that one, which has the registers of both (1024 rows of 1024 columns 288 us, 301).
-    const bool two = grid.x > (unsigned)t.num_sms;
+    // A grid per column (static groups) takes one always: two have no registers left for it, and gain nothing (16384 rows of
+    // 400 columns 517 us with one, 519 with two; 8192 of 1023 1227, 1221).
+    const bool two = grid.x > (unsigned)t.num_sms && !static_groups;
     if (far_form && static_groups) quant_block_kernel<true, true, 1><<<grid, QB_THREADS_FAR, smem, s>>>(uh, ul, ph, pl, a);
     else if (far_form) quant_block_kernel<true, false, 1><<<grid, QB_THREADS_FAR, smem, s>>>(uh, ul, ph, pl, a);
-    else if (static_groups && two) quant_block_kernel<false, true, 2><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
     else if (static_groups) quant_block_kernel<false, true, 1><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
     else if (two) quant_block_kernel<false, false, 2><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
     else quant_block_kernel<false, false, 1><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
@@ -593,7 +594,6 @@ cudaError_t configure_quantize_kernels() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, true, 1>, attr, (int)quant_block_smem_bytes(true, true));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, false, 1>, attr, (int)quant_block_smem_bytes(true, false));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true, 1>, attr, (int)quant_block_smem_bytes(false, true));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true, 2>, attr, (int)quant_block_smem_bytes(false, true));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false, 1>, attr, (int)quant_block_smem_bytes(false, false));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false, 2>, attr, (int)quant_block_smem_bytes(false, false));
     return e;

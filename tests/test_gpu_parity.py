@@ -339,7 +339,9 @@ def test_act_order(n, m, group, B, bf16):
                                                         (768, 33, 64, 128, True, True, 0), (640, 20, 128, 128, False, False, 0),
                                                         (320, 30, 64, 64, True, False, 3), (512, 33, 64, 64, False, True, 3),
                                                         (768, 24, 128, 128, True, True, 0), (1024, 24, 32, 64, True, True, 3),
-                                                        (320, 64, 32, 128, True, True, 3)])
+                                                        (320, 64, 32, 128, True, True, 3),
+                                                        # more rows than a round of CTAs, without the tensor cores
+                                                        (96, 4737, 32, 64, False, False, 3), (129, 4800, 16, 32, True, False, 0)])
 def test_static_groups(n, m, group, B, act, bf16, ndead):
     """Static groups, with and without act_order: grids per group of the caller's columns from the original
     weights (inputs that never fired count as zero weights); the loop replayed by the oracle in the device's
