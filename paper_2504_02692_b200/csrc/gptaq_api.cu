@@ -313,13 +313,13 @@ struct SplitBatch {
 // hi_t / lo_t non-null: the transposed form goes there in the same pass (transpose is then ignored)
 Split16Args split16_args(const float *src, int64_t lds, __half *hi, __half *lo, int64_t ldd, int rows, int cols,
                          bool transpose, int mask, float scale, const unsigned *amax, const SplitBatch &b = SplitBatch(),
-                         __half *hi_t = nullptr, __half *lo_t = nullptr) {
+                         __half *hi_t = nullptr, __half *lo_t = nullptr, float *row_inv = nullptr) {
     Split16Args a;
     a.src = src; a.lds = lds; a.src_bstride = b.src_bstride; a.hi = hi; a.lo = lo; a.ldd = ldd;
     a.dst_bstride = b.dst_bstride;
     a.rows = rows; a.cols = cols; a.rows_last = b.rows_last; a.cols_last = b.cols_last; a.nbatch = b.nbatch;
     a.transpose = hi_t ? 2 : (transpose ? 1 : 0); a.mask = mask; a.scale = scale; a.amax = amax;
-    a.hi_t = hi_t; a.lo_t = lo_t;
+    a.hi_t = hi_t; a.lo_t = lo_t; a.row_inv = row_inv;
     return a;
 }
 cudaError_t launch_split16(const Split16Args &a, cudaStream_t s, const Split16Args *second = nullptr) {
@@ -1294,10 +1294,12 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
     WsLayout wl = ws_layout(h->n, 0);
     float *O = reinterpret_cast<float *>(h->ws + wl.t_off);
     if (h->tensor) {
-        // every operand is
-        // scaled by a power of two into the fp16 range, so its largest magnitude is recorded first (by a
-        // reduction kernel for U and dXX^T, by the producing GEMM's epilogue for O and P).
-        // Workspace: S[0] = U^T (kept for gptaq_quantize), S[1] = U, then P^T (kept), S[2] = dXX^T, then O.
+        // Every operand is scaled by a power of two into the fp16 range, so its largest magnitude is recorded first (by a
+        // reduction kernel for U and dXX^T, by the producing GEMM's epilogue for O and P).  dXX^T and O have a scale per
+        // row: a row goes with the unit of the input that it belongs to, and with one scale for the whole matrix the rows of
+        // inputs 1e4 below the largest kept 13 of their 22 bits.
+        // Workspace: S[0] = U^T (kept for gptaq_quantize), S[1] = U, then P^T (kept), S[2] = dXX^T, then O; the row scales lie
+        // where gptaq_factor had the diagonal blocks of R.
         const int64_t ldt = split_pitch(n);
         const size_t nn = (size_t)n * ldt;
         __half *UT16 = reinterpret_cast<__half *>(h->ws + wl.s_off[0]);
@@ -1305,11 +1307,15 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
         __half *A16 = reinterpret_cast<__half *>(h->ws + wl.s_off[2]);
         unsigned *am = h->hd->tc_amax;
         const float inv_tokens = (float)(1.0 / (double)h->tokens);
-        CU(cudaMemsetAsync(am + AMAX_U, 0, 4 * sizeof(unsigned), s));      // slots U, D, O, P
+        unsigned *amax_d = reinterpret_cast<unsigned *>(h->ws + wl.rinv_off), *amax_o = amax_d + n;
+        float *inv_d = reinterpret_cast<float *>(amax_o + n), *inv_o = inv_d + n;
+        CU(cudaMemsetAsync(am + AMAX_U, 0, 2 * sizeof(unsigned), s));      // slots U, P
         // (of dXX^T only the entries above the diagonal reach O: row j of U starts at column j and M_U keeps j > i)
-        CU(launch_absmax({h->H, n, n, n, SPLIT_UPPER, 1.f, am + AMAX_U}, {h->D, n, n, n, SPLIT_STRICT_UPPER, inv_tokens, am + AMAX_D}, h->num_sms, s));
+        CU(launch_absmax({h->H, n, n, n, SPLIT_UPPER, 1.f, am + AMAX_U, nullptr, nullptr},
+                         {h->D, n, n, n, SPLIT_STRICT_UPPER, inv_tokens, nullptr, amax_d, amax_o}, h->num_sms, s));
         // U and U^T in one pass, dXX^T in the same launch
-        const Split16Args split_d = split16_args(h->D, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, inv_tokens, am + AMAX_D);
+        const Split16Args split_d = split16_args(h->D, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, inv_tokens, amax_d, SplitBatch(),
+                                                 nullptr, nullptr, inv_d);
         CU(launch_split16(split16_args(h->H, n, U16, U16 + nn, ldt, n, n, false, SPLIT_UPPER, 1.f, am + AMAX_U, SplitBatch(), UT16, UT16 + nn), s, &split_d));
         h->launches += 2;
         const SplitOperand Uop{U16, U16 + nn, n, n, ldt}, UTop{UT16, UT16 + nn, n, n, ldt};
@@ -1318,13 +1324,14 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
         // O = ((dXX^T / tokens) U^T) .* M_U  (contraction over k >= column, U[a][k] = 0 below)
         if (!make_tc_maps(&maps, Aop, Uop, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
         TcGemmArgs go = tc_args(O, n, n, n, n, 1.f, 0.f, TC_O, TC_MASK_STRICT_ZERO, h->hd);
-        go.amax_a = am + AMAX_D; go.amax_b = am + AMAX_U; go.amax_out = am + AMAX_O;
+        go.row_inv = inv_d; go.amax_b = am + AMAX_U; go.row_amax_out = amax_o;
         CU(launch_tc_gemm(maps, go, h->num_sms, s));
-        CU(launch_split16(split16_args(O, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, 1.f, am + AMAX_O), s));
+        CU(launch_split16(split16_args(O, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, 1.f, amax_o, SplitBatch(), nullptr,
+                                       nullptr, inv_o), s));
         // P = alpha * O U  (B operand rows are rows of U^T)
         if (!make_tc_maps(&maps, Aop, UTop, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
         TcGemmArgs gp = tc_args(h->D, n, n, n, n, alpha, 0.f, TC_P, TC_MASK_STRICT_ZERO, h->hd);
-        gp.amax_a = am + AMAX_O; gp.amax_b = am + AMAX_U; gp.amax_out = am + AMAX_P;
+        gp.row_inv = inv_o; gp.amax_b = am + AMAX_U; gp.amax_out = am + AMAX_P;
         CU(launch_tc_gemm(maps, gp, h->num_sms, s));
         // P^T for the lazy-batch updates of gptaq_quantize, over the copy of U that is no longer needed
         CU(launch_split16(split16_args(h->D, n, U16, U16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P), s));
@@ -1361,8 +1368,9 @@ gptaq_status_t gptaq_build_P_rowwise(gptaq_handle_t h, float alpha, gptaq_stream
         __half *UT16 = reinterpret_cast<__half *>(h->ws + wl.s_off[0]);
         __half *PT16 = reinterpret_cast<__half *>(h->ws + wl.s_off[1]);
         unsigned *am = h->hd->tc_amax;
-        CU(cudaMemsetAsync(am + AMAX_U, 0, 4 * sizeof(unsigned), s));
-        CU(launch_absmax({h->H, n, n, n, SPLIT_UPPER, 1.f, am + AMAX_U}, {h->D, n, n, n, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P}, h->num_sms, s));
+        CU(cudaMemsetAsync(am + AMAX_U, 0, 2 * sizeof(unsigned), s));
+        CU(launch_absmax({h->H, n, n, n, SPLIT_UPPER, 1.f, am + AMAX_U, nullptr, nullptr},
+                         {h->D, n, n, n, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P, nullptr, nullptr}, h->num_sms, s));
         const Split16Args split_p = split16_args(h->D, n, PT16, PT16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P);
         CU(launch_split16(split16_args(h->H, n, UT16, UT16 + nn, ldt, n, n, true, SPLIT_UPPER, 1.f, am + AMAX_U), s, &split_p));
         h->launches += 2;

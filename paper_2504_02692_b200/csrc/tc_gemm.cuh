@@ -82,6 +82,7 @@ struct TcGemmArgs {
     const unsigned *amax_a, *amax_b;
     const float *row_inv;            // operands with one scale per row of A: 1 / scale of row i (amax_a null)
     unsigned *amax_out;              // if set: receives (atomicMax) the bit pattern of max |C| over what is stored
+    unsigned *row_amax_out;          // ... [M]: of max |C| over what is stored of each row (one batch entry)
     int c_tma;                       // beta == 1, one batch entry: C += through bulk tensor reductions (mapC)
     int diag_off;                    // C is a block of columns of a square matrix: its column j is column j + diag_off there
     // Tile scheduler: CTA b starts with tile b; further tile numbers come from a counter in global memory.  A launch draws
@@ -384,6 +385,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
             if (lane == 0) mbar_arrive(sempty_bar(slot));
             if (t < 0) break;
             tc_decode<TBN>(a, t, ti, BK);
+            const int row = ti.i0 + quarter * 32 + lane;           // within the batch entry
+            // (read before the products are waited for)
+            const float alpha = a.alpha * (a.row_inv && row < ti.Mz ? op_scale * a.row_inv[(long long)ti.z * a.M + row] : op_scale);
 #pragma unroll
             for (int i = 0; i < TBN / 2; ++i) acc[i] = 0.f;
             if (ti.work) {
@@ -407,7 +411,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                 }
                 if (!a.c_tma && !ok) break;
             }
-            const int row = ti.i0 + quarter * 32 + lane;           // within the batch entry
             const int col0 = ti.j0 + half * (TBN / 2);
             if (a.c_tma) {
                 // C += alpha * acc through shared memory and bulk tensor reductions: the four warps of a
@@ -415,8 +418,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                 // like the tensor map's 128-byte mode), one thread hands it to the TMA unit.  Rows and
                 // columns beyond the matrix are clipped by the tensor map.
                 if (named_bar_any(1 + half, 128, !ok)) { ok = false; break; }       // a wait gave up: all leave together
-                float alpha = a.alpha;
-                alpha *= (a.row_inv && row < ti.Mz) ? op_scale * a.row_inv[row] : op_scale;
                 const bool issuer = quarter == 2 && lane == 0;                       // first warp of the half
                 const int r_in = quarter * 32 + lane;
                 const uint32_t box = stg0 + half * TC_STG_BOX_BYTES;
@@ -448,9 +449,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
             if (row >= ti.Mz) continue;
             float *cp = a.C + (long long)ti.z * a.c_bstride + (long long)row * a.ldc + col0;
             const float beta = a.beta;
-            float alpha = a.alpha;
-            alpha *= a.row_inv ? op_scale * a.row_inv[(long long)ti.z * a.M + row] : op_scale;
             const bool vec_ok = (reinterpret_cast<uintptr_t>(cp) & 15) == 0;
+            float row_max = 0.f;
 #pragma unroll
             for (int q = 0; q < TBN / 2 / 4; ++q) {
                 const int c = col0 + 4 * q;
@@ -462,9 +462,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
 #pragma unroll
                     for (int e = 0; e < 4; ++e) if (c + e <= row) v[e] = 0.f;
                 }
-                if (a.amax_out) {
+                if (a.amax_out || a.row_amax_out) {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) if (c + e < ti.Nz) out_max = fmaxf(out_max, fabsf(v[e]));
+                    for (int e = 0; e < 4; ++e) if (c + e < ti.Nz) row_max = fmaxf(row_max, fabsf(v[e]));
                 }
                 const bool keep_all = a.mask != TC_MASK_UPPER_KEEP || c + a.diag_off >= row;
                 if (vec_ok && c + 3 < ti.Nz && keep_all) {
@@ -490,6 +490,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
                     }
                 }
             }
+            out_max = fmaxf(out_max, row_max);
+            if (a.row_amax_out && row_max > 0.f) atomicMax(a.row_amax_out + row, __float_as_uint(row_max));
         }
         if (a.c_tma) bulk_wait0();          // (only the issuing threads have groups outstanding)
         if (a.amax_out) {
@@ -512,8 +514,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
 // FP16 operand preparation.  absmax_kernel (a CTA per row, strided) records max |scale * src| over the
 // (masked) region as a float bit pattern (atomicMax on the bits orders non-negative floats);
 // split16_kernel then writes
-// hi = fp16(s x), lo = fp16(s x - hi), x = scale * src, s = split_scale(recorded maximum), optionally transposed and
-// masked to the (strictly) upper triangle of the source (elements outside are written as zero), tile by tile through
+// hi = fp16(s x), lo = fp16(s x - hi), x = scale * src, s = split_scale(recorded maximum), of the matrix or (plain form
+// only) of the element's row, optionally transposed and masked to the (strictly) upper triangle of the source (elements outside are written as zero), tile by tile through
 // shared memory.  The slot has to be zeroed before the first absmax_kernel into it; several matrices that share a scale
 // are reduced into the same slot.
 //   src element (r, c), r < rows, c < cols, at src[r * lds + c];
@@ -521,7 +523,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
 // ---------------------------------------------------------------------------
 enum SplitMask { SPLIT_ALL = 0, SPLIT_UPPER = 1, SPLIT_STRICT_UPPER = 2 };
 
-struct AbsmaxArgs { const float *src; long long lds; int rows, cols, mask; float scale; unsigned *slot; };
+// slot: one maximum of the whole region.  row_slot (instead): one per row, and row_zero[row] is set to zero on the way.
+struct AbsmaxArgs { const float *src; long long lds; int rows, cols, mask; float scale; unsigned *slot, *row_slot, *row_zero; };
 // (two matrices per launch, blockIdx.y)
 __global__ void __launch_bounds__(256) absmax_kernel(AbsmaxArgs a0, AbsmaxArgs a1) {
     const AbsmaxArgs &a = blockIdx.y ? a1 : a0;
@@ -530,13 +533,16 @@ __global__ void __launch_bounds__(256) absmax_kernel(AbsmaxArgs a0, AbsmaxArgs a
     const int rows = a.rows, cols = a.cols, mask = a.mask;
     const float scale = a.scale;
     unsigned *slot = a.slot;
-    __shared__ float red[8];
+    constexpr int BATCH = 32;                        // rows between two barriers, with a maximum per row
+    __shared__ float red[BATCH][8];
     float m = 0.f;
+    int kept = 0;
     const bool vec = (lds & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
     for (int r = blockIdx.x; r < rows; r += gridDim.x) {
         const int cb = mask == SPLIT_ALL ? 0 : (mask == SPLIT_UPPER ? r : r + 1);     // first column kept
         const float *row = src + (long long)r * lds;
         if (vec) {
+#pragma unroll 4
             for (int c4 = (cb >> 2) + threadIdx.x; 4 * c4 < cols; c4 += 256) {
                 const int c = 4 * c4;
                 float v[4] = {0.f, 0.f, 0.f, 0.f};
@@ -552,14 +558,35 @@ __global__ void __launch_bounds__(256) absmax_kernel(AbsmaxArgs a0, AbsmaxArgs a
         } else {
             for (int c = cb + threadIdx.x; c < cols; c += 256) m = fmaxf(m, fabsf(row[c]));
         }
+        if (a.row_slot) {
+            m *= fabsf(scale);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if ((threadIdx.x & 31) == 0) red[kept][threadIdx.x >> 5] = m;
+            m = 0.f;
+            ++kept;
+            if (kept == BATCH || r + (int)gridDim.x >= rows) {
+                __syncthreads();
+                if ((int)threadIdx.x < kept) {
+                    float x = 0.f;
+                    for (int w = 0; w < 8; ++w) x = fmaxf(x, red[threadIdx.x][w]);
+                    const int row_of = r - (kept - 1 - (int)threadIdx.x) * (int)gridDim.x;
+                    a.row_slot[row_of] = __float_as_uint(x);
+                    a.row_zero[row_of] = 0u;
+                }
+                __syncthreads();
+                kept = 0;
+            }
+        }
     }
+    if (a.row_slot) return;
     m *= fabsf(scale);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    if ((threadIdx.x & 31) == 0) red[0][threadIdx.x >> 5] = m;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) m = fmaxf(m, red[w]);
+        for (int w = 1; w < 8; ++w) m = fmaxf(m, red[0][w]);
         if (m > 0.f) atomicMax(slot, __float_as_uint(m));
     }
 }
@@ -570,8 +597,9 @@ struct Split16Args {
     int rows, cols, rows_last, cols_last, nbatch;      // blockIdx.z walks batch entries
     int transpose, mask;       // transpose 2: both forms, the plain one to (hi, lo), the transposed one to (hi_t, lo_t)
     float scale;
-    const unsigned *amax;
+    const unsigned *amax;      // maximum of the matrix; with row_inv: [rows], of each row
     __half *hi_t, *lo_t;
+    float *row_inv;            // nullptr, or (transpose 0, one batch entry) receives 1 / scale of each row
 };
 
 __device__ __forceinline__ void split16_pack(const float (&x)[4], uint2 &hi, uint2 &lo) {
@@ -603,14 +631,15 @@ __global__ void __launch_bounds__(256) split16_kernel(Split16Args a, Split16Args
         a.lo += (long long)z * a.dst_bstride;
         if (a.transpose == 2) { a.hi_t += (long long)z * a.dst_bstride; a.lo_t += (long long)z * a.dst_bstride; }
     }
-    const float s = a.scale * split_scale(__uint_as_float(*a.amax));
     const int tq = threadIdx.x & 15, ty = threadIdx.x >> 4;        // 16 quads x 16 rows
     // all four loads of the thread first (a store in between would serialise them), none for quads that
     // the mask empties
     float xs[4][4];
+    unsigned am[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int r = r0 + ty + 16 * i, c = c0 + 4 * tq;
+        am[i] = a.amax[a.row_inv && r < a.rows ? r : 0];
 #pragma unroll
         for (int e = 0; e < 4; ++e) xs[i][e] = 0.f;
         const bool any = a.mask == SPLIT_ALL || (a.mask == SPLIT_UPPER ? c + 3 >= r : c + 3 > r);
@@ -629,6 +658,8 @@ __global__ void __launch_bounds__(256) split16_kernel(Split16Args a, Split16Args
         const int rr = ty + 16 * i;
         const int r = r0 + rr, c = c0 + 4 * tq;
         float x[4];
+        const float sr = split_scale_bits(am[i]), s = a.scale * sr;
+        if (a.row_inv && c == 0 && r < a.rows) a.row_inv[r] = 1.f / sr;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const bool keep = a.mask == SPLIT_ALL || (a.mask == SPLIT_UPPER ? c + e >= r : c + e > r);

@@ -951,3 +951,29 @@ def test_captured_quantize_can_be_replayed(n, m, B, group):
 def test_captured_solve_can_be_replayed(n, m, B, group):
     """Launches that overlap their predecessors, and three streams, in one graph."""
     _replays_match(n, m, B, group, True)
+
+
+@pytest.mark.parametrize("n", [516, 520, 1036])
+def test_correction_matrix_rows_of_inputs_in_small_units(n):
+    """Inputs whose units span a factor of 1e4: every row of P is as good as its own size, not only that of the largest.
+    From the device's own U and dXX^T: two products after one another, of factors good to 2^-22 each."""
+    torch.manual_seed(n)
+    tokens, alpha = 2 * n, 0.5
+    unit = torch.logspace(-2, 2, n, device="cuda")[torch.randperm(n, device="cuda")]
+    X = torch.randn(tokens, n, device="cuda") * unit
+    Xfp = X + 0.05 * torch.randn(tokens, n, device="cuda") * unit
+    st = g.LayerState(n, 1, tokens, 32, "cuda")
+    try:
+        g.gptaq_accumulate(st.handle, X, Xfp)
+        D = np.triu(st.D().cpu().numpy().astype(np.float64), 1) / tokens
+        g.gptaq_factor(st.handle, 0.01)
+        g.gptaq_build_P(st.handle, alpha)
+        U = np.triu(st.H().cpu().numpy().astype(np.float64))
+        P = np.triu(st.D().cpu().numpy().astype(np.float64), 1)
+        assert g.gptaq_sync_status(st.handle)[0] == g.GPTAQ_OK
+    finally:
+        st.close()
+    ref = alpha * np.triu(np.triu(D @ U.T, 1) @ U, 1)
+    size = alpha * np.triu(np.triu(abs(D) @ abs(U).T, 1) @ abs(U), 1)
+    err = np.linalg.norm(P - ref, axis=1)[:-1] / np.linalg.norm(size, axis=1)[:-1]        # (the last row is empty)
+    assert err.max() <= 2.0 ** -20, err.max()
