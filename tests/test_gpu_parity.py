@@ -79,8 +79,8 @@ def test_super_panels_and_super_blocks(n, m, B, group, bits):
 
 
 def test_no_damping_keeps_the_unbounded_operand_form():
-    """damp = 0: nothing bounds the entries of the inverse factor in advance, so the block inverse runs with
-    TF32-split operands (no range limits) while the other products keep their fp16-split form."""
+    """damp = 0: nothing bounds the entries of the factor and of its inverse in advance, so rank updates and block inverse are
+    plain float32 products, while P and the lazy-batch updates keep their fp16-split form."""
     cfg = wl.scaled(wl.CONFIGS["cfg2"], name="nodamp", n=768, m=40, batch_tokens=4096, n_batches=2, damp=0.0,
                     outlier_channels=6)
     out = hp.check_layer(cfg, wl.make_weight(cfg), batches_of(cfg))
@@ -977,3 +977,30 @@ def test_correction_matrix_rows_of_inputs_in_small_units(n):
     size = alpha * np.triu(np.triu(abs(D) @ abs(U).T, 1) @ abs(U), 1)
     err = np.linalg.norm(P - ref, axis=1)[:-1] / np.linalg.norm(size, axis=1)[:-1]        # (the last row is empty)
     assert err.max() <= 2.0 ** -20, err.max()
+
+
+@pytest.mark.parametrize("n", [516, 1024, 2052])
+def test_factor_without_damping_of_inputs_in_small_units(n):
+    """Inputs whose units span a factor of 2^26 and no damping: rows of R span as much.  Bound and comparison as in
+    test_factor_panels, for float32 products (2^-24 each) and with the units taken out of the condition number: a scaling of
+    the inputs by powers of two changes no rounding of a float32 factorisation, only the columns of U."""
+    torch.manual_seed(n)
+    unit = 2.0 ** torch.randint(-13, 14, (n,), device="cuda")
+    X = torch.randn(3 * n, n, device="cuda") * unit
+    st = g.LayerState(n, 1, 3 * n, 32, "cuda")
+    try:
+        g.gptaq_set_stats_precision(st.handle, g.GPTAQ_STATS_FP32)
+        g.gptaq_accumulate(st.handle, X, X)
+        H = st.H().cpu().numpy().astype(np.float64)
+        g.gptaq_factor(st.handle, 0.0)
+        U = np.triu(st.H().cpu().numpy().astype(np.float64))
+        assert g.gptaq_sync_status(st.handle)[0] == g.GPTAQ_OK
+    finally:
+        st.close()
+    ref, _ = orc.factor(np.triu(H) + np.triu(H, 1).T, 3 * n, 0.0)
+    u = unit.cpu().numpy()
+    U, ref = U * u, ref * u
+    sv = np.linalg.svd(ref, compute_uv=False)
+    bound = (sv[0] / sv[-1]) ** 2 * np.sqrt(n) * 2.0 ** -24
+    err = np.linalg.norm(U - ref, axis=1) / np.linalg.norm(ref, axis=1)
+    assert err.max() <= bound, (err.max(), bound)
