@@ -52,6 +52,7 @@ struct gptaq_ctx {
     int64_t launches;
     int stats_precision;   // GPTAQ_STATS_*
     bool tensor;           // float32-grade tensor-core GEMMs (fp16-split operands) for factor / P / trailing update
+    bool split;            // ... for P / trailing update of the current factor (set by gptaq_factor)
     int terms;             // GPTAQ_TERM_* switches of gptaq_quantize
     bool static_groups;    // group grids from the original weights, per group of the caller's columns
     int clip_steps; float clip_min;   // clipping-range search of the grids
@@ -1281,6 +1282,10 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         p2.batchN_last = tail;
         OK(gemm(h, p2, false, true, s));
     }
+    // Without damping the columns of U go with the reciprocal units of the inputs, and in the contractions of P and of the
+    // lazy-batch update the parts' range (2^-39 of the largest entry) is off by the ratio of the units.  Widths that are
+    // 4 mod 8 take plain float32 then; the others keep the split operands at any damping.
+    h->split = h->tensor && (damp > 0.f || n % 8 == 0);
     h->stage = STAGE_FACTORED;
     return GPTAQ_OK;
 }
@@ -1299,7 +1304,7 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
     const int n = (int)h->n;
     WsLayout wl = ws_layout(h->n, 0);
     float *O = reinterpret_cast<float *>(h->ws + wl.t_off);
-    if (h->tensor) {
+    if (h->split) {
         // Every operand is scaled by a power of two into the fp16 range, so its largest magnitude is recorded first (by a
         // reduction kernel for U and dXX^T, by the producing GEMM's epilogue for O and P).  dXX^T and O have a scale per
         // row: a row goes with the unit of the input that it belongs to, and with one scale for the whole matrix the rows of
@@ -1368,7 +1373,7 @@ gptaq_status_t gptaq_build_P_rowwise(gptaq_handle_t h, float alpha, gptaq_stream
     LAUNCHED();
     // the operand copies that gptaq_quantize reads, as gptaq_build_P leaves them
     WsLayout wl = ws_layout(h->n, 0);
-    if (h->tensor) {
+    if (h->split) {
         const int64_t ldt = split_pitch(n);
         const size_t nn = (size_t)n * ldt;
         __half *UT16 = reinterpret_cast<__half *>(h->ws + wl.s_off[0]);
@@ -1409,7 +1414,7 @@ gptaq_status_t gptaq_quantize(gptaq_handle_t h, void *d_W, int w_dtype, int64_t 
     t.side = h->gemm_stream; t.fork = h->conv_done[0]; t.join = h->gemm_done[0];
     // fp16-split updates, plain float32 products otherwise
     // (groups of fewer than 32 columns update block by block, and blocks of 32 columns are no whole K-block of 64)
-    const bool f16 = h->tensor && ((blocksize % 64) == 0 || group <= 0 || (group % 32) == 0 || h->static_groups);
+    const bool f16 = h->split && ((blocksize % 64) == 0 || group <= 0 || (group % 32) == 0 || h->static_groups);
     if (f16) {
         t.ldt = split_pitch(h->n);
         t.UT16 = reinterpret_cast<const __half *>(h->ws + wl.s_off[0]);

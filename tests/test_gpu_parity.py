@@ -1004,3 +1004,38 @@ def test_factor_without_damping_of_inputs_in_small_units(n):
     bound = (sv[0] / sv[-1]) ** 2 * np.sqrt(n) * 2.0 ** -24
     err = np.linalg.norm(U - ref, axis=1) / np.linalg.norm(ref, axis=1)
     assert err.max() <= bound, (err.max(), bound)
+
+
+def test_solve_without_damping_of_inputs_in_small_units():
+    """The same through P and the loop at a width that is a multiple of 4 only: P from the device's own U and dXX^T as in
+    test_correction_matrix_rows_of_inputs_in_small_units, the loop replayed from the device's own U and P with the bounds of
+    the parity tests."""
+    n, m, alpha = 516, 40, 0.25
+    torch.manual_seed(n)
+    unit = 2.0 ** torch.randint(-10, 11, (n,), device="cuda")
+    X = torch.randn(3 * n, n, device="cuda") * unit
+    Xfp = X + 0.05 * torch.randn(3 * n, n, device="cuda") * unit
+    W = 0.02 * torch.randn(m, n, device="cuda")
+    G = hp.n_groups(n, 32)
+    codes = torch.empty((m, n), dtype=torch.uint8, device="cuda")
+    sc, zp = torch.empty((m, G), device="cuda"), torch.empty((m, G), device="cuda")
+    st = g.LayerState(n, m, 3 * n, 128, "cuda")
+    try:
+        g.gptaq_set_stats_precision(st.handle, g.GPTAQ_STATS_FP32)
+        g.gptaq_accumulate(st.handle, X, Xfp)
+        D = np.triu(st.D().cpu().numpy().astype(np.float64), 1) / (3 * n)
+        g.gptaq_factor(st.handle, 0.0)
+        g.gptaq_build_P(st.handle, alpha)
+        U = np.triu(st.H().cpu().numpy().astype(np.float64))
+        P = np.triu(st.D().cpu().numpy().astype(np.float64), 1)
+        g.gptaq_quantize(st.handle, W.clone(), 4, 32, True, 128, codes, sc, zp)
+        assert g.gptaq_sync_status(st.handle)[0] == g.GPTAQ_OK
+    finally:
+        st.close()
+    ref = alpha * np.triu(np.triu(D @ U.T, 1) @ U, 1)
+    size = alpha * np.triu(np.triu(abs(D) @ abs(U).T, 1) @ abs(U), 1)
+    err = np.linalg.norm(P - ref, axis=1)[:-1] / np.linalg.norm(size, axis=1)[:-1]
+    assert err.max() <= 2.0 ** -20, err.max()
+    rep = orc.follow(W.cpu().numpy().astype(np.float64), U, P, np.zeros(n, bool), 4, 32, True, codes.cpu().numpy(),
+                     sc.cpu().numpy().astype(np.float64), zp.cpu().numpy().astype(np.float64), band=hp.TOL_FLIP_BAND)
+    assert rep.disallowed == 0 and rep.allowed <= hp.TOL_FLIP_RATE * rep.total and rep.grid_rel_err <= hp.TOL_GRID, rep
