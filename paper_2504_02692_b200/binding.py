@@ -109,10 +109,16 @@ def _ptr(t) -> int | None:
     return int(t)
 
 
+# The current stream's handle without building a Stream object (3 us, as much as a launch).  Not a documented function of
+# torch: where it is missing, the documented way is taken.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int | None:
     if stream is None:
-        # the current stream's handle without building a Stream object (3 us, as much as a launch)
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) or None
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device()) or None
+        return torch.cuda.current_stream().cuda_stream or None
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream or None
     return int(stream) or None

@@ -64,3 +64,21 @@ def test_product_path_has_no_cpu_fallback():
     import sys
     src = open(os.path.join(ROOT, "paper_2504_02692_b200", "binding.py")).read()
     assert "oracle" not in src.replace("no CPU fallback", "")
+
+
+@pytest.mark.parametrize("raw", [True, False])
+def test_the_current_stream_without_torch_s_undocumented_function(monkeypatch, raw):
+    """The handle of torch's current stream is found whether or not this torch has the short way to it (0 is the default
+    stream: no handle)."""
+    from paper_2504_02692_b200 import binding
+
+    class Stream:
+        cuda_stream = 0x1230
+
+    monkeypatch.setattr(binding.torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(binding.torch.cuda, "current_stream", lambda: Stream)
+    monkeypatch.setattr(binding, "_raw_stream", (lambda device: Stream.cuda_stream if device == 3 else -1) if raw else None)
+    assert binding._stream(None) == 0x1230
+    Stream.cuda_stream = 0
+    assert binding._stream(None) is None
+    assert binding._stream(0x50) == 0x50
