@@ -548,8 +548,8 @@ def test_device_side_conditions_are_reported_not_trapped():
     assert status == g.GPTAQ_ERR_NONFINITE
     st.close()
     # a NaN / Inf in the LAST column of W propagates nowhere and quantizes to a finite code: it is
-    # reported from the loaded value, with its row, by both column kernels (full blocks with grids per
-    # 32 columns take column_block_kernel, groups of 8 take column_loop_kernel)
+    # reported from its value before the rounding, with its row, by both column kernels (groups of 8 take
+    # column_loop_kernel, the others quant_block_kernel)
     for group, bad_value, row in ((32, float("nan"), 2), (8, float("inf"), 1), (0, float("nan"), 3)):
         st = g.LayerState(n, 4, 256, 32)
         h = st.handle
@@ -603,16 +603,23 @@ def test_dead_inputs():
 def _stats_only(cfg, bt, precision, scale=1.0):
     st = g.LayerState(cfg.n, 8, cfg.batch_tokens, cfg.blocksize)
     g.gptaq_set_stats_precision(st.handle, precision)
+    g.gptaq_set_kernel_timing(st.handle, True)
     for X, Xfp in bt:
         g.gptaq_accumulate(st.handle, (X * scale).cuda(), (Xfp * scale).cuda())
     assert g.gptaq_sync_status(st.handle)[0] == g.GPTAQ_OK
     H = st.H().cpu().numpy().astype(np.float64)
     D = st.D().cpu().numpy().astype(np.float64)
+    # which kernel ran: the tensor-core one, once per batch at least, beyond 2^25 of tokens * n^2
+    _, launches = g.gptaq_stats_kernel_time(st.handle)
+    tensor = precision != g.GPTAQ_STATS_FP32 and cfg.batch_tokens * cfg.n ** 2 > 2 ** 25
+    assert launches >= len(bt) if tensor else launches == 0
     st.close()
     return H, D
 
 
-@pytest.mark.parametrize("n,tokens,nb", [(256, 64, 1), (384, 1000, 2), (1024, 4112, 2), (2052, 777, 1)])
+# (a small batch that takes float32 products whatever the precision; a single K-block of 64, padded and whole; several)
+@pytest.mark.parametrize("n,tokens,nb", [(256, 64, 1), (1024, 33, 2), (1024, 64, 1), (384, 1000, 2), (1024, 4112, 2),
+                                         (2052, 777, 1)])
 def test_tensor_core_statistics_against_oracle(n, tokens, nb):
     """Tensor-core sums vs float64.  Elementwise error relative to sqrt(H_ii H_jj) is bounded by
     the rounding of the operands: 2^-11 per fp16 factor in the single-term mode; the split mode
@@ -716,9 +723,10 @@ def test_small_float32_products(n, m, tokens, group, B):
 @pytest.mark.parametrize("n", [
     100,           # less than one panel
     129, 257,      # one column beyond a panel: no aligned rows
-    516,           # the next diagonal block is not factored ahead (width a multiple of 4 only)
-    520, 1024,     # one super-panel, its last panel ragged / full
+    516, 520,      # one super-panel on split operands, its last panel ragged; row pitch of their copies padded / not
+    1024,          # ... its last panel full
     1032, 1160,    # a second super-panel of 8 columns / of one panel and 8 columns
+    1153,          # the same in float32 (odd width): no block is factored ahead, the inverse beside the panels all the same
     2504,          # more rows than one warp per 4 of them can take at once
 ])
 def test_factor_panels(n):
