@@ -53,7 +53,8 @@ typedef enum {
     GPTAQ_ERR_BAD_STATE = 2,    /* call out of order */
     GPTAQ_ERR_WORKSPACE = 3,    /* state / workspace / staging buffer too small */
     GPTAQ_ERR_NOT_SPD = 4,      /* device: a pivot of the damped H was <= 0; info = its index */
-    GPTAQ_ERR_NONFINITE = 5,    /* device: NaN/Inf met in H or W; info = row or column index */
+    GPTAQ_ERR_NONFINITE = 5,    /* device: NaN/Inf met in H, in W or in what a column of W receives through U and P;
+                                   info = column of H or row of W */
     GPTAQ_ERR_TIMEOUT = 6,      /* device: a bounded wait ran out; info = where */
     GPTAQ_ERR_UNSUPPORTED = 7,  /* argument combination outside the supported set */
     GPTAQ_ERR_CUDA = 8          /* a CUDA runtime call failed; see gptaq_last_cuda_error */
@@ -64,7 +65,8 @@ enum { GPTAQ_W_FP32 = 0, GPTAQ_W_BF16 = 1 };
 /* Arithmetic of the statistics (Algorithm 1, first step).  In the two tensor-core modes X and
  * X~ - X (the difference taken in float32 first) are rounded to fp16, scaled by a power of two
  * if the batch would leave the fp16 range, and multiplied by tcgen05 MMAs with float32
- * accumulation; they apply for n >= 256 and for n = 128, other small layers always take the float32 path.
+ * accumulation; they apply for n >= 256 and for n = 128, other small layers always take the float32 path,
+ * and so do small batches of any layer (tokens * n^2 <= 2^25), whatever the mode asked for.
  * GPTAQ_STATS_FP16_SPLIT_TENSOR (default): H additionally carries the rounding remainder of X
  *   as a second fp16 term (H = hi hi^T + hi lo^T + lo hi^T, about 22 significant bits), so that
  *   the factor U keeps its accuracy even with few tokens per input channel.

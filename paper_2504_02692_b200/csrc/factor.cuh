@@ -325,8 +325,8 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
             if (tid < 64) solve_rows(o, o1, tid);
             named_bar_arrive(2, DF_CHAIN + DF_HELP);
             named_bar_sync(3, DF_CHAIN);
-            // the next sub-block, less their contribution: 2 x 4 outputs of the upper triangle per thread, mirrored (n = 2052:
-            // 770 us in all with 4 x 4 outputs in 36 threads, 760)
+            // the next sub-block, less their contribution: 2 x 4 outputs of the upper triangle per thread, mirrored (4 x 4 in
+            // 36 threads: 1 % more in all)
             {
                 const int i = o1 + 2 * (tid >> 3), j = o1 + 4 * (tid & 7);
                 if (j + 3 >= i) {

@@ -1,5 +1,5 @@
-// Small kernels of the GPTAQ layer solve: damping, the diagonal-block reverse
-// Cholesky, the per-column quantize-and-propagate loop, and helpers.
+// Small kernels of the GPTAQ layer solve: damping, grids, the column loop for groups of fewer than 32 columns, the row-by-row
+// form of P, column orders and copies.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>

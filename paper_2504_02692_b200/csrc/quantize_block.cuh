@@ -20,7 +20,8 @@
 // shuffled copies that the other lanes need are off the chain -- and a shuffle more at every 8th column.  It takes 110
 // (alone) to 200 cycles (beside the near warps of a block's first step), though: shared memory returns 128 bytes a cycle,
 // and a column's rows of U and P are 64 such words for the chain's four warps and up to 96 for the near warps.
-// A launch of 512 columns takes 80 us: 13 % of it the copies and products between blocks, 8 % filling the slab.
+// A launch of 512 columns takes 75 to 80 us, 138k cycles: 8k of it fill the slab, 6k to 12k are the products between blocks,
+// 6k the group grids, the rest the 64 pieces of 8 columns.
 #pragma once
 #include "tc_gemm.cuh"
 
@@ -192,7 +193,7 @@ __device__ __forceinline__ void clip_pass(const float *w, int n, float lo, float
 
 // Least squared rounding error of one row's group among candidates k0, k0 + stride, ..: ten per pass over the weights while
 // more than four are left, else four (four throughout and clamped by minimum and maximum, 4096 x 4096 with 80 candidates:
-// 1541 us a call; ten per pass 1515; clamped by saturation 1419).
+// 1541 us a call, now 1419).
 __device__ __forceinline__ void clip_search(const float *w, int n, float lo, float hi, int bits, int sym, int steps, float clip_min,
                                             int k0, int stride, float &best, int &kbest) {
     best = INFINITY; kbest = 0;
@@ -307,8 +308,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
     }
-    // the slab and the first rows of U and P all in flight at once (in batches through registers the prologue took 6 us
-    // of a launch, now 3)
+    // the slab and the first rows of U and P all in flight at once (8k cycles; in batches through registers twice that)
     const int cq = FAR ? nblk * (QB_W / 4) : B / 4;                // quads per row, padded columns included
     const bool wvec = (a.ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(a.W) & 15) == 0;       // (i0 is a multiple of 32)
     // a thread: four columns of every RSTEP-th row

@@ -6,8 +6,8 @@
 // per factor, which is what the factorisation, the correction matrix and the propagation of
 // quantization errors need (single TF32/fp16 products flip integer codes).  TMA loads the
 // 128-row (A) and up to 256-row (B) tiles of both parts, one 128-byte row piece per K-block, into
-// 128-byte-swizzled shared memory; one thread issues the MMAs into one of two 128 x 256
-// accumulators; eight epilogue warps drain them.  Accumulation chains in tensor memory are
+// 128-byte-swizzled shared memory; one thread issues the MMAs into one of two accumulators of a
+// tile; eight epilogue warps drain them.  Accumulation chains in tensor memory are
 // cut every TCHUNK K-blocks and added into float32 registers with round-to-nearest (the
 // tensor core truncates its accumulator).  "C += ..." results leave through shared memory
 // as bulk tensor reductions (one request per 128 x 32 box) where C qualifies for a tensor
@@ -18,11 +18,12 @@
 // the non-zero part of triangular operands, a B operand that switches to a second matrix
 // after k_split ([U ; P] of the lazy-batch update), and masked stores.
 //
-// The operands are hi = fp16(s x), lo = fp16(s x - hi) with a power-of-two scale s per operand that puts the largest
-// magnitude at 2^14 (split16_kernel; the scale is recomputed from the recorded maximum wherever it is needed), 64
+// The operands are hi = fp16(s x), lo = fp16(s x - hi) with a power-of-two scale s per operand or per row of A that puts the
+// largest magnitude at 2^14 (split16_kernel; the scale is recomputed from the recorded maximum wherever it is needed), 64
 // contraction steps per 128-byte row and tcgen05.mma.kind::f16: half the operand bytes and twice the MMA rate of TF32
-// parts for the same 22 bits.  (Widths that are multiples of 4 only used to take TF32 parts, because a TMA row pitch has to
-// be a multiple of 16 bytes; the fp16 copies have a padded pitch instead.  777 x 2052: 2142 -> 1673 us.)
+// parts for the same 22 bits, down to 2^-17 of the largest magnitude (below it an absolute 2^-39 of that; TF32 parts have no
+// such limit, so a product whose operands nothing bounds is plain float32).  The row pitch of the copies is padded to a
+// multiple of 16 bytes.
 //
 // Every wait on an mbarrier is bounded; see umma_gemm.cuh.
 #pragma once
@@ -224,7 +225,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
     uint8_t *aligned = smem_raw + (base - raw);
     const uint32_t stg0 = base + TSTAGES * TSTAGE_BYTES;
     const uint32_t bar0 = stg0 + TC_STG_BYTES;
-    // barrier slots (8 bytes each): full[2], empty[2], tfull[2], tempty[2]; then tmem slot, abort flag
+    // barrier slots (8 bytes each): full[TSTAGES], empty[TSTAGES], tfull[2], tempty[2]; then tmem slot, abort flag
     auto full_bar = [&](int s) { return bar0 + 8u * s; };
     auto empty_bar = [&](int s) { return bar0 + 8u * (TSTAGES + s); };
     auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * TSTAGES + b); };
@@ -368,7 +369,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapAhi, const __grid_constant
     } else {
         // ------------------------------------------------------------ epilogue (warps 2..9)
         const int quarter = warp & 3;                 // TMEM lanes 32 * quarter .. + 31
-        const int half = (warp - 2) >> 2;             // columns [128 * half, 128 * half + 128)
+        const int half = (warp - 2) >> 2;             // columns [TBN / 2 * half, TBN / 2 * half + TBN / 2)
         uint32_t ccount = 0;
         bool ok = true;
         float acc[TBN / 2];
