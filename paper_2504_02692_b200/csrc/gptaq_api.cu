@@ -67,7 +67,7 @@ struct gptaq_ctx {
     bool relayout;         // the operand buffers change size: wait for the products in flight first
     int next_buf;
     // tensor maps of a buffer's operands (they lie in the workspace: only the padded token count and the layout matter)
-    struct StatsMaps { CUtensorMap x, d, xlo, dlo; int64_t kp, chunk; int narr; } stats_maps[2];
+    struct StatsMaps { CUtensorMap x, d, xlo, dlo, h, dxx, slots; int64_t kp, chunk; int narr; bool c_tma; } stats_maps[2];
     // partial sums of the cut tiles of the statistics products wait in the workspace (fix_args.scratch) until
     // the sums are needed or the cut changes; fix_pending: they have not been added to H / dXX^T yet
     bool fix_pending;
@@ -448,6 +448,11 @@ gptaq_status_t accumulate_tc(gptaq_ctx *h, const float *X, const float *Xfp, int
                 h->cuda_error = "cuTensorMapEncodeTiled failed";
                 return GPTAQ_ERR_CUDA;
             }
+            // the targets of the sums: bulk reductions where the rows are 16-byte multiples (scattered reductions otherwise)
+            float *scratch = reinterpret_cast<float *>(h->ws + 2 * buf_bytes);
+            mp.c_tma = n % 4 == 0 && make_c_map(&mp.h, h->H, n, n, n) && make_c_map(&mp.dxx, h->D, n, n, n) &&
+                       make_c_map(&mp.slots, scratch, (int64_t)h->num_sms * UBM, UBN, UBN);
+            if (!mp.c_tma) mp.h = mp.dxx = mp.slots = mp.x;         // (placeholders, not dereferenced)
             mp.kp = kp; mp.chunk = chunk; mp.narr = narr;
         }
         StatsGemmArgs ga;
@@ -485,6 +490,7 @@ gptaq_status_t accumulate_tc(gptaq_ctx *h, const float *X, const float *Xfp, int
         // scratch behind the two operand buffers (one partial 128 x 256 tile per CTA at most; the products
         // run one after the other on the internal stream, so one scratch serves both buffers)
         ga.scratch = reinterpret_cast<float *>(h->ws + 2 * buf_bytes);
+        ga.c_tma = mp.c_tma ? 1 : 0;
         const int nitems = ga.full_tiles + cut_items;
         const int sgrid = 2 * std::min(nitems, npairs);
         std::pair<cudaEvent_t, cudaEvent_t> *tev = nullptr;
@@ -507,7 +513,7 @@ gptaq_status_t accumulate_tc(gptaq_ctx *h, const float *X, const float *Xfp, int
             h->fix_args = ga;
             h->fix_pending = true;
         }
-        stats_umma_kernel<<<sgrid, UMMA_THREADS, UMMA_SMEM, gs>>>(mp.x, mp.d, mp.xlo, mp.dlo, ga);
+        stats_umma_kernel<<<sgrid, UMMA_THREADS, UMMA_SMEM, gs>>>(mp.x, mp.d, mp.xlo, mp.dlo, mp.h, mp.dxx, mp.slots, ga);
         LAUNCHED();
         if (tev) CU(cudaEventRecord(tev->second, gs));
         CU(cudaEventRecord(h->gemm_done[buf], gs));

@@ -824,6 +824,13 @@ def test_statistics_cut_by_length(n, tokens, act_order):
     assert (np.abs(err) / np.outer(np.sqrt(d), h)).max() < 2.0 ** -10
 
 
+# (boxes of 32 columns x 128 rows: a last box of 4 columns and of 28, of 4 rows and of 124; a width whose rows are no 16-byte
+# multiples; whole tiles beside cut ones)
+@pytest.mark.parametrize("n,tokens", [(260, 1111), (380, 1111), (388, 2048), (386, 1111), (1916, 1111)])
+def test_statistics_at_the_edges_of_the_boxes(n, tokens):
+    test_statistics_cut_by_length(n, tokens, False)
+
+
 @pytest.mark.parametrize("n", [512, 1024, 1416])
 def test_correction_matrix_sums_keep_their_precision_in_narrow_tiles(n):
     """P from the device's own U and dXX^T where the products take 64-wide tiles.  A chain of 256 contraction steps is 48
