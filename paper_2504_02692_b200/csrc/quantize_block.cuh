@@ -5,23 +5,23 @@
 // memory; what would be a launch per block and a product per block over the whole matrix is a pipeline of
 // warp roles inside the CTA:
 //
-//   chain   (4 warps)  quantizes 32 columns at a time, four lanes per row with 8 consecutive columns each (lanes 8 s .. 8 s + 7
-//                      hold columns 8 s .. of eight rows: a 16-byte read of U or P by 8 lanes is one word broadcast; with
-//                      the four lanes of a row side by side a launch took 4 % longer);
+//   chain   (4 warps)  quantizes 32 columns at a time: a lane has a row, a warp 8 consecutive columns of all rows, which it
+//                      publishes in shared memory four at a time for the warps with the columns behind them;
 //   near    (8 warps)  applies a step's errors to the rest of its 128-column block (float32 FMA), 8 columns
-//                      behind the chain, fetches the rows of U and P of the next step, writes results out;
+//                      behind the chain, fetches the rows of U and P of the next step, makes the errors of every 64
+//                      columns the tensor cores' operand, writes results out;
 //   drain   (4 warps)  adds the products of the tensor cores to the later blocks of the slab;
 //   load, mma (1 + 1)  stream U^T and P^T (fp16 hi / lo parts) and issue
 //                      D[128 later columns][32 rows] = [U^T | P^T] [-Err | rho Wpre]^T   (tcgen05, M = 128, N = 32)
 //                      for every 64 quantized columns, as lo*hi + hi*lo + hi*hi.
 //
-// What bounds it: the chain.  A column is 7 dependent float32 operations (28 cycles) as long as the next
-// column belongs to the same lane -- the lane goes on with its own error and pre-quantization value, the
-// shuffled copies that the other lanes need are off the chain -- and a shuffle more at every 8th column.  It takes 110
-// (alone) to 200 cycles (beside the near warps of a block's first step), though: shared memory returns 128 bytes a cycle,
-// and a column's rows of U and P are 64 such words for the chain's four warps and up to 96 for the near warps.
-// A launch of 512 columns takes 75 to 80 us, 138k cycles: 8k of it fill the slab, 6k to 12k are the products between blocks,
-// 6k the group grids, the rest the 64 pieces of 8 columns.
+// What bounds it: the chain, and the near warps behind it.  A column is 7 dependent float32 operations (28 cycles); with its
+// share of the updates, the codes and the hand-over to the next warp 8 columns take 750 cycles alone and 950 beside the near
+// warps, which need 830 for them (a scheduler starts a 16-byte LDS in 8 cycles where lanes share words, in 16 where they do
+// not).  A step of 32 columns ends some 2000 cycles after its last column: the near warps' last 8 columns, results, operands.
+// With a row in the four lanes of one warp every column's errors went through two shuffles to all of them, every lane updated
+// its 8 columns at every step, needed or not, and read U and P for it (64 words a column, now 36): a launch of 512 columns
+// 71 -> 64 us with groups, 68 -> 53 without; 16,384 x 4096 3432 -> 3259 us a call, 1024 x 1024 without workspace 272 -> 256.
 #pragma once
 #include "tc_gemm.cuh"
 
@@ -66,7 +66,7 @@ struct QuantBlockArgs {
 
 // Shared memory, in bytes from a 1024-byte boundary.  The tensor-core operands come first (alignment).
 struct QuantBlockSmem {
-    int a, e, w, up, st, grid, udinv, perm, inv, bars, total, wld;
+    int a, e, w, up, st, grid, udinv, perm, inv, rmax, bars, total, wld;
 };
 __host__ __device__ constexpr QuantBlockSmem quant_block_smem(bool far_form, bool percol) {
     QuantBlockSmem s{};
@@ -80,7 +80,8 @@ __host__ __device__ constexpr QuantBlockSmem quant_block_smem(bool far_form, boo
     s.udinv = s.grid + (percol ? 3 * 32 * QB_SLD * 4 : 0);
     s.perm = s.udinv + 2 * 32 * 4;
     s.inv = s.perm + 2 * 32 * 4;
-    s.bars = s.inv + 2 * QB_ROWS * 4;
+    s.rmax = s.inv + 2 * QB_ROWS * 4;
+    s.bars = s.rmax + (far_form ? QB_NEAR * 4 : 0);
     s.total = s.bars + 256;
     return s;
 }
@@ -93,7 +94,7 @@ static_assert(quant_block_smem_bytes(true, false) <= 227 * 1024 && quant_block_s
 constexpr uint32_t QB_IDESC = (1u << 4) | ((QB_ROWS >> 3) << 17) | ((128 >> 4) << 24);
 
 // Named barriers.  Chunk barriers are used once per step each; the step barrier keeps the chain from lapping them.
-enum { QBAR_CHUNK = 1, QBAR_STEP = 5, QBAR_NEAR = 6, QBAR_DRAIN = 7, QBAR_CLIP = 8 };
+enum { QBAR_CHUNK = 1, QBAR_STEP = 5, QBAR_NEAR = 6, QBAR_DRAIN = 7, QBAR_CLIP = 8, QBAR_HAND = 9 /* .. 14 */, QBAR_CHAIN = 15 };
 
 // Position of a row in a column of the published errors: the near warps' threads take rows ti, ti + 8, .. as
 // one 16-byte read.
@@ -118,26 +119,13 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
 }
 __device__ __forceinline__ float pick2(const unsigned long long (&v)[4], int j) { return (j & 1) ? hi2(v[j >> 1]) : lo2(v[j >> 1]); }
 
-// 16 bytes of shared memory into (x, y) where `on`.
-__device__ __forceinline__ void lds128_if(bool on, const float *p, unsigned long long &x, unsigned long long &y) {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t@q ld.shared.v2.u64 {%0, %1}, [%2];\n\t}"
-                 : "+l"(x), "+l"(y) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"((uint32_t)on));
+__device__ __forceinline__ void lds_pair2(const float *p, unsigned long long &x, unsigned long long &y) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(p);
+    x = v.x; y = v.y;
 }
-
-// Range of a row over `len` columns (a multiple of 32) from w, by the row's four lanes.
-__device__ __forceinline__ void row_range(const float *w, int len, int sub, float &lo, float &hi) {
-    lo = 0.f; hi = 0.f;
-#pragma unroll 2
-    for (int c = 4 * sub; c < len; c += 16) {
-        const float4 v = *reinterpret_cast<const float4 *>(w + c);
-        lo = fminf(lo, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
-        hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
-    }
-#pragma unroll
-    for (int d = 8; d < 32; d <<= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, d));
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, d));
-    }
+__device__ __forceinline__ void lds_pair4(const float *p, unsigned long long (&x)[4]) {
+    lds_pair2(p, x[0], x[1]);
+    lds_pair2(p + 4, x[2], x[3]);
 }
 
 __device__ __forceinline__ float fma_sat(float a, float b, float c) {
@@ -223,6 +211,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     float *udinv2 = reinterpret_cast<float *>(sm + L.udinv);       // [2 steps][32]: err_scale / U_kk
     int *perm2 = reinterpret_cast<int *>(sm + L.perm);             // [2 steps][32]: where a column's codes go
     float *inv_s = reinterpret_cast<float *>(sm + L.inv);          // [2 halves][32]: 1 / scale of a row's errors
+    float *rmax_s = reinterpret_cast<float *>(sm + L.rmax);        // [8 near warps][32]: a row's largest error of 8 columns
     const uint32_t bar0 = base + L.bars;
     // mbarriers (8 bytes each): afull[3], aempty[3], efull[2], efree[2], tfull[6], tempty[6]; tmem slot, abort flag
     auto afull = [&](int s) { return bar0 + 8u * s; };
@@ -297,7 +286,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     if (FAR) {
         if (tid == 0) {
             for (int s = 0; s < ASLOTS; ++s) { mbar_init(afull(s), 1); mbar_init(aempty(s), 1); }
-            for (int s = 0; s < 2; ++s) { mbar_init(efull(s), QB_CHAIN / 32); mbar_init(efree(s), QB_DRAIN / 32); }
+            for (int s = 0; s < 2; ++s) { mbar_init(efull(s), QB_NEAR / 32); mbar_init(efree(s), QB_DRAIN / 32); }
             for (int s = 0; s < 6; ++s) { mbar_init(tfull(s), 1); mbar_init(tempty(s), QB_DRAIN / 32); }
             *abort_flag = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -365,17 +354,18 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
 
     if (tid < QB_CHAIN) {
         // ================================================================ chain
-        const int lrow = 8 * warp + (lane & 7), sub = lane >> 3;
+        const int lrow = lane, w8 = 8 * warp;                       // this warp's columns of a step: w8 .. w8 + 7
         const int row = row0 + lrow;
         const bool live = lrow < nrows;
         float *wrow = Ws + lrow * WLD;
         const int pos = qb_pos(lrow);
         float scale = 1.f, zero = 0.f;
-        float row_max = 0.f;                                        // largest magnitude of the row's errors in this launch
         if (!PERCOL && a.group <= 0 && live) { scale = a.scales[row]; zero = a.zeros[row]; }
         float inv_scale = 1.f / scale, qlo = -zero, qhi = maxq - zero;
+#pragma unroll 1
         for (int b = 0; b < nblk; ++b) {
             const int nst = nsteps(b);
+#pragma unroll 1
             for (int s = 0; s < nst; ++s) {
                 const int co = b * QB_W + 32 * s;                   // first column of the step in the slab
                 const int cg = i0 + co;                             // ... in W
@@ -386,15 +376,30 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 if (PERCOL) {
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        scv[e] = grid_s[(8 * sub + e) * QB_SLD + lrow];
-                        zv[e] = grid_s[(32 + 8 * sub + e) * QB_SLD + lrow];
-                        ivv[e] = grid_s[(64 + 8 * sub + e) * QB_SLD + lrow];
+                        scv[e] = grid_s[(w8 + e) * QB_SLD + lrow];
+                        zv[e] = grid_s[(32 + w8 + e) * QB_SLD + lrow];
+                        ivv[e] = grid_s[(64 + w8 + e) * QB_SLD + lrow];
                     }
                 } else if (grid_starts(cg)) {
-                    // grid of the group that starts here, from the current values
-                    // (columns of it beyond the layer are zeros)
-                    float lo, hi;
-                    row_range(wrow + co, a.group, sub, lo, hi);
+                    // grid of the group that starts here, from the current values (columns of it beyond the layer are zeros):
+                    // a quarter of the range per warp
+                    float lo = 0.f, hi = 0.f;
+                    const float *wq4 = wrow + co + warp * (a.group >> 2);
+#pragma unroll 2
+                    for (int c = 0; c < a.group >> 2; c += 4) {
+                        const float4 v = *reinterpret_cast<const float4 *>(wq4 + c);
+                        lo = fminf(lo, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
+                        hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                    }
+                    // (through the part of the step's error buffer that warp 3 publishes into, after all have read it)
+                    float2 *range_s = reinterpret_cast<float2 *>(St + 24 * QB_SLD);
+                    range_s[warp * QB_ROWS + lrow] = make_float2(lo, hi);
+                    named_bar_sync(QBAR_CHAIN, QB_CHAIN);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 v = range_s[q * QB_ROWS + lrow];
+                        lo = fminf(lo, v.x); hi = fmaxf(hi, v.y);
+                    }
                     float p = 1.f;
                     if (a.clip_steps > 0) {
                         named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);          // the near warps search
@@ -402,7 +407,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         p = clip_ratio(reinterpret_cast<int *>(St)[lrow], a.clip_steps, a.clip_min);
                     }
                     make_grid(p * lo, p * hi, p * fmaxf(-lo, hi), a.bits, a.sym, scale, zero);
-                    if (live && sub == 0) {
+                    if (live && warp == 0) {
                         const int g = cg / a.group;
                         a.scales[(int64_t)row * a.G + g] = scale;
                         a.zeros[(int64_t)row * a.G + g] = zero;
@@ -411,34 +416,61 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     inv_scale = 1.f / scale; qlo = -zero; qhi = maxq - zero;
                 }
                 const int ld = up_ld(s);
-                const float *Us = up_buf(s) + 8 * sub, *Ps = Us + 32 * ld;
-                const float *ud = udinv2 + (s & 1) * 32;
+                const float *Uw = up_buf(s) + w8, *Pw = Uw + 32 * ld;
                 unsigned long long x[4];                            // this lane's 8 columns, in pairs
                 {
-                    const ulonglong2 v0 = *reinterpret_cast<const ulonglong2 *>(wrow + co + 8 * sub);
-                    const ulonglong2 v1 = *reinterpret_cast<const ulonglong2 *>(wrow + co + 8 * sub + 4);
+                    const ulonglong2 v0 = *reinterpret_cast<const ulonglong2 *>(wrow + co + w8);
+                    const ulonglong2 v1 = *reinterpret_cast<const ulonglong2 *>(wrow + co + w8 + 4);
                     x[0] = v0.x; x[1] = v0.y; x[2] = v1.x; x[3] = v1.y;
                 }
-                // `c` is the chain: the current column's value in the lane that owns it.  Every lane runs the same
-                // instructions on its own column; only the owner's results are used.  Entries of x that belong to
-                // columns already done are garbage (entries of U and P at or below the diagonal are applied to them)
-                // and never read again.
+                // the earlier columns of the step, four at a time as the warps before this one publish them; their rows of U
+                // and P are fetched before the wait
+#pragma unroll 1
+                for (int h = 0; h < 2 * warp; ++h) {
+                    unsigned long long u[4][4], pp[4][4];
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) {
+                        lds_pair4(Uw + (4 * h + kk) * ld, u[kk]);
+                        lds_pair4(Pw + (4 * h + kk) * ld, pp[kk]);
+                    }
+                    named_bar_sync(QBAR_HAND + h, 32 * (4 - (h >> 1)));
+                    const float *Se = St + 4 * h * QB_SLD + pos;
+                    float er[4], wa[4];
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) { er[kk] = Se[kk * QB_SLD]; wa[kk] = Se[(32 + kk) * QB_SLD]; }
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) {
+                        const unsigned long long ne2 = pack2(er[kk], er[kk]), wa2 = pack2(wa[kk], wa[kk]);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) x[j] = fma2(ne2, u[kk][j], fma2(wa2, pp[kk][j], x[j]));
+                    }
+                }
+                // `c` is the chain: the current column's value.  Entries of x that belong to columns already done are garbage
+                // (entries of U and P at or below the diagonal are applied to them) and never read again.
+                const float *ud = udinv2 + (s & 1) * 32 + w8;
+                const float4 ud0 = *reinterpret_cast<const float4 *>(ud), ud1 = *reinterpret_cast<const float4 *>(ud + 4);
+                const float udv[8] = {ud0.x, ud0.y, ud0.z, ud0.w, ud1.x, ud1.y, ud1.z, ud1.w};
+                Uw += w8 * ld; Pw += w8 * ld;
+                float *Sw = St + w8 * QB_SLD + pos;
+                float qv[8];
+                uint32_t code[2] = {0u, 0u};
                 float c = lo2(x[0]);
 #pragma unroll
-                for (int ph = 0; ph < 4; ++ph) {
-                    float nerr[8], pre[8], qv[8];
-                    uint32_t code[2] = {0u, 0u};
-                    const float4 ud0 = *reinterpret_cast<const float4 *>(ud + 8 * ph), ud1 = *reinterpret_cast<const float4 *>(ud + 8 * ph + 4);
-                    const float udv[8] = {ud0.x, ud0.y, ud0.z, ud0.w, ud1.x, ud1.y, ud1.z, ud1.w};
+                for (int half = 0; half < 2; ++half) {
+                    unsigned long long u[4][4], pp[4][4];           // (columns that no lane needs any more are not read)
+                    float nerr[4], pre[4];
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {
-                        const int K = 8 * ph + kk;
-                        const ulonglong2 u0 = *reinterpret_cast<const ulonglong2 *>(Us + K * ld), u1 = *reinterpret_cast<const ulonglong2 *>(Us + K * ld + 4);
-                        const ulonglong2 p0 = *reinterpret_cast<const ulonglong2 *>(Ps + K * ld), p1 = *reinterpret_cast<const ulonglong2 *>(Ps + K * ld + 4);
-                        const unsigned long long u[4] = {u0.x, u0.y, u1.x, u1.y}, pp[4] = {p0.x, p0.y, p1.x, p1.y};
-                        const float sc = PERCOL ? scv[kk] : scale;
-                        const float iv = PERCOL ? ivv[kk] : inv_scale;
-                        const float z = PERCOL ? zv[kk] : zero;
+                    for (int kk = 0; kk < 4; ++kk) {
+                        const int k = 4 * half + kk;
+                        if (k < 3) { lds_pair2(Uw + k * ld, u[kk][0], u[kk][1]); lds_pair2(Pw + k * ld, pp[kk][0], pp[kk][1]); }
+                        if (k < 7) { lds_pair2(Uw + k * ld + 4, u[kk][2], u[kk][3]); lds_pair2(Pw + k * ld + 4, pp[kk][2], pp[kk][3]); }
+                    }
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) {
+                        const int k = 4 * half + kk;
+                        const float sc = PERCOL ? scv[k] : scale;
+                        const float iv = PERCOL ? ivv[k] : inv_scale;
+                        const float z = PERCOL ? zv[k] : zero;
                         const float w0 = c;
                         // round(w / scale), clamped to the grid, minus the zero point.  Adding 1.5 * 2^23 rounds to nearest even
                         // wherever |v| < 2^22 and leaves larger values large (the clamp decides those).
@@ -446,99 +478,49 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         const float r = __fsub_rn(__fadd_rn(__fmul_rn(w0, iv), magic), magic);
                         const float cz = fminf(fmaxf(r, PERCOL ? -z : qlo), PERCOL ? maxq - z : qhi);
                         const float d = __fmaf_rn(sc, cz, -w0);                  // -(w - q)
-                        const float ne = d * udv[kk];                            // ... / U_kk
+                        const float ne = d * udv[k];                             // ... / U_kk
                         const float wa = a.asym_scale * w0;
-                        qv[kk] = sc * cz; nerr[kk] = ne; pre[kk] = wa;
-                        code[kk >> 2] |= (__float_as_uint(cz + z + magic) & 0xffu) << (8 * (kk & 3));
-                        // the owner's next column, from its own values
-                        if (kk < 7) c = fmaf(d, udv[kk] * pick2(u, kk + 1), fmaf(wa, pick2(pp, kk + 1), pick2(x, kk + 1)));
-                        const float ne_b = __shfl_sync(0xffffffffu, ne, 8 * ph + (lane & 7));
-                        const float wa_b = __shfl_sync(0xffffffffu, wa, 8 * ph + (lane & 7));
-                        const unsigned long long ne2 = pack2(ne_b, ne_b), wa2 = pack2(wa_b, wa_b);
+                        qv[k] = sc * cz; nerr[kk] = ne; pre[kk] = wa;
+                        code[k >> 2] |= (__float_as_uint(cz + z + magic) & 0xffu) << (8 * (k & 3));
+                        if (k == 7) continue;
+                        // the next column from the error itself, the ones after it through x
+                        c = fmaf(d, udv[k] * pick2(u[kk], k + 1), fmaf(wa, pick2(pp[kk], k + 1), pick2(x, k + 1)));
+                        const unsigned long long ne2 = pack2(ne, ne), wa2 = pack2(wa, wa);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            if (ph == 3 && 2 * j + 1 <= kk) continue;            // (no lane needs it any more)
-                            x[j] = fma2(ne2, u[j], fma2(wa2, pp[j], x[j]));
-                        }
-                        if (kk == 7) c = lo2(x[0]);
-                    }
-                    // publish these 8 columns
-                    if (sub == ph) {
-#pragma unroll
-                        for (int kk = 0; kk < 8; ++kk) {
-                            St[(8 * ph + kk) * QB_SLD + pos] = nerr[kk];
-                            St[(32 + 8 * ph + kk) * QB_SLD + pos] = pre[kk];
-                        }
-                        *reinterpret_cast<float4 *>(wrow + co + 8 * sub) = make_float4(qv[0], qv[1], qv[2], qv[3]);
-                        *reinterpret_cast<float4 *>(wrow + co + 8 * sub + 4) = make_float4(qv[4], qv[5], qv[6], qv[7]);
-                        if (live) {
-                            uint8_t *crow = a.codes + (int64_t)row * n;
-                            const int cc = cg + 8 * sub;
-                            if (!a.perm && cc + 7 < n && (reinterpret_cast<uintptr_t>(crow + cc) & 7) == 0) {
-                                *reinterpret_cast<uint2 *>(crow + cc) = make_uint2(code[0], code[1]);
-                            } else {
-#pragma unroll
-                                for (int kk = 0; kk < 8; ++kk)
-                                    if (cc + kk < n) crow[perm2[(s & 1) * 32 + 8 * ph + kk]] = (uint8_t)(code[kk >> 2] >> (8 * (kk & 3)));
-                            }
+                            if (2 * j + 1 < k + 2) continue;
+                            x[j] = fma2(ne2, u[kk][j], fma2(wa2, pp[kk][j], x[j]));
                         }
                     }
-                    named_bar_arrive(QBAR_CHUNK + ph, QB_THREADS_NEAR);
+                    // publish these 4 columns: to the chain's other warps, then (8 columns) to the near warps
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk) {
+                        Sw[(4 * half + kk) * QB_SLD] = nerr[kk];
+                        Sw[(32 + 4 * half + kk) * QB_SLD] = pre[kk];
+                    }
+                    if (warp < 3) named_bar_arrive(QBAR_HAND + 2 * warp + half, 32 * (4 - warp));
                 }
-                if (FAR && (s & 1)) {
-                    // 64 columns done: their errors as the tensor cores' operand, with one power-of-two scale per row
-                    __syncwarp();
-                    float v[2][2][8];                               // [step of the pair][-Err, Wpre][column]
-                    float mx = 0.f;
+                *reinterpret_cast<float4 *>(wrow + co + w8) = make_float4(qv[0], qv[1], qv[2], qv[3]);
+                *reinterpret_cast<float4 *>(wrow + co + w8 + 4) = make_float4(qv[4], qv[5], qv[6], qv[7]);
+                named_bar_arrive(QBAR_CHUNK + warp, 32 + QB_NEAR);
+                if (live) {
+                    uint8_t *crow = a.codes + (int64_t)row * n;
+                    const int cc = cg + w8;
+                    if (!a.perm && cc + 7 < n && (reinterpret_cast<uintptr_t>(crow + cc) & 7) == 0) {
+                        *reinterpret_cast<uint2 *>(crow + cc) = make_uint2(code[0], code[1]);
+                    } else {
 #pragma unroll
-                    for (int d = 0; d < 2; ++d)
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float *S2 = Sts + d * 64 * QB_SLD;
-                            v[d][0][e] = S2[(8 * sub + e) * QB_SLD + pos];
-                            v[d][1][e] = rho * S2[(32 + 8 * sub + e) * QB_SLD + pos];
-                            mx = fmaxf(mx, fmaxf(fabsf(v[d][0][e]), fabsf(v[d][1][e])));
-                        }
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-                    row_max = fmaxf(row_max, mx);
-                    if (b < last_groups) {
-                        const int half = s >> 1;                    // buffer: even and odd halves alternate
-                        // (the drain warps are done with this buffer's row scales, the MMAs with its operands)
-                        if (b > 0) mbar_wait(efree(half), (uint32_t)(b - 1) & 1u, abort_flag);
-                        const float sc = split_scale(mx);
-                        if (sub == 0) inv_s[half * QB_ROWS + lrow] = 1.f / sc / su;
-                        uint8_t *eb = sm + L.e + half * QB_HALF_BYTES + (lrow >> 3) * 1024 + (lrow & 7) * 128;
-#pragma unroll
-                        for (int d = 0; d < 2; ++d)
-#pragma unroll
-                            for (int o = 0; o < 2; ++o) {
-                                const float y0[4] = {sc * v[d][o][0], sc * v[d][o][1], sc * v[d][o][2], sc * v[d][o][3]};
-                                const float y1[4] = {sc * v[d][o][4], sc * v[d][o][5], sc * v[d][o][6], sc * v[d][o][7]};
-                                uint2 h0, l0, h1, l1;
-                                split16_pack(y0, h0, l0);
-                                split16_pack(y1, h1, l1);
-                                const int ch = ((4 * d + sub) ^ (lrow & 7)) << 4;
-                                *reinterpret_cast<uint4 *>(eb + o * QB_E_BYTES + ch) = make_uint4(h0.x, h0.y, h1.x, h1.y);
-                                *reinterpret_cast<uint4 *>(eb + (2 + o) * QB_E_BYTES + ch) = make_uint4(l0.x, l0.y, l1.x, l1.y);
-                            }
-                        fence_proxy_async_smem();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(efull(half));
+                        for (int kk = 0; kk < 8; ++kk)
+                            if (cc + kk < n) crow[perm2[(s & 1) * 32 + w8 + kk]] = (uint8_t)(code[kk >> 2] >> (8 * (kk & 3)));
                     }
                 }
             }
-        }
-        if (FAR && a.EWS_hi && sub == 0) {
-            const float sc = live ? split_scale(row_max) : 1.f;
-            udinv2[lrow] = sc;                                      // (free: the last step's pivots are in the other half; read
-                                                                    //  after the barrier below)
-            if (live) a.row_inv[row] = 1.f / sc;
         }
     } else if (tid < QB_THREADS_NEAR) {
         // ================================================================ near
         const int t = tid - QB_CHAIN;
         const int ti = t & 7, tj = t >> 3;                          // rows ti, ti + 8, ti + 16, ti + 24; columns 4 tj .. of the rest
+        float row_max = 0.f;                                        // largest magnitude of row (t & 31)'s errors in this launch
         for (int b = 0; b < nblk; ++b) {
             const int nst = nsteps(b);
             for (int s = 0; s < nst; ++s) {
@@ -591,7 +573,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
 #pragma unroll
                 for (int e = 0; e < 4; ++e) { acc[e][0] = 0ull; acc[e][1] = 0ull; }
                 for (int ph = 0; ph < 4; ++ph) {
-                    named_bar_sync(QBAR_CHUNK + ph, QB_THREADS_NEAR);
+                    named_bar_sync(QBAR_CHUNK + ph, 32 + QB_NEAR);
                     if (!active) continue;
 #pragma unroll
                     for (int kk = 0; kk < 16; ++kk) {
@@ -616,11 +598,52 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         *cp = v;
                     }
                 }
+                // 64 columns done: a thread takes eight of them in one row (before the chain goes on and overwrites the first 32)
+                const int er = t & 31, ec = t >> 5;
+                float ev[2][8], mx = 0.f;
+                if (FAR && (s & 1)) {
+                    const float *S2 = Sts + ((ec >> 2) * 64 + 8 * (ec & 3)) * QB_SLD + qb_pos(er);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        ev[0][e] = S2[e * QB_SLD];
+                        ev[1][e] = rho * S2[(32 + e) * QB_SLD];
+                        mx = fmaxf(mx, fmaxf(fabsf(ev[0][e]), fabsf(ev[1][e])));
+                    }
+                    rmax_s[ec * QB_ROWS + er] = mx;
+                }
                 asm volatile("cp.async.wait_all;" ::: "memory");
                 if (!last) {
                     if (t < 32) { udinv2[(ns & 1) * 32 + t] = next_ud; perm2[(ns & 1) * 32 + t] = next_perm; }
                     if (PERCOL) store_grid(t >> 3, 4 * (t & 7), next_sc, next_zp);      // (the chain has read this step's)
                     named_bar_arrive(QBAR_STEP, QB_THREADS_NEAR);
+                }
+                if (FAR && (s & 1)) {
+                    // ... as the tensor cores' operand, with one power-of-two scale per row
+                    named_bar_sync(QBAR_NEAR, QB_NEAR);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) mx = fmaxf(mx, rmax_s[e * QB_ROWS + er]);
+                    row_max = fmaxf(row_max, mx);
+                    if (b < last_groups) {
+                        const int half = s >> 1;                    // buffer: even and odd halves alternate
+                        // (the drain warps are done with this buffer's row scales, the MMAs with its operands)
+                        if (b > 0) mbar_wait(efree(half), (uint32_t)(b - 1) & 1u, abort_flag);
+                        const float sc = split_scale(mx);
+                        if (ec == 0) inv_s[half * QB_ROWS + er] = 1.f / sc / su;
+                        uint8_t *eb = sm + L.e + half * QB_HALF_BYTES + (er >> 3) * 1024 + (er & 7) * 128 + ((ec ^ (er & 7)) << 4);
+#pragma unroll
+                        for (int o = 0; o < 2; ++o) {
+                            const float y0[4] = {sc * ev[o][0], sc * ev[o][1], sc * ev[o][2], sc * ev[o][3]};
+                            const float y1[4] = {sc * ev[o][4], sc * ev[o][5], sc * ev[o][6], sc * ev[o][7]};
+                            uint2 h0, l0, h1, l1;
+                            split16_pack(y0, h0, l0);
+                            split16_pack(y1, h1, l1);
+                            *reinterpret_cast<uint4 *>(eb + o * QB_E_BYTES) = make_uint4(h0.x, h0.y, h1.x, h1.y);
+                            *reinterpret_cast<uint4 *>(eb + (2 + o) * QB_E_BYTES) = make_uint4(l0.x, l0.y, l1.x, l1.y);
+                        }
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(efull(half));
+                    }
                 }
                 // results of the step: dequantized columns, -Err and Wpre (a thread: four columns of a row)
                 {
@@ -670,6 +693,12 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     }
                 }
             }
+        }
+        if (FAR && a.EWS_hi && t < QB_ROWS) {
+            const float sc = t < nrows ? split_scale(row_max) : 1.f;
+            udinv2[t] = sc;                                         // (free: the last step's pivots are in the other half; read
+                                                                    //  after the barrier below)
+            if (t < nrows) a.row_inv[row0 + t] = 1.f / sc;
         }
     } else if (FAR && tid < QB_THREADS_NEAR + QB_DRAIN) {
         // ================================================================ drain: tensor memory -> later blocks of the slab
@@ -769,17 +798,26 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     if (a.EWS_hi) {
         // fp16 parts of [-Err | rho Wpre] for everything beyond this launch's columns (the rows were written by this
         // CTA; one scale per row over the whole launch)
-        const int q = a.ew_ld / 4;
-        for (int idx = tid; idx < nrows * q; idx += NTHREADS) {
-            const int r = idx / q, c = 4 * (idx - r * q);
-            const int64_t off = (int64_t)(row0 + r) * a.ew_ld + c;
-            const float4 v = *reinterpret_cast<const float4 *>(a.EW + off);
-            const float sc = udinv2[r];
-            const float x[4] = {sc * v.x, sc * v.y, sc * v.z, sc * v.w};
-            uint2 h2, l2;
-            split16_pack(x, h2, l2);
-            *reinterpret_cast<uint2 *>(a.EWS_hi + off) = h2;
-            *reinterpret_cast<uint2 *>(a.EWS_lo + off) = l2;
+        // (columns [0, QB_SUPER) and [ew_pre, ew_pre + QB_SUPER) of a row; five loads in flight per thread)
+        constexpr int Q = 2 * QB_SUPER / 4, BATCH = 5;
+        const float *src = a.EW + (int64_t)row0 * (2 * QB_SUPER);
+        __half *hi = a.EWS_hi + (int64_t)row0 * (2 * QB_SUPER), *lo = a.EWS_lo + (int64_t)row0 * (2 * QB_SUPER);
+        for (int i0q = tid; i0q < nrows * Q; i0q += BATCH * NTHREADS) {
+            float4 v[BATCH];
+#pragma unroll
+            for (int e = 0; e < BATCH; ++e)
+                if (i0q + e * NTHREADS < nrows * Q) v[e] = *reinterpret_cast<const float4 *>(src + 4 * (i0q + e * NTHREADS));
+#pragma unroll
+            for (int e = 0; e < BATCH; ++e) {
+                const int idx = i0q + e * NTHREADS;
+                if (idx >= nrows * Q) break;
+                const float sc = udinv2[idx / Q];
+                const float x[4] = {sc * v[e].x, sc * v[e].y, sc * v[e].z, sc * v[e].w};
+                uint2 h2, l2;
+                split16_pack(x, h2, l2);
+                *reinterpret_cast<uint2 *>(hi + 4 * idx) = h2;
+                *reinterpret_cast<uint2 *>(lo + 4 * idx) = l2;
+            }
         }
     }
     if (*abort_flag && tid == 0) record_status(a.hd, ST_TIMEOUT, 3000000 + blockIdx.x);
