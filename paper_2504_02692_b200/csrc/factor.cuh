@@ -11,7 +11,9 @@
 // 1024-wide layer took 33 us (every CTA of one kernel factored the diagonal block first) + 12 us for the update, now
 // about 20 us (diagonal) + 7 us (rows above).  Factorisation with the inversion that follows it, before and after (the
 // inversion beside the panels included): n = 1024 404 -> 287 us, n = 2052 1118 -> 726 us, n = 4096 2036 -> 1500 to 1700 us,
-// n = 14336 19.8 -> 16.6 ms.
+// n = 14336 19.8 -> 16.6 ms.  Since then: eight columns of a diagonal block at a time, its inverse beside the next block instead of
+// a kernel of its own (11 us on one SM) behind the update, the rows of U gathered as they come: n = 1024 293 -> 254 us, a panel
+// 33 -> 28 us, a layer of 777 x 2052 1337 -> 1278.
 #pragma once
 #include "tc_gemm.cuh"
 
@@ -34,8 +36,8 @@ __device__ __forceinline__ void move_up8(T (&d)[32]) {
 
 // x R^T = a for one row (a: 32 entries) against an upper triangular 32 x 32 block R given by its transpose (Rt[k][i] =
 // R[i][k], pitch FP_LD) and its reciprocal diagonal; emit(k, x_k) receives the results from k = 31 down.
-// The same recurrence with a = unit vector e_l gives column l of R^-1.  ready(k) is called before columns k .. k - 3 are
-// read (k = 31, 27, ..).
+// The same recurrence with a = unit vector e_l gives column l of R^-1.  ready(k) is called before columns k .. k - 7 are
+// read (k = 31, 23, ..).
 template <typename Ready, typename Emit>
 __device__ __forceinline__ void solve32(float (&a)[32], const float *Rt, const float *dinv, Ready ready, Emit emit) {
 #pragma unroll 1
@@ -44,7 +46,7 @@ __device__ __forceinline__ void solve32(float (&a)[32], const float *Rt, const f
 #pragma unroll
         for (int e = 7; e >= 0; --e) {
             const int k = k0 + e;
-            if (e == 7 || e == 3) ready(k);
+            if (e == 7) ready(k);
             const float x = a[24 + e] * dinv[k];
             emit(k, x);
             // entries below k: 24 + e - 1 .. 24 - k0; the rest (below entry 0) reads up to 24 words ahead of the row in shared
@@ -63,92 +65,235 @@ __device__ __forceinline__ void solve32(float (&a)[32], const float *Rt, const f
     }
 }
 
-// 32 x 32 reverse Cholesky of a symmetric block held one full row per lane; R^T to the lower part of Sd (pitch FP_LD).
-// Four columns at a time are signalled to a second warp at named barriers bar0, bar0 + 1, ..  The chain from pivot to
-// pivot is the reciprocal root (hardware estimate plus one Newton step, to about one ulp), the scaling of the column, and
-// two shuffles: the next pivot, and the entry that the next column's own update needs.  The rest of a column's rank-1
-// update waits until the next step's root is under way: the column goes to shared memory (cv: two buffers of 64 floats)
-// and comes back as broadcast float4s one step later.
-// A pivot that is not a positive normal number counts as 1 (the estimate is taken from the pivot as it comes, the test
-// runs beside it); returns the first such column (-1: none).
-__device__ __forceinline__ int chol32(float (&d)[32], int lane, float *Sd, float *dinv, float *cv, int bar0) {
-    int bad_col = -1;
-    float piv = __shfl_sync(0xffffffffu, d[31], 31), cprev = 0.f;
-    cv[lane] = 0.f; cv[32 + lane] = 0.f; cv[64 + lane] = 0.f; cv[96 + lane] = 0.f;
+// Eight columns of the block factorisation, for the rows that a warp holds one per lane (d[24 + e]: entry of the row in column
+// e of the eight).  Leader: the eight rows of the columns' own diagonal block are among them (lanes l0 .. l0 + 7); every lane
+// reads that 8 x 8 block (through `gs`, 64 words) and factors it by itself, so that the chain from pivot to pivot is a
+// reciprocal root (hardware estimate and one Newton step, to about one ulp), a scaling and one FMA, in registers.
+// col[k * FP_LD + i] receives R[i][k] for the lanes up to the diagonal, dinv[k] the reciprocal roots.  x: the row's results.
+// A pivot that is not a positive normal number counts as 1; returns the first such column (-1: none).
+__device__ __forceinline__ int chol8(float (&d)[32], float (&x)[8], int lane, int l0, float *gs, float *col, float *dinv) {
+    if ((lane & ~7) == l0) {
+        *reinterpret_cast<float4 *>(gs + (lane & 7) * 8) = make_float4(d[24], d[25], d[26], d[27]);
+        *reinterpret_cast<float4 *>(gs + (lane & 7) * 8 + 4) = make_float4(d[28], d[29], d[30], d[31]);
+    }
     __syncwarp();
-#pragma unroll 1
-    for (int k0 = 24; k0 >= 0; k0 -= 8) {
-        // d[24 + e] is column k0 + e
+    float g[8][8];                                   // (the upper triangle is used)
 #pragma unroll
-        for (int e = 7; e >= 0; --e) {
-            const int K = k0 + e;
-            float r;
-            asm volatile("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(piv));
-            {
-                // column K + 1 applied to the columns below K (its update of column K came by shuffle); columns below 0 read
-                // what lies ahead in the buffers and are never used
-                const uint32_t buf = (uint32_t)__cvta_generic_to_shared(cv + 64 * ((e + 1) & 1) + 32 + k0 - 24);
-#pragma unroll
-                for (int j4 = 5 + (e + 3) / 4; j4 >= 0; --j4) {
-                    float4 cj;
-                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(cj.x), "=f"(cj.y), "=f"(cj.z), "=f"(cj.w) : "r"(buf + 16 * j4));
-                    if (4 * j4 + 3 < 24 + e) d[4 * j4 + 3] = fmaf(-cprev, cj.w, d[4 * j4 + 3]);
-                    if (4 * j4 + 2 < 24 + e) d[4 * j4 + 2] = fmaf(-cprev, cj.z, d[4 * j4 + 2]);
-                    if (4 * j4 + 1 < 24 + e) d[4 * j4 + 1] = fmaf(-cprev, cj.y, d[4 * j4 + 1]);
-                    if (4 * j4 + 0 < 24 + e) d[4 * j4 + 0] = fmaf(-cprev, cj.x, d[4 * j4 + 0]);
-                }
-            }
-            const bool bad = !(piv >= 1.17549435e-38f) || !(piv < INFINITY);
-            r = r * fmaf(-0.5f * piv, r * r, 1.5f);
-            bad_col = (bad && bad_col < 0) ? K : bad_col;
-            piv = bad ? 1.f : piv;
-            r = bad ? 1.f : r;
-            const float c = lane < K ? d[24 + e] * r : 0.f;
-            // the next column (23 + e) receives its share of this one at once
-            const int nx = K > 0 ? K - 1 : 0;
-            const float ck = __shfl_sync(0xffffffffu, c, nx);
-            const float next = __shfl_sync(0xffffffffu, fmaf(-c, c, d[23 + e]), nx);
-            asm volatile("st.shared.f32 [%0], %1;" ::"r"((uint32_t)__cvta_generic_to_shared(cv + 64 * (e & 1) + 32 + lane)), "f"(c) : "memory");
-            __syncwarp();
-            d[23 + e] = fmaf(-c, ck, d[23 + e]);
-            const float rk = lane == K ? piv * r : c;
-            if (lane <= K) Sd[K * FP_LD + lane] = rk;
-            if (lane == K) dinv[K] = r;
-            piv = next;
-            cprev = c;
-            if (e == 4) named_bar_arrive(bar0 + (24 - k0) / 4, 64);
-            if (e == 0) named_bar_arrive(bar0 + (24 - k0) / 4 + 1, 64);
+    for (int i = 0; i < 8; ++i) {
+        const float4 hi = *reinterpret_cast<const float4 *>(gs + 8 * i + 4);
+        g[i][4] = hi.x; g[i][5] = hi.y; g[i][6] = hi.z; g[i][7] = hi.w;
+        if (i < 4) {
+            const float4 lo = *reinterpret_cast<const float4 *>(gs + 8 * i);
+            g[i][0] = lo.x; g[i][1] = lo.y; g[i][2] = lo.z; g[i][3] = lo.w;
         }
-        move_up8(d);
+    }
+    int bad_col = -1;
+#pragma unroll
+    for (int k = 7; k >= 0; --k) {
+        float piv = g[k][k], r;
+        asm volatile("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(piv));
+        const bool bad = !(piv >= 1.17549435e-38f) || !(piv < INFINITY);
+        r = r * fmaf(-0.5f * piv, r * r, 1.5f);
+        bad_col = (bad && bad_col < 0) ? k : bad_col;
+        piv = bad ? 1.f : piv;
+        r = bad ? 1.f : r;
+#pragma unroll
+        for (int i = k - 1; i >= 0; --i) {
+            g[i][k] *= r;
+#pragma unroll
+            for (int j = i; j < k; ++j) g[i][j] = fmaf(-g[i][k], g[j][k], g[i][j]);
+        }
+        x[k] = d[24 + k] * r;
+#pragma unroll
+        for (int j = k - 1; j >= 0; --j) d[24 + j] = fmaf(-x[k], g[j][k], d[24 + j]);
+        const float rk = lane == l0 + k ? piv * r : x[k];
+        if (lane <= l0 + k) col[k * FP_LD + lane] = rk;
+        if (lane == 0) dinv[k] = r;
     }
     return bad_col;
 }
 
+// ... the rows above: by substitution against the eight columns (R[j][k] at rt[k * FP_LD + j]); col[k * FP_LD + lane] receives
+// the results.
+__device__ __forceinline__ void solve8(float (&d)[32], float (&x)[8], int lane, const float *rt, const float *dinv, float *col) {
+    const float4 r0 = *reinterpret_cast<const float4 *>(dinv), r1 = *reinterpret_cast<const float4 *>(dinv + 4);
+    const float rv[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+    float c[8][8];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) {
+        const float4 lo = *reinterpret_cast<const float4 *>(rt + k * FP_LD);
+        c[k][0] = lo.x; c[k][1] = lo.y; c[k][2] = lo.z; c[k][3] = lo.w;
+        if (k > 4) {
+            const float4 hi = *reinterpret_cast<const float4 *>(rt + k * FP_LD + 4);
+            c[k][4] = hi.x; c[k][5] = hi.y; c[k][6] = hi.z; c[k][7] = hi.w;
+        }
+    }
+#pragma unroll
+    for (int k = 7; k >= 0; --k) {
+        x[k] = d[24 + k] * rv[k];
+#pragma unroll
+        for (int j = k - 1; j >= 0; --j) d[24 + j] = fmaf(-x[k], c[k][j], d[24 + j]);
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) col[k * FP_LD + lane] = x[k];
+}
+
+// d[J0 + j] -= sum over k of x[k] rt[k * FP_LD + j], j < 8
+template <int J0>
+__device__ __forceinline__ void rank8(float (&d)[32], const float (&x)[8], const float *rt) {
+#pragma unroll
+    for (int k = 7; k >= 0; --k)
+#pragma unroll
+        for (int j4 = 0; j4 < 2; ++j4) {
+            const float4 r = *reinterpret_cast<const float4 *>(rt + k * FP_LD + 4 * j4);
+            d[J0 + 4 * j4 + 0] = fmaf(-x[k], r.x, d[J0 + 4 * j4 + 0]); d[J0 + 4 * j4 + 1] = fmaf(-x[k], r.y, d[J0 + 4 * j4 + 1]);
+            d[J0 + 4 * j4 + 2] = fmaf(-x[k], r.z, d[J0 + 4 * j4 + 2]); d[J0 + 4 * j4 + 3] = fmaf(-x[k], r.w, d[J0 + 4 * j4 + 3]);
+        }
+}
+
+// Where the inverses of a block's four 32 x 32 diagonal sub-blocks lie: in the upper part of Rdiag, which R^T leaves free.  Row l
+// (32 consecutive floats) of sub-block c: inv(R_cc)[j][l].
+__device__ __forceinline__ int diag_inverse_at(int c, int l) { return ((c == 3 ? 32 : 0) + l) * NB + (c == 3 ? 64 : 32 * (c + 1)); }
+
 // ---------------------------------------------------------------------------
-// The NB x NB diagonal block [b0, b0 + NB): R_pp^T in the lower part of Rdiag (the rest of Rdiag is undefined) and the
-// inverses of its four 32 x 32 diagonal sub-blocks in Y.  Rows / columns beyond n are padded with the identity.
-// Warp 0 factors the 32 x 32 sub-blocks in registers (lane = row); warps 12 - 15 invert them, four columns behind; the
-// rows above are a product with that inverse (warps 0, 1 the 32 rows right above, whose contribution they then take off
-// the next sub-block; warps 4 - 11 the rows further up, then the rest of the rank-32 update while the next sub-block is
-// being factored).  Warp 16 runs the tensor-core product.
-// What bounds it: the pivot chain (about 150 cycles a column, 5k per sub-block) and the words that shared memory returns
-// (solving the rows 2.2k, the next sub-block 3.5k cycles): solving by substitution, a row per lane, reads R once per row and
-// took as long as the factorisation itself.  The helpers start when the chain's rows are solved: beside that solve their
-// reads delay it (n = 2052 761 -> 755 us in all), kept back until the chain factors again they slow the pivots more (45k
-// against 38k cycles).  Two columns per pivot step (two roots and one round of shuffles for both) took longer, 321 -> 328
-// us at n = 1024: the chain is short of issue slots and shared memory by then, not of latency.
+// U_pp = R_pp^-1 onto the diagonal of H (strict lower part of the block zero), by one CTA: the starting point of U = R^-1.  The
+// 32 x 32 diagonal sub-blocks come inverted from diag_factor_kernel; X12 = -X11 (R12 X22) for 32 -> 64 -> 128.  Bound by
+// shared-memory reads: 4 x 4 outputs per thread.  A second CTA of the next block's diag_factor_kernel, which takes twice as long
+// (as a CTA of panel_solve_kernel it held that up: a panel's rows 7 -> 11 us; as a kernel of its own behind the update, which
+// inverted the sub-blocks itself, it took 11 us a panel and one stream operation more); block 0 has a launch of its own.
 // ---------------------------------------------------------------------------
-constexpr int DF_MAIN = 512, DF_THREADS = DF_MAIN + 32;
-constexpr int DF_CHAIN = 128, DF_HELP = 8 * 32;
+constexpr int ID_THREADS = 256, ID_BAR = 15;
+constexpr int ID_LD = FP_LD;
+constexpr size_t ID_SMEM = (2 * NB * ID_LD + 64 * 68) * sizeof(float);
+
+// C[i][j] = sign * sum_k A[i][k] B[k][j], S x S outputs, 4 x 4 per thread (rows ti + S / 4 e, four columns), all operands
+// row-major in shared memory; `t` counts the (S / 4)^2 threads of one product.
+template <int S>
+__device__ __forceinline__ void tile_product(float *C, int ldc, const float *A, int lda, const float *B, int ldb, int t, float sign) {
+    const int ti = t / (S / 4), tj = t % (S / 4);
+    float acc[4][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < S; k += 4) {
+        float av[4][4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float4 v = *reinterpret_cast<const float4 *>(A + (ti + S / 4 * e) * lda + k);
+            av[e][0] = v.x; av[e][1] = v.y; av[e][2] = v.z; av[e][3] = v.w;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 b = *reinterpret_cast<const float4 *>(B + (k + q) * ldb + 4 * tj);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                acc[e][0] = fmaf(av[e][q], b.x, acc[e][0]); acc[e][1] = fmaf(av[e][q], b.y, acc[e][1]);
+                acc[e][2] = fmaf(av[e][q], b.z, acc[e][2]); acc[e][3] = fmaf(av[e][q], b.w, acc[e][3]);
+            }
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        *reinterpret_cast<float4 *>(C + (ti + S / 4 * e) * ldc + 4 * tj) =
+            make_float4(sign * acc[e][0], sign * acc[e][1], sign * acc[e][2], sign * acc[e][3]);
+}
+
+// by the first ID_THREADS threads of a CTA
+__device__ __forceinline__ void invert_diag_block(float *smem_f, float *H, int n, int b0, const float *Rdiag) {
+    float *S = smem_f, *X = S + NB * ID_LD, *T = X + NB * ID_LD;
+    const int tid = threadIdx.x;
+    float4 v[NB * NB / 4 / ID_THREADS];
+#pragma unroll
+    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) v[it] = *reinterpret_cast<const float4 *>(Rdiag + 4 * (tid + it * ID_THREADS));
+    float y[4 * 32 * 32 / ID_THREADS];
+#pragma unroll
+    for (int it = 0; it < 4 * 32 * 32 / ID_THREADS; ++it) {
+        const int idx = tid + it * ID_THREADS;
+        y[it] = Rdiag[diag_inverse_at(idx >> 10, (idx >> 5) & 31) + (idx & 31)];
+    }
+#pragma unroll
+    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) {
+        const int i = (tid + it * ID_THREADS) >> 5, j4 = (tid + it * ID_THREADS) & 31;
+        // R^T as it comes, left of the sub-block on the diagonal
+        if (j4 < (i >> 5) * 8) *reinterpret_cast<float4 *>(S + i * ID_LD + 4 * j4) = v[it];
+        if ((j4 >> 3) != (i >> 5)) *reinterpret_cast<float4 *>(X + i * ID_LD + 4 * j4) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int it = 0; it < 4 * 32 * 32 / ID_THREADS; ++it) {
+        const int idx = tid + it * ID_THREADS, c = idx >> 10, l = (idx >> 5) & 31, j = idx & 31;
+        X[(32 * c + j) * ID_LD + 32 * c + l] = j <= l ? y[it] : 0.f;
+    }
+    named_bar_sync(ID_BAR, ID_THREADS);
+    // R above the diagonal
+    for (int idx = tid; idx < NB * NB; idx += ID_THREADS) {
+        const int i = idx >> 7, j = idx & 127;
+        if ((j >> 5) < (i >> 5)) S[j * ID_LD + i] = S[i * ID_LD + j];
+    }
+    named_bar_sync(ID_BAR, ID_THREADS);
+    // X12 = -X11 (R12 X22), 32 -> 64 for both pairs, then 64 -> 128 (the triangular operands carry explicit zeros)
+    const int pr = tid >> 6, o = 64 * pr;
+    if (tid < 128) tile_product<32>(T + pr * 32 * 36, 36, S + o * ID_LD + o + 32, ID_LD, X + (o + 32) * ID_LD + o + 32, ID_LD, tid & 63, 1.f);
+    named_bar_sync(ID_BAR, ID_THREADS);
+    if (tid < 128) tile_product<32>(X + o * ID_LD + o + 32, ID_LD, X + o * ID_LD + o, ID_LD, T + pr * 32 * 36, 36, tid & 63, -1.f);
+    named_bar_sync(ID_BAR, ID_THREADS);
+    tile_product<64>(T, 68, S + 64, ID_LD, X + 64 * ID_LD + 64, ID_LD, tid, 1.f);
+    named_bar_sync(ID_BAR, ID_THREADS);
+    tile_product<64>(X + 64, ID_LD, X, ID_LD, T, 68, tid, -1.f);
+    named_bar_sync(ID_BAR, ID_THREADS);
+    const bool vec = (n & 3) == 0 && b0 + NB <= n;
+#pragma unroll 4
+    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) {
+        const int i = (tid + it * ID_THREADS) >> 5, j = 4 * ((tid + it * ID_THREADS) & 31);
+        const float4 x = *reinterpret_cast<const float4 *>(X + i * ID_LD + j);
+        float *dst = H + (int64_t)(b0 + i) * n + b0 + j;
+        if (vec) *reinterpret_cast<float4 *>(dst) = x;
+        else if (b0 + i < n) {
+            const float xe[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) if (b0 + j + e < n) dst[e] = xe[e];
+        }
+    }
+}
+
+__global__ void __launch_bounds__(ID_THREADS, 1) invert_diag_block_kernel(float *H, int n, int b0, const float *Rdiag) {
+    extern __shared__ __align__(16) float smem_f[];
+    pdl_wait();
+    invert_diag_block(smem_f, H, n, b0, Rdiag);
+}
+
+// ---------------------------------------------------------------------------
+// The NB x NB diagonal block [b0, b0 + NB): R_pp^T in the lower part of Rdiag and the inverses of its four 32 x 32 diagonal
+// sub-blocks in the upper part (diag_inverse_at; the rest is undefined).  Rows / columns beyond n are padded with the identity.
+// Warps 0 - 3 hold the 128 rows, one per lane, and go through the 32-column sub-blocks from the right, eight columns at a time:
+// the warp with the sub-block's own rows leads (chol8), those above it follow (solve8).  The helpers (warps 4 - 11) gather the
+// products for the next sub-block's columns as the rows are solved, so that its leader starts soon after the sub-block before is
+// done, and then update what lies further left.  Warp 12 inverts the sub-blocks, eight columns behind the leader; warp 13 runs
+// the tensor-core product.
+// What bounds it (clocks in a copy): eight columns take the leader 900 to 1400 cycles, of which 350 are dependent operations; the
+// rest is the issue of LDS (a scheduler starts one 16-byte form in 8 cycles where all lanes read the same words, else in 16) and
+// of code that a launch runs for the first time.  A warp for all 32 columns of a sub-block, one pivot at a time through shuffles,
+// took 150 cycles a pivot, and the rows above waited for the sub-block's inverse.  Rows that keep the next sub-block's
+// columns up to date by themselves (64 such reads per eight columns) fell 5k cycles behind the leader.
+// ---------------------------------------------------------------------------
+constexpr int DF_HELP = 8 * 32, DF_MAIN = 128 + DF_HELP, DF_THREADS = DF_MAIN + 64;
 constexpr int DF_TILE_BYTES = NB * 64 * 2;           // 128 rows x 64 fp16
-constexpr size_t DF_SMEM = 4 * DF_TILE_BYTES + (size_t)(NB * FP_LD + 2 * 32 * FP_YLD + NB + 128) * sizeof(float) + 64 + 1024;
+constexpr size_t DF_SMEM_BLOCK = 4 * DF_TILE_BYTES + (size_t)(NB * FP_LD + NB + 64 + 32) * sizeof(float) + 32 + 1024;
+constexpr size_t DF_SMEM = DF_SMEM_BLOCK > ID_SMEM ? DF_SMEM_BLOCK : ID_SMEM;
 constexpr uint32_t DF_IDESC = (1u << 4) | ((NB >> 3) << 17) | ((NB >> 4) << 24);     // kind::f16, M = N = 128
+// Named barriers.  COLS + q: eight columns (q = 0: the rightmost) of a sub-block are factored (its leader arrives; the warps above
+// it and the inverter wait); ROWS + q: ... and solved in the rows above (these arrive, the helpers wait); NEXT: the next
+// sub-block's columns are up to date (the helpers arrive, its rows wait); DONE: the last sub-block is factored.  Each is used
+// again in the next sub-block, which nobody enters before all have passed it.
+enum { DBAR_COLS = 1, DBAR_ROWS = 5, DBAR_NEXT = 9, DBAR_DONE = 10 };
 
 struct DiagFactorArgs {
     const float *src; long long lds;     // element (0, 0) of the block and its row pitch; entries j >= i are used
     int n, b0;
     float *Rdiag;                        // [NB][NB]
-    float *Y;                            // [4][32][FP_YLD]: Y[c][l][j] = inv(R_cc)[j][l]
+    float *H; int inv_b0;                // a second CTA inverts the block at inv_b0 (onto the diagonal of H) from inv_Rdiag
+    const float *inv_Rdiag;
     int syrk, pan_col0;                  // 1: subtract rows b0 .. of the panel at columns pan_col0 .. of the split copy times
                                          //    their transpose first (scale of the copy: tc_amax[AMAX_PAN])
     StateHeader *hd;
@@ -161,25 +306,28 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *sm = smem_raw + (base - raw);
     float (*S)[FP_LD] = reinterpret_cast<float (*)[FP_LD]>(sm + 4 * DF_TILE_BYTES);
-    // [2][32][FP_YLD]: inverses of the sub-blocks, Yc[s & 1][l][j] = inv(R_ss)[j][l] (the helpers still read one while the
-    // next is being made)
-    float *Yc = reinterpret_cast<float *>(S + NB);
-    float *dinv = Yc + 2 * 32 * FP_YLD;
-    float *cv = dinv + NB;                           // 2 x (32 words of padding, 32)
-    uint8_t *tailp = reinterpret_cast<uint8_t *>(cv + 128);
+    float *dinv = reinterpret_cast<float *>(S + NB);
+    float *gs = dinv + NB;                           // 8 x 8: the diagonal block of the columns at hand
+    float *rdiag = gs + 64;                          // 1 / R_kk of the sub-block that is being inverted
+    uint8_t *tailp = reinterpret_cast<uint8_t *>(rdiag + 32);
     const uint32_t bar = smem_u32(tailp), bar_mma = bar + 8;
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(tailp + 16);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tailp + 20);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nv = min(NB, a.n - a.b0);
     pdl_launch_dependents();
+    if (blockIdx.x == 1) {
+        pdl_wait();
+        if (tid < ID_THREADS) invert_diag_block(reinterpret_cast<float *>(smem_raw), a.H, a.n, a.inv_b0, a.inv_Rdiag);
+        return;
+    }
     if (tid == 0) {
         mbar_init(bar, 1);
         mbar_init(bar_mma, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (a.syrk && warp == 16) {
+    if (a.syrk && warp == 13) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(const_cast<uint32_t *>(tmem_slot))), "r"(128u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -188,7 +336,7 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
     __syncthreads();
     tc_fence_after();
     pdl_wait();
-    if (warp == 16) {
+    if (warp == 13) {
         if (a.syrk && lane == 0) {
             mbar_expect_tx(bar, 4 * DF_TILE_BYTES);
             for (int t = 0; t < 4; ++t) tma_load_2d(base + t * DF_TILE_BYTES, t < 2 ? &mapHi : &mapLo, a.pan_col0 + 64 * (t & 1), a.b0, bar);
@@ -207,96 +355,67 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
             }
         }
         __syncwarp();
-    } else
-    // the block (all loads in flight before the first store)
-    if (nv == NB && (a.lds & 3) == 0 && (reinterpret_cast<uintptr_t>(a.src) & 15) == 0) {
-        float4 v[NB * NB / 4 / DF_MAIN];
+    } else if (warp < 12) {
+        // the block (all loads in flight before the first store)
+        constexpr int QUADS = NB * NB / 4, ITS = (QUADS + DF_MAIN - 1) / DF_MAIN;
+        if (nv == NB && (a.lds & 3) == 0 && (reinterpret_cast<uintptr_t>(a.src) & 15) == 0) {
+            float4 v[ITS];
 #pragma unroll
-        for (int it = 0; it < NB * NB / 4 / DF_MAIN; ++it) {
-            const int idx = tid + it * DF_MAIN;
-            v[it] = *reinterpret_cast<const float4 *>(a.src + (idx >> 5) * a.lds + 4 * (idx & 31));
-        }
+            for (int it = 0; it < ITS; ++it) {
+                const int idx = tid + it * DF_MAIN;
+                if (idx < QUADS) v[it] = *reinterpret_cast<const float4 *>(a.src + (idx >> 5) * a.lds + 4 * (idx & 31));
+            }
 #pragma unroll
-        for (int it = 0; it < NB * NB / 4 / DF_MAIN; ++it) {
-            const int idx = tid + it * DF_MAIN;
-            *reinterpret_cast<float4 *>(&S[idx >> 5][4 * (idx & 31)]) = v[it];
-        }
-    } else {
-        for (int idx = tid; idx < NB * NB; idx += DF_MAIN) {
-            const int i = idx >> 7, j = idx & 127;
-            S[i][j] = (i < nv && j < nv && j >= i) ? a.src[i * a.lds + j] : (i == j ? 1.f : 0.f);
+            for (int it = 0; it < ITS; ++it) {
+                const int idx = tid + it * DF_MAIN;
+                if (idx < QUADS) *reinterpret_cast<float4 *>(&S[idx >> 5][4 * (idx & 31)]) = v[it];
+            }
+        } else {
+            for (int idx = tid; idx < NB * NB; idx += DF_MAIN) {
+                const int i = idx >> 7, j = idx & 127;
+                S[i][j] = (i < nv && j < nv && j >= i) ? a.src[i * a.lds + j] : (i == j ? 1.f : 0.f);
+            }
         }
     }
     __syncthreads();
     if (a.syrk) {
         const uint32_t tmem = *tmem_slot;
-        // 16 warps, 32 x 32 each
-        const int quarter = warp & 3, c0 = 32 * (warp >> 2), row = 32 * quarter + lane;
-        const bool ok = warp < 16 && mbar_wait(bar_mma, 0u, abort_flag);
+        // 32 x 32 pieces of the upper triangle, one or two per warp
+        const int quarter = warp & 3, row = 32 * quarter + lane;
+        const bool ok = warp < 12 && mbar_wait(bar_mma, 0u, abort_flag);
         __syncwarp();
-        if (ok && c0 + 31 >= 32 * quarter) {
+        if (ok) {
             tc_fence_after();
-            uint32_t v[32];
-            tmem_ld32(tmem + c0 + ((uint32_t)(quarter * 32) << 16), v);
-            tmem_ld_wait();
             const float sc = split_scale(__uint_as_float(a.hd->tc_amax[AMAX_PAN]));
             const float inv = 1.f / (sc * sc);
+            for (int cb = warp >> 2; cb < 4; cb += 3) {
+                if (cb < quarter) continue;
+                const int c0 = 32 * cb;
+                uint32_t v[32];
+                tmem_ld32(tmem + c0 + ((uint32_t)(quarter * 32) << 16), v);
+                tmem_ld_wait();
 #pragma unroll
-            for (int c4 = 0; c4 < 8; ++c4) {
-                float4 x = *reinterpret_cast<float4 *>(&S[row][c0 + 4 * c4]);
-                x.x = fmaf(-inv, __uint_as_float(v[4 * c4]), x.x); x.y = fmaf(-inv, __uint_as_float(v[4 * c4 + 1]), x.y);
-                x.z = fmaf(-inv, __uint_as_float(v[4 * c4 + 2]), x.z); x.w = fmaf(-inv, __uint_as_float(v[4 * c4 + 3]), x.w);
-                *reinterpret_cast<float4 *>(&S[row][c0 + 4 * c4]) = x;
+                for (int c4 = 0; c4 < 8; ++c4) {
+                    float4 x = *reinterpret_cast<float4 *>(&S[row][c0 + 4 * c4]);
+                    x.x = fmaf(-inv, __uint_as_float(v[4 * c4]), x.x); x.y = fmaf(-inv, __uint_as_float(v[4 * c4 + 1]), x.y);
+                    x.z = fmaf(-inv, __uint_as_float(v[4 * c4 + 2]), x.z); x.w = fmaf(-inv, __uint_as_float(v[4 * c4 + 3]), x.w);
+                    *reinterpret_cast<float4 *>(&S[row][c0 + 4 * c4]) = x;
+                }
             }
         }
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
-        if (warp == 16)
+        if (warp == 13)
             asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128u) : "memory");
     }
 
-    // X = S[rows, sub] inv(R_ss)^T, 4 x 4 outputs per thread; into the lower part (transposed: S[o + j][i])
-    auto solve_rows = [&](int o, int i0, int u) {
-        const int i = i0 + 4 * (u >> 3), j = 4 * (u & 7);
-        const float *Ys = Yc + ((o >> 5) & 1) * 32 * FP_YLD;
-        float acc[4][4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-#pragma unroll
-            for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
-#pragma unroll 2
-        for (int l = 0; l < 32; l += 4) {
-            float av[4][4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float4 q = *reinterpret_cast<const float4 *>(&S[i + e][o + l]);
-                av[e][0] = q.x; av[e][1] = q.y; av[e][2] = q.z; av[e][3] = q.w;
-            }
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-                const float4 y = *reinterpret_cast<const float4 *>(Ys + (l + g) * FP_YLD + j);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    acc[0][e] = fmaf(av[e][g], y.x, acc[0][e]); acc[1][e] = fmaf(av[e][g], y.y, acc[1][e]);
-                    acc[2][e] = fmaf(av[e][g], y.z, acc[2][e]); acc[3][e] = fmaf(av[e][g], y.w, acc[3][e]);
-                }
-            }
-        }
-#pragma unroll
-        for (int f = 0; f < 4; ++f)
-            *reinterpret_cast<float4 *>(&S[o + j + f][i]) = make_float4(acc[f][0], acc[f][1], acc[f][2], acc[f][3]);
-    };
-    // products of the solved rows: acc[e][f] = X[i + e] . X[j + f]
-    auto rows_dot = [&](int o, int i, int j, float (&acc)[4][4]) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-#pragma unroll
-            for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
+    // products of the solved rows, nk of them from row k0 of R^T on: acc[e][f] += X[i + e] . X[j + f]
+    auto rows_dot = [&](int k0, int nk, int i, int j, float (&acc)[4][4]) {
 #pragma unroll 4
-        for (int k = 0; k < 32; ++k) {
-            const float4 ri = *reinterpret_cast<const float4 *>(&S[o + k][i]);
-            const float4 rj = *reinterpret_cast<const float4 *>(&S[o + k][j]);
+        for (int k = k0 + nk - 1; k >= k0; --k) {
+            const float4 ri = *reinterpret_cast<const float4 *>(&S[k][i]);
+            const float4 rj = *reinterpret_cast<const float4 *>(&S[k][j]);
             const float av[4] = {ri.x, ri.y, ri.z, ri.w}, bv[4] = {rj.x, rj.y, rj.z, rj.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e)
@@ -304,111 +423,113 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
                 for (int f = 0; f < 4; ++f) acc[e][f] = fmaf(av[e], bv[f], acc[e][f]);
         }
     };
-    // Named barriers: 1 -- a sub-block is factored and inverted and the helpers' last update is done (warps 0 - 15); 2 -- the
-    // rows right above are solved (chain warps arrive, helpers wait); 3 -- the same, among the chain warps; 4 .. 11 -- four
-    // columns of the sub-block are ready for its inverter; 12 -- the rows further up are solved, among the helpers.
-    if (tid < DF_CHAIN) {
-        float d[32];
-        if (warp == 0) {
+    auto subtract = [&](int i, int j, const float (&acc)[4][4]) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) d[j] = (j >= lane) ? S[96 + lane][96 + j] : S[96 + j][96 + lane];
+        for (int e = 0; e < 4; ++e) {
+            float4 *cp = reinterpret_cast<float4 *>(&S[i + e][j]);
+            float4 v = *cp;
+            // (below the diagonal nothing is read before results are written there)
+            v.x -= acc[e][0]; v.y -= acc[e][1]; v.z -= acc[e][2]; v.w -= acc[e][3];
+            *cp = v;
         }
+    };
+    if (warp < 4) {
+        const int row = 32 * warp + lane;
+        float d[32], x[8];                           // the row in this sub-block's columns
 #pragma unroll 1
-        for (int sb = 3; sb >= 0; --sb) {
-            const int o = 32 * sb, o1 = o - 32;
-            if (warp == 0) {
-                const int bad_col = chol32(d, lane, &S[o][o], dinv + o, cv, 4);
-                if (bad_col >= 0 && lane == 0) record_status(a.hd, ST_NOT_SPD, a.b0 + o + bad_col);
+        for (int sb = 3; sb >= warp; --sb) {
+            const int o = 32 * sb;
+            const bool leads = sb == warp;
+            if (sb < 3) named_bar_sync(DBAR_NEXT, DF_HELP + 32 * (sb + 1));
+#pragma unroll
+            for (int j4 = 0; j4 < 8; ++j4) {
+                const float4 v = *reinterpret_cast<const float4 *>(&S[row][o + 4 * j4]);       // (left of the diagonal: never used)
+                d[4 * j4] = v.x; d[4 * j4 + 1] = v.y; d[4 * j4 + 2] = v.z; d[4 * j4 + 3] = v.w;
             }
-            if (sb == 0) break;
-            named_bar_sync(1, DF_MAIN);
-            if (tid < 64) solve_rows(o, o1, tid);
-            named_bar_arrive(2, DF_CHAIN + DF_HELP);
-            named_bar_sync(3, DF_CHAIN);
-            // the next sub-block, less their contribution: 2 x 4 outputs of the upper triangle per thread, mirrored (4 x 4 in
-            // 36 threads: 1 % more in all)
-            {
-                const int i = o1 + 2 * (tid >> 3), j = o1 + 4 * (tid & 7);
-                if (j + 3 >= i) {
-                    float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll 8
-                    for (int k = 0; k < 32; ++k) {
-                        const float2 ri = *reinterpret_cast<const float2 *>(&S[o + k][i]);
-                        const float4 rj = *reinterpret_cast<const float4 *>(&S[o + k][j]);
-                        acc[0][0] = fmaf(ri.x, rj.x, acc[0][0]); acc[0][1] = fmaf(ri.x, rj.y, acc[0][1]);
-                        acc[0][2] = fmaf(ri.x, rj.z, acc[0][2]); acc[0][3] = fmaf(ri.x, rj.w, acc[0][3]);
-                        acc[1][0] = fmaf(ri.y, rj.x, acc[1][0]); acc[1][1] = fmaf(ri.y, rj.y, acc[1][1]);
-                        acc[1][2] = fmaf(ri.y, rj.z, acc[1][2]); acc[1][3] = fmaf(ri.y, rj.w, acc[1][3]);
-                    }
-#pragma unroll
-                    for (int e = 0; e < 2; ++e)
-#pragma unroll
-                        for (int f = 0; f < 4; ++f)
-                            if (j + f >= i + e) {
-                                const float v = S[i + e][j + f] - acc[e][f];
-                                S[i + e][j + f] = v;
-                                if (j + f > i + e) S[j + f][i + e] = v;
-                            }
+#pragma unroll 1
+            for (int q = 0; q < 4; ++q) {
+                const int k0 = 24 - 8 * q;
+                float *rt = &S[o + k0][0];           // rt[k * FP_LD + i]: R[i][o + k0 + k]
+                if (leads) {
+                    const int bad_col = chol8(d, x, lane, k0, gs, rt + o, dinv + o + k0);
+                    named_bar_arrive(DBAR_COLS + q, 32 * (sb + 2));
+                    if (bad_col >= 0 && lane == 0) record_status(a.hd, ST_NOT_SPD, a.b0 + o + k0 + bad_col);
+                    __syncwarp();
+                } else {
+                    named_bar_sync(DBAR_COLS + q, 32 * (sb + 2));
+                    solve8(d, x, lane, rt + o + k0, dinv + o + k0, rt + 32 * warp);
+                    named_bar_arrive(DBAR_ROWS + q, DF_HELP + 32 * sb);
                 }
-            }
-            named_bar_sync(3, DF_CHAIN);
-            if (warp == 0) {
-#pragma unroll
-                for (int j4 = 0; j4 < 8; ++j4) {
-                    const float4 q = *reinterpret_cast<const float4 *>(&S[o1 + lane][o1 + 4 * j4]);
-                    d[4 * j4] = q.x; d[4 * j4 + 1] = q.y; d[4 * j4 + 2] = q.z; d[4 * j4 + 3] = q.w;
-                }
+                // the columns left of these
+                if (k0 >= 8) rank8<16>(d, x, rt + o + k0 - 8);
+                if (k0 >= 16) rank8<8>(d, x, rt + o + k0 - 16);
+                if (k0 >= 24) rank8<0>(d, x, rt + o);
+                move_up8(d);
             }
         }
-    } else if (tid < DF_CHAIN + DF_HELP) {
-        const int t = tid - DF_CHAIN;
+        if (warp == 0) named_bar_arrive(DBAR_DONE, DF_HELP + 32);
+    } else if (warp < 12) {
+        const int t = tid - 128;
+        // R^T of a sub-block's rows, up to the diagonal
+        auto store_rows = [&](int sb) {
+            for (int idx = t; idx < 32 * (NB / 4); idx += DF_HELP) {
+                const int i = 32 * sb + (idx >> 5), j4 = idx & 31;
+                if (j4 < 8 * (sb + 1)) *reinterpret_cast<float4 *>(a.Rdiag + i * NB + 4 * j4) = *reinterpret_cast<const float4 *>(&S[i][4 * j4]);
+            }
+        };
 #pragma unroll 1
         for (int sb = 3; sb >= 1; --sb) {
             const int o = 32 * sb;
-            named_bar_sync(1, DF_MAIN);
-            named_bar_sync(2, DF_CHAIN + DF_HELP);
-            if (t < 2 * (o - 32)) solve_rows(o, 0, t);
-            named_bar_sync(12, DF_HELP);
-            // leading part: S[i][j] -= X[i] . X[j] for i <= j < o, the tiles of the upper triangle numbered row by row; the
-            // last 32 x 32 sub-block is the chain's own
-            const int q = o / 4, ntile = q * (q + 1) / 2 - 36;
-            for (int u = t; u < ntile; u += DF_HELP) {
-                int ti = 0, left = u;
-                while (left >= q - ti) { left -= q - ti; ++ti; }
-                const int i = 4 * ti, j = 4 * (ti + left);
-                float acc[4][4];
-                rows_dot(o, i, j, acc);
+            float acc[4][4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    float4 *cp = reinterpret_cast<float4 *>(&S[i + e][j]);
-                    float4 v = *cp;
-                    v.x -= acc[e][0]; v.y -= acc[e][1]; v.z -= acc[e][2]; v.w -= acc[e][3];
-                    *cp = v;
-                }
+            for (int e = 0; e < 4; ++e)
+#pragma unroll
+                for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
+            // the next sub-block's columns: S[i][j] -= X[i] . X[j], i < o, o - 32 <= j < o
+            const int i = 4 * (t >> 3), j = o - 32 + 4 * (t & 7);
+#pragma unroll 1
+            for (int q = 0; q < 4; ++q) {
+                named_bar_sync(DBAR_ROWS + q, DF_HELP + 32 * sb);
+                if (i < o) rows_dot(o + 24 - 8 * q, 8, i, j, acc);
             }
+            if (i < o) subtract(i, j, acc);
+            named_bar_arrive(DBAR_NEXT, DF_HELP + 32 * sb);
+            // ... and what lies left of them: i <= j < o - 32, the 4 x 4 tiles of the upper triangle numbered row by row
+            const int q4 = (o - 32) / 4, ntile = q4 * (q4 + 1) / 2;
+            if (t < ntile) {
+                int ti = 0, left = t;
+                while (left >= q4 - ti) { left -= q4 - ti; ++ti; }
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
+                rows_dot(o, 32, 4 * ti, 4 * (ti + left), acc);
+                subtract(4 * ti, 4 * (ti + left), acc);
+            }
+            store_rows(sb);
         }
-    } else if (warp < 16) {
-        // warp 12 + c inverts sub-block c (lane = column)
-        const int c = warp - 12, o = 32 * c;
+        named_bar_sync(DBAR_DONE, DF_HELP + 32);
+        store_rows(0);
+    } else if (warp == 12) {
+        // the inverses of the sub-blocks (lane = column), by the reciprocals of the diagonal as it was rounded (with the reciprocal
+        // roots instead U was off by 3 to 5 % more)
 #pragma unroll 1
         for (int sb = 3; sb >= 0; --sb) {
-            if (sb == c) {
-                float y[32];
+            const int o = 32 * sb;
+            float y[32];
 #pragma unroll
-                for (int k = 0; k < 32; ++k) y[k] = (k == lane) ? 1.f : 0.f;
-                float *dst = a.Y + (c * 32 + lane) * FP_YLD;
-                solve32(y, &S[o][o], dinv + o, [&](int k) { named_bar_sync(4 + (31 - k) / 4, 64); },
-                        [&](int k, float v) { Yc[(c & 1) * 32 * FP_YLD + lane * FP_YLD + k] = v; dst[k] = v; });
-            }
-            if (sb > 0) named_bar_sync(1, DF_MAIN);
+            for (int k = 0; k < 32; ++k) y[k] = (k == lane) ? 1.f : 0.f;
+            float *dst = a.Rdiag + diag_inverse_at(sb, lane);
+            solve32(y, &S[o][o], rdiag,
+                    [&](int k) {
+                        named_bar_sync(DBAR_COLS + (31 - k) / 8, 32 * (sb + 2));
+                        if (lane < 8) rdiag[k - lane] = 1.f / S[o + k - lane][o + k - lane];
+                        __syncwarp();
+                    },
+                    [&](int k, float v) { dst[k] = v; });
         }
     }
     __syncthreads();
-#pragma unroll
-    for (int it = 0; it < NB * NB / 4 / DF_MAIN; ++it) {
-        const int idx = tid + it * DF_MAIN;
-        if (warp < 16) *reinterpret_cast<float4 *>(a.Rdiag + 4 * idx) = *reinterpret_cast<const float4 *>(&S[idx >> 5][4 * (idx & 31)]);
-    }
     if (*abort_flag && tid == 0) record_status(a.hd, ST_TIMEOUT, 4000000 + a.b0);
 }
 
@@ -429,7 +550,7 @@ constexpr size_t PS_SMEM = (size_t)(NB * FP_LD + 4 * 32 * FP_YLD + PS_WORKERS * 
 
 struct PanelSolveArgs {
     float *H; int n; int b0;
-    const float *Rdiag, *Y;    // as diag_factor_kernel leaves them (R_pp^T in the lower part)
+    const float *Rdiag;        // as diag_factor_kernel leaves it
     __half *pan_hi, *pan_lo;   // nullptr, or fp16 parts of split_scale(tc_amax[AMAX_PAN]) * row: row pitch pan_ld, this panel
     int pan_ld, pan_col0;      //   at columns pan_col0 .. + NB (several panels side by side)
     int workers;               // warps of a CTA that take rows
@@ -484,7 +605,8 @@ __global__ void __launch_bounds__(PS_THREADS) panel_solve_kernel(PanelSolveArgs 
         const int i = idx >> 5, j4 = idx & 31;
         if (j4 < (i >> 5) * 8) sg_copy16(&S[i][4 * j4], a.Rdiag + 4 * idx);
     }
-    for (int idx = tid; idx < 4 * 32 * FP_YLD / 4; idx += PS_THREADS) sg_copy16(Yt + 4 * idx, a.Y + 4 * idx);
+    for (int idx = tid; idx < 4 * 32 * 8; idx += PS_THREADS)
+        sg_copy16(Yt + (idx >> 3) * FP_YLD + 4 * (idx & 7), a.Rdiag + diag_inverse_at(idx >> 8, (idx >> 3) & 31) + 4 * (idx & 7));
     if (!a.early && g < ngroups) load_rows(g);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
@@ -581,108 +703,6 @@ __global__ void __launch_bounds__(PS_THREADS) panel_solve_kernel(PanelSolveArgs 
                     *reinterpret_cast<uint2 *>(a.pan_lo + row * a.pan_ld + a.pan_col0 + c) = lo;
                 }
             }
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Inverts NB x NB diagonal factors R_pp from block `first` on (one CTA each) and stores the inverse on the
-// diagonal of H (strict lower part of the block zero): the starting point of U = R^-1.  Bound by shared-memory
-// reads: 4 x 4 outputs per thread (one output per thread, and divisions in the substitution, took 36 us; now 11).
-// 32 x 32 diagonal sub-blocks by back substitution (one warp each, lane = column), then
-// X12 = -X11 (R12 X22) for 32 -> 64 -> 128.
-// ---------------------------------------------------------------------------
-constexpr int ID_THREADS = 256;
-constexpr int ID_LD = FP_LD;
-constexpr size_t ID_SMEM = (32 + 2 * NB * ID_LD + 64 * 68 + NB) * sizeof(float);
-
-// C[i][j] = sign * sum_k A[i][k] B[k][j], S x S outputs, 4 x 4 per thread (rows ti + S / 4 e, four columns), all operands
-// row-major in shared memory; `t` counts the (S / 4)^2 threads of one product.
-template <int S>
-__device__ __forceinline__ void tile_product(float *C, int ldc, const float *A, int lda, const float *B, int ldb, int t, float sign) {
-    const int ti = t / (S / 4), tj = t % (S / 4);
-    float acc[4][4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-#pragma unroll
-        for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
-#pragma unroll 4
-    for (int k = 0; k < S; k += 4) {
-        float av[4][4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float4 v = *reinterpret_cast<const float4 *>(A + (ti + S / 4 * e) * lda + k);
-            av[e][0] = v.x; av[e][1] = v.y; av[e][2] = v.z; av[e][3] = v.w;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float4 b = *reinterpret_cast<const float4 *>(B + (k + q) * ldb + 4 * tj);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                acc[e][0] = fmaf(av[e][q], b.x, acc[e][0]); acc[e][1] = fmaf(av[e][q], b.y, acc[e][1]);
-                acc[e][2] = fmaf(av[e][q], b.z, acc[e][2]); acc[e][3] = fmaf(av[e][q], b.w, acc[e][3]);
-            }
-        }
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-        *reinterpret_cast<float4 *>(C + (ti + S / 4 * e) * ldc + 4 * tj) =
-            make_float4(sign * acc[e][0], sign * acc[e][1], sign * acc[e][2], sign * acc[e][3]);
-}
-
-__global__ void __launch_bounds__(ID_THREADS, 1) invert_diag_blocks_kernel(float *H, int n, const float *Rdiag, int first) {
-    extern __shared__ __align__(16) float smem_f[];
-    float *S = smem_f + 32, *X = S + NB * ID_LD,      // (padding: solve32 reads ahead of its block)
-          *T = X + NB * ID_LD, *dinv = T + 64 * 68;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int b0 = (first + blockIdx.x) * NB;
-    const float *src = Rdiag + (int64_t)(first + blockIdx.x) * NB * NB;
-    float4 v[NB * NB / 4 / ID_THREADS];
-#pragma unroll
-    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) v[it] = *reinterpret_cast<const float4 *>(src + 4 * (tid + it * ID_THREADS));
-    if (tid < NB) dinv[tid] = 1.f / src[tid * NB + tid];
-#pragma unroll
-    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) {
-        const int i = (tid + it * ID_THREADS) >> 5, j4 = (tid + it * ID_THREADS) & 31;
-        // R^T as it comes (the substitution below reads it by rows), and R above the diagonal
-        if (4 * j4 <= i) *reinterpret_cast<float4 *>(S + i * ID_LD + 4 * j4) = v[it];
-        *reinterpret_cast<float4 *>(X + i * ID_LD + 4 * j4) = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    __syncthreads();
-    for (int idx = tid; idx < NB * NB; idx += ID_THREADS) {
-        const int i = idx >> 7, j = idx & 127;
-        if (j < i) S[j * ID_LD + i] = S[i * ID_LD + j];
-    }
-    __syncthreads();
-    if (warp < NB / 32) {
-        const int o = 32 * warp;
-        float x[32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) x[i] = (i == lane) ? 1.f : 0.f;
-        solve32(x, S + o * ID_LD + o, dinv + o, [](int) {}, [&](int k, float v) { X[(o + k) * ID_LD + o + lane] = v; });
-    }
-    __syncthreads();
-    // X12 = -X11 (R12 X22), 32 -> 64 for both pairs, then 64 -> 128 (the triangular operands carry explicit zeros)
-    const int pr = tid >> 6, o = 64 * pr;
-    if (tid < 128) tile_product<32>(T + pr * 32 * 36, 36, S + o * ID_LD + o + 32, ID_LD, X + (o + 32) * ID_LD + o + 32, ID_LD, tid & 63, 1.f);
-    __syncthreads();
-    if (tid < 128) tile_product<32>(X + o * ID_LD + o + 32, ID_LD, X + o * ID_LD + o, ID_LD, T + pr * 32 * 36, 36, tid & 63, -1.f);
-    __syncthreads();
-    tile_product<64>(T, 68, S + 64, ID_LD, X + 64 * ID_LD + 64, ID_LD, tid, 1.f);
-    __syncthreads();
-    tile_product<64>(X + 64, ID_LD, X, ID_LD, T, 68, tid, -1.f);
-    __syncthreads();
-    const bool vec = (n & 3) == 0 && b0 + NB <= n;
-    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) {
-        const int i = (tid + it * ID_THREADS) >> 5, j = 4 * ((tid + it * ID_THREADS) & 31);
-        float x[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) x[e] = j + e >= i ? X[i * ID_LD + j + e] : 0.f;
-        float *dst = H + (int64_t)(b0 + i) * n + b0 + j;
-        if (vec) *reinterpret_cast<float4 *>(dst) = make_float4(x[0], x[1], x[2], x[3]);
-        else if (b0 + i < n) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) if (b0 + j + e < n) dst[e] = x[e];
         }
     }
 }

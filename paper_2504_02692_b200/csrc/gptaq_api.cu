@@ -911,7 +911,7 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
         e = cudaFuncSetAttribute(panel_solve_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM);
     if (e == cudaSuccess) e = configure_quantize_kernels();
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(invert_diag_blocks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ID_SMEM);
+        e = cudaFuncSetAttribute(invert_diag_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ID_SMEM);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(stats_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UMMA_SMEM);
     if (e == cudaSuccess)
@@ -1106,7 +1106,7 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         const SplitOperand pan{pan_hi, pan_lo, n, SUPER_NB, SUPER_NB};
         if (!make_tc_maps(&pan_maps, pan, pan, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
     }
-    float *Y = reinterpret_cast<float *>(h->ws + wl.diag_off), *next_diag = Y + 4 * 32 * FP_YLD;
+    float *next_diag = reinterpret_cast<float *>(h->ws + wl.diag_off);
     // rank-NB (or super-panel) update of the columns to the left of panel p, on stream `us` with at most `sms` CTAs
     auto update = [&](int p, cudaStream_t us, int sms) -> gptaq_status_t {
         const int b0 = p * NB;
@@ -1136,24 +1136,21 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
     };
     auto factor_diag = [&](int p, const float *src, int64_t lds, int syrk, int pan_col0) -> gptaq_status_t {
         DiagFactorArgs da;
-        da.src = src; da.lds = lds; da.n = n; da.b0 = p * NB; da.Rdiag = Rinv + (size_t)p * NB * NB; da.Y = Y;
+        da.src = src; da.lds = lds; da.n = n; da.b0 = p * NB; da.Rdiag = Rinv + (size_t)p * NB * NB;
         da.syrk = syrk; da.pan_col0 = pan_col0; da.hd = h->hd;
-        CU(launch_pdl(true, diag_factor_kernel, dim3(1), dim3(DF_THREADS), DF_SMEM, s, pan_maps.a_hi, pan_maps.a_lo, da));
+        // (a second CTA inverts the block before)
+        da.H = H; da.inv_b0 = (p + 1) * NB; da.inv_Rdiag = da.Rdiag + NB * NB;
+        CU(launch_pdl(true, diag_factor_kernel, dim3(p + 1 < nb ? 2 : 1), dim3(DF_THREADS), DF_SMEM, s, pan_maps.a_hi, pan_maps.a_lo, da));
         h->launches++;
         return GPTAQ_OK;
     };
     // U = R^-1 of each diagonal block of SUPER_NB columns, a row of NB x NB blocks at a time and beside the factorisation:
-    //   U[p, p] = R_pp^-1,   U[p, > p] = -R_pp^-1 (R[p, > p] U[> p, > p])   (columns > p of the super-panel)
-    // The product in brackets needs the panels to the right only and runs while block p is being factored; when the last
-    // block is, little is left (by doubling 128 -> 1024 afterwards, every level waiting for the one before, 74 us at n = 1024
-    // and 175 at 4096).  Plain float32 products.  R is overwritten: row p comes after panel p is solved, hence after the
-    // update that reads it.  Nothing of this is put on the chain's own stream, where every event costs 4 us.
+    //   U[p, p] = R_pp^-1 (beside the next diagonal block),   U[p, > p] = -U[p, p] T[p, > p],   T[i, > i] = R[i, > i] U[> i, > i]
+    // T gathers the products of a row of U as soon as that row is there (rows i < p of the super-panel at once, 128 contraction
+    // steps each), so that little is left when the last block is factored.  Plain float32 products.
+    // R is overwritten: row p comes after panel p is solved, hence after the update that reads it.  Nothing of this is put on
+    // the chain's own stream, where every event costs 4 us.
     cudaStream_t is = nb > 1 ? h->inv_stream : s;
-    auto invert_diag = [&](int p, cudaStream_t st) -> gptaq_status_t {
-        invert_diag_blocks_kernel<<<1, ID_THREADS, ID_SMEM, st>>>(H, n, Rinv, p);
-        LAUNCHED();
-        return GPTAQ_OK;
-    };
     auto inverse_row = [&](int p) -> gptaq_status_t {
         const int b0 = p * NB, b1 = b0 + NB, e1 = std::min(b0 / SUPER_NB * SUPER_NB + SUPER_NB, n);
         if (b1 >= e1) return GPTAQ_OK;
@@ -1161,12 +1158,13 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
                                       H + (int64_t)b0 * n + b1, n, NB, e1 - b1, NB, -1.f, 0.f, GEMM_TRI_LEFT);
         return gemm(h, pu, false, true, is);
     };
-    // R[p, > p] U[> p, > p], once panel p + 1 is solved
-    auto inverse_product = [&](int p) -> gptaq_status_t {
-        const int b0 = p * NB, b1 = b0 + NB, e1 = std::min(b0 / SUPER_NB * SUPER_NB + SUPER_NB, n);
-        if (b1 >= e1) return GPTAQ_OK;
-        GemmProblem pt = make_problem(make_operand(H + (int64_t)b0 * n + b1, n, 1), make_operand(H + (int64_t)b1 * n + b1, 1, n),
-                                      T + (int64_t)b0 * n + b1, n, NB, e1 - b1, e1 - b1, 1.f, 0.f, GEMM_TRI_RIGHT);
+    // T[i, p ..] += R[i, p] U[p, p ..] for the rows i < p of the super-panel (the columns of block p receive their first term)
+    auto inverse_gather = [&](int p) -> gptaq_status_t {
+        const int b0 = p * NB, q0 = b0 / SUPER_NB * SUPER_NB, e1 = std::min(q0 + SUPER_NB, n);
+        if (b0 == q0) return GPTAQ_OK;
+        GemmProblem pt = make_problem(make_operand(H + (int64_t)q0 * n + b0, n, 1), make_operand(H + (int64_t)b0 * n + b0, 1, n),
+                                      T + (int64_t)q0 * n + b0, n, b0 - q0, e1 - b0, std::min(NB, n - b0), 1.f, 1.f, GEMM_FULL);
+        pt.fresh = NB;
         return gemm(h, pt, false, true, is);
     };
     // Rows of a panel may be read before the diagonal kernel in front of it has finished, because the update that made them is
@@ -1184,7 +1182,7 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         if (p == 0) break;
         const bool ahead = split && b0 > s0;   // the next panel is in the same super-panel: its block needs this panel only
         PanelSolveArgs pa;
-        pa.H = H; pa.n = n; pa.b0 = b0; pa.Rdiag = Rinv + (size_t)p * NB * NB; pa.Y = Y;
+        pa.H = H; pa.n = n; pa.b0 = b0; pa.Rdiag = Rinv + (size_t)p * NB * NB;
         pa.pan_hi = pan_hi; pa.pan_lo = pan_lo;
         pa.pan_ld = SUPER_NB; pa.pan_col0 = b0 - s0; pa.hd = h->hd;
         pa.next_diag = ahead ? next_diag : nullptr;
@@ -1199,31 +1197,31 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         if (rpt == 1) CU(launch_pdl(true, panel_solve_kernel<1>, pg, dim3(PS_THREADS), PS_SMEM, s, pa));
         else CU(launch_pdl(true, panel_solve_kernel<2>, pg, dim3(PS_THREADS), PS_SMEM, s, pa));
         h->launches++;
-        if (!ahead) {
-            CU(cudaEventRecord(h->inv_ready, s));
-            CU(cudaStreamWaitEvent(is, h->inv_ready, 0));
-            OK(invert_diag(p, is));
-            OK(inverse_row(p));
-            OK(inverse_product(p - 1));
-            OK(update(p, s, h->num_sms));
-            continue;
-        }
-        // the update on the internal stream, the next diagonal block beside it (one SM is left free for it)
-        CU(cudaEventRecord(h->conv_done[0], s));
-        CU(cudaStreamWaitEvent(h->gemm_stream, h->conv_done[0], 0));
-        OK(update(p, h->gemm_stream, h->num_sms - 1));
-        CU(cudaEventRecord(h->gemm_done[0], h->gemm_stream));
-        OK(factor_diag(p - 1, next_diag, NB, 1, b0 - s0));
-        CU(cudaStreamWaitEvent(s, h->gemm_done[0], 0));
-        diag_done = true;
-        OK(invert_diag(p, h->gemm_stream));
-        CU(cudaEventRecord(h->inv_ready, h->gemm_stream));
+        CU(cudaEventRecord(h->inv_ready, s));
         CU(cudaStreamWaitEvent(is, h->inv_ready, 0));
-        OK(inverse_row(p));
-        OK(inverse_product(p - 1));
+        if (ahead) {
+            // the update on the internal stream, the next diagonal block (and this one's inverse) beside it on two SMs left free
+            CU(cudaStreamWaitEvent(h->gemm_stream, h->inv_ready, 0));
+            OK(update(p, h->gemm_stream, h->num_sms - 2));
+            CU(cudaEventRecord(h->gemm_done[0], h->gemm_stream));
+            OK(factor_diag(p - 1, next_diag, NB, 1, b0 - s0));
+            CU(cudaStreamWaitEvent(s, h->gemm_done[0], 0));
+            diag_done = true;
+        } else OK(update(p, s, h->num_sms));
+        // (block p + 1 was inverted beside block p)
+        if (p + 1 < nb) {
+            OK(inverse_row(p + 1));
+            OK(inverse_gather(p + 1));
+        }
     }
-    // (block 0 is inverted on the chain's stream while the inverse's own stream ends with the product of row 0)
-    OK(invert_diag(0, s));
+    if (nb > 1) {
+        CU(cudaEventRecord(h->inv_ready, s));
+        CU(cudaStreamWaitEvent(is, h->inv_ready, 0));
+        OK(inverse_row(1));
+        OK(inverse_gather(1));
+    }
+    CU(launch_pdl(true, invert_diag_block_kernel, dim3(1), dim3(ID_THREADS), ID_SMEM, s, H, n, 0, static_cast<const float *>(Rinv)));
+    h->launches++;
     if (nb > 1) {
         CU(cudaEventRecord(h->inv_done, is));
         CU(cudaStreamWaitEvent(s, h->inv_done, 0));

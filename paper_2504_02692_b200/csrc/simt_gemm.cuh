@@ -50,6 +50,7 @@ struct GemmProblem {
     int paired, pair_mode;
     const float *pair_sub;
     float *pair_C;
+    int fresh;              // columns below this one are written without what C holds (beta counts for the others)
 };
 
 constexpr int GBM = 128, GBN = 128, GBK = 16, GPAD = 4;
@@ -235,7 +236,7 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(GemmProblem pr) {
             bool masked = (mode == GEMM_O || mode == GEMM_P);
             if (j + 3 < N && ((reinterpret_cast<uintptr_t>(cp) & 15) == 0)) {
                 float4 t = make_float4(o[0], o[1], o[2], o[3]);
-                if (beta != 0.f && !masked) {
+                if (beta != 0.f && !masked && j >= pr.fresh) {          // (fresh: a multiple of 4)
                     float4 c = *reinterpret_cast<const float4 *>(cp);
                     t.x += beta * c.x; t.y += beta * c.y; t.z += beta * c.z; t.w += beta * c.w;
                 }
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(GemmProblem pr) {
             } else {
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    if (j + e < N) cp[e] = o[e] + ((beta != 0.f && !masked) ? beta * cp[e] : 0.f);
+                    if (j + e < N) cp[e] = o[e] + ((beta != 0.f && !masked && j + e >= pr.fresh) ? beta * cp[e] : 0.f);
             }
         }
     }
@@ -363,13 +364,18 @@ __global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, 
 #pragma unroll
         for (int f = 0; f < 4; ++f) {
             const int i = i0 + (A_RC ? 4 * ti + e : ti + 8 * e), j = j0 + (B_RC ? 4 * tj + f : tj + 8 * f);
-            cv[e][f] = (add_c && ksplit == 1 && i < M && j < N) ? C[(int64_t)i * pr.ldc + j] : 0.f;
+            cv[e][f] = (add_c && ksplit == 1 && i < M && j < N && j >= pr.fresh) ? C[(int64_t)i * pr.ldc + j] : 0.f;
         }
     for (int t = 0; t < nk; ++t) {
         asm volatile("cp.async.wait_group %0;" ::"n"(SG_STAGES - 2) : "memory");
         __syncthreads();
         fetch(t + SG_STAGES - 1);                                     // into the stage that was read last step
         const float *st = sg_smem + (t % SG_STAGES) * stage_floats;
+        float part[4][4];                                             // (a stage's 32 terms by themselves: shorter chains of roundings)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int f = 0; f < 4; ++f) part[e][f] = 0.f;
 #pragma unroll 2
         for (int k = 0; k < SGK; k += 4) {
             float av[4][4], bv[4][4];
@@ -388,8 +394,12 @@ __global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, 
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
 #pragma unroll
-                    for (int f = 0; f < 4; ++f) acc[e][f] = fmaf(av[q][e], bv[q][f], acc[e][f]);
+                    for (int f = 0; f < 4; ++f) part[e][f] = fmaf(av[q][e], bv[q][f], part[e][f]);
         }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int f = 0; f < 4; ++f) acc[e][f] += part[e][f];
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
 
@@ -421,7 +431,7 @@ __global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, 
 #pragma unroll
     for (int q = 0; q < SGT * SGT / 2 / SG_THREADS; ++q) {
         const int idx = tid + q * SG_THREADS, i = i0 + part * rows + (idx >> 5), j = j0 + (idx & 31);
-        own[q] = (add_c && idx < rows * SGT && i < M && j < N) ? C[(int64_t)i * pr.ldc + j] : 0.f;
+        own[q] = (add_c && idx < rows * SGT && i < M && j < N && j >= pr.fresh) ? C[(int64_t)i * pr.ldc + j] : 0.f;
     }
 #pragma unroll
     for (int q = 0; q < SGT * SGT / 2 / SG_THREADS; ++q) {
@@ -494,7 +504,7 @@ inline GemmProblem make_problem(Operand A, Operand B, float *C, int64_t ldc, int
     GemmProblem p; p.A = A; p.B = B; p.C = C; p.ldc = ldc; p.M = M; p.N = N; p.K = K;
     p.alpha = alpha; p.beta = beta; p.mode = mode; p.batchA = p.batchB = p.batchC = 0;
     p.batchM_last = p.batchN_last = p.batchK_last = 0; p.nbatch = 1;
-    p.paired = p.pair_mode = 0; p.pair_sub = nullptr; p.pair_C = nullptr; return p;
+    p.paired = p.pair_mode = 0; p.pair_sub = nullptr; p.pair_C = nullptr; p.fresh = 0; return p;
 }
 
 }  // namespace gptaq

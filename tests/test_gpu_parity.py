@@ -751,6 +751,12 @@ def test_factor_panels(n):
     assert np.linalg.norm(U - ref) <= bound * np.linalg.norm(ref), (hp.rel_fro(U, ref), bound)
 
 
+# (a diagonal block's pieces of eight columns and sub-blocks of 32, and the block beside which another is inverted)
+@pytest.mark.parametrize("n", [7, 33, 64, 97, 128, 136])
+def test_factor_inside_a_block(n):
+    test_factor_panels(n)
+
+
 @pytest.mark.parametrize("n", [512, 516, 1036, 1284])
 def test_split_operand_row_pitch(n):
     """Tensor-core products whose fp16 operand copies have rows of 8 k and of 8 k + 4 columns (row pitch padded to a multiple
