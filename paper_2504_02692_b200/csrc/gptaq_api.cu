@@ -163,9 +163,9 @@ gptaq_status_t cuda_fail(gptaq_ctx *h, cudaError_t e) {
         h->launches++;                                       \
     } while (0)
 
-gptaq_status_t gemm(gptaq_ctx *h, const GemmProblem &p, bool a_rc, bool b_rc, cudaStream_t s) {
+gptaq_status_t gemm(gptaq_ctx *h, const GemmProblem &p, bool a_rc, bool b_rc, cudaStream_t s, bool pdl = false) {
     if (p.M <= 0 || p.N <= 0 || p.nbatch <= 0) return GPTAQ_OK;
-    cudaError_t e = launch_simt_gemm(p, a_rc, b_rc, s);
+    cudaError_t e = launch_simt_gemm(p, a_rc, b_rc, s, pdl);
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->launches++;
     return GPTAQ_OK;
@@ -326,8 +326,7 @@ Split16Args split16_args(const float *src, int64_t lds, __half *hi, __half *lo, 
 cudaError_t launch_split16(const Split16Args &a, cudaStream_t s, const Split16Args *second = nullptr) {
     if (a.rows <= 0 || a.cols <= 0 || a.nbatch <= 0) return cudaSuccess;
     dim3 grid((a.cols + 63) / 64, (a.rows + 63) / 64, a.nbatch + (second ? 1 : 0));
-    split16_kernel<<<grid, 256, 0, s>>>(a, second ? *second : a);
-    return cudaGetLastError();
+    return launch_pdl(true, split16_kernel, grid, dim3(256), 0, s, a, second ? *second : a);
 }
 
 // Scratch of the statistics kernel's K-split tail: at most one 128 x 256 partial tile per SM.
@@ -434,8 +433,9 @@ gptaq_status_t accumulate_tc(gptaq_ctx *h, const float *X, const float *Xfp, int
         dim3 cgrid(kp / 64, (n + 63) / 64);
         convert_transpose_kernel<0><<<cgrid, 256, 0, s>>>(ca);
         LAUNCHED();
-        convert_transpose_kernel<1><<<std::min<unsigned>(cgrid.x * cgrid.y, 4u * (unsigned)h->num_sms), 256, 0, s>>>(ca);
-        LAUNCHED();
+        CU(launch_pdl(true, convert_transpose_kernel<1>, dim3(std::min<unsigned>(cgrid.x * cgrid.y, 4u * (unsigned)h->num_sms)), dim3(256),
+                      0, s, ca));
+        h->launches++;
         CU(cudaEventRecord(h->conv_done[buf], s));
         CU(cudaStreamWaitEvent(gs, h->conv_done[buf], 0));
         gptaq_ctx::StatsMaps &mp = h->stats_maps[buf];
@@ -585,12 +585,13 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
     // A grid per column (static groups) takes one always: two have no registers left for it, and gain nothing (16384 rows of
     // 400 columns 517 us with one, 519 with two; 8192 of 1023 1227, 1221).
     const bool two = grid.x > (unsigned)t.num_sms && !static_groups;
-    if (far_form && static_groups) quant_block_kernel<true, true, 1><<<grid, QB_THREADS_FAR, smem, s>>>(uh, ul, ph, pl, a);
-    else if (far_form) quant_block_kernel<true, false, 1><<<grid, QB_THREADS_FAR, smem, s>>>(uh, ul, ph, pl, a);
-    else if (static_groups) quant_block_kernel<false, true, 1><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
-    else if (two) quant_block_kernel<false, false, 2><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
-    else quant_block_kernel<false, false, 1><<<grid, QB_THREADS_NEAR, smem, s>>>(uh, ul, ph, pl, a);
-    return cudaGetLastError();
+    // Near form, from the second launch of a call on: it starts while the product before it drains, and reads U and P meanwhile
+    // (the first one waits for all that made them).
+    const bool pdl = !far_form && i0 > 0;
+    auto launch = [&](auto kernel, int threads) { return launch_pdl(pdl, kernel, grid, dim3(threads), smem, s, uh, ul, ph, pl, a); };
+    if (far_form) return static_groups ? launch(quant_block_kernel<true, true, 1>, QB_THREADS_FAR) : launch(quant_block_kernel<true, false, 1>, QB_THREADS_FAR);
+    if (static_groups) return launch(quant_block_kernel<false, true, 1>, QB_THREADS_NEAR);
+    return two ? launch(quant_block_kernel<false, false, 2>, QB_THREADS_NEAR) : launch(quant_block_kernel<false, false, 1>, QB_THREADS_NEAR);
 }
 
 // Raises the shared-memory limits of the kernels of the column loop.
@@ -784,7 +785,7 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
             bop.p2 = t.P + (int64_t)i0 * n + i1;
             bop.k_split = SW;
             GemmProblem pt = make_problem(make_operand(EW, 2 * SW, 1), bop, Wk + i1, ldk, (int)m, n - i1, 2 * SW, 1.f, 1.f, GEMM_FULL);
-            *err = launch_simt_gemm(pt, false, true, s);
+            *err = launch_simt_gemm(pt, false, true, s, steps);
             if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
             ++*launches;
         }
@@ -1087,8 +1088,9 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         permute_symmetric_kernel<<<dim3((n + 255) / 256, n), 256, 0, s>>>(H, T, n, h->perm);
         LAUNCHED();
     }
-    scale_damp_kernel<<<dim3((n + 63) / 64, (n + 15) / 16), 256, 0, s>>>(h->act_order ? T : H, H, n, h->hd, h->dead);
-    LAUNCHED();
+    CU(launch_pdl(true, scale_damp_kernel, dim3((n + 63) / 64, (n + 15) / 16), dim3(256), 0, s, static_cast<const float *>(h->act_order ? T : H),
+                  H, n, static_cast<const StateHeader *>(h->hd), static_cast<const uint8_t *>(h->dead)));
+    h->launches++;
 
     // Rank updates and the inverse on split operands, with damping: the rows of R lie between sqrt(lambda) and
     // sqrt(max diag H_d), those of its inverse between 1 / sqrt of these, and as lambda = damp * mean(diag) the two are at most
@@ -1156,7 +1158,7 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         if (b1 >= e1) return GPTAQ_OK;
         GemmProblem pu = make_problem(make_operand(H + (int64_t)b0 * n + b0, n, 1), make_operand(T + (int64_t)b0 * n + b1, 1, n),
                                       H + (int64_t)b0 * n + b1, n, NB, e1 - b1, NB, -1.f, 0.f, GEMM_TRI_LEFT);
-        return gemm(h, pu, false, true, is);
+        return gemm(h, pu, false, true, is, true);
     };
     // T[i, p ..] += R[i, p] U[p, p ..] for the rows i < p of the super-panel (the columns of block p receive their first term)
     auto inverse_gather = [&](int p) -> gptaq_status_t {
@@ -1165,7 +1167,7 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         GemmProblem pt = make_problem(make_operand(H + (int64_t)q0 * n + b0, n, 1), make_operand(H + (int64_t)b0 * n + b0, 1, n),
                                       T + (int64_t)q0 * n + b0, n, b0 - q0, e1 - b0, std::min(NB, n - b0), 1.f, 1.f, GEMM_FULL);
         pt.fresh = NB;
-        return gemm(h, pt, false, true, is);
+        return gemm(h, pt, false, true, is, true);
     };
     // Rows of a panel may be read before the diagonal kernel in front of it has finished, because the update that made them is
     // waited for by an event.  In a captured graph that event becomes an edge of the same programmatic kind as the one from

@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(1024) diag_stats_kernel(const float *H, int n,
                                                           uint8_t *dead, uint8_t *dead_working) {
     __shared__ double red[1024];
     __shared__ float redmax[1024];
+    pdl_launch_dependents();
     double s = 0.0;
     float mx = 0.f;
     for (int q = threadIdx.x; q < n; q += 1024) {
@@ -107,6 +108,8 @@ __global__ void __launch_bounds__(1024) diag_stats_kernel(const float *H, int n,
 // (src: H itself, or the matrix in sorted order.)
 __global__ void __launch_bounds__(256) scale_damp_kernel(const float *src, float *H, int n, const StateHeader *hd,
                                                          const uint8_t *dead) {
+    pdl_launch_dependents();
+    pdl_wait();
     const int j = blockIdx.x * 64 + 4 * (threadIdx.x & 15), i = blockIdx.y * 16 + (threadIdx.x >> 4);
     if (j >= n || i >= n) return;
     const float inv = hd->inv_tokens, lam = hd->lambda;

@@ -297,7 +297,11 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
     }
-    // the slab and the first rows of U and P all in flight at once (8k cycles; in batches through registers twice that)
+    // the slab and the first rows of U and P all in flight at once (8k cycles; in batches through registers twice that); U and P
+    // without waiting for the launch before this one
+    if (!FAR) pdl_launch_dependents();
+    fetch_up(i0, 0, tid, NTHREADS);
+    if (!FAR) pdl_wait();
     const int cq = FAR ? nblk * (QB_W / 4) : B / 4;                // quads per row, padded columns included
     const bool wvec = (a.ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(a.W) & 15) == 0;       // (i0 is a multiple of 32)
     // a thread: four columns of every RSTEP-th row
@@ -319,7 +323,6 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     }
     // (dead inputs read as zero; the flags are 4-byte aligned and padded beyond n)
     const uint32_t dead4 = fills && wc < cols ? *reinterpret_cast<const uint32_t *>(a.dead + i0 + wc) : 0u;
-    fetch_up(i0, 0, tid, NTHREADS);
     if (tid < 32) { udinv2[tid] = load_pivot(i0 + tid); perm2[tid] = load_perm(i0 + tid); }
     if (PERCOL && tid < QB_NEAR) {
         float sc[4], zp[4];

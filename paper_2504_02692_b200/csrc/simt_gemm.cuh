@@ -295,6 +295,8 @@ template <bool A_RC, bool B_RC>
 __global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, int ksplit) {
     extern __shared__ __align__(16) float sg_smem[];
     const int tid = threadIdx.x;
+    pdl_launch_dependents();
+    pdl_wait();                                                       // (nothing before it: products may follow each other closely)
     const int z = blockIdx.z / ksplit, part = blockIdx.z - z * ksplit;
     int M = pr.M, N = pr.N, K = pr.K;
     if (z == pr.nbatch - 1) {
@@ -462,7 +464,7 @@ inline int64_t simt_tiles(const GemmProblem &pr) {
 constexpr int64_t SIMT_SMALL_TILES = 60;
 
 template <bool A_RC, bool B_RC>
-inline cudaError_t launch_simt_small(const GemmProblem &pr, cudaStream_t s) {
+inline cudaError_t launch_simt_small(const GemmProblem &pr, cudaStream_t s, bool pdl) {
     dim3 grid((pr.N + SGT - 1) / SGT, (pr.M + SGT - 1) / SGT, pr.nbatch);
     // long contractions of few tiles (the statistics of narrow layers) are shared by up to eight CTAs per tile
     int ksplit = 1;
@@ -472,20 +474,23 @@ inline cudaError_t launch_simt_small(const GemmProblem &pr, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(SG_THREADS); cfg.stream = s;
     cfg.dynamicSmemBytes = (size_t)SG_STAGES * (pr.A.sub || pr.paired ? 3 : 2) * SG_TILE * sizeof(float);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = (unsigned)ksplit;
-    cfg.attrs = attr; cfg.numAttrs = ksplit > 1 ? 1 : 0;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = (unsigned)ksplit;
+    cfg.attrs = attr; cfg.numAttrs = ksplit > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, simt_small_kernel<A_RC, B_RC>, pr, ksplit);
 }
 
-inline cudaError_t launch_simt_gemm(const GemmProblem &pr, bool a_rc, bool b_rc, cudaStream_t s) {
+// pdl: the 32 x 32 form may start while the kernel before it drains
+inline cudaError_t launch_simt_gemm(const GemmProblem &pr, bool a_rc, bool b_rc, cudaStream_t s, bool pdl = false) {
     if (pr.M <= 0 || pr.N <= 0 || pr.nbatch <= 0) return cudaSuccess;
     if (simt_tiles(pr) <= SIMT_SMALL_TILES && !pr.B.sub) {
-        if (a_rc && b_rc) return launch_simt_small<true, true>(pr, s);
-        if (a_rc) return launch_simt_small<true, false>(pr, s);
-        if (b_rc) return launch_simt_small<false, true>(pr, s);
-        return launch_simt_small<false, false>(pr, s);
+        if (a_rc && b_rc) return launch_simt_small<true, true>(pr, s, pdl);
+        if (a_rc) return launch_simt_small<true, false>(pr, s, pdl);
+        if (b_rc) return launch_simt_small<false, true>(pr, s, pdl);
+        return launch_simt_small<false, false>(pr, s, pdl);
     }
     dim3 grid((pr.N + GBN - 1) / GBN, (pr.M + GBM - 1) / GBM, pr.nbatch);
     if (a_rc && b_rc) simt_gemm_kernel<true, true><<<grid, 256, 0, s>>>(pr);

@@ -511,6 +511,7 @@ __global__ void __launch_bounds__(256) absmax_kernel(AbsmaxArgs a0, AbsmaxArgs a
     __shared__ float red[BATCH][8];
     float m = 0.f;
     int kept = 0;
+    pdl_launch_dependents();
     const bool vec = (lds & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
     for (int r = blockIdx.x; r < rows; r += gridDim.x) {
         const int cb = mask == SPLIT_ALL ? 0 : (mask == SPLIT_UPPER ? r : r + 1);     // first column kept
@@ -593,6 +594,8 @@ __device__ __forceinline__ void split16_pack(const float (&x)[4], uint2 &hi, uin
 __global__ void __launch_bounds__(256) split16_kernel(Split16Args a, Split16Args second) {
     __shared__ float tile[64][65];
     const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
+    pdl_launch_dependents();
+    pdl_wait();
     {
         int z = blockIdx.z;
         if (z == a.nbatch) { a = second; z = 0; }

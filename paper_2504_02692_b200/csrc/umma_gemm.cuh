@@ -186,6 +186,7 @@ __global__ void __launch_bounds__(256) convert_transpose_kernel(ConvertArgs a) {
     __shared__ uint32_t sl[CVT_WORDS];
     __shared__ uint32_t sdl[CVT_WORDS];
     if (PASS == 1) {
+        pdl_wait();                  // (launched while pass 0 drains: its own start costs nothing)
         const float scx = pick_scale(__uint_as_float(a.amax[0]));
         const float scd = pick_scale(__uint_as_float(a.amax[1]));
         if (scx == 1.f && scd == 1.f) return;
@@ -195,6 +196,7 @@ __global__ void __launch_bounds__(256) convert_transpose_kernel(ConvertArgs a) {
             __syncthreads();
         }
     } else {
+        pdl_launch_dependents();
         convert_tile<0>(a, blockIdx.x * 64, blockIdx.y * 64, 1.f, 1.f, sx, sd, sl, sdl);
     }
 }
