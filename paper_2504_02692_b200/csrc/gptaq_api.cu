@@ -107,7 +107,7 @@ inline int64_t split_pitch(int64_t n) { return (n + 7) / 8 * 8; }
 
 struct WsLayout {
     size_t t_off, rinv_off;
-    size_t diag_off;        // inverses of the current diagonal block's sub-blocks, copy of the next diagonal block
+    size_t diag_off;        // copy of the next diagonal block
     size_t s_off[3];        // split operand matrices, fp16 hi then lo (n x split_pitch(n) each)
     size_t pan_off[2];      // split copy of factor panels, hi / lo: n x SUPER_NB fp16
     // [-Err | Wpre] of a launch: float32, its fp16 hi / lo parts (tensor cores), row scales
@@ -131,7 +131,7 @@ WsLayout ws_layout(int64_t n, int64_t m_max) {
     w.t_off = 0;
     w.rinv_off = w.t_off + mat;
     w.diag_off = w.rinv_off + round_up(nb * NB * NB * sizeof(float), ALIGN);
-    size_t off = w.diag_off + round_up((4 * 32 * FP_YLD + NB * NB) * sizeof(float), ALIGN);
+    size_t off = w.diag_off + round_up(NB * NB * sizeof(float), ALIGN);
     // S0 = U^T, S1 = U then P^T, S2 = dXX^T then O
     const size_t smat = round_up(2 * (size_t)n * (size_t)split_pitch(n) * sizeof(__half), ALIGN);
     for (int i = 0; i < 3; ++i) { w.s_off[i] = off; if (w.tensor) off += smat; }
@@ -245,7 +245,7 @@ bool make_tc_maps(TcMaps *m, const SplitOperand &A, const SplitOperand &B, const
 // Launch with programmatic stream serialization: the kernel may be scheduled while its predecessor
 // drains; it calls pdl_wait() before it touches anything the predecessor wrote.
 // (Measured on a 4096-wide layer: the factorisation's chain of short launches gains 4 %, the quantize
-// chain loses 4 %, so only the former uses it.)
+// chain on the tensor cores loses 4 %, so it alone does not use it.)
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
