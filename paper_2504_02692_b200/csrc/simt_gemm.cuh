@@ -50,7 +50,9 @@ struct GemmProblem {
     int paired, pair_mode;
     const float *pair_sub;
     float *pair_C;
-    int fresh;              // columns below this one are written without what C holds (beta counts for the others)
+    // columns below this one are written without what C holds (beta counts for the others); the 32 x 32 form with K in one piece
+    // knows it alone, the launch refuses it elsewhere
+    int fresh;
 };
 
 constexpr int GBM = 128, GBN = 128, GBK = 16, GPAD = 4;
@@ -236,7 +238,7 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(GemmProblem pr) {
             bool masked = (mode == GEMM_O || mode == GEMM_P);
             if (j + 3 < N && ((reinterpret_cast<uintptr_t>(cp) & 15) == 0)) {
                 float4 t = make_float4(o[0], o[1], o[2], o[3]);
-                if (beta != 0.f && !masked && j >= pr.fresh) {          // (fresh: a multiple of 4)
+                if (beta != 0.f && !masked) {
                     float4 c = *reinterpret_cast<const float4 *>(cp);
                     t.x += beta * c.x; t.y += beta * c.y; t.z += beta * c.z; t.w += beta * c.w;
                 }
@@ -244,7 +246,7 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(GemmProblem pr) {
             } else {
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    if (j + e < N) cp[e] = o[e] + ((beta != 0.f && !masked && j + e >= pr.fresh) ? beta * cp[e] : 0.f);
+                    if (j + e < N) cp[e] = o[e] + ((beta != 0.f && !masked) ? beta * cp[e] : 0.f);
             }
         }
     }
@@ -373,11 +375,11 @@ __global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, 
         __syncthreads();
         fetch(t + SG_STAGES - 1);                                     // into the stage that was read last step
         const float *st = sg_smem + (t % SG_STAGES) * stage_floats;
-        float part[4][4];                                             // (a stage's 32 terms by themselves: shorter chains of roundings)
+        float sum[4][4];                                              // (a stage's 32 terms by themselves: shorter chains of roundings)
 #pragma unroll
         for (int e = 0; e < 4; ++e)
 #pragma unroll
-            for (int f = 0; f < 4; ++f) part[e][f] = 0.f;
+            for (int f = 0; f < 4; ++f) sum[e][f] = 0.f;
 #pragma unroll 2
         for (int k = 0; k < SGK; k += 4) {
             float av[4][4], bv[4][4];
@@ -396,12 +398,12 @@ __global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, 
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
 #pragma unroll
-                    for (int f = 0; f < 4; ++f) part[e][f] = fmaf(av[q][e], bv[q][f], part[e][f]);
+                    for (int f = 0; f < 4; ++f) sum[e][f] = fmaf(av[q][e], bv[q][f], sum[e][f]);
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e)
 #pragma unroll
-            for (int f = 0; f < 4; ++f) acc[e][f] += part[e][f];
+            for (int f = 0; f < 4; ++f) acc[e][f] += sum[e][f];
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
 
@@ -433,7 +435,7 @@ __global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, 
 #pragma unroll
     for (int q = 0; q < SGT * SGT / 2 / SG_THREADS; ++q) {
         const int idx = tid + q * SG_THREADS, i = i0 + part * rows + (idx >> 5), j = j0 + (idx & 31);
-        own[q] = (add_c && idx < rows * SGT && i < M && j < N && j >= pr.fresh) ? C[(int64_t)i * pr.ldc + j] : 0.f;
+        own[q] = (add_c && idx < rows * SGT && i < M && j < N) ? C[(int64_t)i * pr.ldc + j] : 0.f;
     }
 #pragma unroll
     for (int q = 0; q < SGT * SGT / 2 / SG_THREADS; ++q) {
@@ -470,6 +472,7 @@ inline cudaError_t launch_simt_small(const GemmProblem &pr, cudaStream_t s, bool
     int ksplit = 1;
     const int64_t tiles = (int64_t)grid.x * grid.y * grid.z;
     while (ksplit < 8 && tiles * ksplit <= 592 && pr.K / (2 * ksplit) >= 128) ksplit *= 2;      // 592: four CTAs per SM
+    if (pr.fresh > 0 && ksplit > 1) return cudaErrorInvalidValue;
     grid.z *= ksplit;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(SG_THREADS); cfg.stream = s;
@@ -492,6 +495,7 @@ inline cudaError_t launch_simt_gemm(const GemmProblem &pr, bool a_rc, bool b_rc,
         if (b_rc) return launch_simt_small<false, true>(pr, s, pdl);
         return launch_simt_small<false, false>(pr, s, pdl);
     }
+    if (pr.fresh > 0) return cudaErrorInvalidValue;
     dim3 grid((pr.N + GBN - 1) / GBN, (pr.M + GBM - 1) / GBM, pr.nbatch);
     if (a_rc && b_rc) simt_gemm_kernel<true, true><<<grid, 256, 0, s>>>(pr);
     else if (a_rc && !b_rc) simt_gemm_kernel<true, false><<<grid, 256, 0, s>>>(pr);
