@@ -163,9 +163,9 @@ gptaq_status_t cuda_fail(gptaq_ctx *h, cudaError_t e) {
         h->launches++;                                       \
     } while (0)
 
-gptaq_status_t gemm(gptaq_ctx *h, const GemmProblem &p, bool a_rc, bool b_rc, cudaStream_t s, bool pdl = false) {
+gptaq_status_t gemm(gptaq_ctx *h, const GemmProblem &p, bool a_rc, bool b_rc, cudaStream_t s, int early_ctas = 0) {
     if (p.M <= 0 || p.N <= 0 || p.nbatch <= 0) return GPTAQ_OK;
-    cudaError_t e = launch_simt_gemm(p, a_rc, b_rc, s, pdl);
+    cudaError_t e = launch_simt_gemm(p, a_rc, b_rc, s, early_ctas);
     if (e != cudaSuccess) return cuda_fail(h, e);
     h->launches++;
     return GPTAQ_OK;
@@ -242,10 +242,15 @@ bool make_tc_maps(TcMaps *m, const SplitOperand &A, const SplitOperand &B, const
            make_operand_map(&m->b2_hi, b2.hi, b2, TBOX) && make_operand_map(&m->b2_lo, b2.lo, b2, TBOX);
 }
 
-// Launch with programmatic stream serialization: the kernel may be scheduled while its predecessor
+// Launch with programmatic stream serialization where `pdl` is set: the kernel may be scheduled while its predecessor
 // drains; it calls pdl_wait() before it touches anything the predecessor wrote.
-// (Measured on a 4096-wide layer: the factorisation's chain of short launches gains 4 %, the quantize
-// chain on the tensor cores loses 4 %, so it alone does not use it.)
+// So start: the factorisation's chain (4 % of it at n = 4096; the damping up to 3 us up to n = 2052, the inverse of block 0
+// 3 us up to n = 128) and the tensor-core products of gptaq_factor and gptaq_build_P; the second pass of the statistics'
+// conversion (2 to 4 us a call; back to back 4 calls of 4112 tokens at n = 1024 141 -> 135, of 2777 at n = 2052 392 -> 396);
+// split copies and small float32 products of few CTAs (launch_split16, launch_simt_gemm); the column loop without tensor cores
+// from its second launch on (launch_quant_block).  All else is launched plainly: the column loop on the tensor cores and its
+// products (4 % slower so), column_loop_kernel, the statistics products, what a call begins with (copies, permutations, grids,
+// maxima).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -323,10 +328,14 @@ Split16Args split16_args(const float *src, int64_t lds, __half *hi, __half *lo, 
     a.hi_t = hi_t; a.lo_t = lo_t; a.row_inv = row_inv;
     return a;
 }
-cudaError_t launch_split16(const Split16Args &a, cudaStream_t s, const Split16Args *second = nullptr) {
+// Starts early where that takes no more than a CTA per SM: those that are there before their turn hold the SMs that the product in
+// front leaves free, several to an SM, and work there.  us plain / always early / by this rule: gptaq_build_P at n = 640
+// 50 / 49 / 46, 768 54 / 64 / 52, 1024 64 / 72 / 64, 4096 356 / 362 / 356; gptaq_factor at n = 1536 417 / 424 / 418.
+cudaError_t launch_split16(const Split16Args &a, int num_sms, cudaStream_t s, const Split16Args *second = nullptr) {
     if (a.rows <= 0 || a.cols <= 0 || a.nbatch <= 0) return cudaSuccess;
     dim3 grid((a.cols + 63) / 64, (a.rows + 63) / 64, a.nbatch + (second ? 1 : 0));
-    return launch_pdl(true, split16_kernel, grid, dim3(256), 0, s, a, second ? *second : a);
+    const bool early = (int64_t)grid.x * grid.y * grid.z <= num_sms;
+    return launch_pdl(early, split16_kernel, grid, dim3(256), 0, s, a, second ? *second : a);
 }
 
 // Scratch of the statistics kernel's K-split tail: at most one 128 x 256 partial tile per SM.
@@ -586,7 +595,8 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
     // 400 columns 517 us with one, 519 with two; 8192 of 1023 1227, 1221).
     const bool two = grid.x > (unsigned)t.num_sms && !static_groups;
     // Near form, from the second launch of a call on: it starts while the product before it drains, and reads U and P meanwhile
-    // (the first one waits for all that made them).
+    // (1000 rows of 1024 columns 256 -> 242 us a call).  That takes two things: the first launch of a call is a plain one, so that
+    // all that made U and P is done before the call's first kernel begins, in a captured graph too; and nothing in a call writes U or P.
     const bool pdl = !far_form && i0 > 0;
     auto launch = [&](auto kernel, int threads) { return launch_pdl(pdl, kernel, grid, dim3(threads), smem, s, uh, ul, ph, pl, a); };
     if (far_form) return static_groups ? launch(quant_block_kernel<true, true, 1>, QB_THREADS_FAR) : launch(quant_block_kernel<true, false, 1>, QB_THREADS_FAR);
@@ -784,8 +794,10 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
             Operand bop = make_operand(t.U + (int64_t)i0 * n + i1, 1, n);
             bop.p2 = t.P + (int64_t)i0 * n + i1;
             bop.k_split = SW;
+            // (early up to four CTAs per SM, the column loop leaves most of the SMs free: 128 x 1024 194 us plain, 182 early; 256 x 1024,
+            // 448 CTAs at first, 198 and 192; 512 x 1024, 896 CTAs, 213 and 224; 1000 x 1024 242 and 250)
             GemmProblem pt = make_problem(make_operand(EW, 2 * SW, 1), bop, Wk + i1, ldk, (int)m, n - i1, 2 * SW, 1.f, 1.f, GEMM_FULL);
-            *err = launch_simt_gemm(pt, false, true, s, steps);
+            *err = launch_simt_gemm(pt, false, true, s, steps ? 4 * t.num_sms : 0);
             if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
             ++*launches;
         }
@@ -1152,13 +1164,16 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
     // steps each), so that little is left when the last block is factored.  Plain float32 products.
     // R is overwritten: row p comes after panel p is solved, hence after the update that reads it.  Nothing of this is put on
     // the chain's own stream, where every event costs 4 us.
+    // These products start early where they have at most a CTA per SM: more of them sit on SMs that the chain's kernels beside
+    // them want whole (gptaq_factor, us plain / always early / so: n = 512 136 / 134 / 134, 1024 249 / 252 / 247,
+    // 2048 561 / 578 / 559, 4096 1268 / 1313 / 1266).
     cudaStream_t is = nb > 1 ? h->inv_stream : s;
     auto inverse_row = [&](int p) -> gptaq_status_t {
         const int b0 = p * NB, b1 = b0 + NB, e1 = std::min(b0 / SUPER_NB * SUPER_NB + SUPER_NB, n);
         if (b1 >= e1) return GPTAQ_OK;
         GemmProblem pu = make_problem(make_operand(H + (int64_t)b0 * n + b0, n, 1), make_operand(T + (int64_t)b0 * n + b1, 1, n),
                                       H + (int64_t)b0 * n + b1, n, NB, e1 - b1, NB, -1.f, 0.f, GEMM_TRI_LEFT);
-        return gemm(h, pu, false, true, is, true);
+        return gemm(h, pu, false, true, is, h->num_sms);
     };
     // T[i, p ..] += R[i, p] U[p, p ..] for the rows i < p of the super-panel (the columns of block p receive their first term)
     auto inverse_gather = [&](int p) -> gptaq_status_t {
@@ -1167,7 +1182,7 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         GemmProblem pt = make_problem(make_operand(H + (int64_t)q0 * n + b0, n, 1), make_operand(H + (int64_t)b0 * n + b0, 1, n),
                                       T + (int64_t)q0 * n + b0, n, b0 - q0, e1 - b0, std::min(NB, n - b0), 1.f, 1.f, GEMM_FULL);
         pt.fresh = NB;
-        return gemm(h, pt, false, true, is, true);
+        return gemm(h, pt, false, true, is, h->num_sms);
     };
     // Rows of a panel may be read before the diagonal kernel in front of it has finished, because the update that made them is
     // waited for by an event.  In a captured graph that event becomes an edge of the same programmatic kind as the one from
@@ -1253,17 +1268,17 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
             SplitBatch sbt = sb; sbt.cols_last = tail;
             SplitBatch sbc = sb; sbc.rows_last = tail; sbc.cols_last = tail;
             CU(cudaMemsetAsync(am + AMAX_T, 0, sizeof(unsigned), s));
-            CU(launch_split16(split16_args(H + sz, n, A1 + sz, A1 + nn + sz, ldt, (int)sz, (int)sz, false, SPLIT_ALL, 1.f, am + AMAX_PAN, sbt), s));
+            CU(launch_split16(split16_args(H + sz, n, A1 + sz, A1 + nn + sz, ldt, (int)sz, (int)sz, false, SPLIT_ALL, 1.f, am + AMAX_PAN, sbt), h->num_sms, s));
             CU(launch_split16(split16_args(H + sz * n + sz, n, B2 + sz * ldt + sz, B2 + nn + sz * ldt + sz, ldt, (int)sz, (int)sz, true,
-                                           SPLIT_UPPER, 1.f, am + AMAX_INV, sbc), s));
+                                           SPLIT_UPPER, 1.f, am + AMAX_INV, sbc), h->num_sms, s));
             TcGemmArgs g1 = tc_args(T + sz, n, (int)sz, (int)sz, (int)sz, 1.f, 0.f, TC_TRI_RIGHT, TC_MASK_NONE, h->hd);
             g1.nbatch = np; g1.c_bstride = bstride; g1.N_last = tail; g1.K_last = tail;
             g1.a_row0 = 0; g1.a_row_bs = (int)(2 * sz); g1.a_k0 = (int)sz; g1.a_k_bs = (int)(2 * sz);
             g1.b_row0 = (int)sz; g1.b_row_bs = (int)(2 * sz); g1.b_k0 = (int)sz; g1.b_k_bs = (int)(2 * sz);
             g1.amax_a = am + AMAX_PAN; g1.amax_b = am + AMAX_INV; g1.amax_out = am + AMAX_T;
             CU(launch_tc_gemm(m16, g1, h->num_sms, s));
-            CU(launch_split16(split16_args(H, n, A1, A1 + nn, ldt, (int)sz, (int)sz, false, SPLIT_UPPER, 1.f, am + AMAX_INV, sb), s));
-            CU(launch_split16(split16_args(T + sz, n, B2 + sz * ldt, B2 + nn + sz * ldt, ldt, (int)sz, (int)sz, true, SPLIT_ALL, 1.f, am + AMAX_T, sbt), s));
+            CU(launch_split16(split16_args(H, n, A1, A1 + nn, ldt, (int)sz, (int)sz, false, SPLIT_UPPER, 1.f, am + AMAX_INV, sb), h->num_sms, s));
+            CU(launch_split16(split16_args(T + sz, n, B2 + sz * ldt, B2 + nn + sz * ldt, ldt, (int)sz, (int)sz, true, SPLIT_ALL, 1.f, am + AMAX_T, sbt), h->num_sms, s));
             TcGemmArgs g2 = tc_args(H + sz, n, (int)sz, (int)sz, (int)sz, -1.f, 0.f, TC_TRI_LEFT, TC_MASK_NONE, h->hd);
             g2.nbatch = np; g2.c_bstride = bstride; g2.N_last = tail;
             g2.a_row0 = 0; g2.a_row_bs = (int)(2 * sz); g2.a_k0 = 0; g2.a_k_bs = (int)(2 * sz);
@@ -1333,7 +1348,7 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
         // U and U^T in one pass, dXX^T in the same launch
         const Split16Args split_d = split16_args(h->D, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, inv_tokens, amax_d, SplitBatch(),
                                                  nullptr, nullptr, inv_d);
-        CU(launch_split16(split16_args(h->H, n, U16, U16 + nn, ldt, n, n, false, SPLIT_UPPER, 1.f, am + AMAX_U, SplitBatch(), UT16, UT16 + nn), s, &split_d));
+        CU(launch_split16(split16_args(h->H, n, U16, U16 + nn, ldt, n, n, false, SPLIT_UPPER, 1.f, am + AMAX_U, SplitBatch(), UT16, UT16 + nn), h->num_sms, s, &split_d));
         h->launches += 2;
         const SplitOperand Uop{U16, U16 + nn, n, n, ldt}, UTop{UT16, UT16 + nn, n, n, ldt};
         const SplitOperand Aop{A16, A16 + nn, n, n, ldt};
@@ -1344,14 +1359,14 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
         go.row_inv = inv_d; go.amax_b = am + AMAX_U; go.row_amax_out = amax_o;
         CU(launch_tc_gemm(maps, go, h->num_sms, s));
         CU(launch_split16(split16_args(O, n, A16, A16 + nn, ldt, n, n, false, SPLIT_STRICT_UPPER, 1.f, amax_o, SplitBatch(), nullptr,
-                                       nullptr, inv_o), s));
+                                       nullptr, inv_o), h->num_sms, s));
         // P = alpha * O U  (B operand rows are rows of U^T)
         if (!make_tc_maps(&maps, Aop, UTop, nullptr)) { h->cuda_error = "cuTensorMapEncodeTiled failed"; return GPTAQ_ERR_CUDA; }
         TcGemmArgs gp = tc_args(h->D, n, n, n, n, alpha, 0.f, TC_P, TC_MASK_STRICT_ZERO, h->hd);
         gp.row_inv = inv_o; gp.amax_b = am + AMAX_U; gp.amax_out = am + AMAX_P;
         CU(launch_tc_gemm(maps, gp, h->num_sms, s));
         // P^T for the lazy-batch updates of gptaq_quantize, over the copy of U that is no longer needed
-        CU(launch_split16(split16_args(h->D, n, U16, U16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P), s));
+        CU(launch_split16(split16_args(h->D, n, U16, U16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P), h->num_sms, s));
         h->launches += 4;
         h->stage = STAGE_P;
         return GPTAQ_OK;
@@ -1389,7 +1404,7 @@ gptaq_status_t gptaq_build_P_rowwise(gptaq_handle_t h, float alpha, gptaq_stream
         CU(launch_absmax({h->H, n, n, n, SPLIT_UPPER, 1.f, am + AMAX_U, nullptr, nullptr},
                          {h->D, n, n, n, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P, nullptr, nullptr}, h->num_sms, s));
         const Split16Args split_p = split16_args(h->D, n, PT16, PT16 + nn, ldt, n, n, true, SPLIT_STRICT_UPPER, 1.f, am + AMAX_P);
-        CU(launch_split16(split16_args(h->H, n, UT16, UT16 + nn, ldt, n, n, true, SPLIT_UPPER, 1.f, am + AMAX_U), s, &split_p));
+        CU(launch_split16(split16_args(h->H, n, UT16, UT16 + nn, ldt, n, n, true, SPLIT_UPPER, 1.f, am + AMAX_U), h->num_sms, s, &split_p));
         h->launches += 2;
     }
     h->stage = STAGE_P;

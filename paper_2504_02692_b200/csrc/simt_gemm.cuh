@@ -466,7 +466,7 @@ inline int64_t simt_tiles(const GemmProblem &pr) {
 constexpr int64_t SIMT_SMALL_TILES = 60;
 
 template <bool A_RC, bool B_RC>
-inline cudaError_t launch_simt_small(const GemmProblem &pr, cudaStream_t s, bool pdl) {
+inline cudaError_t launch_simt_small(const GemmProblem &pr, cudaStream_t s, int early_ctas) {
     dim3 grid((pr.N + SGT - 1) / SGT, (pr.M + SGT - 1) / SGT, pr.nbatch);
     // long contractions of few tiles (the statistics of narrow layers) are shared by up to eight CTAs per tile
     int ksplit = 1;
@@ -479,21 +479,22 @@ inline cudaError_t launch_simt_small(const GemmProblem &pr, cudaStream_t s, bool
     cfg.dynamicSmemBytes = (size_t)SG_STAGES * (pr.A.sub || pr.paired ? 3 : 2) * SG_TILE * sizeof(float);
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = tiles * ksplit <= early_ctas ? 1 : 0;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = 1; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = (unsigned)ksplit;
     cfg.attrs = attr; cfg.numAttrs = ksplit > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, simt_small_kernel<A_RC, B_RC>, pr, ksplit);
 }
 
-// pdl: the 32 x 32 form may start while the kernel before it drains
-inline cudaError_t launch_simt_gemm(const GemmProblem &pr, bool a_rc, bool b_rc, cudaStream_t s, bool pdl = false) {
+// early_ctas: the 32 x 32 form starts while the kernel before it drains where it has at most so many CTAs.  Those that are there
+// before their turn hold the SMs that were free at that time, several to an SM, and it is there that the product runs.
+inline cudaError_t launch_simt_gemm(const GemmProblem &pr, bool a_rc, bool b_rc, cudaStream_t s, int early_ctas = 0) {
     if (pr.M <= 0 || pr.N <= 0 || pr.nbatch <= 0) return cudaSuccess;
     if (simt_tiles(pr) <= SIMT_SMALL_TILES && !pr.B.sub) {
-        if (a_rc && b_rc) return launch_simt_small<true, true>(pr, s, pdl);
-        if (a_rc) return launch_simt_small<true, false>(pr, s, pdl);
-        if (b_rc) return launch_simt_small<false, true>(pr, s, pdl);
-        return launch_simt_small<false, false>(pr, s, pdl);
+        if (a_rc && b_rc) return launch_simt_small<true, true>(pr, s, early_ctas);
+        if (a_rc) return launch_simt_small<true, false>(pr, s, early_ctas);
+        if (b_rc) return launch_simt_small<false, true>(pr, s, early_ctas);
+        return launch_simt_small<false, false>(pr, s, early_ctas);
     }
     if (pr.fresh > 0) return cudaErrorInvalidValue;
     dim3 grid((pr.N + GBN - 1) / GBN, (pr.M + GBM - 1) / GBM, pr.nbatch);
