@@ -831,8 +831,9 @@ def test_statistics_cut_by_length(n, tokens, act_order):
 
 
 # (boxes of 32 columns x 128 rows: a last box of 4 columns and of 28, of 4 rows and of 124; a width whose rows are no 16-byte
-# multiples; whole tiles beside cut ones)
-@pytest.mark.parametrize("n,tokens", [(260, 1111), (380, 1111), (388, 2048), (386, 1111), (1916, 1111)])
+# multiples; 72 tiles for the 74 pairs of 148 SMs, none of them cut; 90 tiles, of which 74 are whole and 16 cut in two, so that a
+# CTA's boxes go to the sums first and to the partial sums then)
+@pytest.mark.parametrize("n,tokens", [(260, 1111), (380, 1111), (388, 2048), (386, 1111), (1916, 1111), (2052, 2777)])
 def test_statistics_at_the_edges_of_the_boxes(n, tokens):
     test_statistics_cut_by_length(n, tokens, False)
 
@@ -968,10 +969,46 @@ def test_captured_quantize_can_be_replayed(n, m, B, group):
     _replays_match(n, m, B, group, False)
 
 
-@pytest.mark.parametrize("n,m,B,group", [(2048, 300, 128, 128), (520, 9000, 64, 64)])
+@pytest.mark.parametrize("n,m,B,group", [
+    (2048, 300, 128, 128), (520, 9000, 64, 64),
+    (384, 300, 128, 128),       # the column loop without tensor cores: three launches, the later ones overlap the products
+    (129, 5000, 32, 32),        # ... two CTAs to an SM; the second launch has one column
+    (1153, 40, 64, 64),         # factorisation in plain float32
+])
 def test_captured_solve_can_be_replayed(n, m, B, group):
     """Launches that overlap their predecessors, and three streams, in one graph."""
     _replays_match(n, m, B, group, True)
+
+
+@pytest.mark.parametrize("n,m,B,group", [(1024, 1024, 128, 128), (200, 70, 32, 0)])
+def test_captured_static_entry_point_can_be_replayed(n, m, B, group):
+    """The launches after the first read U and P before the product in front of them has ended.  Other U and P before each
+    replay, written on the stream just before it: the first launch of a call has to wait for them."""
+    torch.manual_seed(n)
+    G = hp.n_groups(n, group)
+    new = lambda *shape: torch.empty(shape, device="cuda")
+    U, P, W = new(n, n), new(n, n), 0.02 * torch.randn(m, n, device="cuda")
+    out = (torch.empty((m, n), dtype=torch.uint8, device="cuda"), new(m, G), new(m, G), new(m, n))
+    status = torch.zeros(2, dtype=torch.int64, device="cuda")
+    factors = [(torch.eye(n, device="cuda") + torch.triu(torch.randn(n, n, device="cuda"), 1) / n,
+                torch.triu(torch.randn(n, n, device="cuda"), 1) / n) for _ in range(3)]
+
+    def quantize():
+        g.gptaq_quantize_static(U, P, W, 4, group, False, B, *out, status)
+
+    def with_factors(u, p, call):
+        U.copy_(u)
+        P.copy_(p)
+        call()
+        assert status.tolist()[0] == g.GPTAQ_OK
+        return [t.clone() for t in out]
+
+    want = [with_factors(u, p, quantize) for u, p in factors]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        quantize()
+    for (u, p), w in zip(factors, want):
+        assert [int((x != y).sum()) for x, y in zip(with_factors(u, p, graph.replay), w)] == [0, 0, 0, 0]
 
 
 @pytest.mark.parametrize("n", [516, 520, 1036])
