@@ -589,18 +589,19 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
         return cudaErrorUnknown;
     const dim3 grid((unsigned)((r1 - r0 + QB_ROWS - 1) / QB_ROWS));
     const size_t smem = quant_block_smem_bytes(far_form, static_groups);
-    // Near form, more CTAs than SMs: two to an SM, one works while the other waits for its own chain (16384 rows of 400
-    // columns 455 us, with one 498); below that one, which has the registers of both (1024 rows of 1024 columns 288 us, 301).
-    // A grid per column (static groups) takes one always: two have no registers left for it, and gain nothing (16384 rows of
-    // 400 columns 517 us with one, 519 with two; 8192 of 1023 1227, 1221).
-    const bool two = grid.x > (unsigned)t.num_sms && !static_groups;
+    // Near form, more CTAs than SMs: two to an SM, one works while the other waits for its own chain, although each has 80
+    // registers then and spills some (16384 rows of 400 columns 413 us, with one 435; 8192 of 1023 1092, 1110; static groups 460, 475
+    // and 1133, 1182; with a grid every 32 columns 4768 rows of 500 columns 242, 237, 16384 of 1023 1911, 1954); below that
+    // one, which has the registers of both (1023 columns: 1024 rows 299, two 351; 4736
+    // rows 629, 658).
+    const bool two = grid.x > (unsigned)t.num_sms;
     // Near form, from the second launch of a call on: it starts while the product before it drains, and reads U and P meanwhile
     // (1000 rows of 1024 columns 256 -> 242 us a call).  That takes two things: the first launch of a call is a plain one, so that
     // all that made U and P is done before the call's first kernel begins, in a captured graph too; and nothing in a call writes U or P.
     const bool pdl = !far_form && i0 > 0;
     auto launch = [&](auto kernel, int threads) { return launch_pdl(pdl, kernel, grid, dim3(threads), smem, s, uh, ul, ph, pl, a); };
     if (far_form) return static_groups ? launch(quant_block_kernel<true, true, 1>, QB_THREADS_FAR) : launch(quant_block_kernel<true, false, 1>, QB_THREADS_FAR);
-    if (static_groups) return launch(quant_block_kernel<false, true, 1>, QB_THREADS_NEAR);
+    if (static_groups) return two ? launch(quant_block_kernel<false, true, 2>, QB_THREADS_NEAR) : launch(quant_block_kernel<false, true, 1>, QB_THREADS_NEAR);
     return two ? launch(quant_block_kernel<false, false, 2>, QB_THREADS_NEAR) : launch(quant_block_kernel<false, false, 1>, QB_THREADS_NEAR);
 }
 
@@ -612,6 +613,7 @@ cudaError_t configure_quantize_kernels() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, true, 1>, attr, (int)quant_block_smem_bytes(true, true));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, false, 1>, attr, (int)quant_block_smem_bytes(true, false));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true, 1>, attr, (int)quant_block_smem_bytes(false, true));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true, 2>, attr, (int)quant_block_smem_bytes(false, true));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false, 1>, attr, (int)quant_block_smem_bytes(false, false));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false, 2>, attr, (int)quant_block_smem_bytes(false, false));
     return e;
