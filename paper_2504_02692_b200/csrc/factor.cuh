@@ -7,13 +7,13 @@
 // The chain diagonal -> solve -> update -> next diagonal bounds narrow and ordinary layers, and of it the diagonal block
 // (128 dependent pivots).  Where the next block belongs to the same super-panel its diagonal kernel does not wait for the
 // update: it takes a copy of the block from before the update and subtracts this panel's contribution itself (one
-// 128 x 128 x 128 product on the tensor cores), so that the update runs beside it on another stream.  A panel of a
-// 1024-wide layer took 33 us (every CTA of one kernel factored the diagonal block first) + 12 us for the update, now
-// about 20 us (diagonal) + 7 us (rows above).  Factorisation with the inversion that follows it, before and after (the
-// inversion beside the panels included): n = 1024 404 -> 287 us, n = 2052 1118 -> 726 us, n = 4096 2036 -> 1500 to 1700 us,
-// n = 14336 19.8 -> 16.6 ms.  Since then: eight columns of a diagonal block at a time, its inverse beside the next block instead of
-// a kernel of its own (11 us on one SM) behind the update, the rows of U gathered as they come: n = 1024 293 -> 254 us, a panel
-// 33 -> 28 us, a layer of 777 x 2052 1337 -> 1278.
+// 128 x 128 x 128 product on the tensor cores), so that the update runs beside it on another stream.
+// A panel of a 1024-wide layer is 28 us of the chain, from one diagonal kernel's start to the next one's: the diagonal block 19, the
+// rows above it 7, the launches between.  Its inverse is made beside the next block and the rows of U are gathered as they come; with
+// the inverse as a kernel of its own behind the update (11 us on one SM) and one pivot at a time a panel was 33 us, with
+// every CTA of one kernel factoring the diagonal block first and the update on the chain 45.  Factorisation and inversion in that
+// last form took 404 us at n = 1024, 1118 at 2052, 2036 at 4096; in the one before this and in this, both in turn: n = 1024 292 and
+// 248 us, 2052 731 and 659, 4096 1396 and 1265, 14336 12.5 and 11.5 ms.
 #pragma once
 #include "tc_gemm.cuh"
 

@@ -18,10 +18,13 @@
 // What bounds it: the chain, and the near warps behind it.  A column is 7 dependent float32 operations (28 cycles); with its
 // share of the updates, the codes and the hand-over to the next warp 8 columns take 750 cycles alone and 950 beside the near
 // warps, which need 830 for them (a scheduler starts a 16-byte LDS in 8 cycles where lanes share words, in 16 where they do
-// not).  A step of 32 columns ends some 2000 cycles after its last column: the near warps' last 8 columns, results, operands.
-// With a row in the four lanes of one warp every column's errors went through two shuffles to all of them, every lane updated
-// its 8 columns at every step, needed or not, and read U and P for it (64 words a column, now 36): a launch of 512 columns
-// 71 -> 64 us with groups, 68 -> 53 without; 16,384 x 4096 3432 -> 3259 us a call, 1024 x 1024 without workspace 272 -> 256.
+// not).  A step of 32 columns ends some 2000 cycles after its last column (the near warps' last 8 columns, results, operands),
+// the products between two blocks take 5000.
+// A row in the four lanes of one warp (every column's errors through two shuffles to all of them, 64 words of U and P a column
+// for now 36): 8 columns 900 to 1600 cycles, but the end of a step 100 to 1000 and the products between blocks 2300, because the
+// chain's own warps made the operand; a launch of 512 columns 71 us with groups and 68 without, now 64 and 53.
+// The tensor-core form may have 96 registers and spills 60 bytes (static groups 52), the near form 80 where two CTAs share an SM
+// and spills 112 (140); with one to an SM it takes 160 and spills nothing.
 #pragma once
 #include "tc_gemm.cuh"
 
