@@ -259,6 +259,9 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(GemmProblem pr) {
 // What bounds it: shared-memory reads (two 16-byte reads per 16 FMA: about half the FMA rate of the 128 x 128
 // form), so it pays while those tiles leave the chip idle.  A rank-128 update of 384 columns: 30 us as 128 x 128
 // tiles, 9 here; the statistics of 8192 tokens at n = 200: 2700 us there, 150 here.
+// The 32 terms of a stage are summed by themselves: P of a float32 layer is 30 to 45 % closer to float64 so (n = 100 to 384), for 17
+// to 32 registers more (128 at most, still eight CTAs to an SM; 4 bytes spilled where both operands have K contiguous) and up to 3 % of
+// the time (gptaq_build_P at n = 256 26.8 -> 27.7 us, 777 94.2 -> 93.4).
 // ---------------------------------------------------------------------------
 constexpr int SGT = 32, SGK = 32, SG_LD = SGK + 4, SG_STAGES = 3, SG_THREADS = 64;
 constexpr int SG_TILE = SGT * SG_LD;                  // floats of one operand tile

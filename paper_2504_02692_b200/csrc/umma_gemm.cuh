@@ -41,8 +41,8 @@ constexpr int UEPI_WARPS = 8;
 constexpr int UMMA_THREADS = 64 + 32 * UEPI_WARPS;
 // Staging of the results: per column half one 128 x 32 float32 box (128-byte rows, swizzled), handed to the TMA unit as a bulk
 // reduction.  A 16-byte reduction per thread saturated the L2 (70 G/s) while the next tile's MMAs waited for their accumulators:
-// 4096 x 4096 with 32 x 8192 tokens 13,946 -> 13,589 us in all, n = 14336 141.8 -> 138.4 ms, 8 x 4112 tokens of n = 1024
-// 818 -> 805.
+// 8192 tokens of n = 4096 267 -> 253 us a launch among others, 237 -> 225 alone; 4096 x 4096 with 32 such batches 13,946 -> 13,589 us
+// in all, 8 x 4112 tokens of n = 1024 818 -> 805.  (n = 14336: 3 %, where runs of one build differ by up to 8 %.)
 constexpr int USTG_BOX_BYTES = UBM * 32 * 4;
 constexpr int USTG_BYTES = 2 * USTG_BOX_BYTES;
 constexpr size_t UMMA_SMEM = (size_t)USTAGES * USTAGE_BYTES + USTG_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
