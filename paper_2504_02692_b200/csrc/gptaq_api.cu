@@ -587,8 +587,15 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
     if (far_form && (!make_f16_map(&uh, t.UT16, t.n, t.n, t.ldt, 128) || !make_f16_map(&ul, t.UT16 + nn, t.n, t.n, t.ldt, 128) ||
                      !make_f16_map(&ph, t.PT16, t.n, t.n, t.ldt, 128) || !make_f16_map(&pl, t.PT16 + nn, t.n, t.n, t.ldt, 128)))
         return cudaErrorUnknown;
-    const dim3 grid((unsigned)((r1 - r0 + QB_ROWS - 1) / QB_ROWS));
-    const size_t smem = quant_block_smem_bytes(far_form, static_groups);
+    // Few rows: CTAs of 16 while one round of them takes all rows (m, not this launch's share of it: two halves beside one another
+    // are more than a round).  us a call with 32 and with 16: 64 x 1024 146 and 131, 512 x 1024 with groups 152 and 134, 1003 x 1416
+    // 228 and 206, 2368 x 1416 249 and 232.  Without tensor cores a launch is a quarter as long and the products between two launches,
+    // which start early, meet twice as many CTAs: 512 x 400 85 and 81, 777 x 400 88 and 85, 1003 x 400 91 and 95, hence a third of
+    // the SMs.
+    const bool few = m <= (int64_t)QB_ROWS_FEW * (far_form ? t.num_sms : t.num_sms / 3);
+    const int rows = few ? QB_ROWS_FEW : QB_ROWS;
+    const dim3 grid((unsigned)((r1 - r0 + rows - 1) / rows));
+    const size_t smem = quant_block_smem_bytes(far_form, static_groups, rows);
     // Near form, more CTAs than SMs: two to an SM, one works while the other waits for its own chain, although each has 80
     // registers then and spills some (16384 rows of 400 columns 413 us, with one 435; 8192 of 1023 1092, 1110; static groups 460, 475
     // and 1133, 1182; with a grid every 32 columns 4768 rows of 500 columns 242, 237, 16384 of 1023 1911, 1954); below that
@@ -600,6 +607,10 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
     // all that made U and P is done before the call's first kernel begins, in a captured graph too; and nothing in a call writes U or P.
     const bool pdl = !far_form && i0 > 0;
     auto launch = [&](auto kernel, int threads) { return launch_pdl(pdl, kernel, grid, dim3(threads), smem, s, uh, ul, ph, pl, a); };
+    if (few) {
+        if (far_form) return static_groups ? launch(quant_block_kernel<true, true, 1, QB_ROWS_FEW>, QB_THREADS_FAR) : launch(quant_block_kernel<true, false, 1, QB_ROWS_FEW>, QB_THREADS_FAR);
+        return static_groups ? launch(quant_block_kernel<false, true, 1, QB_ROWS_FEW>, QB_THREADS_NEAR) : launch(quant_block_kernel<false, false, 1, QB_ROWS_FEW>, QB_THREADS_NEAR);
+    }
     if (far_form) return static_groups ? launch(quant_block_kernel<true, true, 1>, QB_THREADS_FAR) : launch(quant_block_kernel<true, false, 1>, QB_THREADS_FAR);
     if (static_groups) return two ? launch(quant_block_kernel<false, true, 2>, QB_THREADS_NEAR) : launch(quant_block_kernel<false, true, 1>, QB_THREADS_NEAR);
     return two ? launch(quant_block_kernel<false, false, 2>, QB_THREADS_NEAR) : launch(quant_block_kernel<false, false, 1>, QB_THREADS_NEAR);
@@ -610,12 +621,16 @@ cudaError_t configure_quantize_kernels() {
     const cudaFuncAttribute attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(column_loop_kernel<4>, attr, 2 * 128 * 128 * (int)sizeof(float));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(column_loop_kernel<2>, attr, 2 * 64 * 64 * (int)sizeof(float));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, true, 1>, attr, (int)quant_block_smem_bytes(true, true));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, false, 1>, attr, (int)quant_block_smem_bytes(true, false));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true, 1>, attr, (int)quant_block_smem_bytes(false, true));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true, 2>, attr, (int)quant_block_smem_bytes(false, true));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false, 1>, attr, (int)quant_block_smem_bytes(false, false));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false, 2>, attr, (int)quant_block_smem_bytes(false, false));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, true, 1>, attr, (int)quant_block_smem_bytes(true, true, QB_ROWS));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, false, 1>, attr, (int)quant_block_smem_bytes(true, false, QB_ROWS));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true, 1>, attr, (int)quant_block_smem_bytes(false, true, QB_ROWS));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true, 2>, attr, (int)quant_block_smem_bytes(false, true, QB_ROWS));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false, 1>, attr, (int)quant_block_smem_bytes(false, false, QB_ROWS));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false, 2>, attr, (int)quant_block_smem_bytes(false, false, QB_ROWS));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, true, 1, QB_ROWS_FEW>, attr, (int)quant_block_smem_bytes(true, true, QB_ROWS_FEW));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<true, false, 1, QB_ROWS_FEW>, attr, (int)quant_block_smem_bytes(true, false, QB_ROWS_FEW));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, true, 1, QB_ROWS_FEW>, attr, (int)quant_block_smem_bytes(false, true, QB_ROWS_FEW));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(quant_block_kernel<false, false, 1, QB_ROWS_FEW>, attr, (int)quant_block_smem_bytes(false, false, QB_ROWS_FEW));
     return e;
 }
 

@@ -1,6 +1,6 @@
 // The column loop of Algorithm 1 over several lazy-batch blocks of columns in ONE launch.
 //
-// Rows of W are independent, so a CTA that owns 32 rows can run the sequential part of the loop over many
+// Rows of W are independent, so a CTA that owns 32 rows (16 where there are few) can run the sequential part of the loop over many
 // lazy-batch blocks without ever meeting another CTA.  Its slab of W (32 x 512 float32) stays in shared
 // memory; what would be a launch per block and a product per block over the whole matrix is a pipeline of
 // warp roles inside the CTA:
@@ -30,19 +30,22 @@
 
 namespace gptaq {
 
-constexpr int QB_ROWS = 32;             // rows of W per CTA
+// Rows of W per CTA, and where there are few of them (launch_quant_block): half the rows are half the work for the near and the
+// drain warps, and the chain, which takes as long for 16 rows as for 32, has less of it beside itself (eight columns 700 to 900 cycles
+// for 750 to 950, a launch of 512 columns 64 -> 57 us).
+constexpr int QB_ROWS = 32, QB_ROWS_FEW = 16;
 constexpr int QB_W = 128;               // columns per block (float32 updates inside, tensor cores beyond)
 constexpr int QB_SUPER = 512;           // most columns per launch
 constexpr int QB_CHAIN = 128, QB_NEAR = 256, QB_DRAIN = 128;
 constexpr int QB_THREADS_NEAR = QB_CHAIN + QB_NEAR;                   // one block per launch, no tensor cores
 constexpr int QB_THREADS_FAR = QB_THREADS_NEAR + QB_DRAIN + 64;
 constexpr int QB_ULD0 = QB_W + 4, QB_ULD1 = QB_W - 32 + 4;            // pitch of U / P rows in the even / odd step's buffer
-constexpr int QB_SLD = QB_ROWS + 4;                                   // pitch of the published errors
+__host__ __device__ constexpr int qb_sld(int rows) { return rows + 4; }   // pitch of the published errors
 // 128 x 64 fp16 tiles of U^T / P^T in flight (one less makes room for the grids per column)
 __host__ __device__ constexpr int qb_aslots(bool percol) { return percol ? 2 : 3; }
 constexpr int QB_A_BYTES = 128 * 64 * 2;
-constexpr int QB_E_BYTES = QB_ROWS * 64 * 2;                          // one K-block (64 columns) of one part of the errors
-constexpr int QB_HALF_BYTES = 4 * QB_E_BYTES;                         // (hi, lo) x (-Err, Wpre) of 64 columns
+__host__ __device__ constexpr int qb_e_bytes(int rows) { return rows * 64 * 2; }          // one K-block (64 columns) of one part of the errors
+__host__ __device__ constexpr int qb_half_bytes(int rows) { return 4 * qb_e_bytes(rows); } // (hi, lo) x (-Err, Wpre) of 64 columns
 constexpr int QB_TMEM_COLS = 256;                                     // 2 halves x 3 blocks x 32 columns, a power of two
 
 struct QuantBlockArgs {
@@ -71,37 +74,38 @@ struct QuantBlockArgs {
 struct QuantBlockSmem {
     int a, e, w, up, st, grid, udinv, perm, inv, rmax, bars, total, wld;
 };
-__host__ __device__ constexpr QuantBlockSmem quant_block_smem(bool far_form, bool percol) {
+__host__ __device__ constexpr QuantBlockSmem quant_block_smem(bool far_form, bool percol, int rows) {
     QuantBlockSmem s{};
     s.wld = (far_form ? QB_SUPER : QB_W) + 4;
     s.a = 0;
     s.e = s.a + (far_form ? qb_aslots(percol) * QB_A_BYTES : 0);
-    s.w = s.e + (far_form ? 2 * QB_HALF_BYTES : 0);
-    s.up = s.w + QB_ROWS * s.wld * 4;
+    s.w = s.e + (far_form ? 2 * qb_half_bytes(rows) : 0);
+    s.up = s.w + rows * s.wld * 4;
     s.st = s.up + 2 * 32 * (QB_ULD0 + QB_ULD1) * 4;
-    s.grid = s.st + 2 * 64 * QB_SLD * 4;
-    s.udinv = s.grid + (percol ? 3 * 32 * QB_SLD * 4 : 0);
+    s.grid = s.st + 2 * 64 * qb_sld(rows) * 4;
+    s.udinv = s.grid + (percol ? 3 * 32 * qb_sld(rows) * 4 : 0);
     s.perm = s.udinv + 2 * 32 * 4;
     s.inv = s.perm + 2 * 32 * 4;
-    s.rmax = s.inv + 2 * QB_ROWS * 4;
+    s.rmax = s.inv + 2 * rows * 4;
     s.bars = s.rmax + (far_form ? QB_NEAR * 4 : 0);
     s.total = s.bars + 256;
     return s;
 }
-constexpr size_t quant_block_smem_bytes(bool far_form, bool percol) {
-    return (size_t)quant_block_smem(far_form, percol).total + 1024;        // (alignment slack)
+constexpr size_t quant_block_smem_bytes(bool far_form, bool percol, int rows) {
+    return (size_t)quant_block_smem(far_form, percol, rows).total + 1024;        // (alignment slack)
 }
-static_assert(quant_block_smem_bytes(true, false) <= 227 * 1024 && quant_block_smem_bytes(true, true) <= 227 * 1024, "shared memory of one SM");
+static_assert(quant_block_smem_bytes(true, false, QB_ROWS) <= 227 * 1024 && quant_block_smem_bytes(true, true, QB_ROWS) <= 227 * 1024, "shared memory of one SM");
 
-// kind::f16 instruction descriptor: fp16 A and B (K-major), fp32 D, M = 128, N = QB_ROWS.
-constexpr uint32_t QB_IDESC = (1u << 4) | ((QB_ROWS >> 3) << 17) | ((128 >> 4) << 24);
+// kind::f16 instruction descriptor: fp16 A and B (K-major), fp32 D, M = 128, N = rows.
+__host__ __device__ constexpr uint32_t qb_idesc(int rows) { return (1u << 4) | ((uint32_t)(rows >> 3) << 17) | ((128 >> 4) << 24); }
 
 // Named barriers.  Chunk barriers are used once per step each; the step barrier keeps the chain from lapping them.
 enum { QBAR_CHUNK = 1, QBAR_STEP = 5, QBAR_NEAR = 6, QBAR_DRAIN = 7, QBAR_CLIP = 8, QBAR_HAND = 9 /* .. 14 */, QBAR_CHAIN = 15 };
 
 // Position of a row in a column of the published errors: the near warps' threads take rows ti, ti + 8, .. as
 // one 16-byte read.
-__device__ __forceinline__ int qb_pos(int row) { return (row & 7) * 4 + (row >> 3); }
+template <int ROWS>
+__device__ __forceinline__ int qb_pos(int row) { return (row & 7) * (ROWS / 8) + (row >> 3); }
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
@@ -195,7 +199,7 @@ __device__ __forceinline__ void clip_search(const float *w, int n, float lo, flo
 
 // FAR: several blocks per launch, updates between them on the tensor cores.  PERCOL: static groups, a grid per column.
 // CTAS: CTAs that share an SM (shared memory allows one of the tensor-core form).
-template <bool FAR, bool PERCOL, int CTAS>
+template <bool FAR, bool PERCOL, int CTAS, int ROWS = QB_ROWS>
 __global__ void __launch_bounds__(FAR ? QB_THREADS_FAR : QB_THREADS_NEAR, CTAS)
 quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_constant__ CUtensorMap mapUlo,
                    const __grid_constant__ CUtensorMap mapPhi, const __grid_constant__ CUtensorMap mapPlo, QuantBlockArgs a) {
@@ -203,14 +207,15 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *sm = smem_raw + (base - raw);
-    constexpr QuantBlockSmem L = quant_block_smem(FAR, PERCOL);
+    constexpr QuantBlockSmem L = quant_block_smem(FAR, PERCOL, ROWS);
+    constexpr int SLD = qb_sld(ROWS), E_BYTES = qb_e_bytes(ROWS), HALF_BYTES = qb_half_bytes(ROWS), RPT = ROWS / 8;
     constexpr int ASLOTS = qb_aslots(PERCOL);
     constexpr int WLD = L.wld;
     constexpr int NTHREADS = FAR ? QB_THREADS_FAR : QB_THREADS_NEAR;
     float *Ws = reinterpret_cast<float *>(sm + L.w);               // [32][WLD]: the slab
     float *UPs = reinterpret_cast<float *>(sm + L.up);             // rows of U and P of the current and the next step
-    float *Sts = reinterpret_cast<float *>(sm + L.st);             // [2 steps][64][QB_SLD]: -Err, then Wpre, of 32 columns
-    float *grid_s = reinterpret_cast<float *>(sm + L.grid);        // PERCOL: scales, zero points, 1 / scales, [32 columns][QB_SLD] each
+    float *Sts = reinterpret_cast<float *>(sm + L.st);             // [2 steps][64][SLD]: -Err, then Wpre, of 32 columns
+    float *grid_s = reinterpret_cast<float *>(sm + L.grid);        // PERCOL: scales, zero points, 1 / scales, [32 columns][SLD] each
     float *udinv2 = reinterpret_cast<float *>(sm + L.udinv);       // [2 steps][32]: err_scale / U_kk
     int *perm2 = reinterpret_cast<int *>(sm + L.perm);             // [2 steps][32]: where a column's codes go
     float *inv_s = reinterpret_cast<float *>(sm + L.inv);          // [2 halves][32]: 1 / scale of a row's errors
@@ -228,8 +233,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = a.n, i0 = a.i0, B = a.bw;
-    const int row0 = a.row_first + blockIdx.x * QB_ROWS;
-    const int nrows = min(QB_ROWS, a.m - row0);
+    const int row0 = a.row_first + blockIdx.x * ROWS;
+    const int nrows = min(ROWS, a.m - row0);
     const int cols = a.i1 - i0;
     const int nblk = FAR ? (cols + QB_W - 1) / QB_W : 1;
     auto nsteps = [&](int b) { return min(B / 32, (cols - b * QB_W + 31) / 32); };     // 32-column steps of block b
@@ -279,9 +284,9 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     auto store_grid = [&](int r, int c, const float (&sc)[4], const float (&zp)[4]) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            grid_s[(c + e) * QB_SLD + r] = sc[e];
-            grid_s[(32 + c + e) * QB_SLD + r] = zp[e];
-            grid_s[(64 + c + e) * QB_SLD + r] = 1.f / sc[e];
+            grid_s[(c + e) * SLD + r] = sc[e];
+            grid_s[(32 + c + e) * SLD + r] = zp[e];
+            grid_s[(64 + c + e) * SLD + r] = 1.f / sc[e];
         }
     };
 
@@ -289,7 +294,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     if (FAR) {
         if (tid == 0) {
             for (int s = 0; s < ASLOTS; ++s) { mbar_init(afull(s), 1); mbar_init(aempty(s), 1); }
-            for (int s = 0; s < 2; ++s) { mbar_init(efull(s), QB_NEAR / 32); mbar_init(efree(s), QB_DRAIN / 32); }
+            for (int s = 0; s < 2; ++s) { mbar_init(efull(s), 8 * ROWS / 32); mbar_init(efree(s), QB_DRAIN / 32); }
             for (int s = 0; s < 6; ++s) { mbar_init(tfull(s), 1); mbar_init(tempty(s), QB_DRAIN / 32); }
             *abort_flag = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -315,7 +320,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         const bool whole = wvec && wc + 3 < cols;
         const float *src = a.W + (int64_t)(row0 + wr0) * a.ldw + i0 + wc;
         float *dst = Ws + wr0 * WLD + wc;
-        for (int r = wr0; r < QB_ROWS; r += RSTEP) {
+        for (int r = wr0; r < ROWS; r += RSTEP) {
             if (whole && r < nrows) cp_async16(dst, src);
             else {
 #pragma unroll
@@ -327,7 +332,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     // (dead inputs read as zero; the flags are 4-byte aligned and padded beyond n)
     const uint32_t dead4 = fills && wc < cols ? *reinterpret_cast<const uint32_t *>(a.dead + i0 + wc) : 0u;
     if (tid < 32) { udinv2[tid] = load_pivot(i0 + tid); perm2[tid] = load_perm(i0 + tid); }
-    if (PERCOL && tid < QB_NEAR) {
+    if (PERCOL && tid < 8 * ROWS) {
         float sc[4], zp[4];
         load_grid(tid >> 3, i0 + 4 * (tid & 7), sc, zp);
         store_grid(tid >> 3, 4 * (tid & 7), sc, zp);
@@ -335,7 +340,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     asm volatile("cp.async.wait_all;" ::: "memory");
     if (fills && dead4) {
         float4 *wp = reinterpret_cast<float4 *>(Ws + wr0 * WLD + wc);                  // (the words that this thread has copied)
-        for (int r = wr0; r < QB_ROWS; r += RSTEP, wp += RSTEP * WLD / 4) {
+        for (int r = wr0; r < ROWS; r += RSTEP, wp += RSTEP * WLD / 4) {
             float4 v = *wp;
             if (dead4 & 0xffu) v.x = 0.f;
             if (dead4 & 0xff00u) v.y = 0.f;
@@ -360,11 +365,12 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
 
     if (tid < QB_CHAIN) {
         // ================================================================ chain
-        const int lrow = lane, w8 = 8 * warp;                       // this warp's columns of a step: w8 .. w8 + 7
+        const int lrow = lane & (ROWS - 1), w8 = 8 * warp;          // (16 rows: the upper lanes do the same as the lower ones)
+                             // this warp's columns of a step: w8 .. w8 + 7
         const int row = row0 + lrow;
         const bool live = lrow < nrows;
         float *wrow = Ws + lrow * WLD;
-        const int pos = qb_pos(lrow);
+        const int pos = qb_pos<ROWS>(lrow);
         float scale = 1.f, zero = 0.f;
         if (!PERCOL && a.group <= 0 && live) { scale = a.scales[row]; zero = a.zeros[row]; }
         float inv_scale = 1.f / scale, qlo = -zero, qhi = maxq - zero;
@@ -377,14 +383,14 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 const int cg = i0 + co;                             // ... in W
                 if (b + s > 0) named_bar_sync(QBAR_STEP, QB_THREADS_NEAR);
                 if (FAR && s == 0 && b > 0) named_bar_sync(QBAR_DRAIN, QB_CHAIN + QB_DRAIN);
-                float *St = Sts + (s & 1) * 64 * QB_SLD;
+                float *St = Sts + (s & 1) * 64 * SLD;
                 float scv[8], ivv[8], zv[8];
                 if (PERCOL) {
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        scv[e] = grid_s[(w8 + e) * QB_SLD + lrow];
-                        zv[e] = grid_s[(32 + w8 + e) * QB_SLD + lrow];
-                        ivv[e] = grid_s[(64 + w8 + e) * QB_SLD + lrow];
+                        scv[e] = grid_s[(w8 + e) * SLD + lrow];
+                        zv[e] = grid_s[(32 + w8 + e) * SLD + lrow];
+                        ivv[e] = grid_s[(64 + w8 + e) * SLD + lrow];
                     }
                 } else if (grid_starts(cg)) {
                     // grid of the group that starts here, from the current values (columns of it beyond the layer are zeros):
@@ -398,12 +404,12 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
                     }
                     // (through the part of the step's error buffer that warp 3 publishes into, after all have read it)
-                    float2 *range_s = reinterpret_cast<float2 *>(St + 24 * QB_SLD);
-                    range_s[warp * QB_ROWS + lrow] = make_float2(lo, hi);
+                    float2 *range_s = reinterpret_cast<float2 *>(St + 24 * SLD);
+                    range_s[warp * ROWS + lrow] = make_float2(lo, hi);
                     named_bar_sync(QBAR_CHAIN, QB_CHAIN);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        const float2 v = range_s[q * QB_ROWS + lrow];
+                        const float2 v = range_s[q * ROWS + lrow];
                         lo = fminf(lo, v.x); hi = fmaxf(hi, v.y);
                     }
                     float p = 1.f;
@@ -413,7 +419,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         p = clip_ratio(reinterpret_cast<int *>(St)[lrow], a.clip_steps, a.clip_min);
                     }
                     make_grid(p * lo, p * hi, p * fmaxf(-lo, hi), a.bits, a.sym, scale, zero);
-                    if (live && warp == 0) {
+                    if (live && warp == 0 && lane < ROWS) {
                         const int g = cg / a.group;
                         a.scales[(int64_t)row * a.G + g] = scale;
                         a.zeros[(int64_t)row * a.G + g] = zero;
@@ -440,10 +446,10 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         lds_pair4(Pw + (4 * h + kk) * ld, pp[kk]);
                     }
                     named_bar_sync(QBAR_HAND + h, 32 * (4 - (h >> 1)));
-                    const float *Se = St + 4 * h * QB_SLD + pos;
+                    const float *Se = St + 4 * h * SLD + pos;
                     float er[4], wa[4];
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) { er[kk] = Se[kk * QB_SLD]; wa[kk] = Se[(32 + kk) * QB_SLD]; }
+                    for (int kk = 0; kk < 4; ++kk) { er[kk] = Se[kk * SLD]; wa[kk] = Se[(32 + kk) * SLD]; }
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
                         const unsigned long long ne2 = pack2(er[kk], er[kk]), wa2 = pack2(wa[kk], wa[kk]);
@@ -457,7 +463,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 const float4 ud0 = *reinterpret_cast<const float4 *>(ud), ud1 = *reinterpret_cast<const float4 *>(ud + 4);
                 const float udv[8] = {ud0.x, ud0.y, ud0.z, ud0.w, ud1.x, ud1.y, ud1.z, ud1.w};
                 Uw += w8 * ld; Pw += w8 * ld;
-                float *Sw = St + w8 * QB_SLD + pos;
+                float *Sw = St + w8 * SLD + pos;
                 float qv[8];
                 uint32_t code[2] = {0u, 0u};
                 float c = lo2(x[0]);
@@ -501,15 +507,15 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     // publish these 4 columns: to the chain's other warps, then (8 columns) to the near warps
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
-                        Sw[(4 * half + kk) * QB_SLD] = nerr[kk];
-                        Sw[(32 + 4 * half + kk) * QB_SLD] = pre[kk];
+                        Sw[(4 * half + kk) * SLD] = nerr[kk];
+                        Sw[(32 + 4 * half + kk) * SLD] = pre[kk];
                     }
                     if (warp < 3) named_bar_arrive(QBAR_HAND + 2 * warp + half, 32 * (4 - warp));
                 }
                 *reinterpret_cast<float4 *>(wrow + co + w8) = make_float4(qv[0], qv[1], qv[2], qv[3]);
                 *reinterpret_cast<float4 *>(wrow + co + w8 + 4) = make_float4(qv[4], qv[5], qv[6], qv[7]);
                 named_bar_arrive(QBAR_CHUNK + warp, 32 + QB_NEAR);
-                if (live) {
+                if (live && lane < ROWS) {
                     uint8_t *crow = a.codes + (int64_t)row * n;
                     const int cc = cg + w8;
                     if (!a.perm && cc + 7 < n && (reinterpret_cast<uintptr_t>(crow + cc) & 7) == 0) {
@@ -525,8 +531,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     } else if (tid < QB_THREADS_NEAR) {
         // ================================================================ near
         const int t = tid - QB_CHAIN;
-        const int ti = t & 7, tj = t >> 3;                          // rows ti, ti + 8, ti + 16, ti + 24; columns 4 tj .. of the rest
-        float row_max = 0.f;                                        // largest magnitude of row (t & 31)'s errors in this launch
+        const int ti = t & 7, tj = t >> 3;                          // rows ti, ti + 8, ..; columns 4 tj .. of the rest
+        float row_max = 0.f;                                        // largest magnitude of row t % ROWS's errors in this launch
         for (int b = 0; b < nblk; ++b) {
             const int nst = nsteps(b);
             for (int s = 0; s < nst; ++s) {
@@ -540,12 +546,12 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 if (!last) {
                     fetch_up(i0 + nb * QB_W, ns, t, QB_NEAR);
                     if (t < 32) { next_ud = load_pivot(ncol + t); next_perm = load_perm(ncol + t); }
-                    if (PERCOL) load_grid(t >> 3, ncol + 4 * (t & 7), next_sc, next_zp);
+                    if (PERCOL && t < 8 * ROWS) load_grid(t >> 3, ncol + 4 * (t & 7), next_sc, next_zp);
                 }
                 if (a.clip_steps > 0 && grid_starts(i0 + co)) {
-                    // clipping-range search: thread = (row, one eighth of the candidates)
+                    // clipping-range search: thread = (row, a share of the candidates)
                     named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);     // the group's values are current
-                    const int r = t & 31, cgi = t >> 5;
+                    const int r = t & (ROWS - 1), cgi = t / ROWS;
                     const float *w = Ws + r * WLD + co;
                     float lo = 0.f, hi = 0.f, best;
                     int kb;
@@ -554,16 +560,16 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         lo = fminf(lo, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
                         hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
                     }
-                    clip_search(w, a.group, lo, hi, a.bits, a.sym, a.clip_steps, a.clip_min, cgi, QB_NEAR / 32, best, kb);
-                    float *scratch = Sts + (s & 1) * 64 * QB_SLD;   // (the chain writes there only after this search)
+                    clip_search(w, a.group, lo, hi, a.bits, a.sym, a.clip_steps, a.clip_min, cgi, QB_NEAR / ROWS, best, kb);
+                    float *scratch = Sts + (s & 1) * 64 * SLD;   // (the chain writes there only after this search)
                     float *be = scratch + 64;
                     int *bk = reinterpret_cast<int *>(be + QB_NEAR);
                     be[t] = best; bk[t] = kb;
                     named_bar_sync(QBAR_NEAR, QB_NEAR);
-                    if (t < QB_ROWS) {
-                        for (int g = 1; g < QB_NEAR / 32; ++g) {
-                            const float e = be[g * 32 + t];
-                            const int k = bk[g * 32 + t];
+                    if (t < ROWS) {
+                        for (int g = 1; g < QB_NEAR / ROWS; ++g) {
+                            const float e = be[g * ROWS + t];
+                            const int k = bk[g * ROWS + t];
                             if (e < best || (e == best && k < kb)) { best = e; kb = k; }
                         }
                         reinterpret_cast<int *>(scratch)[t] = kb;
@@ -573,22 +579,29 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 }
                 const int ld = up_ld(s);
                 const float *Ub = up_buf(s) + 32 + 4 * tj, *Pb = Ub + 32 * ld;      // (columns beyond the step's own 32)
-                const float *St = Sts + (s & 1) * 64 * QB_SLD;
+                const float *St = Sts + (s & 1) * 64 * SLD;
                 const bool active = 32 + 4 * tj < B - 32 * s;
-                unsigned long long acc[4][2];
+                unsigned long long acc[RPT][2];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) { acc[e][0] = 0ull; acc[e][1] = 0ull; }
+                for (int e = 0; e < RPT; ++e) { acc[e][0] = 0ull; acc[e][1] = 0ull; }
                 for (int ph = 0; ph < 4; ++ph) {
                     named_bar_sync(QBAR_CHUNK + ph, 32 + QB_NEAR);
                     if (!active) continue;
 #pragma unroll
                     for (int kk = 0; kk < 16; ++kk) {
                         const int k = 8 * ph + (kk & 7);
-                        const float4 av = *reinterpret_cast<const float4 *>(St + (k + (kk < 8 ? 0 : 32)) * QB_SLD + 4 * ti);
+                        const float *ap = St + (k + (kk < 8 ? 0 : 32)) * SLD + RPT * ti;
+                        float ae[4];
+                        if (RPT == 4) {
+                            const float4 av = *reinterpret_cast<const float4 *>(ap);
+                            ae[0] = av.x; ae[1] = av.y; ae[2] = av.z; ae[3] = av.w;
+                        } else {
+                            const float2 av = *reinterpret_cast<const float2 *>(ap);
+                            ae[0] = av.x; ae[1] = av.y;
+                        }
                         const ulonglong2 bv = *reinterpret_cast<const ulonglong2 *>((kk < 8 ? Ub : Pb) + k * ld);
-                        const float ae[4] = {av.x, av.y, av.z, av.w};
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
+                        for (int e = 0; e < RPT; ++e) {
                             const unsigned long long aa = pack2(ae[e], ae[e]);
                             acc[e][0] = fma2(aa, bv.x, acc[e][0]);
                             acc[e][1] = fma2(aa, bv.y, acc[e][1]);
@@ -597,7 +610,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 }
                 if (active) {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
+                    for (int e = 0; e < RPT; ++e) {
                         float4 *cp = reinterpret_cast<float4 *>(Ws + (ti + 8 * e) * WLD + co + 32 + 4 * tj);
                         float4 v = *cp;
                         v.x += lo2(acc[e][0]); v.y += hi2(acc[e][0]); v.z += lo2(acc[e][1]); v.w += hi2(acc[e][1]);
@@ -605,37 +618,37 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     }
                 }
                 // 64 columns done: a thread takes eight of them in one row (before the chain goes on and overwrites the first 32)
-                const int er = t & 31, ec = t >> 5;
+                const int er = t & (ROWS - 1), ec = t / ROWS;
                 float ev[2][8], mx = 0.f;
-                if (FAR && (s & 1)) {
-                    const float *S2 = Sts + ((ec >> 2) * 64 + 8 * (ec & 3)) * QB_SLD + qb_pos(er);
+                if (FAR && (s & 1) && ec < 8) {
+                    const float *S2 = Sts + ((ec >> 2) * 64 + 8 * (ec & 3)) * SLD + qb_pos<ROWS>(er);
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        ev[0][e] = S2[e * QB_SLD];
-                        ev[1][e] = rho * S2[(32 + e) * QB_SLD];
+                        ev[0][e] = S2[e * SLD];
+                        ev[1][e] = rho * S2[(32 + e) * SLD];
                         mx = fmaxf(mx, fmaxf(fabsf(ev[0][e]), fabsf(ev[1][e])));
                     }
-                    rmax_s[ec * QB_ROWS + er] = mx;
+                    rmax_s[ec * ROWS + er] = mx;
                 }
                 asm volatile("cp.async.wait_all;" ::: "memory");
                 if (!last) {
                     if (t < 32) { udinv2[(ns & 1) * 32 + t] = next_ud; perm2[(ns & 1) * 32 + t] = next_perm; }
-                    if (PERCOL) store_grid(t >> 3, 4 * (t & 7), next_sc, next_zp);      // (the chain has read this step's)
+                    if (PERCOL && t < 8 * ROWS) store_grid(t >> 3, 4 * (t & 7), next_sc, next_zp);      // (the chain has read this step's)
                     named_bar_arrive(QBAR_STEP, QB_THREADS_NEAR);
                 }
                 if (FAR && (s & 1)) {
                     // ... as the tensor cores' operand, with one power-of-two scale per row
                     named_bar_sync(QBAR_NEAR, QB_NEAR);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) mx = fmaxf(mx, rmax_s[e * QB_ROWS + er]);
+                    for (int e = 0; e < 8; ++e) mx = fmaxf(mx, rmax_s[e * ROWS + er]);
                     row_max = fmaxf(row_max, mx);
-                    if (b < last_groups) {
+                    if (b < last_groups && ec < 8) {
                         const int half = s >> 1;                    // buffer: even and odd halves alternate
                         // (the drain warps are done with this buffer's row scales, the MMAs with its operands)
                         if (b > 0) mbar_wait(efree(half), (uint32_t)(b - 1) & 1u, abort_flag);
                         const float sc = split_scale(mx);
-                        if (ec == 0) inv_s[half * QB_ROWS + er] = 1.f / sc / su;
-                        uint8_t *eb = sm + L.e + half * QB_HALF_BYTES + (er >> 3) * 1024 + (er & 7) * 128 + ((ec ^ (er & 7)) << 4);
+                        if (ec == 0) inv_s[half * ROWS + er] = 1.f / sc / su;
+                        uint8_t *eb = sm + L.e + half * HALF_BYTES + (er >> 3) * 1024 + (er & 7) * 128 + ((ec ^ (er & 7)) << 4);
 #pragma unroll
                         for (int o = 0; o < 2; ++o) {
                             const float y0[4] = {sc * ev[o][0], sc * ev[o][1], sc * ev[o][2], sc * ev[o][3]};
@@ -643,8 +656,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                             uint2 h0, l0, h1, l1;
                             split16_pack(y0, h0, l0);
                             split16_pack(y1, h1, l1);
-                            *reinterpret_cast<uint4 *>(eb + o * QB_E_BYTES) = make_uint4(h0.x, h0.y, h1.x, h1.y);
-                            *reinterpret_cast<uint4 *>(eb + (2 + o) * QB_E_BYTES) = make_uint4(l0.x, l0.y, l1.x, l1.y);
+                            *reinterpret_cast<uint4 *>(eb + o * E_BYTES) = make_uint4(h0.x, h0.y, h1.x, h1.y);
+                            *reinterpret_cast<uint4 *>(eb + (2 + o) * E_BYTES) = make_uint4(l0.x, l0.y, l1.x, l1.y);
                         }
                         fence_proxy_async_smem();
                         __syncwarp();
@@ -655,9 +668,9 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 {
                     const int r = t >> 3, c4 = 4 * (t & 7);
                     const int cw = co + c4;                         // column in the slab
-                    const float4 v = *reinterpret_cast<const float4 *>(Ws + r * WLD + cw);
+                    const float4 v = r < ROWS ? *reinterpret_cast<const float4 *>(Ws + r * WLD + cw) : make_float4(0.f, 0.f, 0.f, 0.f);
                     const int left = cols - cw;                     // columns that exist from here on
-                    if (r < nrows && left > 0) {
+                    if (r < nrows && left > 0) {                    // (r < ROWS, too)
                         float *dst = a.W + (int64_t)(row0 + r) * a.ldw + i0 + cw;
                         if (left >= 4 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) *reinterpret_cast<float4 *>(dst) = v;
                         else {
@@ -674,21 +687,20 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     auto magnitude = [](float v) { return __float_as_uint(v) & 0x7fffffffu; };
                     if (!a.EW) {
                         const int k = t >> 3;                       // column k, rows ti, ti + 8, ..
-                        const float4 e = *reinterpret_cast<const float4 *>(St + k * QB_SLD + 4 * ti);
-                        const float4 p = *reinterpret_cast<const float4 *>(St + (32 + k) * QB_SLD + 4 * ti);
-                        const uint32_t big[4] = {max(magnitude(e.x), magnitude(p.x)), max(magnitude(e.y), magnitude(p.y)),
-                                                 max(magnitude(e.z), magnitude(p.z)), max(magnitude(e.w), magnitude(p.w))};
+                        const float *ep = St + k * SLD + RPT * ti, *pp = ep + 32 * SLD;
 #pragma unroll
-                        for (int f = 0; f < 4; ++f)
-                            if (big[f] >= 0x7f800000u && ti + 8 * f < nrows) record_status(a.hd, ST_NONFINITE, row0 + ti + 8 * f);
+                        for (int f = 0; f < RPT; ++f) {
+                            const uint32_t big = max(magnitude(ep[f]), magnitude(pp[f]));
+                            if (big >= 0x7f800000u && ti + 8 * f < nrows) record_status(a.hd, ST_NONFINITE, row0 + ti + 8 * f);
+                        }
                     } else if (r < nrows) {
-                        const int pos = qb_pos(r);
+                        const int pos = qb_pos<ROWS>(r);
                         float e4[4], p4[4];
                         uint32_t big = 0u;
 #pragma unroll
                         for (int f = 0; f < 4; ++f) {
-                            e4[f] = St[(c4 + f) * QB_SLD + pos];
-                            const float p = St[(32 + c4 + f) * QB_SLD + pos];
+                            e4[f] = St[(c4 + f) * SLD + pos];
+                            const float p = St[(32 + c4 + f) * SLD + pos];
                             big = max(big, max(magnitude(e4[f]), magnitude(p)));
                             p4[f] = rho * p;
                         }
@@ -700,7 +712,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 }
             }
         }
-        if (FAR && a.EWS_hi && t < QB_ROWS) {
+        if (FAR && a.EWS_hi && t < ROWS) {
             const float sc = t < nrows ? split_scale(row_max) : 1.f;
             udinv2[t] = sc;                                         // (free: the last step's pivots are in the other half; read
                                                                     //  after the barrier below)
@@ -717,16 +729,17 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     const int slot = half * 3 + (j - 1);            // (used once per earlier block: b = 0 .. j - 1)
                     mbar_wait(tfull(slot), (uint32_t)b & 1u, abort_flag);
                     tc_fence_after();
-                    uint32_t v[32];
-                    tmem_ld32(tmem_base + slot * QB_ROWS + ((uint32_t)(quarter * 32) << 16), v);
+                    uint32_t v[ROWS];
+                    if constexpr (ROWS == 32) tmem_ld32(tmem_base + slot * ROWS + ((uint32_t)(quarter * 32) << 16), v);
+                    else tmem_ld16(tmem_base + slot * ROWS + ((uint32_t)(quarter * 32) << 16), v);
                     tmem_ld_wait();
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty(slot));
                     float *wp = Ws + j * QB_W + quarter * 32 + lane;
 #pragma unroll
-                    for (int r4 = 0; r4 < QB_ROWS / 4; ++r4) {
-                        const float4 iv = *reinterpret_cast<const float4 *>(inv_s + half * QB_ROWS + 4 * r4);
+                    for (int r4 = 0; r4 < ROWS / 4; ++r4) {
+                        const float4 iv = *reinterpret_cast<const float4 *>(inv_s + half * ROWS + 4 * r4);
                         float *w4 = wp + 4 * r4 * WLD;
                         w4[0] = fmaf(__uint_as_float(v[4 * r4]), iv.x, w4[0]);
                         w4[WLD] = fmaf(__uint_as_float(v[4 * r4 + 1]), iv.y, w4[WLD]);
@@ -770,25 +783,25 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
             for (int b = 0; ok && b < last_groups; ++b)
                 for (int half = 0; ok && half < 2; ++half) {
                     if (!mbar_wait(efull(half), (uint32_t)b & 1u, abort_flag)) { ok = false; break; }
-                    const uint32_t eb = base + L.e + half * QB_HALF_BYTES;
+                    const uint32_t eb = base + L.e + half * HALF_BYTES;
                     for (int j = b + 1; ok && j < nblk; ++j) {
                         const int acc = half * 3 + (j - 1);
                         if (b > 0 && !mbar_wait(tempty(acc), (uint32_t)(b - 1) & 1u, abort_flag)) { ok = false; break; }
                         tc_fence_after();
-                        const uint32_t d = tmem_base + acc * QB_ROWS;
+                        const uint32_t d = tmem_base + acc * ROWS;
                         for (int t4 = 0; t4 < 4; ++t4) {
                             if (!mbar_wait(afull(slot), phase, abort_flag)) { ok = false; break; }
                             tc_fence_after();
                             const uint64_t ad = make_kmajor_desc(base + L.a + slot * QB_A_BYTES);
-                            const uint64_t bh = make_kmajor_desc(eb + (t4 >> 1) * QB_E_BYTES);
-                            const uint64_t bl = make_kmajor_desc(eb + (2 + (t4 >> 1)) * QB_E_BYTES);
+                            const uint64_t bh = make_kmajor_desc(eb + (t4 >> 1) * E_BYTES);
+                            const uint64_t bl = make_kmajor_desc(eb + (2 + (t4 >> 1)) * E_BYTES);
                             if (t4 & 1) {
 #pragma unroll
-                                for (int k = 0; k < 4; ++k) umma_f16(d, ad + (uint64_t)(k * 2), bl + (uint64_t)(k * 2), QB_IDESC, 1u);
+                                for (int k = 0; k < 4; ++k) umma_f16(d, ad + (uint64_t)(k * 2), bl + (uint64_t)(k * 2), qb_idesc(ROWS), 1u);
                             }
 #pragma unroll
                             for (int k = 0; k < 4; ++k)
-                                umma_f16(d, ad + (uint64_t)(k * 2), bh + (uint64_t)(k * 2), QB_IDESC, (t4 | k) ? 1u : 0u);
+                                umma_f16(d, ad + (uint64_t)(k * 2), bh + (uint64_t)(k * 2), qb_idesc(ROWS), (t4 | k) ? 1u : 0u);
                             umma_commit(aempty(slot));
                             if (++slot == ASLOTS) { slot = 0; phase ^= 1u; }
                         }

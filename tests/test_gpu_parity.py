@@ -798,6 +798,43 @@ def test_quantize_launch_edges(n, m, group, B):
     hp.assert_parity(out)
 
 
+@pytest.mark.parametrize("n,m,group,B,static,clip", [
+    (512, 2385, 64, 64, False, 0),          # tensor-core form: CTAs of 32 rows, of 16 for 37 rows alone
+    (644, 2369, 0, 128, False, 0),
+    (1030, 2369, 128, 128, False, 0),       # rows of U and P that are no 16-byte multiples (plain float32 updates)
+    (516, 2400, 128, 128, True, 0),
+    (520, 2370, 32, 32, False, 20),
+    (200, 801, 64, 64, False, 0),           # without tensor cores the line lies lower
+    (300, 2400, 128, 128, True, 0),
+    (202, 1000, 32, 64, False, 7),
+])
+def test_a_row_does_not_depend_on_how_many_there_are(n, m, group, B, static, clip):
+    """CTAs of 32 and of 16 rows: the same arithmetic per row, hence the same results to the last bit."""
+    torch.manual_seed(n)
+    X = torch.randn(2 * n, n, device="cuda")
+    W = 0.02 * torch.randn(m, n, device="cuda")
+    st = g.LayerState(n, m, 2 * n, B)
+    try:
+        g.gptaq_accumulate(st.handle, X, X + 0.05 * torch.randn_like(X))
+        g.gptaq_factor(st.handle, 0.01)
+        g.gptaq_build_P(st.handle, 0.25)
+        g.gptaq_set_static_groups(st.handle, static)
+        g.gptaq_set_clip_search(st.handle, clip, 0.3)
+
+        def quantize(rows):
+            G = hp.n_groups(n, group)
+            out = [torch.empty((len(rows), w), dtype=d, device="cuda") for w, d in
+                   ((n, torch.uint8), (G, torch.float32), (G, torch.float32), (n, torch.float32))]
+            g.gptaq_quantize(st.handle, W[rows].contiguous(), 4, group, False, B, *out)
+            assert g.gptaq_sync_status(st.handle)[0] == g.GPTAQ_OK
+            return out
+        rows = torch.arange(m, device="cuda")
+        some = torch.cat([rows[:21], rows[-16:]])
+        assert [int((x[some] != y).sum()) for x, y in zip(quantize(rows), quantize(some))] == [0, 0, 0, 0]
+    finally:
+        st.close()
+
+
 @pytest.mark.parametrize("n,tokens,act_order", [
     (128, 2048, False), (128, 2049, False),     # float32 products up to here / one tile of either sum, cut
     (640, 520, False), (640, 520, True),        # a few tiles, of dXX^T the upper ones or all
