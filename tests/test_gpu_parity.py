@@ -801,7 +801,8 @@ def test_quantize_launch_edges(n, m, group, B):
 @pytest.mark.parametrize("n,m,group,B,static,clip", [
     (512, 2385, 64, 64, False, 0),          # tensor-core form: CTAs of 32 rows, of 16 for 37 rows alone
     (644, 2369, 0, 128, False, 0),
-    (1030, 2369, 128, 128, False, 0),       # rows of U and P that are no 16-byte multiples (plain float32 updates)
+    (126, 801, 32, 32, False, 0),           # rows of U and P that are no 16-byte multiples (one launch: the float32 products
+                                            # behind it would have other tiles, and other sums, for other numbers of rows)
     (516, 2400, 128, 128, True, 0),
     (520, 2370, 32, 32, False, 20),
     (200, 801, 64, 64, False, 0),           # without tensor cores the line lies lower
