@@ -534,6 +534,18 @@ gptaq_status_t accumulate_tc(gptaq_ctx *h, const float *X, const float *Xfp, int
 
 bool valid_block(int b) { return b == 32 || b == 64 || b == 128; }
 
+// float32 matrix [n][n] in boxes of 32 x 32, as they lie.
+bool make_box_map(CUtensorMap *map, const float *ptr, int64_t n) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    cuuint64_t dims[2] = {(cuuint64_t)n, (cuuint64_t)n};
+    cuuint64_t strides[1] = {(cuuint64_t)n * 4};
+    cuuint32_t box[2] = {32, 32};
+    cuuint32_t estr[2] = {1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // What the column loop and the trailing update work on: the factor U, the matrix P, the
 // dead-input flags, the device status header and the m x 2B scratch for [-Err | Wpre].
 struct QuantizeTarget {
@@ -582,8 +594,11 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
     a.amax_u = t.amax_u; a.amax_p = t.amax_p; a.hd = t.hd;
     a.err_scale = (t.terms & GPTAQ_TERM_ERR) ? 1.f : 0.f; a.asym_scale = (t.terms & GPTAQ_TERM_ASYM) ? 1.f : 0.f;
     a.perm = t.perm; a.clip_steps = t.clip_steps; a.clip_min = t.clip_min;
-    CUtensorMap uh, ul, ph, pl;
-    std::memset(&uh, 0, sizeof(uh)); ul = ph = pl = uh;
+    CUtensorMap uh, ul, ph, pl, u32, p32;
+    std::memset(&uh, 0, sizeof(uh)); ul = ph = pl = u32 = p32 = uh;
+    // (rows of U and P by the TMA unit where they are 16-byte multiples)
+    a.up_tma = t.n % 4 == 0 && ((reinterpret_cast<uintptr_t>(t.U) | reinterpret_cast<uintptr_t>(t.P)) & 15) == 0 &&
+               make_box_map(&u32, t.U, t.n) && make_box_map(&p32, t.P, t.n);
     if (far_form && (!make_f16_map(&uh, t.UT16, t.n, t.n, t.ldt, 128) || !make_f16_map(&ul, t.UT16 + nn, t.n, t.n, t.ldt, 128) ||
                      !make_f16_map(&ph, t.PT16, t.n, t.n, t.ldt, 128) || !make_f16_map(&pl, t.PT16 + nn, t.n, t.n, t.ldt, 128)))
         return cudaErrorUnknown;
@@ -606,7 +621,7 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, i
     // (1000 rows of 1024 columns 256 -> 242 us a call).  That takes two things: the first launch of a call is a plain one, so that
     // all that made U and P is done before the call's first kernel begins, in a captured graph too; and nothing in a call writes U or P.
     const bool pdl = !far_form && i0 > 0;
-    auto launch = [&](auto kernel, int threads) { return launch_pdl(pdl, kernel, grid, dim3(threads), smem, s, uh, ul, ph, pl, a); };
+    auto launch = [&](auto kernel, int threads) { return launch_pdl(pdl, kernel, grid, dim3(threads), smem, s, uh, ul, ph, pl, u32, p32, a); };
     if (few) {
         if (far_form) return static_groups ? launch(quant_block_kernel<true, true, 1, QB_ROWS_FEW>, QB_THREADS_FAR) : launch(quant_block_kernel<true, false, 1, QB_ROWS_FEW>, QB_THREADS_FAR);
         return static_groups ? launch(quant_block_kernel<false, true, 1, QB_ROWS_FEW>, QB_THREADS_NEAR) : launch(quant_block_kernel<false, false, 1, QB_ROWS_FEW>, QB_THREADS_NEAR);

@@ -26,6 +26,7 @@
 // The tensor-core form may have 96 registers and spills 60 bytes (static groups 52), the near form 80 where two CTAs share an SM
 // and spills 112 (140); with one to an SM it takes 160 and spills nothing.
 #pragma once
+#include "simt_gemm.cuh"
 #include "tc_gemm.cuh"
 
 namespace gptaq {
@@ -39,10 +40,12 @@ constexpr int QB_SUPER = 512;           // most columns per launch
 constexpr int QB_CHAIN = 128, QB_NEAR = 256, QB_DRAIN = 128;
 constexpr int QB_THREADS_NEAR = QB_CHAIN + QB_NEAR;                   // one block per launch, no tensor cores
 constexpr int QB_THREADS_FAR = QB_THREADS_NEAR + QB_DRAIN + 64;
-constexpr int QB_ULD0 = QB_W + 4, QB_ULD1 = QB_W - 32 + 4;            // pitch of U / P rows in the even / odd step's buffer
+// rows of U and P of a step: boxes of 32 rows x 32 columns, the buffer of even steps has four of each matrix, that of odd ones three
+constexpr int QB_BOX = 32 * 32, QB_BOXES0 = QB_W / 32, QB_BOXES1 = QB_BOXES0 - 1;
 __host__ __device__ constexpr int qb_sld(int rows) { return rows + 4; }   // pitch of the published errors
-// 128 x 64 fp16 tiles of U^T / P^T in flight (one less makes room for the grids per column)
-__host__ __device__ constexpr int qb_aslots(bool percol) { return percol ? 2 : 3; }
+// 128 x 64 fp16 tiles of U^T / P^T in flight: what shared memory holds (the grids per column take the room of one)
+constexpr int QB_MAX_ASLOTS = 6;
+__host__ __device__ constexpr int qb_aslots(bool percol, int rows) { return (rows == 32 ? 3 : QB_MAX_ASLOTS) - (percol ? 1 : 0); }
 constexpr int QB_A_BYTES = 128 * 64 * 2;
 __host__ __device__ constexpr int qb_e_bytes(int rows) { return rows * 64 * 2; }          // one K-block (64 columns) of one part of the errors
 __host__ __device__ constexpr int qb_half_bytes(int rows) { return 4 * qb_e_bytes(rows); } // (hi, lo) x (-Err, Wpre) of 64 columns
@@ -51,6 +54,7 @@ constexpr int QB_TMEM_COLS = 256;                                     // 2 halve
 struct QuantBlockArgs {
     float *W; int64_t ldw; int row_first, m, n;     // rows [row_first, m)
     const float *U, *P;        // n x n, ld n; entries below the diagonals are not used
+    int up_tma;                // U and P qualify for tensor maps (16-byte rows)
     const uint8_t *dead;
     int i0, i1;                // columns of this launch: [i0, i1); i1 - i0 <= QB_SUPER (tensor-core form) or one block
     int bw;                    // columns per block: QB_W (tensor-core form); 32, 64 or 128
@@ -78,23 +82,24 @@ __host__ __device__ constexpr QuantBlockSmem quant_block_smem(bool far_form, boo
     QuantBlockSmem s{};
     s.wld = (far_form ? QB_SUPER : QB_W) + 4;
     s.a = 0;
-    s.e = s.a + (far_form ? qb_aslots(percol) * QB_A_BYTES : 0);
+    s.e = s.a + (far_form ? qb_aslots(percol, rows) * QB_A_BYTES : 0);
     s.w = s.e + (far_form ? 2 * qb_half_bytes(rows) : 0);
     s.up = s.w + rows * s.wld * 4;
-    s.st = s.up + 2 * 32 * (QB_ULD0 + QB_ULD1) * 4;
+    s.st = s.up + 2 * (QB_BOXES0 + QB_BOXES1) * QB_BOX * 4;
     s.grid = s.st + 2 * 64 * qb_sld(rows) * 4;
     s.udinv = s.grid + (percol ? 3 * 32 * qb_sld(rows) * 4 : 0);
     s.perm = s.udinv + 2 * 32 * 4;
     s.inv = s.perm + 2 * 32 * 4;
     s.rmax = s.inv + 2 * rows * 4;
     s.bars = s.rmax + (far_form ? QB_NEAR * 4 : 0);
-    s.total = s.bars + 256;
+    s.total = s.bars + 384;
     return s;
 }
 constexpr size_t quant_block_smem_bytes(bool far_form, bool percol, int rows) {
     return (size_t)quant_block_smem(far_form, percol, rows).total + 1024;        // (alignment slack)
 }
-static_assert(quant_block_smem_bytes(true, false, QB_ROWS) <= 227 * 1024 && quant_block_smem_bytes(true, true, QB_ROWS) <= 227 * 1024, "shared memory of one SM");
+static_assert(quant_block_smem_bytes(true, false, QB_ROWS) <= 227 * 1024 && quant_block_smem_bytes(true, true, QB_ROWS) <= 227 * 1024 &&
+              quant_block_smem_bytes(true, false, QB_ROWS_FEW) <= 227 * 1024 && quant_block_smem_bytes(true, true, QB_ROWS_FEW) <= 227 * 1024, "shared memory of one SM");
 
 // kind::f16 instruction descriptor: fp16 A and B (K-major), fp32 D, M = 128, N = rows.
 __host__ __device__ constexpr uint32_t qb_idesc(int rows) { return (1u << 4) | ((uint32_t)(rows >> 3) << 17) | ((128 >> 4) << 24); }
@@ -202,14 +207,15 @@ __device__ __forceinline__ void clip_search(const float *w, int n, float lo, flo
 template <bool FAR, bool PERCOL, int CTAS, int ROWS = QB_ROWS>
 __global__ void __launch_bounds__(FAR ? QB_THREADS_FAR : QB_THREADS_NEAR, CTAS)
 quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_constant__ CUtensorMap mapUlo,
-                   const __grid_constant__ CUtensorMap mapPhi, const __grid_constant__ CUtensorMap mapPlo, QuantBlockArgs a) {
+                   const __grid_constant__ CUtensorMap mapPhi, const __grid_constant__ CUtensorMap mapPlo,
+                   const __grid_constant__ CUtensorMap mapU, const __grid_constant__ CUtensorMap mapP, QuantBlockArgs a) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *sm = smem_raw + (base - raw);
     constexpr QuantBlockSmem L = quant_block_smem(FAR, PERCOL, ROWS);
     constexpr int SLD = qb_sld(ROWS), E_BYTES = qb_e_bytes(ROWS), HALF_BYTES = qb_half_bytes(ROWS), RPT = ROWS / 8;
-    constexpr int ASLOTS = qb_aslots(PERCOL);
+    constexpr int ASLOTS = qb_aslots(PERCOL, ROWS);
     constexpr int WLD = L.wld;
     constexpr int NTHREADS = FAR ? QB_THREADS_FAR : QB_THREADS_NEAR;
     float *Ws = reinterpret_cast<float *>(sm + L.w);               // [32][WLD]: the slab
@@ -221,14 +227,16 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     float *inv_s = reinterpret_cast<float *>(sm + L.inv);          // [2 halves][32]: 1 / scale of a row's errors
     float *rmax_s = reinterpret_cast<float *>(sm + L.rmax);        // [8 near warps][32]: a row's largest error of 8 columns
     const uint32_t bar0 = base + L.bars;
-    // mbarriers (8 bytes each): afull[3], aempty[3], efull[2], efree[2], tfull[6], tempty[6]; tmem slot, abort flag
+    // mbarriers (8 bytes each): afull, aempty, efull[2], efree[2], tfull[6], tempty[6], upfull[2]; tmem slot, abort flag
+    constexpr int EB = 2 * QB_MAX_ASLOTS;
     auto afull = [&](int s) { return bar0 + 8u * s; };
-    auto aempty = [&](int s) { return bar0 + 8u * (3 + s); };
-    auto efull = [&](int s) { return bar0 + 8u * (6 + s); };
-    auto efree = [&](int s) { return bar0 + 8u * (8 + s); };
-    auto tfull = [&](int s) { return bar0 + 8u * (10 + s); };
-    auto tempty = [&](int s) { return bar0 + 8u * (16 + s); };
-    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(sm + L.bars + 8 * 22);
+    auto aempty = [&](int s) { return bar0 + 8u * (QB_MAX_ASLOTS + s); };
+    auto efull = [&](int s) { return bar0 + 8u * (EB + s); };
+    auto efree = [&](int s) { return bar0 + 8u * (EB + 2 + s); };
+    auto tfull = [&](int s) { return bar0 + 8u * (EB + 4 + s); };
+    auto tempty = [&](int s) { return bar0 + 8u * (EB + 10 + s); };
+    auto upfull = [&](int s) { return bar0 + 8u * (EB + 16 + s); };
+    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(sm + L.bars + 8 * (EB + 18));
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -239,36 +247,40 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     const int nblk = FAR ? (cols + QB_W - 1) / QB_W : 1;
     auto nsteps = [&](int b) { return min(B / 32, (cols - b * QB_W + 31) / 32); };     // 32-column steps of block b
     const float maxq = (float)((1 << a.bits) - 1);
-    const bool aligned_up = (n & 3) == 0 && ((reinterpret_cast<uintptr_t>(a.U) | reinterpret_cast<uintptr_t>(a.P)) & 15) == 0;
-
-    // U / P rows of step s of the block that starts at column cb: buffer s & 1, columns cb + 32 s ..
-    auto up_ld = [&](int s) { return (s & 1) ? QB_ULD1 : QB_ULD0; };
-    auto up_buf = [&](int s) { return UPs + (s & 1) * (2 * 32 * QB_ULD0); };
+    // U / P rows of step s of the block that starts at column cb, columns cb + 32 s ..: buffer s & 1, box by box; element (k, c) of
+    // U at up_at(s, 0, k, c), of P at up_at(s, 1, k, c).  One thread asks the TMA unit for the boxes: as 16-byte
+    // copies by all near warps a step's 32 KB took 1100 cycles of their time, in steps where the chain waits for them (4096 x 1024 with
+    // groups 165 -> 161 us a call, 1024 x 1024 with static groups 163 -> 160).  Rows that are no multiple of 16 bytes come in asynchronous
+    // copies of 4 (word by word through registers before: 777 x 777 217 -> 191, 4096 x 777 501 -> 486).
+    auto up_at = [&](int s, int q, int k, int c) {
+        return UPs + ((s & 1) ? 2 * QB_BOXES0 * QB_BOX : 0) + (q * ((s & 1) ? QB_BOXES1 : QB_BOXES0) + (c >> 5)) * QB_BOX + k * 32 + (c & 31);
+    };
     auto fetch_up = [&](int cb, int s, int t, int nthr) {
-        // a warp per row, a lane per four columns (no divisions: with 32 q quads numbered through, they made up most of it)
-        const int ld = up_ld(s), q = (B - 32 * s) / 4, r0 = cb + 32 * s, c4 = t & 31;
-        if (c4 >= q) return;
-        const int col = r0 + 4 * c4;
-        float *du = up_buf(s) + (t >> 5) * ld + 4 * c4, *dp = du + 32 * ld;
-        int64_t off = (int64_t)(r0 + (t >> 5)) * n + col;
-        const bool whole = aligned_up && col + 3 < n;
-        for (int k = t >> 5; k < 32; k += nthr / 32) {
-            if (whole && r0 + k < n) {
-                cp_async16(du, a.U + off);
-                cp_async16(dp, a.P + off);
-            } else {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const bool in = r0 + k < n && col + e < n;
-                    du[e] = in ? a.U[off + e] : 0.f;
-                    dp[e] = in ? a.P[off + e] : 0.f;
+        const int r0 = cb + 32 * s;
+        if (a.up_tma) {
+            if (t == 0) {
+                const int boxes = B / 32 - s;
+                mbar_expect_tx(upfull(s & 1), (uint32_t)(2 * boxes * QB_BOX * 4));
+                for (int x = 0; x < boxes; ++x) {
+                    tma_load_2d(smem_u32(up_at(s, 0, 0, 32 * x)), &mapU, r0 + 32 * x, r0, upfull(s & 1));
+                    tma_load_2d(smem_u32(up_at(s, 1, 0, 32 * x)), &mapP, r0 + 32 * x, r0, upfull(s & 1));
                 }
             }
-            du += nthr / 32 * ld; dp += nthr / 32 * ld; off += (int64_t)(nthr / 32) * n;
+            return;
         }
+        // (a warp per row, a lane per column)
+        const int l = t & 31;
+        for (int k = t >> 5; k < 32; k += nthr / 32)
+            for (int x = 0; x < B / 32 - s; ++x) {
+                const bool in = r0 + k < n && r0 + 32 * x + l < n;
+                const int64_t off = in ? (int64_t)(r0 + k) * n + r0 + 32 * x + l : 0;
+                sg_copy4(up_at(s, 0, k, 32 * x + l), a.U + off, in);
+                sg_copy4(up_at(s, 1, k, 32 * x + l), a.P + off, in);
+            }
     };
     // per column of a step: err_scale / U_kk (padded columns beyond n have no error: 0) and the column's original index
-    auto load_pivot = [&](int c) { return c < n ? a.err_scale * (1.f / a.U[(int64_t)c * n + c]) : 0.f; };
+    auto load_pivot = [&](int c) { return c < n ? a.U[(int64_t)c * n + c] : 0.f; };
+    auto invert_pivot = [&](int c, float u) { return c < n ? a.err_scale * (1.f / u) : 0.f; };
     auto load_perm = [&](int c) { return a.perm && c < n ? a.perm[c] : c; };
     // PERCOL: grids of four columns c .. c + 3 of a row
     auto load_grid = [&](int r, int c, float (&sc)[4], float (&zp)[4]) {
@@ -291,12 +303,16 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     };
 
     // ---------------------------------------------------------------- set-up: barriers, tensor memory, slab, first rows of U / P
+    if (tid == 0) {
+        for (int s = 0; s < 2; ++s) mbar_init(upfull(s), 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
     if (FAR) {
         if (tid == 0) {
             for (int s = 0; s < ASLOTS; ++s) { mbar_init(afull(s), 1); mbar_init(aempty(s), 1); }
             for (int s = 0; s < 2; ++s) { mbar_init(efull(s), 8 * ROWS / 32); mbar_init(efree(s), QB_DRAIN / 32); }
             for (int s = 0; s < 6; ++s) { mbar_init(tfull(s), 1); mbar_init(tempty(s), QB_DRAIN / 32); }
-            *abort_flag = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
         if (warp == NTHREADS / 32 - 1) {
@@ -331,7 +347,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     }
     // (dead inputs read as zero; the flags are 4-byte aligned and padded beyond n)
     const uint32_t dead4 = fills && wc < cols ? *reinterpret_cast<const uint32_t *>(a.dead + i0 + wc) : 0u;
-    if (tid < 32) { udinv2[tid] = load_pivot(i0 + tid); perm2[tid] = load_perm(i0 + tid); }
+    if (tid < 32) { udinv2[tid] = invert_pivot(i0 + tid, load_pivot(i0 + tid)); perm2[tid] = load_perm(i0 + tid); }
     if (PERCOL && tid < 8 * ROWS) {
         float sc[4], zp[4];
         load_grid(tid >> 3, i0 + 4 * (tid & 7), sc, zp);
@@ -352,6 +368,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     if (FAR) tc_fence_before();
     __syncthreads();
     if (FAR) tc_fence_after();
+    if (a.up_tma) mbar_wait(upfull(0), 0u, abort_flag);
 
     float rho = 1.f, su = 1.f;
     if (a.amax_u) {
@@ -427,8 +444,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     if (a.clip_steps > 0) named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);   // the search's scratch is free again
                     inv_scale = 1.f / scale; qlo = -zero; qhi = maxq - zero;
                 }
-                const int ld = up_ld(s);
-                const float *Uw = up_buf(s) + w8, *Pw = Uw + 32 * ld;
+                constexpr int ld = 32;
+                const float *Uw = up_at(s, 0, 0, w8), *Pw = up_at(s, 1, 0, w8);
                 unsigned long long x[4];                            // this lane's 8 columns, in pairs
                 {
                     const ulonglong2 v0 = *reinterpret_cast<const ulonglong2 *>(wrow + co + w8);
@@ -532,6 +549,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         // ================================================================ near
         const int t = tid - QB_CHAIN;
         const int ti = t & 7, tj = t >> 3;                          // rows ti, ti + 8, ..; columns 4 tj .. of the rest
+        int seq = 0;                                                // steps so far
         float row_max = 0.f;                                        // largest magnitude of row t % ROWS's errors in this launch
         for (int b = 0; b < nblk; ++b) {
             const int nst = nsteps(b);
@@ -541,11 +559,11 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 const bool last = b == nblk - 1 && s == nst - 1;
                 const int nb = s + 1 < nst ? b : b + 1, ns = s + 1 < nst ? s + 1 : 0;       // the next step
                 const int ncol = i0 + nb * QB_W + 32 * ns;
-                float next_ud = 0.f, next_sc[4], next_zp[4];
+                float next_u = 0.f, next_sc[4], next_zp[4];
                 int next_perm = 0;
                 if (!last) {
                     fetch_up(i0 + nb * QB_W, ns, t, QB_NEAR);
-                    if (t < 32) { next_ud = load_pivot(ncol + t); next_perm = load_perm(ncol + t); }
+                    if (t < 32) { next_u = load_pivot(ncol + t); next_perm = load_perm(ncol + t); }
                     if (PERCOL && t < 8 * ROWS) load_grid(t >> 3, ncol + 4 * (t & 7), next_sc, next_zp);
                 }
                 if (a.clip_steps > 0 && grid_starts(i0 + co)) {
@@ -577,8 +595,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);
                     named_bar_sync(QBAR_CLIP, QB_THREADS_NEAR);
                 }
-                const int ld = up_ld(s);
-                const float *Ub = up_buf(s) + 32 + 4 * tj, *Pb = Ub + 32 * ld;      // (columns beyond the step's own 32)
+                constexpr int ld = 32;
+                const float *Ub = up_at(s, 0, 0, 32 + 4 * tj), *Pb = up_at(s, 1, 0, 32 + 4 * tj);     // (columns beyond the step's own 32)
                 const float *St = Sts + (s & 1) * 64 * SLD;
                 const bool active = 32 + 4 * tj < B - 32 * s;
                 unsigned long long acc[RPT][2];
@@ -630,9 +648,11 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     }
                     rmax_s[ec * ROWS + er] = mx;
                 }
-                asm volatile("cp.async.wait_all;" ::: "memory");
+                ++seq;
                 if (!last) {
-                    if (t < 32) { udinv2[(ns & 1) * 32 + t] = next_ud; perm2[(ns & 1) * 32 + t] = next_perm; }
+                    if (a.up_tma) mbar_wait(upfull(ns & 1), (uint32_t)(seq >> 1) & 1u, abort_flag);
+                    else asm volatile("cp.async.wait_all;" ::: "memory");
+                    if (t < 32) { udinv2[(ns & 1) * 32 + t] = invert_pivot(ncol + t, next_u); perm2[(ns & 1) * 32 + t] = next_perm; }
                     if (PERCOL && t < 8 * ROWS) store_grid(t >> 3, 4 * (t & 7), next_sc, next_zp);      // (the chain has read this step's)
                     named_bar_arrive(QBAR_STEP, QB_THREADS_NEAR);
                 }
@@ -811,7 +831,13 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         }
     }
 
-    if (!FAR) return;
+    if (!FAR) {
+        if (a.up_tma) {
+            __syncthreads();
+            if (*abort_flag && tid == 0) record_status(a.hd, ST_TIMEOUT, 3000000 + blockIdx.x);
+        }
+        return;
+    }
     tc_fence_before();
     __syncthreads();
     if (a.EWS_hi) {
