@@ -45,6 +45,9 @@ __device__ __forceinline__ float split_scale_bits(unsigned amax) {
     return __uint_as_float(min(267u - (amax >> 23), 241u) << 23);       // biased exponents: 127 + 14 - (e - 126)
 }
 
+// 1 / s for a power of two s whose reciprocal is normal, too.
+__device__ __forceinline__ float pow2_inverse(float s) { return __uint_as_float(0x7f000000u - __float_as_uint(s)); }
+
 // Programmatic dependent launch: a kernel launched with the stream-serialization attribute may be
 // scheduled while its predecessor in the stream drains; pdl_wait() returns once the predecessor has
 // completed and its writes are visible (a no-op for a plain launch), pdl_launch_dependents() lets the

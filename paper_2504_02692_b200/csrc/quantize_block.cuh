@@ -12,8 +12,8 @@
 //                      columns the tensor cores' operand, writes results out;
 //   drain   (4 warps)  adds the products of the tensor cores to the later blocks of the slab;
 //   load, mma (1 + 1)  stream U^T and P^T (fp16 hi / lo parts) and issue
-//                      D[128 later columns][32 rows] = [U^T | P^T] [-Err | rho Wpre]^T   (tcgen05, M = 128, N = 32)
-//                      for every 64 quantized columns, as lo*hi + hi*lo + hi*hi.
+//                      D[128 later columns][32 rows] = [U^T | P^T] [-Err | rho Wpre]^T   (tcgen05, M = 128)
+//                      for every 64 quantized columns; hi*hi and the small terms hi*lo + lo*hi have a column each.
 //
 // What bounds it: the chain, and the near warps behind it.  A column is 7 dependent float32 operations (28 cycles); with its
 // share of the updates, the codes and the hand-over to the next warp 8 columns take 750 cycles alone and 950 beside the near
@@ -49,7 +49,8 @@ __host__ __device__ constexpr int qb_aslots(bool percol, int rows) { return (row
 constexpr int QB_A_BYTES = 128 * 64 * 2;
 __host__ __device__ constexpr int qb_e_bytes(int rows) { return rows * 64 * 2; }          // one K-block (64 columns) of one part of the errors
 __host__ __device__ constexpr int qb_half_bytes(int rows) { return 4 * qb_e_bytes(rows); } // (hi, lo) x (-Err, Wpre) of 64 columns
-constexpr int QB_TMEM_COLS = 256;                                     // 2 halves x 3 blocks x 32 columns, a power of two
+// tensor memory: 2 halves x 3 blocks x 2 groups (hi hi; hi lo + lo hi) of a column per row, a power of two
+__host__ __device__ constexpr int qb_tmem_cols(int rows) { return rows == 32 ? 512 : 256; }
 
 struct QuantBlockArgs {
     float *W; int64_t ldw; int row_first, m, n;     // rows [row_first, m)
@@ -101,8 +102,8 @@ constexpr size_t quant_block_smem_bytes(bool far_form, bool percol, int rows) {
 static_assert(quant_block_smem_bytes(true, false, QB_ROWS) <= 227 * 1024 && quant_block_smem_bytes(true, true, QB_ROWS) <= 227 * 1024 &&
               quant_block_smem_bytes(true, false, QB_ROWS_FEW) <= 227 * 1024 && quant_block_smem_bytes(true, true, QB_ROWS_FEW) <= 227 * 1024, "shared memory of one SM");
 
-// kind::f16 instruction descriptor: fp16 A and B (K-major), fp32 D, M = 128, N = rows.
-__host__ __device__ constexpr uint32_t qb_idesc(int rows) { return (1u << 4) | ((uint32_t)(rows >> 3) << 17) | ((128 >> 4) << 24); }
+// kind::f16 instruction descriptor: fp16 A and B (K-major), fp32 D, M = 128, N = cols.
+__host__ __device__ constexpr uint32_t qb_idesc(int cols) { return (1u << 4) | ((uint32_t)(cols >> 3) << 17) | ((128 >> 4) << 24); }
 
 // Named barriers.  Chunk barriers are used once per step each; the step barrier keeps the chain from lapping them.
 enum { QBAR_CHUNK = 1, QBAR_STEP = 5, QBAR_NEAR = 6, QBAR_DRAIN = 7, QBAR_CLIP = 8, QBAR_HAND = 9 /* .. 14 */, QBAR_CHAIN = 15 };
@@ -317,7 +318,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         }
         if (warp == NTHREADS / 32 - 1) {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                         ::"r"(smem_u32(const_cast<uint32_t *>(tmem_slot))), "r"((uint32_t)QB_TMEM_COLS) : "memory");
+                         ::"r"(smem_u32(const_cast<uint32_t *>(tmem_slot))), "r"((uint32_t)qb_tmem_cols(ROWS)) : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
     }
@@ -376,6 +377,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         const float ap = __uint_as_float(*a.amax_p);
         rho = ap > 0.f ? su / split_scale(ap) : 0.f;
     }
+    const float inv_su = 1.f / su;
     const int last_groups = nblk - 1;                               // blocks 0 .. nblk - 2 have later blocks in this launch
     // a grid is made at column c (groups have 32, 64 or 128 columns)
     auto grid_starts = [&](int c) { return !PERCOL && a.group > 0 && (c & (a.group - 1)) == 0; };
@@ -666,8 +668,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         const int half = s >> 1;                    // buffer: even and odd halves alternate
                         // (the drain warps are done with this buffer's row scales, the MMAs with its operands)
                         if (b > 0) mbar_wait(efree(half), (uint32_t)(b - 1) & 1u, abort_flag);
-                        const float sc = split_scale(mx);
-                        if (ec == 0) inv_s[half * ROWS + er] = 1.f / sc / su;
+                        const float sc = split_scale_bits(__float_as_uint(mx));
+                        if (ec == 0) inv_s[half * ROWS + er] = pow2_inverse(sc) * inv_su;
                         uint8_t *eb = sm + L.e + half * HALF_BYTES + (er >> 3) * 1024 + (er & 7) * 128 + ((ec ^ (er & 7)) << 4);
 #pragma unroll
                         for (int o = 0; o < 2; ++o) {
@@ -676,8 +678,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                             uint2 h0, l0, h1, l1;
                             split16_pack(y0, h0, l0);
                             split16_pack(y1, h1, l1);
-                            *reinterpret_cast<uint4 *>(eb + o * E_BYTES) = make_uint4(h0.x, h0.y, h1.x, h1.y);
-                            *reinterpret_cast<uint4 *>(eb + (2 + o) * E_BYTES) = make_uint4(l0.x, l0.y, l1.x, l1.y);
+                            *reinterpret_cast<uint4 *>(eb + 2 * o * E_BYTES) = make_uint4(h0.x, h0.y, h1.x, h1.y);
+                            *reinterpret_cast<uint4 *>(eb + (2 * o + 1) * E_BYTES) = make_uint4(l0.x, l0.y, l1.x, l1.y);
                         }
                         fence_proxy_async_smem();
                         __syncwarp();
@@ -733,10 +735,10 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
             }
         }
         if (FAR && a.EWS_hi && t < ROWS) {
-            const float sc = t < nrows ? split_scale(row_max) : 1.f;
+            const float sc = t < nrows ? split_scale_bits(__float_as_uint(row_max)) : 1.f;
             udinv2[t] = sc;                                         // (free: the last step's pivots are in the other half; read
                                                                     //  after the barrier below)
-            if (t < nrows) a.row_inv[row0 + t] = 1.f / sc;
+            if (t < nrows) a.row_inv[row0 + t] = pow2_inverse(sc);
         }
     } else if (FAR && tid < QB_THREADS_NEAR + QB_DRAIN) {
         // ================================================================ drain: tensor memory -> later blocks of the slab
@@ -749,9 +751,10 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     const int slot = half * 3 + (j - 1);            // (used once per earlier block: b = 0 .. j - 1)
                     mbar_wait(tfull(slot), (uint32_t)b & 1u, abort_flag);
                     tc_fence_after();
-                    uint32_t v[ROWS];
-                    if constexpr (ROWS == 32) tmem_ld32(tmem_base + slot * ROWS + ((uint32_t)(quarter * 32) << 16), v);
-                    else tmem_ld16(tmem_base + slot * ROWS + ((uint32_t)(quarter * 32) << 16), v);
+                    uint32_t v[ROWS], l[ROWS];                      // hi hi; hi lo + lo hi
+                    const uint32_t taddr = tmem_base + slot * 2 * ROWS + ((uint32_t)(quarter * 32) << 16);
+                    if constexpr (ROWS == 32) { tmem_ld32(taddr, v); tmem_ld32(taddr + ROWS, l); }
+                    else { tmem_ld16(taddr, v); tmem_ld16(taddr + ROWS, l); }
                     tmem_ld_wait();
                     tc_fence_before();
                     __syncwarp();
@@ -761,10 +764,10 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     for (int r4 = 0; r4 < ROWS / 4; ++r4) {
                         const float4 iv = *reinterpret_cast<const float4 *>(inv_s + half * ROWS + 4 * r4);
                         float *w4 = wp + 4 * r4 * WLD;
-                        w4[0] = fmaf(__uint_as_float(v[4 * r4]), iv.x, w4[0]);
-                        w4[WLD] = fmaf(__uint_as_float(v[4 * r4 + 1]), iv.y, w4[WLD]);
-                        w4[2 * WLD] = fmaf(__uint_as_float(v[4 * r4 + 2]), iv.z, w4[2 * WLD]);
-                        w4[3 * WLD] = fmaf(__uint_as_float(v[4 * r4 + 3]), iv.w, w4[3 * WLD]);
+                        w4[0] = fmaf(__uint_as_float(v[4 * r4]) + __uint_as_float(l[4 * r4]), iv.x, w4[0]);
+                        w4[WLD] = fmaf(__uint_as_float(v[4 * r4 + 1]) + __uint_as_float(l[4 * r4 + 1]), iv.y, w4[WLD]);
+                        w4[2 * WLD] = fmaf(__uint_as_float(v[4 * r4 + 2]) + __uint_as_float(l[4 * r4 + 2]), iv.z, w4[2 * WLD]);
+                        w4[3 * WLD] = fmaf(__uint_as_float(v[4 * r4 + 3]) + __uint_as_float(l[4 * r4 + 3]), iv.w, w4[3 * WLD]);
                     }
                     if (half == 1 && j == b + 1) named_bar_arrive(QBAR_DRAIN, QB_CHAIN + QB_DRAIN);
                 }
@@ -780,9 +783,9 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
             for (int b = 0; ok && b < last_groups; ++b)
                 for (int half = 0; ok && half < 2; ++half)
                     for (int j = b + 1; ok && j < nblk; ++j)
-                        for (int t4 = 0; t4 < 4; ++t4) {            // U lo, U hi, P lo, P hi
+                        for (int t4 = 0; t4 < 4; ++t4) {            // U hi, U lo, P hi, P lo
                             if (!mbar_wait(aempty(slot), phase ^ 1u, abort_flag)) { ok = false; break; }
-                            const CUtensorMap *map = t4 == 0 ? &mapUlo : (t4 == 1 ? &mapUhi : (t4 == 2 ? &mapPlo : &mapPhi));
+                            const CUtensorMap *map = t4 == 0 ? &mapUhi : (t4 == 1 ? &mapUlo : (t4 == 2 ? &mapPhi : &mapPlo));
                             mbar_expect_tx(afull(slot), QB_A_BYTES);
                             tma_load_2d(base + L.a + slot * QB_A_BYTES, map, i0 + b * QB_W + 64 * half, i0 + j * QB_W, afull(slot));
                             ++issued;
@@ -808,20 +811,23 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         const int acc = half * 3 + (j - 1);
                         if (b > 0 && !mbar_wait(tempty(acc), (uint32_t)(b - 1) & 1u, abort_flag)) { ok = false; break; }
                         tc_fence_after();
-                        const uint32_t d = tmem_base + acc * ROWS;
+                        const uint32_t d = tmem_base + acc * 2 * ROWS;
                         for (int t4 = 0; t4 < 4; ++t4) {
                             if (!mbar_wait(afull(slot), phase, abort_flag)) { ok = false; break; }
                             tc_fence_after();
                             const uint64_t ad = make_kmajor_desc(base + L.a + slot * QB_A_BYTES);
-                            const uint64_t bh = make_kmajor_desc(eb + (t4 >> 1) * E_BYTES);
-                            const uint64_t bl = make_kmajor_desc(eb + (2 + (t4 >> 1)) * E_BYTES);
+                            // [hi | lo] of the errors are the rows of one operand: a tile of hi takes both in one pass (an MMA of
+                            // 128 rows takes 95 cycles with 16 columns and 115 with 64): 16 MMAs for 24 where the chain waits for
+                            // a block, 2300 -> 1820 cycles
+                            const uint64_t bd = make_kmajor_desc(eb + (t4 >> 1) * 2 * E_BYTES);
                             if (t4 & 1) {
 #pragma unroll
-                                for (int k = 0; k < 4; ++k) umma_f16(d, ad + (uint64_t)(k * 2), bl + (uint64_t)(k * 2), qb_idesc(ROWS), 1u);
-                            }
+                                for (int k = 0; k < 4; ++k) umma_f16(d + ROWS, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), qb_idesc(ROWS), 1u);
+                            } else {
 #pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                umma_f16(d, ad + (uint64_t)(k * 2), bh + (uint64_t)(k * 2), qb_idesc(ROWS), (t4 | k) ? 1u : 0u);
+                                for (int k = 0; k < 4; ++k)
+                                    umma_f16(d, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), qb_idesc(2 * ROWS), (t4 | k) ? 1u : 0u);
+                            }
                             umma_commit(aempty(slot));
                             if (++slot == ASLOTS) { slot = 0; phase ^= 1u; }
                         }
@@ -868,7 +874,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     if (*abort_flag && tid == 0) record_status(a.hd, ST_TIMEOUT, 3000000 + blockIdx.x);
     if (warp == NTHREADS / 32 - 1) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"((uint32_t)QB_TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"((uint32_t)qb_tmem_cols(ROWS)) : "memory");
     }
 }
 
