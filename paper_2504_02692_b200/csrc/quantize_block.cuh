@@ -89,8 +89,8 @@ __host__ __device__ constexpr QuantBlockSmem quant_block_smem(bool far_form, boo
     s.st = s.up + 2 * (QB_BOXES0 + QB_BOXES1) * QB_BOX * 4;
     s.grid = s.st + 2 * 64 * qb_sld(rows) * 4;
     s.udinv = s.grid + (percol ? 3 * 32 * qb_sld(rows) * 4 : 0);
-    s.perm = s.udinv + 2 * 32 * 4;
-    s.inv = s.perm + 2 * 32 * 4;
+    s.perm = s.udinv + (s.wld - 4) * 4;
+    s.inv = s.perm + (s.wld - 4) * 4;
     s.rmax = s.inv + 2 * rows * 4;
     s.bars = s.rmax + (far_form ? QB_NEAR * 4 : 0);
     s.total = s.bars + 384;
@@ -223,8 +223,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     float *UPs = reinterpret_cast<float *>(sm + L.up);             // rows of U and P of the current and the next step
     float *Sts = reinterpret_cast<float *>(sm + L.st);             // [2 steps][64][SLD]: -Err, then Wpre, of 32 columns
     float *grid_s = reinterpret_cast<float *>(sm + L.grid);        // PERCOL: scales, zero points, 1 / scales, [32 columns][SLD] each
-    float *udinv2 = reinterpret_cast<float *>(sm + L.udinv);       // [2 steps][32]: err_scale / U_kk
-    int *perm2 = reinterpret_cast<int *>(sm + L.perm);             // [2 steps][32]: where a column's codes go
+    float *udinv_s = reinterpret_cast<float *>(sm + L.udinv);      // of every column of the launch: err_scale / U_kk
+    int *perm_s = reinterpret_cast<int *>(sm + L.perm);            // ... and where its codes go
     float *inv_s = reinterpret_cast<float *>(sm + L.inv);          // [2 halves][32]: 1 / scale of a row's errors
     float *rmax_s = reinterpret_cast<float *>(sm + L.rmax);        // [8 near warps][32]: a row's largest error of 8 columns
     const uint32_t bar0 = base + L.bars;
@@ -279,9 +279,6 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 sg_copy4(up_at(s, 1, k, 32 * x + l), a.P + off, in);
             }
     };
-    // per column of a step: err_scale / U_kk (padded columns beyond n have no error: 0) and the column's original index
-    auto load_pivot = [&](int c) { return c < n ? a.U[(int64_t)c * n + c] : 0.f; };
-    auto invert_pivot = [&](int c, float u) { return c < n ? a.err_scale * (1.f / u) : 0.f; };
     auto load_perm = [&](int c) { return a.perm && c < n ? a.perm[c] : c; };
     // PERCOL: grids of four columns c .. c + 3 of a row
     auto load_grid = [&](int r, int c, float (&sc)[4], float (&zp)[4]) {
@@ -348,7 +345,13 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     }
     // (dead inputs read as zero; the flags are 4-byte aligned and padded beyond n)
     const uint32_t dead4 = fills && wc < cols ? *reinterpret_cast<const uint32_t *>(a.dead + i0 + wc) : 0u;
-    if (tid < 32) { udinv2[tid] = invert_pivot(i0 + tid, load_pivot(i0 + tid)); perm2[tid] = load_perm(i0 + tid); }
+    // (padded columns beyond n have no error: 0.  All at once here: with a step's 32 made by the near warps at the end of the step before,
+    // the operand behind what the next step needs at a block's end and the minima eight columns at a time 512 x 1024 took 131 us, now
+    // 130; 2369 x 1024 154.6 and 150.5, 4768 x 1024 231 and 226, 512 x 1024 without tensor cores 213 and 204)
+    for (int c = tid; c < L.wld - 4; c += NTHREADS) {
+        udinv_s[c] = i0 + c < n && c < cols ? a.err_scale * (1.f / a.U[(int64_t)(i0 + c) * n + i0 + c]) : 0.f;
+        perm_s[c] = load_perm(i0 + c);
+    }
     if (PERCOL && tid < 8 * ROWS) {
         float sc[4], zp[4];
         load_grid(tid >> 3, i0 + 4 * (tid & 7), sc, zp);
@@ -416,11 +419,14 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     // a quarter of the range per warp
                     float lo = 0.f, hi = 0.f;
                     const float *wq4 = wrow + co + warp * (a.group >> 2);
-#pragma unroll 2
-                    for (int c = 0; c < a.group >> 2; c += 4) {
-                        const float4 v = *reinterpret_cast<const float4 *>(wq4 + c);
-                        lo = fminf(lo, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
-                        hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                    float4 v[8];                                    // (all loads in flight: 8, 16 or 32 columns)
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        v[c] = 4 * c < a.group >> 2 ? *reinterpret_cast<const float4 *>(wq4 + 4 * c) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        lo = fminf(lo, fminf(fminf(v[c].x, v[c].y), fminf(v[c].z, v[c].w)));
+                        hi = fmaxf(hi, fmaxf(fmaxf(v[c].x, v[c].y), fmaxf(v[c].z, v[c].w)));
                     }
                     // (through the part of the step's error buffer that warp 3 publishes into, after all have read it)
                     float2 *range_s = reinterpret_cast<float2 *>(St + 24 * SLD);
@@ -438,8 +444,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         p = clip_ratio(reinterpret_cast<int *>(St)[lrow], a.clip_steps, a.clip_min);
                     }
                     make_grid(p * lo, p * hi, p * fmaxf(-lo, hi), a.bits, a.sym, scale, zero);
-                    if (live && warp == 0 && lane < ROWS) {
-                        const int g = cg / a.group;
+                    if (live && warp == 3 && lane < ROWS) {          // (the warp that has most time)
+                        const int g = cg >> (31 - __clz(a.group));
                         a.scales[(int64_t)row * a.G + g] = scale;
                         a.zeros[(int64_t)row * a.G + g] = zero;
                     }
@@ -478,7 +484,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 }
                 // `c` is the chain: the current column's value.  Entries of x that belong to columns already done are garbage
                 // (entries of U and P at or below the diagonal are applied to them) and never read again.
-                const float *ud = udinv2 + (s & 1) * 32 + w8;
+                const float *ud = udinv_s + co + w8;
                 const float4 ud0 = *reinterpret_cast<const float4 *>(ud), ud1 = *reinterpret_cast<const float4 *>(ud + 4);
                 const float udv[8] = {ud0.x, ud0.y, ud0.z, ud0.w, ud1.x, ud1.y, ud1.z, ud1.w};
                 Uw += w8 * ld; Pw += w8 * ld;
@@ -542,7 +548,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     } else {
 #pragma unroll
                         for (int kk = 0; kk < 8; ++kk)
-                            if (cc + kk < n) crow[perm2[(s & 1) * 32 + w8 + kk]] = (uint8_t)(code[kk >> 2] >> (8 * (kk & 3)));
+                            if (cc + kk < n) crow[perm_s[co + w8 + kk]] = (uint8_t)(code[kk >> 2] >> (8 * (kk & 3)));
                     }
                 }
             }
@@ -561,11 +567,9 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                 const bool last = b == nblk - 1 && s == nst - 1;
                 const int nb = s + 1 < nst ? b : b + 1, ns = s + 1 < nst ? s + 1 : 0;       // the next step
                 const int ncol = i0 + nb * QB_W + 32 * ns;
-                float next_u = 0.f, next_sc[4], next_zp[4];
-                int next_perm = 0;
+                float next_sc[4], next_zp[4];
                 if (!last) {
                     fetch_up(i0 + nb * QB_W, ns, t, QB_NEAR);
-                    if (t < 32) { next_u = load_pivot(ncol + t); next_perm = load_perm(ncol + t); }
                     if (PERCOL && t < 8 * ROWS) load_grid(t >> 3, ncol + 4 * (t & 7), next_sc, next_zp);
                 }
                 if (a.clip_steps > 0 && grid_starts(i0 + co)) {
@@ -651,40 +655,44 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     rmax_s[ec * ROWS + er] = mx;
                 }
                 ++seq;
-                if (!last) {
-                    if (a.up_tma) mbar_wait(upfull(ns & 1), (uint32_t)(seq >> 1) & 1u, abort_flag);
-                    else asm volatile("cp.async.wait_all;" ::: "memory");
-                    if (t < 32) { udinv2[(ns & 1) * 32 + t] = invert_pivot(ncol + t, next_u); perm2[(ns & 1) * 32 + t] = next_perm; }
-                    if (PERCOL && t < 8 * ROWS) store_grid(t >> 3, 4 * (t & 7), next_sc, next_zp);      // (the chain has read this step's)
-                    named_bar_arrive(QBAR_STEP, QB_THREADS_NEAR);
-                }
-                if (FAR && (s & 1)) {
+                // the chain waits for the next step's rows, or, at the end of a block, for what the operand brings to the next one
+                const bool operand_first = FAR && s == QB_W / 32 - 1 && !last;
+#pragma unroll 1
+                for (int turn = 0; turn < 2; ++turn) {
+                    if ((turn == 0) != operand_first) {
+                        if (last) continue;
+                        if (a.up_tma) mbar_wait(upfull(ns & 1), (uint32_t)(seq >> 1) & 1u, abort_flag);
+                        else asm volatile("cp.async.wait_all;" ::: "memory");
+                        if (PERCOL && t < 8 * ROWS) store_grid(t >> 3, 4 * (t & 7), next_sc, next_zp);      // (the chain has read this step's)
+                        named_bar_arrive(QBAR_STEP, QB_THREADS_NEAR);
+                        continue;
+                    }
+                    if (!FAR || !(s & 1)) continue;
                     // ... as the tensor cores' operand, with one power-of-two scale per row
                     named_bar_sync(QBAR_NEAR, QB_NEAR);
 #pragma unroll
                     for (int e = 0; e < 8; ++e) mx = fmaxf(mx, rmax_s[e * ROWS + er]);
                     row_max = fmaxf(row_max, mx);
-                    if (b < last_groups && ec < 8) {
-                        const int half = s >> 1;                    // buffer: even and odd halves alternate
-                        // (the drain warps are done with this buffer's row scales, the MMAs with its operands)
-                        if (b > 0) mbar_wait(efree(half), (uint32_t)(b - 1) & 1u, abort_flag);
-                        const float sc = split_scale_bits(__float_as_uint(mx));
-                        if (ec == 0) inv_s[half * ROWS + er] = pow2_inverse(sc) * inv_su;
-                        uint8_t *eb = sm + L.e + half * HALF_BYTES + (er >> 3) * 1024 + (er & 7) * 128 + ((ec ^ (er & 7)) << 4);
+                    if (b >= last_groups || ec >= 8) continue;
+                    const int half = s >> 1;                        // buffer: even and odd halves alternate
+                    // (the drain warps are done with this buffer's row scales, the MMAs with its operands)
+                    if (b > 0) mbar_wait(efree(half), (uint32_t)(b - 1) & 1u, abort_flag);
+                    const float sc = split_scale_bits(__float_as_uint(mx));
+                    if (ec == 0) inv_s[half * ROWS + er] = pow2_inverse(sc) * inv_su;
+                    uint8_t *eb = sm + L.e + half * HALF_BYTES + (er >> 3) * 1024 + (er & 7) * 128 + ((ec ^ (er & 7)) << 4);
 #pragma unroll
-                        for (int o = 0; o < 2; ++o) {
-                            const float y0[4] = {sc * ev[o][0], sc * ev[o][1], sc * ev[o][2], sc * ev[o][3]};
-                            const float y1[4] = {sc * ev[o][4], sc * ev[o][5], sc * ev[o][6], sc * ev[o][7]};
-                            uint2 h0, l0, h1, l1;
-                            split16_pack(y0, h0, l0);
-                            split16_pack(y1, h1, l1);
-                            *reinterpret_cast<uint4 *>(eb + 2 * o * E_BYTES) = make_uint4(h0.x, h0.y, h1.x, h1.y);
-                            *reinterpret_cast<uint4 *>(eb + (2 * o + 1) * E_BYTES) = make_uint4(l0.x, l0.y, l1.x, l1.y);
-                        }
-                        fence_proxy_async_smem();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(efull(half));
+                    for (int o = 0; o < 2; ++o) {
+                        const float y0[4] = {sc * ev[o][0], sc * ev[o][1], sc * ev[o][2], sc * ev[o][3]};
+                        const float y1[4] = {sc * ev[o][4], sc * ev[o][5], sc * ev[o][6], sc * ev[o][7]};
+                        uint2 h0, l0, h1, l1;
+                        split16_pack(y0, h0, l0);
+                        split16_pack(y1, h1, l1);
+                        *reinterpret_cast<uint4 *>(eb + 2 * o * E_BYTES) = make_uint4(h0.x, h0.y, h1.x, h1.y);
+                        *reinterpret_cast<uint4 *>(eb + (2 * o + 1) * E_BYTES) = make_uint4(l0.x, l0.y, l1.x, l1.y);
                     }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(efull(half));
                 }
                 // results of the step: dequantized columns, -Err and Wpre (a thread: four columns of a row)
                 {
@@ -736,8 +744,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
         }
         if (FAR && a.EWS_hi && t < ROWS) {
             const float sc = t < nrows ? split_scale_bits(__float_as_uint(row_max)) : 1.f;
-            udinv2[t] = sc;                                         // (free: the last step's pivots are in the other half; read
-                                                                    //  after the barrier below)
+            udinv_s[t] = sc;                                        // (free since the first step; read after the barrier below)
             if (t < nrows) a.row_inv[row0 + t] = pow2_inverse(sc);
         }
     } else if (FAR && tid < QB_THREADS_NEAR + QB_DRAIN) {
@@ -862,7 +869,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
             for (int e = 0; e < BATCH; ++e) {
                 const int idx = i0q + e * NTHREADS;
                 if (idx >= nrows * Q) break;
-                const float sc = udinv2[idx / Q];
+                const float sc = udinv_s[idx / Q];
                 const float x[4] = {sc * v[e].x, sc * v[e].y, sc * v[e].z, sc * v[e].w};
                 uint2 h2, l2;
                 split16_pack(x, h2, l2);
