@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(256) simt_gemm_kernel(GemmProblem pr) {
 // through three 32-deep stages of asynchronous copies; the K range of a tile may be shared by a cluster of CTAs,
 // whose partial sums meet in distributed shared memory in a fixed order (deterministic, no scratch).
 // What bounds it: shared-memory reads (two 16-byte reads per 16 FMA: about half the FMA rate of the 128 x 128
-// form), so it pays while those tiles leave the chip idle.  A rank-128 update of 384 columns: 30 us as 128 x 128
+// form), so it pays while those tiles leave the chip idle (simt_small_limit).  A rank-128 update of 384 columns: 30 us as 128 x 128
 // tiles, 9 here; the statistics of 8192 tokens at n = 200: 2700 us there, 150 here.
 // The 32 terms of a stage are summed by themselves: P of a float32 layer is 30 to 45 % closer to float64 so (n = 100 to 384), for 17
 // to 32 registers more (128 at most, still eight CTAs to an SM; 4 bytes spilled where both operands have K contiguous) and up to 3 % of
@@ -464,9 +464,27 @@ __global__ void __launch_bounds__(SG_THREADS) simt_small_kernel(GemmProblem pr, 
 inline int64_t simt_tiles(const GemmProblem &pr) {
     return (int64_t)pr.nbatch * ((pr.M + GBM - 1) / GBM) * ((pr.N + GBN - 1) / GBN);
 }
-// Up to here the 32 x 32 form is the faster one: T tiles on 148 SMs cost ceil(T / 148) x 128 cycles per contraction
-// step as 128 x 128 tiles and about 16 T / 148 x 20 as 32 x 32 tiles.
+// Two sums in one launch (the statistics of narrow layers): up to here.
 constexpr int64_t SIMT_SMALL_TILES = 60;
+
+// Rows of 16-byte multiples, so that the loads of the 128 x 128 form are float4?
+inline bool simt_aligned(const Operand &o) {
+    return ((o.rs == 1 ? o.ks : o.rs) & 3) == 0 &&
+           ((reinterpret_cast<uintptr_t>(o.p) | reinterpret_cast<uintptr_t>(o.p2) | reinterpret_cast<uintptr_t>(o.sub)) & 15) == 0;
+}
+// 128 x 128 tiles up to which the 32 x 32 form is the faster one.  What it loses in reads of shared memory it gains in a chip that is
+// full and in shorter last tiles of triangular products, whose K range the 128 x 128 form goes through on one SM; and its copies do
+// not care for alignment, where the other form loads word by word into registers.  us a call, 128 x 128 beyond 60 tiles and by these limits:
+//   unaligned  n = 1027 factor 707 / 434, P 620 / 132; 2049 2263 / 1116, 1308 / 384; 4097 (1089 tiles) 6287 / 3974, 3275 / 2270;
+//              2500 tiles are 5 % slower (trailing updates of 16000 x 2597)
+//   aligned    factor without damping n = 2052 1466 / 954, P 720 / 300, factor 4096 3204 / 2814 (up to 600 tiles 2876);
+//              trailing updates of 1024 to 4096 x 1024 240 / 240, 303 / 277, 359 / 324, 488 / 451 (up to 300 tiles 462)
+//   token sums 4096 tokens of n = 1024 605 / 431, 2832 of 1416 937 / 1018 with more than 100
+inline int64_t simt_small_limit(const GemmProblem &pr, bool a_rc, bool b_rc) {
+    if (!simt_aligned(pr.A) || !simt_aligned(pr.B)) return 1200;
+    if (a_rc && b_rc) return 100;
+    return pr.mode == GEMM_FULL ? 200 : 300;
+}
 
 template <bool A_RC, bool B_RC>
 inline cudaError_t launch_simt_small(const GemmProblem &pr, cudaStream_t s, int early_ctas) {
@@ -493,7 +511,7 @@ inline cudaError_t launch_simt_small(const GemmProblem &pr, cudaStream_t s, int 
 // before their turn hold the SMs that were free at that time, several to an SM, and it is there that the product runs.
 inline cudaError_t launch_simt_gemm(const GemmProblem &pr, bool a_rc, bool b_rc, cudaStream_t s, int early_ctas = 0) {
     if (pr.M <= 0 || pr.N <= 0 || pr.nbatch <= 0) return cudaSuccess;
-    if (simt_tiles(pr) <= SIMT_SMALL_TILES && !pr.B.sub) {
+    if (simt_tiles(pr) <= simt_small_limit(pr, a_rc, b_rc) && !pr.B.sub) {
         if (a_rc && b_rc) return launch_simt_small<true, true>(pr, s, early_ctas);
         if (a_rc) return launch_simt_small<true, false>(pr, s, early_ctas);
         if (b_rc) return launch_simt_small<false, true>(pr, s, early_ctas);

@@ -752,6 +752,16 @@ def test_factor_panels(n):
 
 
 # (a diagonal block's pieces of eight columns and sub-blocks of 32, and the block beside which another is inverted)
+@pytest.mark.parametrize("n,m,damp", [
+    (1027, 150, 0.01),          # odd rows, 81 tiles of 128 x 128 and more: the 32 x 32 form all the same
+    (1156, 130, 0.0),           # aligned rows, plain float32 without damping, 100 tiles
+])
+def test_float32_products_of_many_tiles(n, m, damp):
+    cfg = wl.scaled(wl.CONFIGS["cfg2"], name="tiles", n=n, m=m, batch_tokens=5 * n, n_batches=2, damp=damp, outlier_channels=4)
+    out = hp.check_layer(cfg, wl.make_weight(cfg), batches_of(cfg), rows=np.arange(0, m, 7))
+    hp.assert_parity(out)
+
+
 @pytest.mark.parametrize("n", [7, 33, 64, 97, 128, 136])
 def test_factor_inside_a_block(n):
     test_factor_panels(n)
