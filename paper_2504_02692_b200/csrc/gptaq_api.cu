@@ -18,6 +18,7 @@
 #include "umma_gemm.cuh"
 #include "tc_gemm.cuh"
 #include "factor.cuh"
+#include "narrow.cuh"
 #include "quantize_block.cuh"
 
 using namespace gptaq;
@@ -956,6 +957,8 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
         e = cudaFuncSetAttribute(panel_solve_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM);
     if (e == cudaSuccess) e = configure_quantize_kernels();
     if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(p_narrow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)np_smem(NP_MAX_N));
+    if (e == cudaSuccess)
         e = cudaFuncSetAttribute(invert_diag_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ID_SMEM);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(stats_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UMMA_SMEM);
@@ -1403,13 +1406,21 @@ gptaq_status_t gptaq_build_P(gptaq_handle_t h, float alpha, gptaq_stream_t strea
         h->stage = STAGE_P;
         return GPTAQ_OK;
     }
+    const float scale = (float)((double)alpha / (double)h->tokens);
+    if (n <= NP_MAX_N) {
+        CU(launch_pdl(true, p_narrow_kernel, dim3((n + NP_ROWS - 1) / NP_ROWS), dim3(NP_THREADS), np_smem(n), s, h->D,
+                      static_cast<const float *>(h->H), n, scale));
+        h->launches++;
+        h->stage = STAGE_P;
+        return GPTAQ_OK;
+    }
     // O = (dXX^T U^T) .* M_U
     GemmProblem po = make_problem(make_operand(h->D, n, 1), make_operand(h->H, n, 1), O, n, n, n, n,
                                   1.f, 0.f, GEMM_O);
     OK(gemm(h, po, false, false, s));
     // P = (alpha / tokens) * O U
     GemmProblem pp = make_problem(make_operand(O, n, 1), make_operand(h->H, 1, n), h->D, n, n, n, n,
-                                  (float)((double)alpha / (double)h->tokens), 0.f, GEMM_P);
+                                  scale, 0.f, GEMM_P);
     OK(gemm(h, pp, false, true, s));
     h->stage = STAGE_P;
     return GPTAQ_OK;

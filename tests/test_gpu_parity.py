@@ -751,7 +751,6 @@ def test_factor_panels(n):
     assert np.linalg.norm(U - ref) <= bound * np.linalg.norm(ref), (hp.rel_fro(U, ref), bound)
 
 
-# (a diagonal block's pieces of eight columns and sub-blocks of 32, and the block beside which another is inverted)
 @pytest.mark.parametrize("n,m,damp", [
     (1027, 150, 0.01),          # odd rows, 81 tiles of 128 x 128 and more: the 32 x 32 form all the same
     (1156, 130, 0.0),           # aligned rows, plain float32 without damping, 100 tiles
@@ -762,9 +761,35 @@ def test_float32_products_of_many_tiles(n, m, damp):
     hp.assert_parity(out)
 
 
+# (a diagonal block's pieces of eight columns and sub-blocks of 32, and the block beside which another is inverted)
 @pytest.mark.parametrize("n", [7, 33, 64, 97, 128, 136])
 def test_factor_inside_a_block(n):
     test_factor_panels(n)
+
+
+@pytest.mark.parametrize("n", [1, 3, 31, 33, 97, 126, 128, 255, 383, 384, 385])
+def test_correction_matrix_of_narrow_layers(n):
+    """One launch up to n = 384, two products beyond: P from the device's own U and dXX^T against float64; sums of up to n float32
+    products in short pieces, 2^-21 of the sum of their sizes leaves a factor of eight over one rounding each."""
+    torch.manual_seed(n)
+    tokens, alpha = 4 * n + 40, 0.5
+    X = torch.randn(tokens, n, device="cuda")
+    st = g.LayerState(n, 8, tokens, 32)
+    try:
+        g.gptaq_set_stats_precision(st.handle, g.GPTAQ_STATS_FP32)
+        g.gptaq_accumulate(st.handle, X, X + 0.3 * torch.randn_like(X))
+        D = np.triu(st.D().cpu().numpy().astype(np.float64), 1) / tokens
+        g.gptaq_factor(st.handle, 0.05)
+        g.gptaq_build_P(st.handle, alpha)
+        U = np.triu(st.H().cpu().numpy().astype(np.float64))
+        P = st.D().cpu().numpy().astype(np.float64)
+        assert g.gptaq_sync_status(st.handle)[0] == g.GPTAQ_OK
+    finally:
+        st.close()
+    ref = alpha * np.triu(np.triu(D @ U.T, 1) @ U, 1)
+    size = alpha * np.triu(np.triu(abs(D) @ abs(U).T, 1) @ abs(U), 1)
+    assert np.array_equal(np.tril(P), np.zeros_like(P))
+    assert np.linalg.norm(P - ref) <= 2.0 ** -21 * np.linalg.norm(size)
 
 
 @pytest.mark.parametrize("n", [512, 516, 1036, 1284])
