@@ -200,32 +200,10 @@ __device__ __forceinline__ void tile_product(float *C, int ldc, const float *A, 
             make_float4(sign * acc[e][0], sign * acc[e][1], sign * acc[e][2], sign * acc[e][3]);
 }
 
-// by the first ID_THREADS threads of a CTA
-__device__ __forceinline__ void invert_diag_block(float *smem_f, float *H, int n, int b0, const float *Rdiag) {
-    float *S = smem_f, *X = S + NB * ID_LD, *T = X + NB * ID_LD;
+// By the first ID_THREADS threads of a CTA, from R^T left of the sub-blocks on the diagonal (in S) and their inverses (in X, zeros
+// elsewhere).
+__device__ __forceinline__ void invert_products(float *S, float *X, float *T, float *H, int n, int b0) {
     const int tid = threadIdx.x;
-    float4 v[NB * NB / 4 / ID_THREADS];
-#pragma unroll
-    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) v[it] = *reinterpret_cast<const float4 *>(Rdiag + 4 * (tid + it * ID_THREADS));
-    float y[4 * 32 * 32 / ID_THREADS];
-#pragma unroll
-    for (int it = 0; it < 4 * 32 * 32 / ID_THREADS; ++it) {
-        const int idx = tid + it * ID_THREADS;
-        y[it] = Rdiag[diag_inverse_at(idx >> 10, (idx >> 5) & 31) + (idx & 31)];
-    }
-#pragma unroll
-    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) {
-        const int i = (tid + it * ID_THREADS) >> 5, j4 = (tid + it * ID_THREADS) & 31;
-        // R^T as it comes, left of the sub-block on the diagonal
-        if (j4 < (i >> 5) * 8) *reinterpret_cast<float4 *>(S + i * ID_LD + 4 * j4) = v[it];
-        if ((j4 >> 3) != (i >> 5)) *reinterpret_cast<float4 *>(X + i * ID_LD + 4 * j4) = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-#pragma unroll
-    for (int it = 0; it < 4 * 32 * 32 / ID_THREADS; ++it) {
-        const int idx = tid + it * ID_THREADS, c = idx >> 10, l = (idx >> 5) & 31, j = idx & 31;
-        X[(32 * c + j) * ID_LD + 32 * c + l] = j <= l ? y[it] : 0.f;
-    }
-    named_bar_sync(ID_BAR, ID_THREADS);
     // R above the diagonal
     for (int idx = tid; idx < NB * NB; idx += ID_THREADS) {
         const int i = idx >> 7, j = idx & 127;
@@ -257,6 +235,35 @@ __device__ __forceinline__ void invert_diag_block(float *smem_f, float *H, int n
     }
 }
 
+// by the first ID_THREADS threads of a CTA
+__device__ __forceinline__ void invert_diag_block(float *smem_f, float *H, int n, int b0, const float *Rdiag) {
+    float *S = smem_f, *X = S + NB * ID_LD, *T = X + NB * ID_LD;
+    const int tid = threadIdx.x;
+    float4 v[NB * NB / 4 / ID_THREADS];
+#pragma unroll
+    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) v[it] = *reinterpret_cast<const float4 *>(Rdiag + 4 * (tid + it * ID_THREADS));
+    float y[4 * 32 * 32 / ID_THREADS];
+#pragma unroll
+    for (int it = 0; it < 4 * 32 * 32 / ID_THREADS; ++it) {
+        const int idx = tid + it * ID_THREADS;
+        y[it] = Rdiag[diag_inverse_at(idx >> 10, (idx >> 5) & 31) + (idx & 31)];
+    }
+#pragma unroll
+    for (int it = 0; it < NB * NB / 4 / ID_THREADS; ++it) {
+        const int i = (tid + it * ID_THREADS) >> 5, j4 = (tid + it * ID_THREADS) & 31;
+        // R^T as it comes, left of the sub-block on the diagonal
+        if (j4 < (i >> 5) * 8) *reinterpret_cast<float4 *>(S + i * ID_LD + 4 * j4) = v[it];
+        if ((j4 >> 3) != (i >> 5)) *reinterpret_cast<float4 *>(X + i * ID_LD + 4 * j4) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int it = 0; it < 4 * 32 * 32 / ID_THREADS; ++it) {
+        const int idx = tid + it * ID_THREADS, c = idx >> 10, l = (idx >> 5) & 31, j = idx & 31;
+        X[(32 * c + j) * ID_LD + 32 * c + l] = j <= l ? y[it] : 0.f;
+    }
+    named_bar_sync(ID_BAR, ID_THREADS);
+    invert_products(S, X, T, H, n, b0);
+}
+
 __global__ void __launch_bounds__(ID_THREADS, 1) invert_diag_block_kernel(float *H, int n, int b0, const float *Rdiag) {
     extern __shared__ __align__(16) float smem_f[];
     pdl_wait();
@@ -281,6 +288,7 @@ constexpr int DF_HELP = 8 * 32, DF_MAIN = 128 + DF_HELP, DF_THREADS = DF_MAIN + 
 constexpr int DF_TILE_BYTES = NB * 64 * 2;           // 128 rows x 64 fp16
 constexpr size_t DF_SMEM_BLOCK = 4 * DF_TILE_BYTES + (size_t)(NB * FP_LD + NB + 64 + 32) * sizeof(float) + 32 + 1024;
 constexpr size_t DF_SMEM = DF_SMEM_BLOCK > ID_SMEM ? DF_SMEM_BLOCK : ID_SMEM;
+constexpr size_t DF_SMEM_WHOLE = ID_SMEM + (NB + 64 + 32) * sizeof(float) + 32 + 1024;
 constexpr uint32_t DF_IDESC = (1u << 4) | ((NB >> 3) << 17) | ((NB >> 4) << 24);     // kind::f16, M = N = 128
 // Named barriers.  COLS + q: eight columns (q = 0: the rightmost) of a sub-block are factored (its leader arrives; the warps above
 // it and the inverter wait); ROWS + q: ... and solved in the rows above (these arrive, the helpers wait); NEXT: the next
@@ -297,16 +305,25 @@ struct DiagFactorArgs {
     int syrk, pan_col0;                  // 1: subtract rows b0 .. of the panel at columns pan_col0 .. of the split copy times
                                          //    their transpose first (scale of the copy: tc_amax[AMAX_PAN])
     StateHeader *hd;
+    // WHOLE: the layer has one block, src is its sum H as it was accumulated
+    float inv_tokens, damp;
+    uint8_t *dead, *dead_working;
 };
 
+// WHOLE (n <= NB): what diag_stats_kernel, scale_damp_kernel and invert_diag_block_kernel do for a wider layer happens here too, with the
+// same arithmetic: gptaq_factor at n = 128 36.6 us as four launches, 31.4 so, n = 100 39.2 and 31.7 (U bit-identical; with R_pp through
+// global memory as between the launches 37.7 and 35.8).
+template <bool WHOLE>
 __global__ void __launch_bounds__(DF_THREADS, 1)
 diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ CUtensorMap mapLo, DiagFactorArgs a) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *sm = smem_raw + (base - raw);
-    float (*S)[FP_LD] = reinterpret_cast<float (*)[FP_LD]>(sm + 4 * DF_TILE_BYTES);
-    float *dinv = reinterpret_cast<float *>(S + NB);
+    // (WHOLE: the inverse's other operands behind it)
+    float (*S)[FP_LD] = reinterpret_cast<float (*)[FP_LD]>(sm + (WHOLE ? 0 : 4 * DF_TILE_BYTES));
+    float *X = reinterpret_cast<float *>(S + NB), *T = X + NB * ID_LD;
+    float *dinv = WHOLE ? T + 64 * 68 : reinterpret_cast<float *>(S + NB);
     float *gs = dinv + NB;                           // 8 x 8: the diagonal block of the columns at hand
     float *rdiag = gs + 64;                          // 1 / R_kk of the sub-block that is being inverted
     uint8_t *tailp = reinterpret_cast<uint8_t *>(rdiag + 32);
@@ -316,7 +333,7 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nv = min(NB, a.n - a.b0);
     pdl_launch_dependents();
-    if (blockIdx.x == 1) {
+    if (!WHOLE && blockIdx.x == 1) {
         pdl_wait();
         if (tid < ID_THREADS) invert_diag_block(reinterpret_cast<float *>(smem_raw), a.H, a.n, a.inv_b0, a.inv_Rdiag);
         return;
@@ -327,7 +344,7 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (a.syrk && warp == 13) {
+    if (!WHOLE && a.syrk && warp == 13) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(const_cast<uint32_t *>(tmem_slot))), "r"(128u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -336,7 +353,53 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
     __syncthreads();
     tc_fence_after();
     pdl_wait();
-    if (warp == 13) {
+    if constexpr (WHOLE) {
+        double *sum = reinterpret_cast<double *>(T);
+        float *top = reinterpret_cast<float *>(sum + NB);
+        float d = tid < nv ? a.src[tid * a.lds + tid] : 0.f;
+        const float raw = d;
+        bool dd = false;
+        constexpr int BATCH = 13, ROUNDS = (NB * NB + BATCH * DF_THREADS - 1) / (BATCH * DF_THREADS);      // (loads in flight)
+#pragma unroll 1
+        for (int r = 0; r < ROUNDS; ++r) {
+            float v[BATCH];
+#pragma unroll
+            for (int e = 0; e < BATCH; ++e) {
+                const int idx = tid + (r * BATCH + e) * DF_THREADS, i = idx >> 7, j = idx & 127;
+                v[e] = i < nv && j < nv && j > i ? a.src[i * a.lds + j] : 0.f;
+            }
+#pragma unroll
+            for (int e = 0; e < BATCH; ++e) {
+                const int idx = tid + (r * BATCH + e) * DF_THREADS, i = idx >> 7, j = idx & 127;
+                if (i < NB && (i != j || i >= nv)) S[i][j] = i == j ? 1.f : v[e] * a.inv_tokens;
+                if (i < NB && (i >> 5) != (j >> 5)) X[i * ID_LD + j] = 0.f;
+            }
+        }
+        if (tid < NB) {
+            if (tid < nv) {
+                if (!isfinite(d)) record_status(a.hd, ST_NONFINITE, tid);
+                dd = d == 0.f;
+                a.dead[tid] = dd ? 1 : 0;
+                if (a.dead_working) a.dead_working[tid] = dd ? 1 : 0;
+                d = dd ? 1.f : d * a.inv_tokens;
+                sum[tid] = dd ? 1.0 : (double)raw * (double)a.inv_tokens;
+                top[tid] = d;
+            } else { sum[tid] = 0.0; top[tid] = 0.f; }
+        }
+        for (int w = NB / 2; w > 0; w >>= 1) {
+            __syncthreads();
+            if (tid < w) { sum[tid] += sum[tid + w]; top[tid] = fmaxf(top[tid], top[tid + w]); }
+        }
+        __syncthreads();
+        const float lambda = (float)((double)a.damp * sum[0] / (double)a.n);
+        if (tid == 0) {
+            a.hd->lambda = lambda;
+            a.hd->inv_tokens = a.inv_tokens;
+            a.hd->tc_amax[AMAX_PAN] = __float_as_uint(sqrtf(top[0] + lambda));
+            a.hd->tc_amax[AMAX_INV] = lambda > 0.f ? __float_as_uint(rsqrtf(lambda)) : 0u;
+        }
+        if (tid < nv) S[tid][tid] = d + lambda;
+    } else if (warp == 13) {
         if (a.syrk && lane == 0) {
             mbar_expect_tx(bar, 4 * DF_TILE_BYTES);
             for (int t = 0; t < 4; ++t) tma_load_2d(base + t * DF_TILE_BYTES, t < 2 ? &mapHi : &mapLo, a.pan_col0 + 64 * (t & 1), a.b0, bar);
@@ -378,7 +441,7 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
         }
     }
     __syncthreads();
-    if (a.syrk) {
+    if (!WHOLE && a.syrk) {
         const uint32_t tmem = *tmem_slot;
         // 32 x 32 pieces of the upper triangle, one or two per warp
         const int quarter = warp & 3, row = 32 * quarter + lane;
@@ -474,7 +537,7 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
         auto store_rows = [&](int sb) {
             for (int idx = t; idx < 32 * (NB / 4); idx += DF_HELP) {
                 const int i = 32 * sb + (idx >> 5), j4 = idx & 31;
-                if (j4 < 8 * (sb + 1)) *reinterpret_cast<float4 *>(a.Rdiag + i * NB + 4 * j4) = *reinterpret_cast<const float4 *>(&S[i][4 * j4]);
+                if (!WHOLE && j4 < 8 * (sb + 1)) *reinterpret_cast<float4 *>(a.Rdiag + i * NB + 4 * j4) = *reinterpret_cast<const float4 *>(&S[i][4 * j4]);
             }
         };
 #pragma unroll 1
@@ -519,18 +582,19 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
             float y[32];
 #pragma unroll
             for (int k = 0; k < 32; ++k) y[k] = (k == lane) ? 1.f : 0.f;
-            float *dst = a.Rdiag + diag_inverse_at(sb, lane);
+            float *dst = WHOLE ? X + o * ID_LD + o + lane : a.Rdiag + diag_inverse_at(sb, lane);
             solve32(y, &S[o][o], rdiag,
                     [&](int k) {
                         named_bar_sync(DBAR_COLS + (31 - k) / 8, 32 * (sb + 2));
                         if (lane < 8) rdiag[k - lane] = 1.f / S[o + k - lane][o + k - lane];
                         __syncwarp();
                     },
-                    [&](int k, float v) { dst[k] = v; });
+                    [&](int k, float v) { dst[WHOLE ? k * ID_LD : k] = !WHOLE || k <= lane ? v : 0.f; });
         }
     }
     __syncthreads();
     if (*abort_flag && tid == 0) record_status(a.hd, ST_TIMEOUT, 4000000 + a.b0);
+    if (WHOLE && tid < ID_THREADS) invert_products(&S[0][0], X, T, a.H, a.n, 0);
 }
 
 // ---------------------------------------------------------------------------

@@ -950,7 +950,9 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
     cudaError_t e = cudaGetDevice(&h->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(diag_factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DF_SMEM);
+        e = cudaFuncSetAttribute(diag_factor_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DF_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(diag_factor_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DF_SMEM_WHOLE);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(panel_solve_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM);
     if (e == cudaSuccess)
@@ -1121,12 +1123,25 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
     float *Rinv = reinterpret_cast<float *>(h->ws + wl.rinv_off);
     float *H = h->H;
 
-    diag_stats_kernel<<<1, 1024, 0, s>>>(H, n, (float)(1.0 / (double)h->tokens), damp, h->hd, h->dead_raw, h->act_order ? nullptr : h->dead);
+    const float inv_tokens = (float)(1.0 / (double)h->tokens);
+    if (nb == 1 && !h->act_order) {
+        DiagFactorArgs da = {};
+        da.src = H; da.lds = n; da.n = n; da.H = H; da.hd = h->hd;
+        da.inv_tokens = inv_tokens; da.damp = damp; da.dead = h->dead_raw; da.dead_working = h->dead;
+        CUtensorMap none;
+        std::memset(&none, 0, sizeof(none));
+        CU(launch_pdl(false, diag_factor_kernel<true>, dim3(1), dim3(DF_THREADS), DF_SMEM_WHOLE, s, none, none, da));
+        h->launches++;
+        h->split = false;
+        h->stage = STAGE_FACTORED;
+        return GPTAQ_OK;
+    }
+    diag_stats_kernel<<<1, 1024, 0, s>>>(H, n, inv_tokens, damp, h->hd, h->dead_raw, h->act_order ? nullptr : h->dead);
     LAUNCHED();
     if (h->act_order) {
         // columns in order of decreasing diag(H): dXX^T and H are permuted on both sides, through T (H stays there until it
         // is scaled)
-        rank_desc_kernel<<<(n + RANK_COLS - 1) / RANK_COLS, 256, 0, s>>>(H, n, (float)(1.0 / (double)h->tokens), h->dead_raw, h->perm, h->dead);
+        rank_desc_kernel<<<(n + RANK_COLS - 1) / RANK_COLS, 256, 0, s>>>(H, n, inv_tokens, h->dead_raw, h->perm, h->dead);
         LAUNCHED();
         const int rows = perm_rows(n, sizeof(float));
         gather_cols_kernel<float><<<std::min((n + rows - 1) / rows, h->num_sms * 8), 256, rows * n * sizeof(float), s>>>(h->D, n, T, n, n, n, h->perm, h->perm, rows);
@@ -1184,12 +1199,12 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         return gemm(h, ps, false, false, us);
     };
     auto factor_diag = [&](int p, const float *src, int64_t lds, int syrk, int pan_col0) -> gptaq_status_t {
-        DiagFactorArgs da;
+        DiagFactorArgs da = {};
         da.src = src; da.lds = lds; da.n = n; da.b0 = p * NB; da.Rdiag = Rinv + (size_t)p * NB * NB;
         da.syrk = syrk; da.pan_col0 = pan_col0; da.hd = h->hd;
         // (a second CTA inverts the block before)
         da.H = H; da.inv_b0 = (p + 1) * NB; da.inv_Rdiag = da.Rdiag + NB * NB;
-        CU(launch_pdl(true, diag_factor_kernel, dim3(p + 1 < nb ? 2 : 1), dim3(DF_THREADS), DF_SMEM, s, pan_maps.a_hi, pan_maps.a_lo, da));
+        CU(launch_pdl(true, diag_factor_kernel<false>, dim3(p + 1 < nb ? 2 : 1), dim3(DF_THREADS), DF_SMEM, s, pan_maps.a_hi, pan_maps.a_lo, da));
         h->launches++;
         return GPTAQ_OK;
     };
