@@ -576,14 +576,15 @@ struct QuantizeTarget {
 };
 
 // One launch of quant_block_kernel: columns [i0, i1) of the loop for rows [r0, r1) of m, SW columns per launch at most.
-cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, int64_t r0, int64_t r1, int64_t m, int i0, int i1, int SW,
+// src: the caller's weights, read instead of W by a launch that takes all columns (or nullptr).
+cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, const void *src, int64_t lds, int w_dtype, int64_t r0, int64_t r1, int64_t m, int i0, int i1, int SW,
                                int bits, int group, int sym, uint8_t *codes, float *scales, float *zeros, int G,
                                bool static_groups, cudaStream_t s) {
     const bool far_form = t.UT16 != nullptr;
     const size_t nn = (size_t)t.n * t.ldt;
     QuantBlockArgs a;
     std::memset(&a, 0, sizeof(a));
-    a.W = W; a.ldw = ldw; a.row_first = (int)r0; a.m = (int)r1; a.n = t.n; a.U = t.U; a.P = t.P; a.dead = t.dead;
+    a.W = W; a.ldw = ldw; a.src = src; a.lds = lds; a.src_bf16 = src && w_dtype == GPTAQ_W_BF16; a.row_first = (int)r0; a.m = (int)r1; a.n = t.n; a.U = t.U; a.P = t.P; a.dead = t.dead;
     a.i0 = i0; a.i1 = i1; a.bw = far_form ? QB_W : SW;
     a.bits = bits; a.group = group; a.sym = sym;
     a.codes = codes; a.scales = scales; a.zeros = zeros; a.G = G;
@@ -681,6 +682,20 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
     float *EW = t.EW;
     float *Wk = static_cast<float *>(d_W);
     int64_t ldk = ldw;
+    // grids per output channel, per group of whole 32-column steps, or per column (static groups): quant_block_kernel.
+    // Smaller groups take column_loop_kernel (one warp per row, any group).
+    const bool static_groups = t.static_groups && group > 0;
+    const bool steps = group <= 0 || (group % 32) == 0 || static_groups;
+    const bool tensor = t.UT16 != nullptr;
+    // columns per launch: as many as the slab holds (and the scratch has room for the errors of), else the caller's block
+    const int SW = !steps ? blocksize : tensor ? QB_SUPER : (n <= QB_W || t.ew_floats >= m * 2 * QB_W) ? QB_W : blocksize;
+    // A single launch for all columns reads the caller's weights itself, and makes the grids per channel of a single block (whose
+    // columns are then a group like another): the copy or the grids' launch is 3 to 30 us a call (1003 x 128 with groups 21.3 -> 17.2,
+    // 333 x 128 from bfloat16 19.5 -> 14.3, 512 x 512 with groups 60 -> 55, 8192 x 128 29.5 -> 24.6).
+    const bool direct = steps && !t.perm && n <= SW;
+    const bool grid_inside = direct && group <= 0 && n <= QB_W && t.clip_steps == 0;
+    const int kernel_group = grid_inside ? QB_W : group;
+    const void *src = nullptr;
     if (t.perm) {
         // working copy in sorted column order (the caller's d_Wq; checked to be a second buffer)
         const size_t esz = w_dtype == GPTAQ_W_BF16 ? sizeof(__nv_bfloat16) : sizeof(float);
@@ -696,7 +711,8 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
         Wk = d_Wq; ldk = n;
     } else if (w_dtype == GPTAQ_W_BF16 || (d_Wq && d_Wq != d_W)) {
         Wk = d_Wq; ldk = n;
-        if (group > 0) {
+        if (direct) src = d_W;
+        else if (group > 0) {
             const dim3 grid((unsigned)((n + 1023) / 1024), (unsigned)std::min<int64_t>((m + WIDEN_ROWS - 1) / WIDEN_ROWS, 65535));
             if (w_dtype == GPTAQ_W_BF16)
                 widen_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(d_W), ldw, d_Wq, n, (int)m, n);
@@ -706,7 +722,6 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
     }
 
     const int G = group > 0 ? (n + group - 1) / group : 1;
-    const bool static_groups = t.static_groups && group > 0;
     if (static_groups) {
         // grids of the original weights (the caller's d_W in its own column order is still untouched)
         const unsigned sg_grid = (unsigned)(((int64_t)m * G + 7) / 8);
@@ -720,25 +735,20 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
                                                                    t.clip_min);
         QLAUNCHED();
     }
-    if (group <= 0) {
+    if (group <= 0 && !grid_inside) {
         // (from the caller's rows, with the working copy made on the way; in sorted order that exists already)
         const unsigned rg = (unsigned)((m + 7) / 8);
-        float *copy = t.perm || Wk == d_W ? nullptr : Wk;
-        if (w_dtype == GPTAQ_W_BF16 && copy)
+        const bool own = t.perm || Wk == d_W;
+        float *copy = own || direct ? nullptr : Wk;
+        if (w_dtype == GPTAQ_W_BF16 && !own)
             row_grid_kernel<__nv_bfloat16><<<rg, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(d_W), ldw, copy, ldk, (int)m, n, t.dead, bits,
                                                               sym, d_scales, d_zeros, t.clip_steps, t.clip_min);
         else
-            row_grid_kernel<float><<<rg, 256, 0, s>>>(copy ? static_cast<const float *>(d_W) : Wk, copy ? ldw : ldk, copy, ldk, (int)m, n, t.dead,
+            row_grid_kernel<float><<<rg, 256, 0, s>>>(own ? Wk : static_cast<const float *>(d_W), own ? ldk : ldw, copy, ldk, (int)m, n, t.dead,
                                                       bits, sym, d_scales, d_zeros, t.clip_steps, t.clip_min);
         QLAUNCHED();
     }
 
-    // grids per output channel, per group of whole 32-column steps, or per column (static groups): quant_block_kernel.
-    // Smaller groups take column_loop_kernel (one warp per row, any group).
-    const bool steps = group <= 0 || (group % 32) == 0 || static_groups;
-    const bool tensor = t.UT16 != nullptr;
-    // columns per launch: as many as the slab holds (and the scratch has room for the errors of), else the caller's block
-    const int SW = !steps ? blocksize : tensor ? QB_SUPER : (n <= QB_W || t.ew_floats >= m * 2 * QB_W) ? QB_W : blocksize;
     TcMaps maps;
     if (tensor) {
         const size_t nn = (size_t)n * t.ldt, me = (size_t)m * 2 * SW;
@@ -761,7 +771,7 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
             const int i1 = std::min(i0 + SW, n);
             for (const Part &p : parts) {
                 if (p.r0 == p.r1) continue;
-                *err = launch_quant_block(t, Wk, ldk, p.r0, p.r1, m, i0, i1, SW, bits, group, sym, d_codes, d_scales, d_zeros, G,
+                *err = launch_quant_block(t, Wk, ldk, src, ldw, w_dtype, p.r0, p.r1, m, i0, i1, SW, bits, kernel_group, sym, d_codes, d_scales, d_zeros, G,
                                           static_groups, p.s);
                 if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
                 ++*launches;
@@ -785,7 +795,7 @@ gptaq_status_t quantize_core(const QuantizeTarget &t, void *d_W, int w_dtype, in
     } else for (int i0 = 0; i0 < n; i0 += SW) {
         const int i1 = std::min(i0 + SW, n);
         if (steps) {
-            *err = launch_quant_block(t, Wk, ldk, 0, m, m, i0, i1, SW, bits, group, sym, d_codes, d_scales, d_zeros, G,
+            *err = launch_quant_block(t, Wk, ldk, src, ldw, w_dtype, 0, m, m, i0, i1, SW, bits, kernel_group, sym, d_codes, d_scales, d_zeros, G,
                                       static_groups, s);
             if (*err != cudaSuccess) return GPTAQ_ERR_CUDA;
             ++*launches;

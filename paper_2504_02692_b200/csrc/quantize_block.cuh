@@ -54,6 +54,8 @@ __host__ __device__ constexpr int qb_tmem_cols(int rows) { return rows == 32 ? 5
 
 struct QuantBlockArgs {
     float *W; int64_t ldw; int row_first, m, n;     // rows [row_first, m)
+    // where the values come from: nullptr (W itself), or the caller's weights, float32 or bfloat16 (a launch that takes all columns)
+    const void *src; int64_t lds; int src_bf16;
     const float *U, *P;        // n x n, ld n; entries below the diagonals are not used
     int up_tma;                // U and P qualify for tensor maps (16-byte rows)
     const uint8_t *dead;
@@ -325,22 +327,38 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     fetch_up(i0, 0, tid, NTHREADS);
     if (!FAR) pdl_wait();
     const int cq = FAR ? nblk * (QB_W / 4) : B / 4;                // quads per row, padded columns included
-    const bool wvec = (a.ldw & 3) == 0 && (reinterpret_cast<uintptr_t>(a.W) & 15) == 0;       // (i0 is a multiple of 32)
+    // (i0 is a multiple of 32)
+    const float *from = a.src ? static_cast<const float *>(a.src) : a.W;
+    const int64_t ldf = a.src ? a.lds : a.ldw;
+    const bool wvec = (ldf & 3) == 0 && (reinterpret_cast<uintptr_t>(from) & (a.src_bf16 ? 7 : 15)) == 0;
     // a thread: four columns of every RSTEP-th row
     constexpr int WQ = FAR ? QB_SUPER / 4 : QB_W / 4, RSTEP = NTHREADS / WQ;
     const int wq = tid % WQ, wr0 = tid / WQ, wc = 4 * wq;
     const bool fills = wr0 < RSTEP && wq < cq;
     if (fills) {
         const bool whole = wvec && wc + 3 < cols;
-        const float *src = a.W + (int64_t)(row0 + wr0) * a.ldw + i0 + wc;
+        const int64_t off = (int64_t)(row0 + wr0) * ldf + i0 + wc;
+        const float *src = from + off;
+        const __nv_bfloat16 *src16 = static_cast<const __nv_bfloat16 *>(a.src) + off;
         float *dst = Ws + wr0 * WLD + wc;
-        for (int r = wr0; r < ROWS; r += RSTEP) {
+        if (a.src_bf16) {
+#pragma unroll 4
+            for (int r = wr0; r < ROWS; r += RSTEP, src16 += (int64_t)RSTEP * ldf, dst += RSTEP * WLD) {
+                Quad<__nv_bfloat16> q;
+                if (whole && r < nrows) q = *reinterpret_cast<const Quad<__nv_bfloat16> *>(src16);
+                else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) q.v[e] = r < nrows && wc + e < cols ? src16[e] : __float2bfloat16(0.f);
+                }
+                *reinterpret_cast<float4 *>(dst) = make_float4((float)q.v[0], (float)q.v[1], (float)q.v[2], (float)q.v[3]);
+            }
+        } else for (int r = wr0; r < ROWS; r += RSTEP) {
             if (whole && r < nrows) cp_async16(dst, src);
             else {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) dst[e] = r < nrows && wc + e < cols ? src[e] : 0.f;
             }
-            src += (int64_t)RSTEP * a.ldw; dst += RSTEP * WLD;
+            src += (int64_t)RSTEP * ldf; dst += RSTEP * WLD;
         }
     }
     // (dead inputs read as zero; the flags are 4-byte aligned and padded beyond n)

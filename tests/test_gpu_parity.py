@@ -871,6 +871,45 @@ def test_a_row_does_not_depend_on_how_many_there_are(n, m, group, B, static, cli
         st.close()
 
 
+@pytest.mark.parametrize("n,m,group,B,clip,static", [
+    (96, 70, 0, 32, 0, False), (128, 800, 0, 128, 0, False),        # one block: grids per channel inside the launch
+    (97, 33, 0, 64, 5, False),                                      # ... before it where ranges are searched
+    (100, 45, 32, 64, 0, False), (512, 40, 128, 128, 0, False),     # one launch, groups
+    (512, 2400, 0, 128, 0, False), (508, 50, 64, 64, 0, True),      # (508: several launches, a working copy)
+])
+def test_a_single_launch_reads_the_callers_weights(n, m, group, B, clip, static):
+    """From a second buffer, from bfloat16 and from rows at odd addresses: as in place on float32 copies, bit for bit."""
+    torch.manual_seed(n)
+    X = torch.randn(3 * n, n, device="cuda")
+    X[:, n // 3] = 0.0                                              # a dead input
+    wide = (0.02 * torch.randn(m, n + 5, device="cuda")).bfloat16()
+    st = g.LayerState(n, m, 3 * n, B)
+    try:
+        g.gptaq_accumulate(st.handle, X, X + 0.05 * torch.randn_like(X))
+        g.gptaq_factor(st.handle, 0.01)
+        g.gptaq_build_P(st.handle, 0.25)
+        g.gptaq_set_static_groups(st.handle, static)
+        g.gptaq_set_clip_search(st.handle, clip, 0.3)
+        G = hp.n_groups(n, group)
+
+        def quantize(W, in_place):
+            out = [torch.empty((m, w), dtype=d, device="cuda") for w, d in ((n, torch.uint8), (G, torch.float32), (G, torch.float32))]
+            Wq = None if in_place else torch.empty((m, n), device="cuda")
+            g.gptaq_quantize(st.handle, W, 4, group, False, B, *out, Wq)
+            assert g.gptaq_sync_status(st.handle)[0] == g.GPTAQ_OK
+            return out + [W if in_place else Wq]
+        view = wide[:, 1:n + 1]
+        want = quantize(view.float().contiguous(), True)
+        floats = wide.float()
+        for W in (view, view.contiguous(), floats[:, 1:n + 1], view.float().contiguous()):
+            before = W.clone()
+            got = quantize(W, False)
+            assert [int((x != y).sum()) for x, y in zip(got, want)] == [0, 0, 0, 0]
+            assert torch.equal(W, before)
+    finally:
+        st.close()
+
+
 @pytest.mark.parametrize("n,tokens,act_order", [
     (128, 2048, False), (128, 2049, False),     # float32 products up to here / one tile of either sum, cut
     (640, 520, False), (640, 520, True),        # a few tiles, of dXX^T the upper ones or all
