@@ -1206,7 +1206,8 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         // A[0:b0, 0:b0] -= R[0:b0, blk] R[0:b0, blk]^T  (upper part)
         Operand rp = make_operand(H + b0, n, 1);
         GemmProblem ps = make_problem(rp, rp, H, n, b0, b0, std::min(NB, n - b0), -1.f, 1.f, GEMM_UPPER_TILES);
-        return gemm(h, ps, false, false, us);
+        // (early where it has a CTA per SM at most: gptaq_factor 384 120 -> 116, 777 293 -> 286, 1027 434 -> 428 us)
+        return gemm(h, ps, false, false, us, h->num_sms);
     };
     auto factor_diag = [&](int p, const float *src, int64_t lds, int syrk, int pan_col0) -> gptaq_status_t {
         DiagFactorArgs da = {};
