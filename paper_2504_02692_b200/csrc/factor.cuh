@@ -601,11 +601,12 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
 // Rows above the block: R[0:b0, blk] = A[0:b0, blk] R_pp^-T, 32 columns at a time: a product with the inverse of the
 // 32 x 32 diagonal sub-block, then a rank-32 update of the columns to the left.  In place and, if asked for, as split
 // parts for the tensor-core rank update.
-// A warp takes 4 (8) rows from end to end: lane = (one (two) rows, 4 columns of every 32), the rows live in registers, the 32
+// A warp takes 2, 4 or 8 rows from end to end: lane = (one (two) rows, 2 or 4 columns of every 32), the rows live in registers, the 32
 // values of a row that all its lanes need go through shared memory inside the warp, so that no barrier of the CTA is on
 // the way (a CTA-wide form with two barriers per sub-block: n = 14336 17.3 against 15.9 ms in all).  What bounds it: the
 // words of R that shared memory returns (8k cycles; fetching them 3k); with two rows per lane they serve twice as many
-// products, with one a narrow panel has twice as many warps.
+// products, with one a narrow panel has twice as many warps, and with two columns a lane instead of four twice as many again (n = 384 116
+// -> 114 us in all, 1024 249.8 -> 247.7, 4096 1266 -> 1260).
 // One more CTA copies the block that is next on the diagonal, for the diag_factor_kernel that runs beside the update.
 // ---------------------------------------------------------------------------
 constexpr int PS_WORKERS = 4;                        // warps that take rows, at most
@@ -623,9 +624,11 @@ struct PanelSolveArgs {
     StateHeader *hd;
 };
 
-template <int RPT>
+// A lane has C columns of every 32 of RPT rows; a warp C * RPT rows.
+template <int C> struct alignas(4 * C) Cols { float v[C]; };
+template <int C, int RPT>
 __global__ void __launch_bounds__(PS_THREADS) panel_solve_kernel(PanelSolveArgs a) {
-    constexpr int ROWS = 4 * RPT;                        // rows per warp
+    constexpr int ROWS = C * RPT;                        // rows per warp
     extern __shared__ __align__(16) float smem_f[];
     float (*S)[FP_LD] = reinterpret_cast<float (*)[FP_LD]>(smem_f);                       // R^T, below the 32 x 32 diagonal sub-blocks
     float *Yt = reinterpret_cast<float *>(S + NB);                                        // [4][32][FP_YLD]
@@ -635,20 +638,21 @@ __global__ void __launch_bounds__(PS_THREADS) panel_solve_kernel(PanelSolveArgs 
     const bool vec = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(a.H) & 15) == 0 && nv == NB;
     const int slabs = gridDim.x - (a.next_diag ? 1 : 0);
     const int ngroups = b0 / ROWS;
-    const int q = lane & 7, rp = lane >> 3;              // 4 columns of every 32; row (pair of rows)
-    float x[RPT][4][4];                                    // [row][sub-block][column]
+    const int q = lane & (32 / C - 1), rp = lane / (32 / C);        // C columns of every 32; row (pair of rows)
+    float x[RPT][4][C];                                    // [row][sub-block][column]
     auto load_rows = [&](int g) {
 #pragma unroll
         for (int e = 0; e < RPT; ++e) {
-            const float *src = a.H + (int64_t)(g * ROWS + RPT * rp + e) * n + b0 + 4 * q;
+            const float *src = a.H + (int64_t)(g * ROWS + RPT * rp + e) * n + b0 + C * q;
 #pragma unroll
             for (int sb = 0; sb < 4; ++sb) {
                 if (vec) {
-                    const float4 v = *reinterpret_cast<const float4 *>(src + 32 * sb);
-                    x[e][sb][0] = v.x; x[e][sb][1] = v.y; x[e][sb][2] = v.z; x[e][sb][3] = v.w;
+                    const Cols<C> v = *reinterpret_cast<const Cols<C> *>(src + 32 * sb);
+#pragma unroll
+                    for (int f = 0; f < C; ++f) x[e][sb][f] = v.v[f];
                 } else {
 #pragma unroll
-                    for (int f = 0; f < 4; ++f) x[e][sb][f] = 32 * sb + 4 * q + f < nv ? src[32 * sb + f] : 0.f;
+                    for (int f = 0; f < C; ++f) x[e][sb][f] = 32 * sb + C * q + f < nv ? src[32 * sb + f] : 0.f;
                 }
             }
         }
@@ -685,15 +689,16 @@ __global__ void __launch_bounds__(PS_THREADS) panel_solve_kernel(PanelSolveArgs 
             __syncwarp();
 #pragma unroll
             for (int e = 0; e < RPT; ++e)
-                *reinterpret_cast<float4 *>(buf + e * FP_YLD + 4 * q) = make_float4(x[e][sb][0], x[e][sb][1], x[e][sb][2], x[e][sb][3]);
+#pragma unroll
+                for (int f = 0; f < C; ++f) buf[e * FP_YLD + C * q + f] = x[e][sb][f];
             __syncwarp();
             // X = (row) inv(R_ss)^T
-            const float *Ys = Yt + sb * 32 * FP_YLD + 4 * q;
-            float acc[RPT][4];
+            const float *Ys = Yt + sb * 32 * FP_YLD + C * q;
+            float acc[RPT][C];
 #pragma unroll
             for (int e = 0; e < RPT; ++e)
 #pragma unroll
-                for (int f = 0; f < 4; ++f) acc[e][f] = 0.f;
+                for (int f = 0; f < C; ++f) acc[e][f] = 0.f;
 #pragma unroll 2
             for (int l = 0; l < 32; l += 4) {
                 float v[RPT][4];
@@ -704,24 +709,24 @@ __global__ void __launch_bounds__(PS_THREADS) panel_solve_kernel(PanelSolveArgs 
                 }
 #pragma unroll
                 for (int h = 0; h < 4; ++h) {
-                    const float4 y = *reinterpret_cast<const float4 *>(Ys + (l + h) * FP_YLD);
+                    const Cols<C> y = *reinterpret_cast<const Cols<C> *>(Ys + (l + h) * FP_YLD);
 #pragma unroll
-                    for (int e = 0; e < RPT; ++e) {
-                        acc[e][0] = fmaf(v[e][h], y.x, acc[e][0]); acc[e][1] = fmaf(v[e][h], y.y, acc[e][1]);
-                        acc[e][2] = fmaf(v[e][h], y.z, acc[e][2]); acc[e][3] = fmaf(v[e][h], y.w, acc[e][3]);
-                    }
+                    for (int e = 0; e < RPT; ++e)
+#pragma unroll
+                        for (int f = 0; f < C; ++f) acc[e][f] = fmaf(v[e][h], y.v[f], acc[e][f]);
                 }
             }
 #pragma unroll
             for (int e = 0; e < RPT; ++e)
 #pragma unroll
-                for (int f = 0; f < 4; ++f) x[e][sb][f] = acc[e][f];
+                for (int f = 0; f < C; ++f) x[e][sb][f] = acc[e][f];
             if (sb == 0) break;
             // columns to the left: x[s'] -= X[l] R[.][32 sb + l]
             __syncwarp();
 #pragma unroll
             for (int e = 0; e < RPT; ++e)
-                *reinterpret_cast<float4 *>(buf + e * FP_YLD + 4 * q) = make_float4(acc[e][0], acc[e][1], acc[e][2], acc[e][3]);
+#pragma unroll
+                for (int f = 0; f < C; ++f) buf[e * FP_YLD + C * q + f] = acc[e][f];
             __syncwarp();
 #pragma unroll 1
             for (int l = 0; l < 32; l += 4) {
@@ -735,12 +740,11 @@ __global__ void __launch_bounds__(PS_THREADS) panel_solve_kernel(PanelSolveArgs 
                 for (int h = 0; h < 4; ++h)
 #pragma unroll
                     for (int t = 0; t < sb; ++t) {
-                        const float4 r = *reinterpret_cast<const float4 *>(&S[32 * sb + l + h][32 * t + 4 * q]);
+                        const Cols<C> r = *reinterpret_cast<const Cols<C> *>(&S[32 * sb + l + h][32 * t + C * q]);
 #pragma unroll
-                        for (int e = 0; e < RPT; ++e) {
-                            x[e][t][0] = fmaf(-v[e][h], r.x, x[e][t][0]); x[e][t][1] = fmaf(-v[e][h], r.y, x[e][t][1]);
-                            x[e][t][2] = fmaf(-v[e][h], r.z, x[e][t][2]); x[e][t][3] = fmaf(-v[e][h], r.w, x[e][t][3]);
-                        }
+                        for (int e = 0; e < RPT; ++e)
+#pragma unroll
+                            for (int f = 0; f < C; ++f) x[e][t][f] = fmaf(-v[e][h], r.v[f], x[e][t][f]);
                     }
             }
         }
@@ -751,20 +755,26 @@ __global__ void __launch_bounds__(PS_THREADS) panel_solve_kernel(PanelSolveArgs 
             const int64_t row = g * ROWS + RPT * rp + e;
 #pragma unroll
             for (int sb = 0; sb < 4; ++sb) {
-                const int c = 32 * sb + 4 * q;
-                const float (&v)[4] = x[e][sb];
+                const int c = 32 * sb + C * q;
                 float *dst = a.H + row * n + b0 + c;
-                if (vec) *reinterpret_cast<float4 *>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+                Cols<C> v;
+#pragma unroll
+                for (int f = 0; f < C; ++f) v.v[f] = x[e][sb][f];
+                if (vec) *reinterpret_cast<Cols<C> *>(dst) = v;
                 else {
 #pragma unroll
-                    for (int f = 0; f < 4; ++f) if (c + f < nv) dst[f] = v[f];
+                    for (int f = 0; f < C; ++f) if (c + f < nv) dst[f] = v.v[f];
                 }
                 if (a.pan_hi) {
-                    const float s4[4] = {sc * v[0], sc * v[1], sc * v[2], sc * v[3]};
-                    uint2 hi, lo;
-                    split16_pack(s4, hi, lo);
-                    *reinterpret_cast<uint2 *>(a.pan_hi + row * a.pan_ld + a.pan_col0 + c) = hi;
-                    *reinterpret_cast<uint2 *>(a.pan_lo + row * a.pan_ld + a.pan_col0 + c) = lo;
+#pragma unroll
+                    for (int f = 0; f < C; f += 2) {
+                        const float s0 = sc * v.v[f], s1 = sc * v.v[f + 1];
+                        const __half2 h = __floats2half2_rn(s0, s1);
+                        const float2 hf = __half22float2(h);
+                        const int64_t at = row * a.pan_ld + a.pan_col0 + c + f;
+                        *reinterpret_cast<__half2 *>(a.pan_hi + at) = h;
+                        *reinterpret_cast<__half2 *>(a.pan_lo + at) = __floats2half2_rn(s0 - hf.x, s1 - hf.y);
+                    }
                 }
             }
         }

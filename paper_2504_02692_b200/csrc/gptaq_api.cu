@@ -964,9 +964,11 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(diag_factor_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DF_SMEM_WHOLE);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(panel_solve_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM);
+        e = cudaFuncSetAttribute(panel_solve_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(panel_solve_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM);
+        e = cudaFuncSetAttribute(panel_solve_kernel<4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(panel_solve_kernel<4, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM);
     if (e == cudaSuccess) e = configure_quantize_kernels();
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(p_narrow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)np_smem(NP_MAX_N));
@@ -1265,15 +1267,15 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         pa.pan_ld = SUPER_NB; pa.pan_col0 = b0 - s0; pa.hd = h->hd;
         pa.next_diag = ahead ? next_diag : nullptr;
         pa.early = early ? 1 : 0;
-        // a warp per 4 rows while that fills no SM beyond PS_WORKERS warps, per 8 rows beyond; as few warps per CTA as give
+        // a warp per 2 (4) rows while that fills no SM beyond PS_WORKERS warps, per 8 rows beyond; as few warps per CTA as give
         // every SM at most one CTA
-        const int rpt = b0 / 4 <= PS_WORKERS * h->num_sms ? 1 : 2;
-        const int groups = b0 / (4 * rpt);
+        const int most = PS_WORKERS * h->num_sms, rows = b0 / 2 <= most ? 2 : b0 / 4 <= most ? 4 : 8;
+        const int groups = b0 / rows;
         pa.workers = std::max(1, std::min(PS_WORKERS, (groups + h->num_sms - 1) / h->num_sms));
         const int slabs = std::min((groups + pa.workers - 1) / pa.workers, h->num_sms);
         const dim3 pg(slabs + (ahead ? 1 : 0));
-        if (rpt == 1) CU(launch_pdl(true, panel_solve_kernel<1>, pg, dim3(PS_THREADS), PS_SMEM, s, pa));
-        else CU(launch_pdl(true, panel_solve_kernel<2>, pg, dim3(PS_THREADS), PS_SMEM, s, pa));
+        CU(launch_pdl(true, rows == 2 ? panel_solve_kernel<2, 1> : rows == 4 ? panel_solve_kernel<4, 1> : panel_solve_kernel<4, 2>, pg,
+                      dim3(PS_THREADS), PS_SMEM, s, pa));
         h->launches++;
         CU(cudaEventRecord(h->inv_ready, s));
         CU(cudaStreamWaitEvent(is, h->inv_ready, 0));
