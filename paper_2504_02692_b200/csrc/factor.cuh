@@ -160,7 +160,8 @@ __device__ __forceinline__ int diag_inverse_at(int c, int l) { return ((c == 3 ?
 // 32 x 32 diagonal sub-blocks come inverted from diag_factor_kernel; X12 = -X11 (R12 X22) for 32 -> 64 -> 128.  Bound by
 // shared-memory reads: 4 x 4 outputs per thread.  A second CTA of the next block's diag_factor_kernel, which takes twice as long
 // (as a CTA of panel_solve_kernel it held that up: a panel's rows 7 -> 11 us; as a kernel of its own behind the update, which
-// inverted the sub-blocks itself, it took 11 us a panel and one stream operation more); block 0 has a launch of its own.
+// inverted the sub-blocks itself, it took 11 us a panel and one stream operation more).  Block 1 has a launch of its own, beside block 0,
+// which inverts itself.
 // ---------------------------------------------------------------------------
 constexpr int ID_THREADS = 256, ID_BAR = 15;
 constexpr int ID_LD = FP_LD;
@@ -266,7 +267,6 @@ __device__ __forceinline__ void invert_diag_block(float *smem_f, float *H, int n
 
 __global__ void __launch_bounds__(ID_THREADS, 1) invert_diag_block_kernel(float *H, int n, int b0, const float *Rdiag) {
     extern __shared__ __align__(16) float smem_f[];
-    pdl_wait();
     invert_diag_block(smem_f, H, n, b0, Rdiag);
 }
 
@@ -288,6 +288,8 @@ constexpr int DF_HELP = 8 * 32, DF_MAIN = 128 + DF_HELP, DF_THREADS = DF_MAIN + 
 constexpr int DF_TILE_BYTES = NB * 64 * 2;           // 128 rows x 64 fp16
 constexpr size_t DF_SMEM_BLOCK = 4 * DF_TILE_BYTES + (size_t)(NB * FP_LD + NB + 64 + 32) * sizeof(float) + 32 + 1024;
 constexpr size_t DF_SMEM = DF_SMEM_BLOCK > ID_SMEM ? DF_SMEM_BLOCK : ID_SMEM;
+constexpr size_t DF_SMEM_LAST = 4 * DF_TILE_BYTES + ID_SMEM + (NB + 64 + 32) * sizeof(float) + 32 + 1024;
+static_assert(DF_SMEM_LAST <= 227 * 1024, "shared memory of one SM");
 constexpr size_t DF_SMEM_WHOLE = ID_SMEM + (NB + 64 + 32) * sizeof(float) + 32 + 1024;
 constexpr uint32_t DF_IDESC = (1u << 4) | ((NB >> 3) << 17) | ((NB >> 4) << 24);     // kind::f16, M = N = 128
 // Named barriers.  COLS + q: eight columns (q = 0: the rightmost) of a sub-block are factored (its leader arrives; the warps above
@@ -305,25 +307,28 @@ struct DiagFactorArgs {
     int syrk, pan_col0;                  // 1: subtract rows b0 .. of the panel at columns pan_col0 .. of the split copy times
                                          //    their transpose first (scale of the copy: tc_amax[AMAX_PAN])
     StateHeader *hd;
-    // WHOLE: the layer has one block, src is its sum H as it was accumulated
+    // DF_WHOLE: the layer has one block, src is its sum H as it was accumulated
     float inv_tokens, damp;
     uint8_t *dead, *dead_working;
 };
 
-// WHOLE (n <= NB): what diag_stats_kernel, scale_damp_kernel and invert_diag_block_kernel do for a wider layer happens here too, with the
-// same arithmetic: gptaq_factor at n = 128 36.6 us as four launches, 31.4 so, n = 100 39.2 and 31.7 (U bit-identical; with R_pp through
+// DF_LAST (block 0): the block's inverse follows at once, from the factor as it lies in shared memory (as a kernel of its own it
+// followed 2 us later and loaded it first).  DF_WHOLE (n <= NB): what diag_stats_kernel and scale_damp_kernel do for a wider layer happens here, too, with the same
+// arithmetic: gptaq_factor at n = 128 36.6 us as four launches, 31.4 so, n = 100 39.2 and 31.7 (U bit-identical; with R_pp through
 // global memory as between the launches 37.7 and 35.8).
-template <bool WHOLE>
+enum { DF_BLOCK = 0, DF_LAST = 1, DF_WHOLE = 2 };
+template <int MODE>
 __global__ void __launch_bounds__(DF_THREADS, 1)
 diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_constant__ CUtensorMap mapLo, DiagFactorArgs a) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *sm = smem_raw + (base - raw);
-    // (WHOLE: the inverse's other operands behind it)
+    constexpr bool WHOLE = MODE == DF_WHOLE, INVERT = MODE != DF_BLOCK;
+    // (the inverse's other operands behind it)
     float (*S)[FP_LD] = reinterpret_cast<float (*)[FP_LD]>(sm + (WHOLE ? 0 : 4 * DF_TILE_BYTES));
     float *X = reinterpret_cast<float *>(S + NB), *T = X + NB * ID_LD;
-    float *dinv = WHOLE ? T + 64 * 68 : reinterpret_cast<float *>(S + NB);
+    float *dinv = INVERT ? T + 64 * 68 : reinterpret_cast<float *>(S + NB);
     float *gs = dinv + NB;                           // 8 x 8: the diagonal block of the columns at hand
     float *rdiag = gs + 64;                          // 1 / R_kk of the sub-block that is being inverted
     uint8_t *tailp = reinterpret_cast<uint8_t *>(rdiag + 32);
@@ -352,6 +357,9 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (INVERT)
+        for (int idx = tid; idx < NB * NB; idx += DF_THREADS)
+            if ((idx >> 12) != ((idx & 127) >> 5)) X[(idx >> 7) * ID_LD + (idx & 127)] = 0.f;
     pdl_wait();
     if constexpr (WHOLE) {
         double *sum = reinterpret_cast<double *>(T);
@@ -372,7 +380,6 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
             for (int e = 0; e < BATCH; ++e) {
                 const int idx = tid + (r * BATCH + e) * DF_THREADS, i = idx >> 7, j = idx & 127;
                 if (i < NB && (i != j || i >= nv)) S[i][j] = i == j ? 1.f : v[e] * a.inv_tokens;
-                if (i < NB && (i >> 5) != (j >> 5)) X[i * ID_LD + j] = 0.f;
             }
         }
         if (tid < NB) {
@@ -537,7 +544,7 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
         auto store_rows = [&](int sb) {
             for (int idx = t; idx < 32 * (NB / 4); idx += DF_HELP) {
                 const int i = 32 * sb + (idx >> 5), j4 = idx & 31;
-                if (!WHOLE && j4 < 8 * (sb + 1)) *reinterpret_cast<float4 *>(a.Rdiag + i * NB + 4 * j4) = *reinterpret_cast<const float4 *>(&S[i][4 * j4]);
+                if (!INVERT && j4 < 8 * (sb + 1)) *reinterpret_cast<float4 *>(a.Rdiag + i * NB + 4 * j4) = *reinterpret_cast<const float4 *>(&S[i][4 * j4]);
             }
         };
 #pragma unroll 1
@@ -582,19 +589,19 @@ diag_factor_kernel(const __grid_constant__ CUtensorMap mapHi, const __grid_const
             float y[32];
 #pragma unroll
             for (int k = 0; k < 32; ++k) y[k] = (k == lane) ? 1.f : 0.f;
-            float *dst = WHOLE ? X + o * ID_LD + o + lane : a.Rdiag + diag_inverse_at(sb, lane);
+            float *dst = INVERT ? X + o * ID_LD + o + lane : a.Rdiag + diag_inverse_at(sb, lane);
             solve32(y, &S[o][o], rdiag,
                     [&](int k) {
                         named_bar_sync(DBAR_COLS + (31 - k) / 8, 32 * (sb + 2));
                         if (lane < 8) rdiag[k - lane] = 1.f / S[o + k - lane][o + k - lane];
                         __syncwarp();
                     },
-                    [&](int k, float v) { dst[WHOLE ? k * ID_LD : k] = !WHOLE || k <= lane ? v : 0.f; });
+                    [&](int k, float v) { dst[INVERT ? k * ID_LD : k] = !INVERT || k <= lane ? v : 0.f; });
         }
     }
     __syncthreads();
     if (*abort_flag && tid == 0) record_status(a.hd, ST_TIMEOUT, 4000000 + a.b0);
-    if (WHOLE && tid < ID_THREADS) invert_products(&S[0][0], X, T, a.H, a.n, 0);
+    if (INVERT && tid < ID_THREADS) invert_products(&S[0][0], X, T, a.H, a.n, a.b0);
 }
 
 // ---------------------------------------------------------------------------

@@ -960,9 +960,13 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
     cudaError_t e = cudaGetDevice(&h->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(diag_factor_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DF_SMEM);
+        e = cudaFuncSetAttribute(invert_diag_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ID_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(diag_factor_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DF_SMEM_WHOLE);
+        e = cudaFuncSetAttribute(diag_factor_kernel<DF_LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DF_SMEM_LAST);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(diag_factor_kernel<DF_BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DF_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(diag_factor_kernel<DF_WHOLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DF_SMEM_WHOLE);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(panel_solve_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM);
     if (e == cudaSuccess)
@@ -972,8 +976,6 @@ gptaq_status_t gptaq_create(gptaq_handle_t *out, int64_t n, void *d_state, size_
     if (e == cudaSuccess) e = configure_quantize_kernels();
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(p_narrow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)np_smem(NP_MAX_N));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(invert_diag_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ID_SMEM);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(stats_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UMMA_SMEM);
     if (e == cudaSuccess)
@@ -1142,7 +1144,7 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         da.inv_tokens = inv_tokens; da.damp = damp; da.dead = h->dead_raw; da.dead_working = h->dead;
         CUtensorMap none;
         std::memset(&none, 0, sizeof(none));
-        CU(launch_pdl(false, diag_factor_kernel<true>, dim3(1), dim3(DF_THREADS), DF_SMEM_WHOLE, s, none, none, da));
+        CU(launch_pdl(false, diag_factor_kernel<DF_WHOLE>, dim3(1), dim3(DF_THREADS), DF_SMEM_WHOLE, s, none, none, da));
         h->launches++;
         h->split = false;
         h->stage = STAGE_FACTORED;
@@ -1215,9 +1217,10 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         DiagFactorArgs da = {};
         da.src = src; da.lds = lds; da.n = n; da.b0 = p * NB; da.Rdiag = Rinv + (size_t)p * NB * NB;
         da.syrk = syrk; da.pan_col0 = pan_col0; da.hd = h->hd;
-        // (a second CTA inverts the block before)
+        // (a second CTA inverts the block before; block 0 has its own inverse to make, block 1 is inverted beside it)
         da.H = H; da.inv_b0 = (p + 1) * NB; da.inv_Rdiag = da.Rdiag + NB * NB;
-        CU(launch_pdl(true, diag_factor_kernel<false>, dim3(p + 1 < nb ? 2 : 1), dim3(DF_THREADS), DF_SMEM, s, pan_maps.a_hi, pan_maps.a_lo, da));
+        CU(launch_pdl(true, p ? diag_factor_kernel<DF_BLOCK> : diag_factor_kernel<DF_LAST>, dim3(p > 0 && p + 1 < nb ? 2 : 1), dim3(DF_THREADS),
+                      p ? DF_SMEM : DF_SMEM_LAST, s, pan_maps.a_hi, pan_maps.a_lo, da));
         h->launches++;
         return GPTAQ_OK;
     };
@@ -1281,11 +1284,14 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
         CU(cudaStreamWaitEvent(is, h->inv_ready, 0));
         if (ahead) {
             // the update on the internal stream, the next diagonal block (and this one's inverse) beside it on two SMs left free
-            CU(cudaStreamWaitEvent(h->gemm_stream, h->inv_ready, 0));
-            OK(update(p, h->gemm_stream, h->num_sms - 2));
-            CU(cudaEventRecord(h->gemm_done[0], h->gemm_stream));
+            // (p = 1: block 0 is all that the update would reach)
+            if (p > 1) {
+                CU(cudaStreamWaitEvent(h->gemm_stream, h->inv_ready, 0));
+                OK(update(p, h->gemm_stream, h->num_sms - 2));
+                CU(cudaEventRecord(h->gemm_done[0], h->gemm_stream));
+            }
             OK(factor_diag(p - 1, next_diag, NB, 1, b0 - s0));
-            CU(cudaStreamWaitEvent(s, h->gemm_done[0], 0));
+            if (p > 1) CU(cudaStreamWaitEvent(s, h->gemm_done[0], 0));
             diag_done = true;
         } else OK(update(p, s, h->num_sms));
         // (block p + 1 was inverted beside block p)
@@ -1293,15 +1299,19 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
             OK(inverse_row(p + 1));
             OK(inverse_gather(p + 1));
         }
+        if (p == 1) {
+            // Row 1 of the inverse need not wait for block 0: block 1 is inverted beside it by a kernel of its own, and block 0 by its own
+            // diagonal kernel (gptaq_factor, us: both behind block 0 n = 384 114, 500 154, 640 162, 777 284, 2048 549; so 108, 147, 156,
+            // 277, 545).
+            CU(cudaStreamWaitEvent(h->gemm_stream, h->inv_ready, 0));
+            invert_diag_block_kernel<<<1, ID_THREADS, ID_SMEM, h->gemm_stream>>>(H, n, NB, Rinv + NB * NB);
+            LAUNCHED();
+            CU(cudaEventRecord(h->conv_done[0], h->gemm_stream));
+            CU(cudaStreamWaitEvent(is, h->conv_done[0], 0));
+            OK(inverse_row(1));
+            OK(inverse_gather(1));
+        }
     }
-    if (nb > 1) {
-        CU(cudaEventRecord(h->inv_ready, s));
-        CU(cudaStreamWaitEvent(is, h->inv_ready, 0));
-        OK(inverse_row(1));
-        OK(inverse_gather(1));
-    }
-    CU(launch_pdl(true, invert_diag_block_kernel, dim3(1), dim3(ID_THREADS), ID_SMEM, s, H, n, 0, static_cast<const float *>(Rinv)));
-    h->launches++;
     if (nb > 1) {
         CU(cudaEventRecord(h->inv_done, is));
         CU(cudaStreamWaitEvent(s, h->inv_done, 0));
