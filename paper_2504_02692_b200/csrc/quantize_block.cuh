@@ -77,6 +77,7 @@ struct QuantBlockArgs {
     int clip_steps; float clip_min;
 };
 
+static_assert(64 * qb_sld(QB_ROWS_FEW) >= 24 * qb_sld(QB_ROWS_FEW) + 8 * QB_ROWS_FEW + 2 * QB_NEAR, "scratch of the clipping search");
 // Shared memory, in bytes from a 1024-byte boundary.  The tensor-core operands come first (alignment).
 struct QuantBlockSmem {
     int a, e, w, up, st, grid, udinv, perm, inv, rmax, bars, total, wld;
@@ -170,6 +171,7 @@ __device__ __forceinline__ void clip_pass(const float *w, int n, float lo, float
         sc2[h] = pack2(sc[0], sc[1]); nz[h] = pack2(-(magic + z[0]), -(magic + z[1]));
         err[h] = 0ull;
     }
+#pragma unroll 1
     for (int c = 0; c < n; c += 4) {
         const float4 v = *reinterpret_cast<const float4 *>(w + c);
         const float x[4] = {v.x, v.y, v.z, v.w};
@@ -196,7 +198,9 @@ __device__ __forceinline__ void clip_pass(const float *w, int n, float lo, float
 
 // Least squared rounding error of one row's group among candidates k0, k0 + stride, ..: ten per pass over the weights while
 // more than four are left, else four (four throughout and clamped by minimum and maximum, 4096 x 4096 with 80 candidates:
-// 1541 us a call, now 1419).
+// 1541 us a call, then 1419).  What bounds it is the number of its instructions, two cycles each on a scheduler whatever their pipe: an
+// integer minimum in place of the two saturating FMAs of a pair, on codes rounded as subnormal numbers, took as long.  Four
+// columns a round: unrolled further the registers ran out (4096 x 1024 251 us, now 242 with the range from the chain's own).
 __device__ __forceinline__ void clip_search(const float *w, int n, float lo, float hi, int bits, int sym, int steps, float clip_min,
                                             int k0, int stride, float &best, int &kbest) {
     best = INFINITY; kbest = 0;
@@ -255,6 +259,8 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
     // copies by all near warps a step's 32 KB took 1100 cycles of their time, in steps where the chain waits for them (4096 x 1024 with
     // groups 165 -> 161 us a call, 1024 x 1024 with static groups 163 -> 160).  Rows that are no multiple of 16 bytes come in asynchronous
     // copies of 4 (word by word through registers before: 777 x 777 217 -> 191, 4096 x 777 501 -> 486).
+    // a step's error buffer, before its first column is quantized: the four quarters of the group's ranges
+    auto range_at = [&](float *st) { return reinterpret_cast<float2 *>(st + 24 * SLD); };
     auto up_at = [&](int s, int q, int k, int c) {
         return UPs + ((s & 1) ? 2 * QB_BOXES0 * QB_BOX : 0) + (q * ((s & 1) ? QB_BOXES1 : QB_BOXES0) + (c >> 5)) * QB_BOX + k * 32 + (c & 31);
     };
@@ -447,7 +453,7 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                         hi = fmaxf(hi, fmaxf(fmaxf(v[c].x, v[c].y), fmaxf(v[c].z, v[c].w)));
                     }
                     // (through the part of the step's error buffer that warp 3 publishes into, after all have read it)
-                    float2 *range_s = reinterpret_cast<float2 *>(St + 24 * SLD);
+                    float2 *range_s = range_at(St);
                     range_s[warp * ROWS + lrow] = make_float2(lo, hi);
                     named_bar_sync(QBAR_CHAIN, QB_CHAIN);
 #pragma unroll
@@ -597,14 +603,14 @@ quant_block_kernel(const __grid_constant__ CUtensorMap mapUhi, const __grid_cons
                     const float *w = Ws + r * WLD + co;
                     float lo = 0.f, hi = 0.f, best;
                     int kb;
-                    for (int c = 0; c < a.group; c += 4) {          // (columns beyond the layer are zeros)
-                        const float4 v = *reinterpret_cast<const float4 *>(w + c);
-                        lo = fminf(lo, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
-                        hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                    float *scratch = Sts + (s & 1) * 64 * SLD;      // (the chain writes there only after this search)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {                   // the range, a quarter from each chain warp
+                        const float2 v = range_at(scratch)[q * ROWS + r];
+                        lo = fminf(lo, v.x); hi = fmaxf(hi, v.y);
                     }
                     clip_search(w, a.group, lo, hi, a.bits, a.sym, a.clip_steps, a.clip_min, cgi, QB_NEAR / ROWS, best, kb);
-                    float *scratch = Sts + (s & 1) * 64 * SLD;   // (the chain writes there only after this search)
-                    float *be = scratch + 64;
+                    float *be = scratch + 24 * SLD + 8 * ROWS;      // (behind the ranges, which other warps still read)
                     int *bk = reinterpret_cast<int *>(be + QB_NEAR);
                     be[t] = best; bk[t] = kb;
                     named_bar_sync(QBAR_NEAR, QB_NEAR);
