@@ -245,8 +245,8 @@ bool make_tc_maps(TcMaps *m, const SplitOperand &A, const SplitOperand &B, const
 
 // Launch with programmatic stream serialization where `pdl` is set: the kernel may be scheduled while its predecessor
 // drains; it calls pdl_wait() before it touches anything the predecessor wrote.
-// So start: the factorisation's chain (4 % of it at n = 4096; the damping up to 3 us up to n = 2052, the inverse of block 0
-// 3 us up to n = 128) and the tensor-core products of gptaq_factor and gptaq_build_P; the second pass of the statistics'
+// So start: the factorisation's chain (4 % of it at n = 4096; the damping up to 3 us up to n = 2052), the tensor-core products of
+// gptaq_factor and gptaq_build_P and the correction matrix of narrow layers; the second pass of the statistics'
 // conversion (2 to 4 us a call; back to back 4 calls of 4112 tokens at n = 1024 141 -> 135, of 2777 at n = 2052 392 -> 396);
 // split copies and small float32 products of few CTAs (launch_split16, launch_simt_gemm); the column loop without tensor cores
 // from its second launch on (launch_quant_block).  All else is launched plainly: the column loop on the tensor cores and its
@@ -614,10 +614,9 @@ cudaError_t launch_quant_block(const QuantizeTarget &t, float *W, int64_t ldw, c
     const dim3 grid((unsigned)((r1 - r0 + rows - 1) / rows));
     const size_t smem = quant_block_smem_bytes(far_form, static_groups, rows);
     // Near form, more CTAs than SMs: two to an SM, one works while the other waits for its own chain, although each has 80
-    // registers then and spills some (16384 rows of 400 columns 413 us, with one 435; 8192 of 1023 1092, 1110; static groups 460, 475
-    // and 1133, 1182; with a grid every 32 columns 4768 rows of 500 columns 242, 237, 16384 of 1023 1911, 1954); below that
-    // one, which has the registers of both (1023 columns: 1024 rows 299, two 351; 4736
-    // rows 629, 658).
+    // registers then and spills some (16384 rows of 400 columns 375 us, with one 390; 8192 of 1023 899, 907; static groups 416, 435
+    // and 939, 972; with a grid every 32 columns 4768 rows of 500 columns 204, 213, 16384 of 1023 1740, 1770); below that
+    // one, which has the registers of both (1023 columns: 2048 rows 355, two 408; 4736 rows 535, 584).
     const bool two = grid.x > (unsigned)t.num_sms;
     // Near form, from the second launch of a call on: it starts while the product before it drains, and reads U and P meanwhile
     // (1000 rows of 1024 columns 256 -> 242 us a call).  That takes two things: the first launch of a call is a plain one, so that
@@ -1303,11 +1302,15 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
             // Row 1 of the inverse need not wait for block 0: block 1 is inverted beside it by a kernel of its own, and block 0 by its own
             // diagonal kernel (gptaq_factor, us: both behind block 0 n = 384 114, 500 154, 640 162, 777 284, 2048 549; so 108, 147, 156,
             // 277, 545).
-            CU(cudaStreamWaitEvent(h->gemm_stream, h->inv_ready, 0));
-            invert_diag_block_kernel<<<1, ID_THREADS, ID_SMEM, h->gemm_stream>>>(H, n, NB, Rinv + NB * NB);
+            // (on the rows' own stream where no row is under way there, one event less)
+            cudaStream_t bs = nb > 2 ? h->gemm_stream : is;
+            if (bs != is) CU(cudaStreamWaitEvent(bs, h->inv_ready, 0));
+            invert_diag_block_kernel<<<1, ID_THREADS, ID_SMEM, bs>>>(H, n, NB, Rinv + NB * NB);
             LAUNCHED();
-            CU(cudaEventRecord(h->conv_done[0], h->gemm_stream));
-            CU(cudaStreamWaitEvent(is, h->conv_done[0], 0));
+            if (bs != is) {
+                CU(cudaEventRecord(h->conv_done[0], bs));
+                CU(cudaStreamWaitEvent(is, h->conv_done[0], 0));
+            }
             OK(inverse_row(1));
             OK(inverse_gather(1));
         }
