@@ -8,12 +8,13 @@
 // (128 dependent pivots).  Where the next block belongs to the same super-panel its diagonal kernel does not wait for the
 // update: it takes a copy of the block from before the update and subtracts this panel's contribution itself (one
 // 128 x 128 x 128 product on the tensor cores), so that the update runs beside it on another stream.
-// A panel of a 1024-wide layer is 28 us of the chain, from one diagonal kernel's start to the next one's: the diagonal block 19, the
-// rows above it 7, the launches between.  Its inverse is made beside the next block and the rows of U are gathered as they come; with
-// the inverse as a kernel of its own behind the update (11 us on one SM) and one pivot at a time a panel was 33 us, with
-// every CTA of one kernel factoring the diagonal block first and the update on the chain 45.  Factorisation and inversion in that
-// last form took 404 us at n = 1024, 1118 at 2052, 2036 at 4096; in the one before this and in this, both in turn: n = 1024 292 and
-// 248 us, 2052 731 and 659, 4096 1396 and 1265, 14336 12.5 and 11.5 ms.
+// A panel of a 1024-wide layer is 28 us of the chain, from one diagonal kernel's start to the next one's: the diagonal block 19 (14.5
+// of them the factorisation, 3 until the block is loaded and updated), the rows above it 7, the launches between.  Its inverse is made
+// beside the next block and the rows of U are gathered as they come, block 1's beside block 0, which inverts itself: behind the last
+// block only row 0 of U is left (n = 384 114 -> 108 us, 777 284 -> 277).  A layer of one block is a single launch (n = 128 36 -> 31).
+// The inverse as a kernel of its own behind the update (11 us on one SM) and one pivot at a time made a panel 33 us, every CTA of one
+// kernel factoring the diagonal block first and the update on the chain 45.  gptaq_factor, us, in that last form: n = 1024 404,
+// 2052 1118, 4096 2036; in the one between 292, 731, 1396; now 246, 653, 1255 to 1275.
 #pragma once
 #include "tc_gemm.cuh"
 

@@ -1171,8 +1171,8 @@ static gptaq_status_t factor_core(gptaq_ctx *h, float damp, cudaStream_t s) {
     // sqrt(max diag H_d), those of its inverse between 1 / sqrt of these, and as lambda = damp * mean(diag) the two are at most
     // sqrt(n / damp) apart (453 at n = 2052, damp = 0.01), while the parts keep their 22 bits down to 2^-17 of the largest entry.
     // Without damping nothing bounds them: plain float32 (units of the inputs that span 1e4, relative error of U at n = 2052
-    // 1.9e-6 with split rank updates, 2.2e-7 without; n = 1024 / 2052 / 4096 / 8192 0.29 -> 0.33, 1.26 -> 1.51, 2.37 -> 3.29,
-    // 8.5 -> 14.4 ms).
+    // 1.9e-6 with split rank updates, 2.2e-7 without; n = 1024 / 2052 / 4096 / 8192 split 0.29, 1.26, 2.37,
+    // 8.5 ms when that was last built, plain now 0.29, 0.95, 2.81, 14.1).
     const bool split = h->tensor && damp > 0.f;
     // reverse Cholesky H_d = R R^T, R upper, from the last block column upwards
     __half *pan_hi = split ? reinterpret_cast<__half *>(h->ws + wl.pan_off[0]) : nullptr;

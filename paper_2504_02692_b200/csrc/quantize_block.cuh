@@ -18,13 +18,14 @@
 // What bounds it: the chain, and the near warps behind it.  A column is 7 dependent float32 operations (28 cycles); with its
 // share of the updates, the codes and the hand-over to the next warp 8 columns take 750 cycles alone and 950 beside the near
 // warps, which need 830 for them (a scheduler starts a 16-byte LDS in 8 cycles where lanes share words, in 16 where they do
-// not).  A step of 32 columns ends some 2000 cycles after its last column (the near warps' last 8 columns, results, operands),
-// the products between two blocks take 5000.
-// A row in the four lanes of one warp (every column's errors through two shuffles to all of them, 64 words of U and P a column
-// for now 36): 8 columns 900 to 1600 cycles, but the end of a step 100 to 1000 and the products between blocks 2300, because the
-// chain's own warps made the operand; a launch of 512 columns 71 us with groups and 68 without, now 64 and 53.
-// The tensor-core form may have 96 registers and spills 60 bytes (static groups 52), the near form 80 where two CTAs share an SM
-// and spills 112 (140); with one to an SM it takes 160 and spills nothing.
+// not).  A step of 32 columns ends 1500 to 2000 cycles after its last column (the near warps' last 8 columns, results), the products
+// between two blocks take 4000 to 5000 (operand, streamed tiles, MMAs, adding them up).
+// A launch of 512 columns of 4096 rows by itself (ncu; the second and the first of two: the first also writes the
+// operand of the update beyond it) with a group grid per 128 columns and without: with 4-byte copies of U and P, the operand of a
+// block's end behind the next step's rows and hi and lo parts in turn 69.6 / 74.9 and 67.6 / 71.6 us, now 64.1 / 69.0 and 62.1 / 67.5;
+// of 512 rows, with 16 of them a CTA, 65.5 / 70.9 and 63.6 / 67.6, now 53.9 / 57.5 and 53.0 / 56.4.
+// Spills (32 rows; 16): the tensor-core form has 96 registers and spills 64 bytes (44), static groups 60 (56); the near form has 80
+// where two CTAs share an SM and spills 100 (static groups 132), with one to an SM up to 158 and spills nothing.
 #pragma once
 #include "simt_gemm.cuh"
 #include "tc_gemm.cuh"
